@@ -379,24 +379,27 @@ hp_status hp_reconstruct_device_noalloc(hp_ctx *ctx, uint32_t n_events, uint64_t
  * Autotuner.  The clustering kernel has launch parameters whose best values
  * depend on the launch shape (how many (event, module) items, how many
  * digis per item):
- *   tile_slots     capacity of the shared-memory tile of the block tier:
- *                  items with more digis are clustered in global scratch;
- *   blocks_per_sm  resident clustering blocks per SM, 1, 2 or 3 (1 allows
- *                  the largest tile; 3 caps the kernel at 40 registers a
- *                  thread and needs a smaller tile);
+ *   tile_slots     runs (horizontal stretches of surviving pixels) that a
+ *                  block's shared memory holds: items with more are
+ *                  clustered in global scratch;
+ *   blocks_per_sm  resident clustering blocks per SM, 1, 2 or 3: with 1 a
+ *                  block is four groups of threads that cluster items of
+ *                  their own (the largest items take the whole block and the
+ *                  largest tile), with 2 two groups, with 3 one;
  *   ticket_items   (event, module) items per work-queue ticket, 16, 8, 4
  *                  or 2 (halved for launches too small to fill the GPU: down
  *                  to 4 for items of under 64 digis on average, to 1 for
  *                  larger ones);
- *   warp_max       largest item (digis) clustered by a single warp, 32 or 64;
- *   label_store    how the items above the warp tier look up a pixel's
- *                  neighbours: HP_STORE_BITMAP,
- *                  module-sized occupancy and survivor bitmaps with
- *                  row-major slots, one block (512 threads) an item; or
- *                  HP_STORE_HASH, an open-addressing table keyed by linear
+ *   warp_max       32 or 64: items of up to eight times as many digis are
+ *                  clustered together, a ticket's worth at a time (with the
+ *                  hash store, items of up to warp_max digis);
+ *   label_store    how the items above these look up a pixel's neighbours:
+ *                  HP_STORE_BITMAP, module-sized bitmaps with the runs of a
+ *                  module in row-major order, one group of threads an item;
+ *                  or HP_STORE_HASH, an open-addressing table keyed by linear
  *                  pixel index with two slots a digi, so that its memory
  *                  follows the item's size, for items up to the hash
- *                  store's capacity (larger ones take the bitmap tiers);
+ *                  store's capacity (larger ones take the bitmaps);
  *   item_threads   threads clustering one item of the hash store, 128, 256
  *                  or 512 (a block runs 512 / item_threads items side by
  *                  side, each in its share of the block's shared memory;
@@ -408,9 +411,9 @@ hp_status hp_reconstruct_device_noalloc(hp_ctx *ctx, uint32_t n_events, uint64_t
  * (host, device, graph and serving paths).  A bucket without an entry takes
  * the entry of the nearest tuned bucket (distance |d items_log2| +
  * 4 |d digis_per_item_log2|, at most 8), else the defaults: 4096 slots, 2
- * blocks, 16 items, 64 digis, bitmap store, or, for a mean of 1024 digis
- * per item or more, the single-block tile with 4 items a ticket and 32
- * digis, bitmap store.
+ * blocks, 16 items, warp_max 64, bitmap store, or, for a mean of 1024 digis
+ * per item or more, the single-block tile with 4 items a ticket and
+ * warp_max 32, bitmap store.
  *
  * hp_autotune times every candidate (hp_tuning_candidates) on the given
  * device-resident inputs, `reps` passes each after one warm-up, on a private

@@ -32,24 +32,23 @@ constexpr int kHistThreads = 512;
 constexpr int kHistCap = 4096;       // (event, module) bins a block can histogram in shared memory
 constexpr int kCCThreads = 512;      // threads of a clustering block
 constexpr int kGroup = kCCThreads / 32; // most (event, module) items per work-queue ticket, one per warp
-constexpr int kWarpMax = 64;         // items with at most this many digis are clustered by one warp
-constexpr int kSmemSlots = 4096;     // digis of an item a block clusters in shared memory (default tile)
+constexpr int kWarpMax = 64;         // default of Tuning::warp_max
+constexpr int kSmemSlots = 4096;     // runs of an item a block clusters in shared memory (default tile)
 constexpr int kMaxTileSlots = 16384; // largest tile considered (one block per SM)
 
 // Launch parameters of the clustering kernel, chosen per launch shape by the
 // autotuner (defaults: the values above, two resident blocks per SM).
 struct Tuning {
-    uint32_t tile_slots = kSmemSlots; // block-tier capacity in shared memory; larger items use global scratch
-    uint32_t blocks_per_sm = 2;       // 1 (largest tile), 2 (up to 64 registers a thread) or 3 (up to 40, smaller tile)
+    uint32_t tile_slots = kSmemSlots; // runs in a block's shared memory; items with more use global scratch
+    uint32_t blocks_per_sm = 2;       // 1 (four groups a block, largest tile), 2 (two groups) or 3 (one group)
     uint32_t ticket_max = kGroup;     // items per ticket before halving for small launches (<= kGroup)
-    uint32_t warp_max = kWarpMax;     // 32 or 64: largest item of the warp tier
-    uint32_t label_store = 0;         // kStoreBitmap or kStoreHash: pixel lookup of the items above the warp tier
+    uint32_t warp_max = kWarpMax;     // 32 or 64: an eighth of the packed tier's largest item (hash store: all of it)
+    uint32_t label_store = 0;         // kStoreBitmap or kStoreHash: pixel lookup of the items above the packed tier
     uint32_t item_threads = kCCThreads; // threads clustering one item of the hash store: 128, 256 or 512
 };
 
-// Pixel lookup of the clustering items above the warp tier: module-sized
-// occupancy and survivor bitmaps (one block an item), or an open-addressing
-// hash table keyed by linear pixel index, sized by the item's digi count
+// Pixel lookup of the clustering items above the packed tier: module-sized
+// bitmaps (a group of threads an item), or an open-addressing hash table keyed by linear pixel index, sized by the item's digi count
 // (item_threads threads an item, several items of a block side by side).
 constexpr uint32_t kStoreBitmap = 0;
 constexpr uint32_t kStoreHash = 1;
@@ -78,17 +77,16 @@ __host__ __device__ inline uint32_t hash_capacity(size_t smem, uint32_t tile_slo
     return (uint32_t)cap;
 }
 
-// Whether a launch of N digis in EM items has block-tier items on average
-// (64 digis or more an item) rather than warp-tier ones.
+// Whether a launch of N digis in EM items has items of 64 digis or more on
+// average.
 __host__ __device__ inline bool large_items(uint64_t N, uint64_t EM) { return N >= 64ull * EM; }
 
 // Items per work-queue ticket of a launch of EM items on `grid` clustering
-// blocks: `gmax`, halved while a launch would have too few tickets per
-// block.  Warp-tier items (small on average) keep at least four a ticket, so
-// that a block's warps work on several at once, and want two tickets a
-// block; block-tier items go down to one a ticket and want four a block, so
-// that a small launch's large items spread over blocks instead of queueing
-// in one ticket (one per block: the grid is sized to match, see the runtime).
+// groups: `gmax`, halved while a launch would have too few tickets per
+// group.  Small items keep at least four a ticket, so that they share the
+// packed tier's phases, and want two tickets a group; larger items go down to
+// one a ticket and want four a group, so that a small launch's items spread
+// over groups instead of queueing in one ticket.
 __host__ __device__ inline uint32_t ticket_items(uint64_t EM, unsigned grid, uint32_t gmax, uint64_t N)
 {
     const bool large = large_items(N, EM);
@@ -161,7 +159,8 @@ constexpr uint32_t kOutChunk = 128;
 // per-item counts and the chained-scan state.
 struct Workspace {
     uint32_t *ctl;        // [16]: 0 item ticket, 1 launch error bits, 2 arena bump, 3 prefix frontier,
-                          //       4 offsets chunk ticket, 6 clusters of the launch (offsets_kernel)
+                          //       4 offsets chunk ticket, 5 large items and 7 their ticket,
+                          //       6 clusters of the launch (offsets_kernel)
     uint32_t *event_err;  // [E]
     uint32_t *count;      // [E*M] digis of each item (reserved part, then the total: scan_kernel);
                           //       then each item's first output position (offsets_kernel)
@@ -175,11 +174,23 @@ struct Workspace {
     uint32_t *bucket_w;   // [N]
     uint32_t *bucket_i;   // [N] index of the digi within its event
     Staging staging;      // [N] each array
+    uint32_t *large;      // [E*M] items of more than cc.large_digis digis, ctl[5] of them (scan_kernel)
     uint32_t *chunk_item; // [N / kOutChunk + 2] item holding the first position of each output chunk
-    unsigned long long *exact; // [cc_grid * 2 * tile_slots] 64-bit moments of heavy clusters
+    unsigned long long *exact; // [cc_grid * 2 * run_exact_slots] 64-bit moments of heavy clusters
     unsigned char *big;   // scratch of items too large for shared memory
     uint64_t big_slots;   // slots per block (slab mode) or in total (arena mode)
     int big_arena;        // 1: bump-allocated arena, 0: one slab per block
+};
+
+// Sizes of the clustering kernel of one launch, worked out on the host.
+struct ClusterPlan {
+    uint32_t items, ticket_items, tickets; // (event, module) items, items a ticket, tickets
+    uint32_t workers;                      // groups of all blocks
+    uint32_t smem, slice;                  // dynamic shared memory of a block, and of each of its groups
+    uint32_t runs, whole_runs;             // run records in a group's slice, and in the whole block's
+    uint32_t exact_slots;                  // 64-bit moment slots of a block
+    uint32_t pack_digis, pack_item;        // packed tier: digis of a pack, and of its largest item
+    uint32_t large_digis;                  // items of more digis are clustered by a whole block
 };
 
 struct Launch {
@@ -192,6 +203,7 @@ struct Launch {
     Outputs out;
     Workspace ws;
     int cc_grid;             // blocks of the clustering kernel
+    ClusterPlan cc;          // sizes of the clustering kernel (cluster_plan)
     int copy_grid = 1216;    // most blocks of the output copy (8 an SM of a 152-SM GPU)
     int sm_count = 152;      // SMs of the device (grids of the persistent histogram and scatter)
     Tuning tune;
@@ -216,13 +228,73 @@ __host__ __device__ inline unsigned bucket_grid(uint64_t N, int sm_count)
 // parent, padded to 8-byte multiples so every slot range stays 8-byte aligned.
 constexpr size_t kBigSlotBytes = 8 + 16 + 8 + 4 + 4;
 
-// Dynamic shared memory of a clustering block: the tile's slot arrays (charge,
-// count, 32-bit moments, parent: 20 bytes a slot), then the occupancy and
-// survivor bitmaps and the survivor prefix (a word each per 32 pixels).
-__host__ __device__ inline size_t cc_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots)
+// Dynamic shared memory of a clustering block of the hash label store: 20
+// bytes a slot and three words per 32 pixels of a module.
+__host__ __device__ inline size_t hash_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots)
 {
     const size_t nwords = ((size_t)R * C + 31) / 32;
     return (size_t)tile_slots * (8 + 8 + 4) + nwords * 4 * 3;
+}
+
+constexpr uint32_t kHashListBytes = (kCCThreads / 32) * 64 * 2; // of these, the run tier's warp lists
+
+// The run tier of the clustering kernel.  A group of threads clusters an item
+// in a slice of the block's shared memory: a survivor bitmap with rows of
+// ceil(C / 32) words, the first run of every word (16 bits), and the records
+// of the runs (20 bytes each), which lie over the bitmap of all digis.
+constexpr size_t kRunBytes = 20;
+constexpr size_t kBigRunBytes = 24; // a record in global scratch
+__host__ __device__ inline uint32_t run_words(uint32_t R, uint32_t C) { return (R * ((C + 31) / 32) + 3) & ~3u; }
+__host__ __device__ inline size_t run_fixed_bytes(uint32_t R, uint32_t C)
+{
+    const size_t nw = run_words(R, C);
+    return nw * 4 + ((nw * 2 + 15) & ~(size_t)15);
+}
+// Runs that a slice of `bytes` holds.
+__host__ __device__ inline uint32_t run_capacity(size_t bytes, uint32_t R, uint32_t C)
+{
+    const size_t fixed = run_fixed_bytes(R, C);
+    return bytes > fixed ? (uint32_t)((bytes - fixed) / kRunBytes) : 0u;
+}
+// Dynamic shared memory of a block of `groups` groups whose whole holds
+// tile_slots runs: at least slices of 256 runs, and of the bitmaps.
+__host__ __device__ inline size_t run_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots, uint32_t groups)
+{
+    const size_t fixed = run_fixed_bytes(R, C), bits = (size_t)run_words(R, C) * 4;
+    auto at_least = [&](size_t runs) { return fixed + (kRunBytes * runs > bits ? kRunBytes * runs : bits); };
+    const size_t whole = at_least(tile_slots), parts = groups * ((at_least(256) + 15) & ~(size_t)15);
+    return whole > parts ? whole : parts;
+}
+// 64-bit moment slots of a block (its groups' slices hold no more runs together).
+__host__ __device__ inline uint32_t run_exact_slots(uint32_t R, uint32_t C, uint32_t tile_slots, uint32_t groups)
+{
+    return run_capacity(run_smem_bytes(R, C, tile_slots, groups), R, C);
+}
+// Digis of a pack of the packed tier (36 bytes each) in a slice of `bytes`
+// with moment scratch for `cap` runs; and the largest item it takes.
+__host__ __device__ inline uint32_t pack_capacity(size_t bytes, uint32_t cap)
+{
+    uint32_t p = bytes / 36 < 1023 ? (uint32_t)(bytes / 36) : 1023u;
+    return p < cap ? p : cap;
+}
+__host__ __device__ inline uint32_t pack_max(uint32_t warp_max) { return 8 * warp_max; }
+
+// Threads and groups of a clustering block for 1, 2 and 3 resident blocks per SM.
+constexpr int kRunThreads1 = 1024, kRunGroups1 = 4;
+constexpr int kRunThreads2 = 512, kRunGroups2 = 2;
+constexpr int kRunThreads3 = 256, kRunGroups3 = 1;
+__host__ __device__ inline uint32_t run_groups(uint32_t blocks_per_sm)
+{
+    return blocks_per_sm >= 3 ? kRunGroups3 : blocks_per_sm == 2 ? kRunGroups2 : kRunGroups1;
+}
+// Digis above which an item is a whole block's: one and a half times the
+// runs of a group's slice (0.6 runs a digi are usual; an item with more runs
+// than the slice holds is finished in global scratch).
+inline uint32_t large_digis(uint32_t R, uint32_t C, const Tuning &t)
+{
+    const uint32_t groups = run_groups(t.blocks_per_sm);
+    if (t.label_store == kStoreHash || groups == 1) return 0xFFFFFFFFu;
+    return run_capacity((run_smem_bytes(R, C, t.tile_slots, groups) / groups) & ~(size_t)15, R, C) / 2 * 3;
 }
 // Lay out the workspace for (E, M, N) in `base` (nullptr: only compute size).
 size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t R, uint32_t C, int cc_grid,

@@ -13,38 +13,29 @@
 //   scatter_kernel  bucket scatter: each digi's word and in-event index go to
 //                   its item's bucket (block-local ranks in shared memory,
 //                   one global atomic per non-empty bin to reserve a range)
-//   cc_kernel       persistent clustering: blocks take tickets of up to
-//                   kGroup consecutive items (the count is a tuning
-//                   parameter); small items (up to 32 or 64 digis) are
-//                   clustered by one warp in registers, larger items by the
-//                   whole block on a shared-memory pixel bitmap with
-//                   rank-addressed union-find (items beyond the tile keep
-//                   their slot arrays in global scratch), or, with the hash
-//                   label store (a tuning choice), by groups of 128-512
-//                   threads on a hash table of the item's pixels; kept clusters are
-//                   staged per item and written in (event, module, id) order
-//                   once their ticket's prefix is known (a cooperative
-//                   frontier over the tickets' cluster counts)
+//   cc_kernel       persistent clustering: groups of threads take tickets of
+//                   up to kGroup consecutive items (the count is a tuning
+//                   parameter); a ticket's small items go together through
+//                   the packed tier (a hash table of their pixels), larger
+//                   ones one by one through the run tier (bitmaps of the
+//                   module, union-find over horizontal runs), in shared
+//                   memory, or in global scratch if their runs do not fit;
+//                   cc_hash_kernel (the hash label store, a tuning choice)
+//                   has groups of 128-512 threads cluster the items between
+//                   on a hash table each; kept clusters are staged per item
+//                   in id order
 //   offsets_kernel  each item's first output position (prefix over the items'
 //                   kept-cluster counts, chained across chunks)
 //   copy_kernel     staged clusters to their ordered output positions; per-event
 //                   status codes
 //
-// Clustering of one module (block tier): set a bit per digi in an occupancy
-// bitmap (a bit already set is a duplicate) and a bit per surviving pixel in
-// a survivor bitmap; an exclusive prefix popcount over the survivor bitmap
-// gives every surviving pixel a dense slot = its rank in row-major order, so
-// slot order is linear-pixel order.  Every pixel starts linked to the first
-// pixel of its horizontal run; runs of adjacent rows that touch (8-adjacency)
-// are joined by atomicMin linking of roots (smaller slot wins), so every root
-// is the smallest slot, i.e. the smallest linear index, of its cluster.
-// Charge, pixel count and the two moments sum(q * row), sum(q * col)
-// accumulate per root with 32-bit shared-memory atomics (the charge always
-// fits, the configuration bounds every cluster's charge; an item with a
-// cluster heavy enough to overflow the moments is re-summed exactly in 64
-// bits; 64-bit shared atomics measured slower); the ordinal of a
-// kept cluster is the rank of its root among kept roots in slot order, so the
-// per-module output is already sorted by id.
+// Labels are unique and the order of clusters fixed, so every tier gives the
+// same result: the id of a cluster is its smallest linear pixel index, the
+// root of its tree in every union-find here; charge, pixel count and the two
+// moments sum(q * row), sum(q * col) accumulate per root in 32 bits (the
+// charge always fits: the configuration bounds every cluster's), and an item
+// with a cluster heavy enough to overflow the moments sums them again in 64
+// bits.
 #include <algorithm>
 #include <climits>
 #include <cstdint>
@@ -69,7 +60,7 @@ constexpr uint32_t kSpinLimit = 1u << 24;          // iterations of a blocking w
 constexpr unsigned long long kWaitNs = 1000000000ull; // and at most one second of it
 
 struct ItemCtx {
-    uint32_t e, m, b, n;
+    uint32_t b, n;
     int32_t gain, ped;
     int32_t *label_e;    // label of the event's first digi, or null
     uint16_t *label16_e; // compact label of the event's first digi, or null (then label_e is null)
@@ -132,18 +123,6 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *t
     return __shfl_sync(kFull, ws - wt, warp) + x - v;
 }
 
-// s / Q as a float offset, with s an exact integer moment: exact operands and
-// one rounding when they fit the float mantissa, else integer quotient plus a
-// rounded remainder fraction.
-__device__ __forceinline__ float centroid(int32_t origin, long long s, int32_t Q)
-{
-    if (s > -16777216LL && s < 16777216LL && Q < 16777216)
-        return (float)origin + (float)s / (float)Q;
-    const long long qt = s / Q;
-    const long long rem = s - qt * Q;
-    return (float)(origin + qt) + (float)rem / (float)Q;
-}
-
 // Event and module of work item `item` (one division, by the thread that
 // sets up the item's record).
 __device__ __forceinline__ void item_coords(uint64_t item, uint32_t M, uint32_t *e, uint32_t *m)
@@ -162,26 +141,25 @@ __device__ __forceinline__ void item_coords(uint64_t item, uint32_t M, uint32_t 
 // (the division by the module count and the calibration loads happen there,
 // not in every thread of the block).
 struct ItemRec {
-    uint32_t e, m;
+    uint32_t e;
     int32_t gain, ped;
-    uint64_t label_off; // the event's first digi
+    uint32_t label_off; // the event's first digi (a launch has fewer than 2^32)
 };
 
 __device__ __forceinline__ ItemRec make_rec(const Launch &L, uint64_t item)
 {
     ItemRec r;
-    item_coords(item, L.g.M, &r.e, &r.m);
-    r.gain = L.g.gain[r.m];
-    r.ped = L.g.ped[r.m];
-    r.label_off = L.offsets[r.e];
+    uint32_t m;
+    item_coords(item, L.g.M, &r.e, &m);
+    r.gain = L.g.gain[m];
+    r.ped = L.g.ped[m];
+    r.label_off = (uint32_t)L.offsets[r.e];
     return r;
 }
 
 __device__ __forceinline__ ItemCtx make_item(const Launch &L, const ItemRec &rec, uint32_t b, uint32_t n)
 {
     ItemCtx it;
-    it.e = rec.e;
-    it.m = rec.m;
     it.b = b;
     it.n = n;
     it.gain = rec.gain;
@@ -454,7 +432,8 @@ __global__ void __launch_bounds__(kHistThreads, 3) hist_kernel(const Launch L)
 // (their runs are reserved, by offset, in blk_off) and count2[] those of
 // blocks with many keys (placed step by step by the scatter); the scan sets
 // boff = the item's bucket start, cursor = the start of the step-by-step
-// part (after every reserved run) and count = the item's total.
+// part (after every reserved run) and count = the item's total.  Items of
+// more than cc.large_digis digis are listed for the clustering kernel.
 __global__ void __launch_bounds__(256) scan_kernel(const Launch L)
 {
     __shared__ uint32_t tmp[256 / 32 + 1];
@@ -471,6 +450,7 @@ __global__ void __launch_bounds__(256) scan_kernel(const Launch L)
     uint32_t run = block_exclusive_scan<256>(local, tmp, &total) + (uint32_t)L.offsets[e];
     for (uint32_t m = m0; m < m1; ++m) {
         const uint32_t c1 = L.ws.count[kb + m], n = c1 + L.ws.count2[kb + m];
+        if (n > L.cc.large_digis) L.ws.large[atomicAdd(&L.ws.ctl[5], 1u)] = (uint32_t)(kb + m);
         L.ws.boff[kb + m] = run;
         L.ws.cursor[kb + m] = run + c1;
         L.ws.count[kb + m] = n;
@@ -617,253 +597,20 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
 
 // ---------------------------------------------------------------- clustering
 
-// After the unions, a root's parent entry holds kMark | its linear pixel index.
-constexpr uint32_t kMark = 0x80000000u;
-// Moments accumulate in 32 bits relative to the root pixel (|drow| < 256,
-// |dcol| < 512): they cannot overflow while Q <= INT32_MAX / 512.  Items with
-// a heavier cluster recompute the moments in 64 bits.
+// Moments accumulate in 32 bits: sum(q * col) and sum(q * (row - root row))
+// cannot overflow while Q <= INT32_MAX / 512 (row < 256, col < 512).  Items
+// with a heavier cluster recompute them in 64 bits.
 constexpr int32_t kQSafe32 = 0x7FFFFFFF / 512;
-
-// Per-item arrays of the block tier: shared memory, or global scratch for
-// items beyond the shared-memory capacity.
-struct Tile {
-    uint32_t *parent;          // union-find parent of a slot; kMark | lin for roots after marking
-    int32_t *q;                // root: charge Q
-    uint32_t *np;              // root: pixel count
-    int2 *m;                   // root: sum q*row, sum q*col
-    unsigned long long *exact; // root: the same two moments in 64 bits (heavy clusters only)
-};
-
-struct BlockShared {
-    uint32_t flag;
-    uint32_t heavy;
-    uint32_t big_off;
-    uint32_t scan_tmp[kCCThreads / 32 + 1];
-};
-
-// Find with path splitting (each visited node is re-pointed to its
-// grandparent).  Parent entries only ever point to a smaller slot of the same
-// tree, so a plain store that races with a link elsewhere leaves a valid
-// ancestor behind; a link that loses such a race is retried by its union.
-__device__ __forceinline__ uint32_t uf_find_halving(uint32_t *parent, uint32_t x)
-{
-    volatile uint32_t *p = parent;
-    uint32_t y = p[x];
-    while (y != x) {
-        const uint32_t z = p[y];
-        if (z != y) p[x] = z;
-        x = y;
-        y = z;
-    }
-    return x;
-}
-
 constexpr uint32_t kNoSlot = 0xFFFFFFFFu;
 
-// Lock-free union of the trees of a and b, for all 32 lanes of a warp in
-// lockstep (lanes with b == kNoSlot idle; the whole warp must call it): the
-// larger root is linked under the smaller with atomicMin, and a lost race
-// re-runs with the new parent.
-__device__ __forceinline__ void warp_union(uint32_t *parent, uint32_t a, uint32_t b)
+// Barrier of the `threads` threads of one group (named barrier `id` >= 1;
+// barrier 0 is the block's __syncthreads).  The compiler's own builtin, not
+// inline assembly: like __syncthreads it is convergent, so the compiler
+// never duplicates it into paths that a warp's threads take apart.
+__device__ __forceinline__ void group_sync(uint32_t id, uint32_t threads)
 {
-    bool done = b == kNoSlot;
-    while (__any_sync(kFull, !done)) {
-        if (!done) {
-            a = uf_find_halving(parent, a);
-            b = uf_find_halving(parent, b);
-            if (a == b) {
-                done = true;
-            } else {
-                if (a < b) {
-                    const uint32_t t = a;
-                    a = b;
-                    b = t;
-                }
-                const uint32_t old = atomicMin(&parent[a], b);
-                if (old == a)
-                    done = true;
-                else
-                    a = old;
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ uint32_t rank_of(const uint32_t *sbits, const uint32_t *spre, uint32_t lin)
-{
-    return spre[lin >> 5] + __popc(sbits[lin >> 5] & ((1u << (lin & 31)) - 1u));
-}
-
-__device__ __forceinline__ bool has_bit(const uint32_t *bits, uint32_t lin)
-{
-    return (bits[lin >> 5] >> (lin & 31)) & 1u;
-}
-
-// Number of surviving pixels immediately to the left of pixel lin in its row
-// (the pixel's offset in its horizontal run), read from the survivor bitmap
-// 32 bits at a time.
-__device__ __forceinline__ uint32_t run_offset(const uint32_t *sbits, uint32_t lin, uint32_t row0)
-{
-    uint32_t off = 0, pos = lin;
-    while (pos > row0) {
-        const uint32_t bt = (pos - 1) & 31;
-        const uint32_t x = ~sbits[(pos - 1) >> 5] << (31 - bt); // bit pos-1 moved to the top
-        const uint32_t ones = x ? (uint32_t)__clz(x) : bt + 1;  // set bits from pos-1 downwards
-        const uint32_t take = min(ones, pos - row0);
-        off += take;
-        pos -= take;
-        if (take < bt + 1) break;
-    }
-    return off;
-}
-
-// One item of at most 32 * K digis, clustered by one warp in registers:
-// digi j is held by lane j % 32 in register slot j / 32.  Adjacency is a bit
-// mask over the item's digis per held digi; the cluster id (the smallest
-// linear index) spreads over the adjacency by min-propagation; cluster sums
-// run over the digis sharing an id.  Returns the number of kept clusters
-// (all lanes).
-template <int K>
-__device__ uint32_t warp_item(const Launch &L, const ItemCtx &it)
-{
-    using Mask = typename std::conditional<K == 1, uint32_t, unsigned long long>::type;
-    const uint32_t lane = threadIdx.x & 31;
-    const int R = (int)L.g.R, C = (int)L.g.C;
-    const uint32_t n = it.n;
-    int r[K], c[K], q[K], lin[K], lab[K];
-    uint32_t idx[K];
-    bool have[K], surv[K];
-    Mask adj[K];
-    bool bad = false;
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        const uint32_t j = lane + 32 * k;
-        have[k] = j < n;
-        const uint32_t w = have[k] ? L.ws.bucket_w[it.b + j] : 0u;
-        idx[k] = have[k] ? L.ws.bucket_i[it.b + j] : 0u;
-        r[k] = (int)(w & 0xFFu);
-        c[k] = (int)((w >> 8) & 0x1FFu);
-        const int adc = (int)((w >> 17) & 0xFFu);
-        if (have[k] && (r[k] >= R || c[k] >= C || adc == 0 || (w >> 25) != 0)) bad = true;
-        lin[k] = have[k] ? r[k] * C + c[k] : -1 - (int)j;
-        q[k] = adc * it.gain - it.ped;
-        surv[k] = have[k] && q[k] >= L.g.pixel_thr;
-        adj[k] = 0;
-    }
-    if (__any_sync(kFull, bad)) {
-        if (lane == 0) atomicOr(it.err_e, kErrBadDigi);
-        return 0;
-    }
-    Mask smask = (Mask)__ballot_sync(kFull, surv[0]);
-    if constexpr (K == 2) smask |= (Mask)__ballot_sync(kFull, surv[1]) << 32;
-    bool dup = false;
-    for (uint32_t j = 0; j < n; ++j) {
-        const uint32_t sl = j & 31, sk = j >> 5;
-        const int lj = __shfl_sync(kFull, (K == 2 && sk) ? lin[K - 1] : lin[0], sl);
-        const int rj = __shfl_sync(kFull, (K == 2 && sk) ? r[K - 1] : r[0], sl);
-        const int cj = __shfl_sync(kFull, (K == 2 && sk) ? c[K - 1] : c[0], sl);
-        const bool sj = (smask >> j) & 1u;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const uint32_t me = lane + 32 * k;
-            if (me == j) continue;
-            if (have[k] && lj == lin[k]) dup = true;
-            if (surv[k] && sj && abs(rj - r[k]) <= 1 && abs(cj - c[k]) <= 1) adj[k] |= (Mask)1 << j;
-        }
-    }
-    if (__any_sync(kFull, dup)) {
-        if (lane == 0) atomicOr(it.err_e, kErrDup);
-        return 0;
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k) lab[k] = surv[k] ? lin[k] : INT_MAX;
-    for (uint32_t round = 0; round < n; ++round) {
-        int nl[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) nl[k] = lab[k];
-        for (uint32_t j = 0; j < n; ++j) {
-            const int lj = __shfl_sync(kFull, (K == 2 && (j >> 5)) ? lab[K - 1] : lab[0], j & 31);
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if ((adj[k] >> j) & 1u) nl[k] = min(nl[k], lj);
-        }
-        bool changed = false;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            changed |= nl[k] != lab[k];
-            lab[k] = nl[k];
-        }
-        if (!__any_sync(kFull, changed)) break;
-    }
-    // sums over the digis of each held digi's cluster, about the cluster's id pixel
-    // (|sums| < 64 * 32263 * 63 < 2^31)
-    int Q[K], np[K], Sr[K], Sc[K], rr[K], rc[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        Q[k] = np[k] = Sr[k] = Sc[k] = 0;
-        rr[k] = surv[k] ? lab[k] / C : 0;
-        rc[k] = surv[k] ? lab[k] - rr[k] * C : 0;
-    }
-    for (uint32_t j = 0; j < n; ++j) {
-        const uint32_t sl = j & 31;
-        const bool hi = K == 2 && (j >> 5);
-        const int labj = __shfl_sync(kFull, hi ? lab[K - 1] : lab[0], sl);
-        const int qj = __shfl_sync(kFull, hi ? q[K - 1] : q[0], sl);
-        const int rj = __shfl_sync(kFull, hi ? r[K - 1] : r[0], sl);
-        const int cj = __shfl_sync(kFull, hi ? c[K - 1] : c[0], sl);
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            if (surv[k] && labj == lab[k]) {
-                Q[k] += qj;
-                ++np[k];
-                Sr[k] += qj * (rj - rr[k]);
-                Sc[k] += qj * (cj - rc[k]);
-            }
-        }
-    }
-    bool kept[K], lead[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        lead[k] = surv[k] && lin[k] == lab[k];
-        kept[k] = surv[k] && Q[k] >= L.g.cluster_thr;
-    }
-    Mask kl = (Mask)__ballot_sync(kFull, lead[0] && kept[0]);
-    if constexpr (K == 2) kl |= (Mask)__ballot_sync(kFull, lead[K - 1] && kept[K - 1]) << 32;
-    uint32_t ord[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) ord[k] = 0;
-    for (uint32_t j = 0; j < n; ++j) {
-        const int lj = __shfl_sync(kFull, (K == 2 && (j >> 5)) ? lin[K - 1] : lin[0], j & 31);
-        if ((kl >> j) & 1u) {
-#pragma unroll
-            for (int k = 0; k < K; ++k)
-                if (lj < lab[k]) ++ord[k]; // the rank of the digi's cluster (lab = lin for its lead)
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-        if (lead[k] && kept[k]) {
-            L.ws.staging.put(it.b + ord[k], lab[k], Q[k], np[k], centroid(rr[k], Sr[k], Q[k]),
-                             centroid(rc[k], Sc[k], Q[k]));
-        }
-        if (it.label_e && have[k]) it.label_e[idx[k]] = !surv[k] ? -1 : (kept[k] ? lab[k] : -2);
-        if (it.label16_e && have[k])
-            it.label16_e[idx[k]] = !surv[k] ? kLab16Below : (kept[k] ? (uint16_t)ord[k] : kLab16Dropped);
-    }
-    if constexpr (K == 1)
-        return __popc(kl);
-    else
-        return __popcll(kl);
-}
-
-// Apply f(k, word) to every digi of the item owned by this thread.  The
-// loop is kept rolled so that the block tier stays small in the instruction
-// cache; the item's bucket (read-only here) is re-read through L1.
-template <class F>
-__device__ __forceinline__ void for_digis(const uint32_t *bw, uint32_t n, F &&f)
-{
-#pragma unroll 1
-    for (uint32_t k = threadIdx.x; k < n; k += kCCThreads) f(k, __ldg(bw + k));
+    __syncwarp();
+    __barrier_sync_count(id, threads);
 }
 
 // Centroid coordinate sum / Q from an exact, non-negative moment: one float
@@ -882,703 +629,1073 @@ __device__ __forceinline__ float centroid_abs(long long sum, int32_t Q)
     return (float)qt + (float)(sum - qt * Q) / (float)Q;
 }
 
-// One item clustered by the whole block (see the file comment).  kBig: the
-// tile lives in global scratch instead of shared memory.  Returns the number
-// of kept clusters (uniform over the block).
-template <bool kBig>
-__device__ uint32_t block_item(const Launch &L, const ItemCtx &it, uint32_t *abits, uint32_t *sbits, uint32_t *spre,
-                               const Tile &t, BlockShared &bs)
+// Static shared memory of one group of threads that clusters items on its
+// own (GT threads: its own named barrier, its own tickets).
+struct GroupShared {
+    uint32_t ticket;
+    uint32_t flag, heavy, pixels, extras;
+    uint32_t bucket_end;           // end of the ticket's buckets
+    uint32_t pack_end;             // packed tier: end of the planned pack (an item of the ticket); run tier: scratch slot
+    uint32_t tmp[32];              // scans; packed tier: kept clusters of each item
+    uint32_t n[kGroup], b[kGroup]; // digis and bucket start of the ticket's items
+    ItemRec rec[kGroup];
+    uint16_t pack[kGroup + 1];     // packed tier: first packed digi of each item, and the total
+};
+
+template <int GT, bool kWhole>
+__device__ __forceinline__ void gsync(uint32_t bar)
 {
-    const uint32_t R = L.g.R, C = L.g.C, nwords = (R * C + 31) >> 5;
-    const int32_t thr = L.g.pixel_thr, cthr = L.g.cluster_thr;
-    const uint32_t tid = threadIdx.x, n = it.n, lane = tid & 31, warp = tid >> 5;
-    const uint32_t *bw = L.ws.bucket_w + it.b;
-    const uint32_t *bi = L.ws.bucket_i + it.b;
+    if constexpr (kWhole)
+        __syncthreads();
+    else
+        group_sync(bar, GT);
+}
+
+// Exclusive scan of one value per thread over the group, with one barrier:
+// every thread's accesses before the call are visible to the group after it.
+template <int GT, bool kWhole>
+__device__ __forceinline__ uint32_t group_exclusive_scan(uint32_t v, uint32_t *tmp, uint32_t gt, uint32_t bar,
+                                                         uint32_t *total)
+{
+    constexpr int kWarps = GT / 32;
+    const uint32_t lane = gt & 31, warp = gt >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, x, o);
+        if ((int)lane >= o) x += y;
+    }
+    if (lane == 31) tmp[warp] = x;
+    gsync<GT, kWhole>(bar);
+    const uint32_t wt = lane < kWarps ? tmp[lane] : 0u;
+    uint32_t ws = wt;
+#pragma unroll
+    for (int o = 1; o < kWarps; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, ws, o);
+        if ((int)lane >= o) ws += y;
+    }
+    *total = __shfl_sync(kFull, ws, kWarps - 1);
+    return __shfl_sync(kFull, ws - wt, warp) + x - v;
+}
+
+// Shared memory by 32-bit address, with the byte offset as an immediate: the
+// run tier's records are five words, and with one address a record all its
+// fields cost no further address arithmetic.
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+template <int kOff = 0>
+__device__ __forceinline__ uint32_t lds(uint32_t a)
+{
+    uint32_t v;
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(a), "n"(kOff) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t lds_u16(uint32_t a)
+{
+    uint16_t v;
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+    return v;
+}
+template <int kOff = 0>
+__device__ __forceinline__ void sts(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u32 [%0+%1], %2;" ::"r"(a), "n"(kOff), "r"(v) : "memory");
+}
+template <int kOff = 0>
+__device__ __forceinline__ void reds_add(uint32_t a, uint32_t v)
+{
+    asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(a), "n"(kOff), "r"(v) : "memory");
+}
+template <int kOff = 0>
+__device__ __forceinline__ uint32_t atoms_add(uint32_t a, uint32_t v)
+{
+    uint32_t old;
+    asm volatile("atom.shared.add.u32 %0, [%1+%2], %3;" : "=r"(old) : "r"(a), "n"(kOff), "r"(v) : "memory");
+    return old;
+}
+__device__ __forceinline__ void reds_or(uint32_t a, uint32_t v)
+{
+    asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+__device__ __forceinline__ uint32_t atoms_min(uint32_t a, uint32_t v)
+{
+    uint32_t old;
+    asm volatile("atom.shared.min.u32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
+    return old;
+}
+
+// ---- run tier
+//
+// One item by a group of GT threads on a survivor bitmap whose rows start at
+// word boundaries (W = ceil(C / 32) words a row).  The unit of the union-find
+// and of the sums is the run: a maximal stretch of surviving pixels inside
+// one bitmap word.  Runs are numbered in word order, which is row-major
+// order, so the smallest run of a cluster holds its smallest linear index
+// (the id), and the runs of the row above that touch a run are consecutive.
+// Phases, one group barrier between them:
+//   1 the item's words; both bitmaps (all digis, survivors) cleared
+//   2 a bit per digi and per survivor; a digi whose bit is taken is found by
+//     counting: the set bits must be as many as the digis
+//   3 runs per word by a scan over the words; run records initialised (they
+//     lie over the bitmap of all digis, free from here on)
+//   4 every survivor adds its charge and q * col to its run; a run's first
+//     pixel stores the run's position
+//   5 a run links itself, by a plain store, under the first run above that
+//     it touches (or the run that ends the word to its left); runs with
+//     further contacts (one in ten or so) go to a list
+//   6 the listed runs are united with those, by find and link
+//   7 every run finds its root and adds its sums to it
+//   8 the position of the root into every run (the label of its digis);
+//     kept roots counted
+//   9 labels of the digis; kept roots staged in run (= id) order
+//
+// What bounds it: instruction issue and the latency of shared memory; an item
+// is a chain of ten barriers, so several groups a block work on items of
+// their own, every phase issues its loads four digis or two runs at a time,
+// and the frequent conditions are predicates, not branches.  Runs, not
+// pixels, are the nodes because there are 0.6 of them a digi in blob-like
+// data (0.5 to 0.8): against a node and four atomics a pixel (the tier this
+// replaced) a pixel needs no rank and two atomics, and a run looks at one word
+// above it instead of eight pixels.  27.7M digis in 16,384 items: 24 -> 14
+// warp instructions a digi, 934 -> 564 us; 29.4M digis in 14,848 items with
+// 13,000-digi ones among them: 1,374 -> 614 us (its records are 20 bytes, so
+// these fit a block's shared memory now).
+//
+// Run records, in shared memory or (kBig) global scratch:
+//   word 0  union-find parent << kRunShift | (roots) pixels of the cluster
+//   word 1  row | col << 8 of the first pixel (the digi word's layout), and
+//           length << 17; from phase 8 on the root's position and a flag
+//   word 2  charge, word 3 sum q * col: of the run, then (roots) the cluster
+//   word 4  the list of phase 5; then (roots) sum q * (row - root's row)
+//   word 5  (kBig only, whose word 0 is the parent alone) pixels
+constexpr int kRunDigis = 8; // digis a thread holds at once
+constexpr uint32_t kRunShift = 18, kRunPixels = (1u << kRunShift) - 1u;
+constexpr uint32_t kRunKept = 1u << 31, kRunDropped = 1u << 30, kRunPos = 0x1FFFFu;
+
+template <bool kBig>
+struct Runs;
+template <>
+struct Runs<false> {
+    uint32_t base;
+    using At = uint32_t;
+    __device__ __forceinline__ At at(uint32_t i) const { return base + i * (uint32_t)kRunBytes; }
+    template <int f>
+    __device__ __forceinline__ static uint32_t ld(At a) { return lds<4 * f>(a); }
+    template <int f>
+    __device__ __forceinline__ static void st(At a, uint32_t v) { sts<4 * f>(a, v); }
+    template <int f>
+    __device__ __forceinline__ static void red(At a, uint32_t v) { reds_add<4 * f>(a, v); }
+    template <int f>
+    __device__ __forceinline__ static uint32_t add(At a, uint32_t v) { return atoms_add<4 * f>(a, v); }
+    __device__ __forceinline__ uint32_t parent(uint32_t i) const { return ld<0>(at(i)) >> kRunShift; }
+    __device__ __forceinline__ void set_parent(uint32_t i, uint32_t p) const { st<0>(at(i), p << kRunShift); }
+    __device__ __forceinline__ uint32_t min_parent(uint32_t i, uint32_t p) const
+    {
+        return atoms_min(at(i), p << kRunShift) >> kRunShift;
+    }
+    // a pixel's charge and charge * column into its run, if in != 0; the
+    // run's position, if head != 0 (predicated: no branch among the lanes)
+    __device__ __forceinline__ static void add_pixel(At a, uint32_t q, uint32_t qc, uint32_t in, uint32_t head,
+                                                     uint32_t pos)
+    {
+        asm volatile("{\n\t"
+                     ".reg .pred p, h;\n\t"
+                     "setp.ne.u32 p, %3, 0;\n\t"
+                     "setp.ne.u32 h, %4, 0;\n\t"
+                     "@p red.shared.add.u32 [%0+8], %1;\n\t"
+                     "@p red.shared.add.u32 [%0+12], %2;\n\t"
+                     "@h st.shared.u32 [%0+4], %5;\n\t"
+                     "}" ::"r"(a), "r"(q), "r"(qc), "r"(in), "r"(head), "r"(pos) : "memory");
+    }
+    __device__ __forceinline__ static void add_pixels(At a, uint32_t v) { red<0>(a, v); }
+    __device__ __forceinline__ static uint32_t pixels(At a) { return ld<0>(a) & kRunPixels; }
+    __device__ __forceinline__ static void set_ordinal(At a, uint32_t i, uint32_t v) { st<0>(a, (i << kRunShift) | v); }
+    __device__ __forceinline__ static void init(At a, uint32_t i)
+    {
+        st<0>(a, i << kRunShift);
+        st<2>(a, 0);
+        st<3>(a, 0);
+        st<4>(a, 0);
+    }
+};
+template <>
+struct Runs<true> {
+    uint32_t *base;
+    using At = uint32_t *;
+    __device__ __forceinline__ At at(uint32_t i) const { return base + (size_t)i * (kBigRunBytes / 4); }
+    template <int f>
+    __device__ __forceinline__ static uint32_t ld(At a) { return *(volatile uint32_t *)(a + f); }
+    template <int f>
+    __device__ __forceinline__ static void st(At a, uint32_t v) { *(volatile uint32_t *)(a + f) = v; }
+    template <int f>
+    __device__ __forceinline__ static void red(At a, uint32_t v) { atomicAdd(a + f, v); }
+    template <int f>
+    __device__ __forceinline__ static uint32_t add(At a, uint32_t v) { return atomicAdd(a + f, v); }
+    __device__ __forceinline__ uint32_t parent(uint32_t i) const { return ld<0>(at(i)); }
+    __device__ __forceinline__ void set_parent(uint32_t i, uint32_t p) const { st<0>(at(i), p); }
+    __device__ __forceinline__ uint32_t min_parent(uint32_t i, uint32_t p) const { return atomicMin(at(i), p); }
+    __device__ __forceinline__ static void add_pixel(At a, uint32_t q, uint32_t qc, uint32_t in, uint32_t head,
+                                                     uint32_t pos)
+    {
+        if (in) {
+            atomicAdd(a + 2, q);
+            atomicAdd(a + 3, qc);
+            if (head) st<1>(a, pos);
+        }
+    }
+    __device__ __forceinline__ static void add_pixels(At a, uint32_t v) { atomicAdd(a + 5, v); }
+    __device__ __forceinline__ static uint32_t pixels(At a) { return ld<5>(a); }
+    __device__ __forceinline__ static void set_ordinal(At a, uint32_t, uint32_t v) { st<5>(a, v); }
+    __device__ __forceinline__ static void init(At a, uint32_t i)
+    {
+        st<0>(a, i);
+        st<2>(a, 0);
+        st<3>(a, 0);
+        st<4>(a, 0);
+        st<5>(a, 0);
+    }
+};
+
+// Find with path halving (each visited run is re-pointed to its
+// grandparent).  Parents only ever point to a smaller run of the same tree,
+// so a plain store that races with a link elsewhere leaves a valid ancestor
+// behind; a link that loses such a race is retried by its union.
+template <class A>
+__device__ __forceinline__ uint32_t run_find(const A &a, uint32_t x)
+{
+    uint32_t y = a.parent(x);
+    while (y != x) {
+        const uint32_t z = a.parent(y);
+        if (z != y) a.set_parent(x, z);
+        x = y;
+        y = z;
+    }
+    return x;
+}
+
+// Lock-free union of the trees of x and y by one thread: the larger root is
+// linked under the smaller with an atomic minimum; a link that finds its
+// root already linked elsewhere retries from the new parent.
+template <class A>
+__device__ __forceinline__ void run_union(const A &a, uint32_t x, uint32_t y)
+{
+    for (;;) {
+        x = run_find(a, x);
+        y = run_find(a, y);
+        if (x == y) return;
+        const uint32_t hi = max(x, y), lo = min(x, y), old = a.min_parent(hi, lo);
+        if (old == hi) return;
+        x = old;
+        y = lo;
+    }
+}
+
+// What a run at position p sees of the bitmap: its word, the word above and
+// that word's first run, the words beside both (those left of the row's
+// first word read as themselves and are not used), and the first run of the
+// word after the one above.  All loads are independent of each other.
+struct RunView {
+    uint32_t word, left, up, up_left, up_right, pre, next;
+};
+__device__ __forceinline__ RunView run_view(uint32_t sb, uint32_t rp, uint32_t W, uint32_t p)
+{
+    const uint32_t r = p & 0xFFu, cw = (p >> 13) & 0xFu, wi = r * W + cw, wu = r ? wi - W : wi;
+    const uint32_t a = sb + 4 * wi, u = sb + 4 * wu, ra = rp + 2 * wu, back = cw ? 4u : 0u;
+    RunView v;
+    v.word = lds(a);
+    v.up = lds(u);
+    v.pre = lds_u16(ra);
+    v.left = lds(a - back);
+    v.up_left = lds(u - back);
+    v.up_right = lds<4>(u); // (past the last word lies the table of first runs)
+    v.next = lds_u16(ra + 2);
+    return v;
+}
+// Runs that touch run i (position p) before it: [*k, *end) of the row above,
+// and *left, the run that ends the word to its left (kNoSlot: none).
+// Returns its length.
+__device__ __forceinline__ uint32_t run_contacts(const RunView &v, uint32_t W, uint32_t i, uint32_t p, uint32_t *k,
+                                                 uint32_t *end, uint32_t *left)
+{
+    const uint32_t cw = (p >> 13) & 0xFu, b = (p >> 8) & 31u;
+    const uint32_t len = (uint32_t)__clz(__brev(~(v.word >> b))); // 32 for a full word
+    const bool above = (p & 0xFFu) != 0, left_edge = b == 0 && cw != 0, right_edge = b + len == 32 && cw + 1 < W;
+    const uint32_t u = above ? v.up : 0u, hu = u & ~(u << 1);
+    const uint32_t mask = (kFull >> (32 - len)) << b, t = u & (mask | (mask << 1) | (mask >> 1));
+    uint32_t k0 = 0, e0 = 0;
+    if (t) {
+        k0 = v.pre + __popc(hu & (t ^ (t - 1))) - 1u;      // heads up to t's lowest bit
+        e0 = v.pre + __popc(hu & (kFull >> __clz(t)));     // and up to its highest
+    }
+    if (left_edge && above && (v.up_left >> 31)) { // the run that ends the word before
+        if (!e0) e0 = v.pre;
+        k0 = v.pre - 1u;
+    }
+    if (right_edge && above && (v.up_right & 1u)) { // the run that starts the word after
+        if (!e0) k0 = v.next;
+        e0 = v.next + 1u;
+    }
+    *k = k0;
+    *end = e0;
+    *left = left_edge && (v.left >> 31) ? i - 1u : kNoSlot;
+    return len;
+}
+
+// The item's digis, four at a time so that their loads overlap:
+// f(k, j, x) for the thread's digis j .. j + 3 with words x[4] (kNoDigi for
+// those past the last), held in w[k] .. w[k + 3] with kSingle (all of them
+// loaded by load_digis), else loaded here.
+constexpr uint32_t kNoDigi = 0xFFFFFFFFu; // an invalid word (row 255, column 511)
+template <int GT>
+__device__ __forceinline__ void load_digis(uint32_t (&w)[kRunDigis], const uint32_t *bw, uint32_t mine)
+{
+#pragma unroll
+    for (int k = 0; k < kRunDigis; ++k) w[k] = (uint32_t)k < mine ? __ldg(bw + k * GT) : kNoDigi;
+}
+template <int GT, bool kSingle, class F>
+__device__ __forceinline__ void each_four(uint32_t (&w)[kRunDigis], const uint32_t *bw, uint32_t mine, F &&f)
+{
+    // bw points at the thread's first digi, mine = how many it has
+    if constexpr (kSingle) {
+#pragma unroll
+        for (int k = 0; k < kRunDigis; k += 4) {
+            if ((uint32_t)k < mine) {
+                uint32_t x[4] = {w[k], w[k + 1], w[k + 2], w[k + 3]};
+                f(k, (uint32_t)k, x);
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (uint32_t base = 0; base < mine; base += 4) {
+            uint32_t x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = base + u < mine ? __ldg(bw + (size_t)(base + u) * GT) : kNoDigi;
+            f(0, base, x);
+        }
+    }
+}
+
+template <int GT, bool kWhole, bool kBig, bool kSingle>
+__device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx &it, uint32_t sb, uint32_t rp,
+                                                 const Runs<kBig> a, unsigned long long *exact, uint32_t nruns,
+                                                 uint32_t (&w)[kRunDigis], GroupShared &gs, uint16_t *wlist,
+                                                 uint32_t gt, uint32_t bar)
+{
+    using A = Runs<kBig>;
+    const uint32_t C = L.g.C, W = (C + 31) >> 5;
+    const int32_t cthr = L.g.cluster_thr;
+    const uint32_t n = it.n, lane = gt & 31, warp = gt >> 5;
+    const uint32_t mine = n > gt ? (n - gt - 1) / GT + 1 : 0u;
+    const uint32_t *bw = L.ws.bucket_w + it.b + gt;
+    const uint32_t *bi = L.ws.bucket_i + it.b + gt;
     const int32_t gain = it.gain, ped = it.ped;
-    auto lin_of = [C](uint32_t w) { return (w & 0xFFu) * C + ((w >> 8) & 0x1FFu); };
-    auto charge = [gain, ped](uint32_t w) { return (int32_t)((w >> 17) & 0xFFu) * gain - ped; };
-
-    for (uint32_t i = tid; i < nwords; i += kCCThreads) {
-        abits[i] = 0;
-        sbits[i] = 0;
-    }
-    if (tid == 0) {
-        bs.flag = 0;
-        bs.heavy = 0;
-    }
-    __syncthreads();
-
-    // occupancy and survivor bitmaps; validation and duplicate detection
-    {   // the item's words are loaded four per thread at a time, so that
-        // their latencies overlap instead of adding up
-        auto body = [&](uint32_t w) {
-            const uint32_t r = w & 0xFFu, c = (w >> 8) & 0x1FFu, adc = (w >> 17) & 0xFFu;
-            if (r >= R || c >= C || adc == 0 || (w >> 25) != 0) {
-                atomicOr(&bs.flag, kErrBadDigi);
-                return;
-            }
-            const uint32_t lin = r * C + c, bit = 1u << (lin & 31);
-            if (atomicOr(&abits[lin >> 5], bit) & bit) atomicOr(&bs.flag, kErrDup);
-            if (charge(w) >= thr) atomicOr(&sbits[lin >> 5], bit);
-        };
-#pragma unroll 1
-        for (uint32_t k0 = tid; k0 < n; k0 += 4 * kCCThreads) {
-            uint32_t wv[4];
+    // runs of four digis, kNoSlot for those below threshold and past the last
+    auto runs_of = [&](const uint32_t (&x)[4], uint32_t (&run)[4], uint32_t (&in)[4], uint32_t (&head)[4]) {
+        uint32_t word[4], pre[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t k = k0 + u * kCCThreads;
-                wv[u] = k < n ? __ldg(bw + k) : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (k0 + u * kCCThreads < n) body(wv[u]);
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t wi = x[u] == kNoDigi ? 0u : (x[u] & 0xFFu) * W + ((x[u] >> 13) & 0xFu);
+            word[u] = lds(sb + 4 * wi);
+            pre[u] = lds_u16(rp + 2 * wi);
         }
-    }
-    __syncthreads();
-    const uint32_t flag = bs.flag;
-    if (flag) {
-        if (tid == 0) atomicOr(it.err_e, flag);
-        __syncthreads();
-        return 0;
-    }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t b = x[u] == kNoDigi ? 0u : 1u << ((x[u] >> 8) & 31u), h = word[u] & ~(word[u] << 1);
+            in[u] = word[u] & b;
+            head[u] = h & b;
+            run[u] = in[u] ? pre[u] + __popc(h & (b | (b - 1u))) - 1u : kNoSlot;
+        }
+    };
 
-    // exclusive prefix popcount of the survivor bitmap -> dense slots
-    const uint32_t per = (nwords + kCCThreads - 1) / kCCThreads;
-    const uint32_t w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
-    uint32_t local = 0;
-    for (uint32_t i = w0; i < w1; ++i) local += __popc(sbits[i]);
-    uint32_t S;
-    uint32_t run = block_exclusive_scan<kCCThreads>(local, bs.scan_tmp, &S);
-    for (uint32_t i = w0; i < w1; ++i) {
-        spre[i] = run;
-        run += __popc(sbits[i]);
-    }
-    // the per-root accumulators of every slot, cleared in slot order
-    for (uint32_t s = tid; s < S; s += kCCThreads) {
-        t.q[s] = 0;
-        t.np[s] = 0;
-        t.m[s] = make_int2(0, 0);
-    }
-    __syncthreads();
-    // every surviving pixel starts in its horizontal run: parent = the run's
-    // first pixel, whose slot is the pixel's slot minus its run offset
-    for_digis(bw, n, [&](uint32_t, uint32_t w) {
-        const uint32_t r = w & 0xFFu, lin = lin_of(w);
-        if (!has_bit(sbits, lin)) return;
-        const uint32_t s = rank_of(sbits, spre, lin);
-        t.parent[s] = s - run_offset(sbits, lin, r * C);
+    // 3 (rest)
+    for (uint32_t i = gt; i < nruns; i += GT) A::init(a.at(i), i);
+    gsync<GT, kWhole>(bar);
+
+    // 4
+    each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t, const uint32_t (&x)[4]) {
+        uint32_t run[4], in[4], head[4];
+        runs_of(x, run, in, head);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t q = ((x[u] >> 17) & 0xFFu) * (uint32_t)gain - (uint32_t)ped;
+            A::add_pixel(a.at(in[u] ? run[u] : 0u), q, q * ((x[u] >> 8) & 0x1FFu), in[u], head[u], x[u] & kRunPos);
+            if constexpr (kSingle) w[k + u] = run[u];
+        }
     });
-    __syncthreads();
+    gsync<GT, kWhole>(bar);
 
-    // Join runs of adjacent rows.  For a pixel p whose upper neighbour U
-    // survives, one union per maximal stretch of such pixels (at p = the run
-    // head, or where the upper-left pixel does not survive) joins p's run to
-    // U's run; a run head whose U is empty checks its upper-left pixel, a run
-    // tail whose U is empty its upper-right one.  Every 8-adjacency between
-    // two runs passes through one of these.  The lanes of a warp walk the
-    // item in step, two digis a lane (64 consecutive digis a warp), and union
-    // the pairs of both in one lockstep round.
-    for (uint32_t k0 = 2 * (tid - lane); k0 < n; k0 += 2 * kCCThreads) {
-        uint32_t s[2] = {0u, 0u}, nb0[2] = {kNoSlot, kNoSlot}, nb1[2] = {kNoSlot, kNoSlot};
+    // 5: two runs a thread at a time
+    for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
+        uint32_t i[2] = {i0, i0 + GT}, p[2];
+        RunView v[2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t k = k0 + 32 * h + lane;
-            if (k < n) {
-                const uint32_t w = __ldg(bw + k);
-                const uint32_t r = w & 0xFFu, c = (w >> 8) & 0x1FFu, lin = r * C + c;
-                if (r > 0 && has_bit(sbits, lin)) {
-                    s[h] = rank_of(sbits, spre, lin);
-                    const uint32_t up = lin - C;
-                    const bool head = c == 0 || !has_bit(sbits, lin - 1);
-                    const bool tail = c + 1 == C || !has_bit(sbits, lin + 1);
-                    const bool ul = c > 0 && has_bit(sbits, up - 1);
-                    if (has_bit(sbits, up)) {
-                        if (head || !ul) nb0[h] = rank_of(sbits, spre, up);
-                    } else {
-                        if (head && ul) nb0[h] = rank_of(sbits, spre, up - 1);
-                        if (tail && c + 1 < C && has_bit(sbits, up + 1)) nb1[h] = rank_of(sbits, spre, up + 1);
-                    }
-                }
-            }
-        }
-        // gather the warp's union pairs onto consecutive lanes, then union them
-        const uint32_t m00 = __ballot_sync(kFull, nb0[0] != kNoSlot), m01 = __ballot_sync(kFull, nb1[0] != kNoSlot);
-        const uint32_t m10 = __ballot_sync(kFull, nb0[1] != kNoSlot), m11 = __ballot_sync(kFull, nb1[1] != kNoSlot);
-        const uint32_t e0 = __popc(m00), e1 = e0 + __popc(m01), e2 = e1 + __popc(m10), total = e2 + __popc(m11);
-        for (uint32_t base = 0; base < total; base += 32) {
-            const uint32_t p = base + lane;
-            const uint32_t seg = p < e0 ? 0u : p < e1 ? 1u : p < e2 ? 2u : 3u;
-            const uint32_t mask = seg == 0 ? m00 : seg == 1 ? m01 : seg == 2 ? m10 : m11;
-            const uint32_t first = seg == 0 ? 0u : seg == 1 ? e0 : seg == 2 ? e1 : e2;
-            const uint32_t src = p < total ? __fns(mask, 0, (int)(p - first) + 1) : 0u;
-            const uint32_t a0 = __shfl_sync(kFull, s[0], src), a1 = __shfl_sync(kFull, s[1], src);
-            const uint32_t b00 = __shfl_sync(kFull, nb0[0], src), b01 = __shfl_sync(kFull, nb1[0], src);
-            const uint32_t b10 = __shfl_sync(kFull, nb0[1], src), b11 = __shfl_sync(kFull, nb1[1], src);
-            const uint32_t a = seg < 2 ? a0 : a1;
-            const uint32_t bb = seg == 0 ? b00 : seg == 1 ? b01 : seg == 2 ? b10 : b11;
-            warp_union(t.parent, a, p < total ? bb : kNoSlot);
+        for (int u = 0; u < 2; ++u) p[u] = i[u] < nruns ? A::template ld<1>(a.at(i[u])) : 0u;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) v[u] = run_view(sb, rp, W, p[u]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (i[u] >= nruns) break;
+            uint32_t k, end, left;
+            const uint32_t len = run_contacts(v[u], W, i[u], p[u], &k, &end, &left);
+            const typename A::At r = a.at(i[u]);
+            A::template st<1>(r, p[u] | (len << 17));
+            if (k < end)
+                a.set_parent(i[u], k);
+            else if (left != kNoSlot)
+                a.set_parent(i[u], left);
+            if (end > k + 1 || (k < end && left != kNoSlot))
+                A::template st<4>(a.at(atomicAdd(&gs.extras, 1u)), i[u]);
         }
     }
-    __syncthreads();
+    gsync<GT, kWhole>(bar);
 
-    // Charge, size and absolute moments per root.  Each pixel walks to its
-    // root (the smallest slot); a root's own pixel marks it with kMark | its
-    // linear index (the cluster id), the others compress to it.  Moments
-    // accumulate in 32 bits; a cluster heavier than kQSafe32 (possible
-    // overflow) sends the item through the exact 64-bit pass below.
-    for_digis(bw, n, [&](uint32_t, uint32_t w) {
-        const uint32_t r = w & 0xFFu, c = (w >> 8) & 0x1FFu, lin = r * C + c;
-        if (!has_bit(sbits, lin)) return;
-        const uint32_t s = rank_of(sbits, spre, lin);
-        const volatile uint32_t *vp = t.parent;
-        uint32_t x = s, p = vp[s];
-        while (p != x && !(p & kMark)) {
-            x = p;
-            p = vp[x];
-        }
-        t.parent[s] = x == s ? (kMark | lin) : x;
-        const int32_t q = charge(w);
-        const int32_t old = atomicAdd(&t.q[x], q);
-        if (old + q > kQSafe32) bs.heavy = 1;
-        atomicAdd(&t.np[x], 1u);
-        atomicAdd(&t.m[x].x, q * (int32_t)r);
-        atomicAdd(&t.m[x].y, q * (int32_t)c);
-    });
-    __syncthreads();
-    const bool heavy = bs.heavy != 0;
-    if (heavy) {
-        for (uint32_t s = tid; s < S; s += kCCThreads) {
-            t.exact[2 * s] = 0;
-            t.exact[2 * s + 1] = 0;
-        }
-        __syncthreads();
-        for_digis(bw, n, [&](uint32_t, uint32_t w) {
-            const uint32_t r = w & 0xFFu, c = (w >> 8) & 0x1FFu, lin = r * C + c;
-            if (!has_bit(sbits, lin)) return;
-            const uint32_t s = rank_of(sbits, spre, lin);
-            const uint32_t p = t.parent[s];
-            const uint32_t x = (p & kMark) ? s : p;
-            const long long q = charge(w);
-            atomicAdd(&t.exact[2 * x], (unsigned long long)(q * (long long)r));
-            atomicAdd(&t.exact[2 * x + 1], (unsigned long long)(q * (long long)c));
-        });
-        __syncthreads();
-    }
-
-    if (it.label_e) { // loads of four digis (word and index) issued together, as for the bitmaps
-        auto label_of = [&](uint32_t w) -> int32_t {
-            const uint32_t lin = lin_of(w);
-            int32_t lab = -1;
-            if (has_bit(sbits, lin)) {
-                const uint32_t s = rank_of(sbits, spre, lin);
-                const uint32_t p = t.parent[s];
-                const uint32_t x = (p & kMark) ? s : p;
-                const uint32_t px = (p & kMark) ? p : t.parent[x];
-                lab = t.q[x] >= cthr ? (int32_t)(px & ~kMark) : -2;
+    // 6
+    for (uint32_t e = gt, ne = gs.extras; e < ne; e += GT) {
+        const typename A::At re = a.at(e);
+        const uint32_t i = A::template ld<4>(re);
+        A::template st<4>(re, 0);
+        const uint32_t p = A::template ld<1>(a.at(i)) & kRunPos;
+        const RunView v = run_view(sb, rp, W, p);
+        uint32_t k, end, left;
+        run_contacts(v, W, i, p, &k, &end, &left);
+        for (++k;; ++k) { // the first contact is linked already
+            uint32_t y = k;
+            if (k >= end) {
+                if (left == kNoSlot) break;
+                y = left;
+                left = kNoSlot;
             }
-            return lab;
-        };
-#pragma unroll 1
-        for (uint32_t k0 = tid; k0 < n; k0 += 4 * kCCThreads) {
-            uint32_t wv[4], iv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t k = k0 + u * kCCThreads;
-                const bool in = k < n;
-                wv[u] = in ? __ldg(bw + k) : 0u;
-                iv[u] = in ? __ldg(bi + k) : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (k0 + u * kCCThreads < n) it.label_e[iv[u]] = label_of(wv[u]);
+            run_union(a, i, y);
         }
     }
+    gsync<GT, kWhole>(bar);
 
-    // Kept roots in slot order (= id order): every warp takes a contiguous
-    // range of 32-slot chunks and ballots them (into abits, free since the
-    // bitmaps were built), one scan of the warp totals gives each warp's
-    // first ordinal, and the warp walks its chunks again in order.
-    const uint32_t chunks = (S + 31) >> 5;
-    constexpr uint32_t kWarps = kCCThreads / 32;
-    const uint32_t cpw = (chunks + kWarps - 1) / kWarps;
+    // 7: only roots receive sums, so a run's own are still its own; two runs
+    // a thread at a time
+    for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
+        const uint32_t i1 = i0 + GT < nruns ? i0 + GT : i0;
+        uint32_t x0 = i0, x1 = i1, y0 = a.parent(i0), y1 = a.parent(i1);
+        while (y0 != x0 || y1 != x1) {
+            x0 = y0;
+            x1 = y1;
+            y0 = a.parent(x0);
+            y1 = a.parent(x1);
+        }
+        const uint32_t i[2] = {i0, i1}, x[2] = {x0, x1};
+        uint32_t p[2], q[2], mc[2], px[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const typename A::At r = a.at(i[u]);
+            p[u] = A::template ld<1>(r);
+            q[u] = A::template ld<2>(r);
+            mc[u] = A::template ld<3>(r);
+            px[u] = A::template ld<1>(a.at(x[u]));
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (u == 1 && i1 == i0) break;
+            const typename A::At rx = a.at(x[u]);
+            if (x[u] != i[u]) {
+                a.set_parent(i[u], x[u]);
+                if ((int32_t)(A::template add<2>(rx, q[u]) + q[u]) > kQSafe32) gs.heavy = 1;
+                A::template red<3>(rx, mc[u]);
+                A::template red<4>(rx, q[u] * ((p[u] & 0xFFu) - (px[u] & 0xFFu)));
+            } else if ((int32_t)q[u] > kQSafe32) {
+                gs.heavy = 1;
+            }
+            A::add_pixels(rx, p[u] >> 17);
+        }
+    }
+    uint32_t iv[kSingle ? kRunDigis : 1] = {}; // in-event indices for the labels
+    auto index_of = [&](int k, uint32_t j) {
+        if constexpr (kSingle)
+            return iv[k];
+        else
+            return __ldg(bi + (size_t)j * GT);
+    };
+    if constexpr (kSingle) {
+        if (it.label_e || it.label16_e) {
+#pragma unroll
+            for (int k = 0; k < kRunDigis; ++k)
+                if ((uint32_t)k < mine) iv[k] = __ldg(bi + k * GT);
+        }
+    }
+    gsync<GT, kWhole>(bar);
+    const bool heavy = gs.heavy != 0;
+    if (heavy) { // both moments of every root again, in 64 bits
+        for (uint32_t i = gt; i < nruns; i += GT) {
+            exact[2 * (size_t)i] = 0;
+            exact[2 * (size_t)i + 1] = 0;
+        }
+        gsync<GT, kWhole>(bar);
+        for (uint32_t j = 0; j < mine; ++j) {
+            const uint32_t x[4] = {__ldg(bw + (size_t)j * GT), kNoDigi, kNoDigi, kNoDigi};
+            uint32_t run[4], in[4], head[4];
+            runs_of(x, run, in, head);
+            if (!in[0]) continue;
+            const size_t y = a.parent(run[0]);
+            const long long q = (long long)((int32_t)((x[0] >> 17) & 0xFFu) * gain - ped);
+            atomicAdd(&exact[2 * y], (unsigned long long)(q * (long long)(x[0] & 0xFFu)));
+            atomicAdd(&exact[2 * y + 1], (unsigned long long)(q * (long long)((x[0] >> 8) & 0x1FFu)));
+        }
+        gsync<GT, kWhole>(bar);
+    }
+
+    // 8: a warp takes a contiguous range of 32-run chunks
+    constexpr uint32_t kWarps = GT / 32;
+    const uint32_t chunks = (nruns + 31) >> 5, cpw = (chunks + kWarps - 1) / kWarps;
     const uint32_t wc0 = min(chunks, warp * cpw), wc1 = min(chunks, wc0 + cpw);
     uint32_t wrun = 0;
     for (uint32_t ch = wc0; ch < wc1; ++ch) {
-        const uint32_t s = (ch << 5) + lane;
-        const bool kept = s < S && (t.parent[s] & kMark) && t.q[s] >= cthr;
-        const uint32_t bal = __ballot_sync(kFull, kept);
-        if (lane == 0) abits[ch] = bal;
-        wrun += __popc(bal);
+        const uint32_t i = (ch << 5) + lane;
+        bool lead = false;
+        if (i < nruns) {
+            const uint32_t x = a.parent(i);
+            const typename A::At rx = a.at(x);
+            const bool kept = (int32_t)A::template ld<2>(rx) >= cthr;
+            lead = kept && x == i;
+            A::template st<1>(a.at(i), (A::template ld<1>(rx) & kRunPos) | (lead ? kRunKept : kept ? 0u : kRunDropped));
+        }
+        wrun += __popc(__ballot_sync(kFull, lead));
     }
-    if (lane == 0) bs.scan_tmp[warp] = wrun;
-    __syncthreads();
-    uint32_t K, woff;
+    if (lane == 0) gs.tmp[warp] = wrun;
+    gsync<GT, kWhole>(bar);
+    uint32_t K, ord;
     {
-        const uint32_t wt = lane < kWarps ? bs.scan_tmp[lane] : 0u;
+        const uint32_t wt = lane < kWarps ? gs.tmp[lane] : 0u;
         uint32_t ws = wt;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
+        for (int o = 1; o < (int)kWarps; o <<= 1) {
             const uint32_t y = __shfl_up_sync(kFull, ws, o);
             if ((int)lane >= o) ws += y;
         }
         K = __shfl_sync(kFull, ws, kWarps - 1);
-        woff = __shfl_sync(kFull, ws - wt, warp);
+        ord = __shfl_sync(kFull, ws - wt, warp);
     }
-    auto stage = [&](uint32_t s, uint32_t ord) {
-        const int32_t Q = t.q[s];
-        long long mr, mc;
-        if (heavy) {
-            mr = (long long)t.exact[2 * s];
-            mc = (long long)t.exact[2 * s + 1];
-        } else {
-            const int2 mm = t.m[s];
-            mr = mm.x;
-            mc = mm.y;
-        }
-        L.ws.staging.put(it.b + ord, (int32_t)(t.parent[s] & ~kMark), Q, (int32_t)t.np[s], centroid_abs(mr, Q),
-                         centroid_abs(mc, Q));
-        if (it.label16_e) t.np[s] = ord; // read back by the compact labels
-    };
-    // (the compact labels look digis up in the survivor bitmap afterwards, so
-    // with them the kept roots are not compacted into its space)
-    if (S <= 2 * nwords && !it.label16_e) {
-        // compact the kept roots (their slots, by ordinal, into the survivor
-        // bitmap's space, free now) so that every lane stages a cluster
-        uint16_t *kslot = reinterpret_cast<uint16_t *>(sbits);
-        uint32_t run = woff;
-        for (uint32_t ch = wc0; ch < wc1; ++ch) {
-            const uint32_t bal = abits[ch];
-            if ((bal >> lane) & 1u) kslot[run + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)((ch << 5) + lane);
-            run += __popc(bal);
-        }
-        __syncthreads();
-        for (uint32_t o = tid; o < K; o += kCCThreads) stage(kslot[o], o);
-    } else {
-        uint32_t run = woff;
-        for (uint32_t ch = wc0; ch < wc1; ++ch) {
-            const uint32_t bal = abits[ch];
-            if ((bal >> lane) & 1u) stage((ch << 5) + lane, run + __popc(bal & ((1u << lane) - 1u)));
-            run += __popc(bal);
-        }
-    }
-    if (it.label16_e) { // compact labels: the ordinal of the digi's root, kept in t.np by the staging
-        __syncthreads();
-#pragma unroll 1
-        for (uint32_t k0 = tid; k0 < n; k0 += 4 * kCCThreads) {
-            uint32_t wv[4], iv[4];
+
+    // 9: labels (the stores drain behind the staging)
+    if (it.label_e) {
+        each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
+            uint32_t run[4], in[4], head[4], at[4], p[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t k = k0 + u * kCCThreads;
-                const bool in = k < n;
-                wv[u] = in ? __ldg(bw + k) : 0u;
-                iv[u] = in ? __ldg(bi + k) : 0u;
+            for (int u = 0; u < 4; ++u) at[u] = j + u < mine ? index_of(k + u, j + u) : 0u;
+            if constexpr (kSingle) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) run[u] = x[u];
+            } else {
+                runs_of(x, run, in, head);
             }
 #pragma unroll
+            for (int u = 0; u < 4; ++u) p[u] = A::template ld<1>(a.at(run[u] == kNoSlot ? 0u : run[u]));
+#pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (k0 + u * kCCThreads >= n) continue;
-                const uint32_t lin = lin_of(wv[u]);
-                uint16_t v = kLab16Below;
-                if (has_bit(sbits, lin)) {
-                    const uint32_t sl = rank_of(sbits, spre, lin);
-                    const uint32_t p = t.parent[sl];
-                    const uint32_t x = (p & kMark) ? sl : p;
-                    v = t.q[x] >= cthr ? (uint16_t)t.np[x] : kLab16Dropped;
+                const uint32_t id = (p[u] & 0xFFu) * C + ((p[u] >> 8) & 0x1FFu);
+                const int32_t lab = run[u] == kNoSlot ? -1 : p[u] & kRunDropped ? -2 : (int32_t)id;
+                if (j + u < mine) it.label_e[at[u]] = lab;
+            }
+        });
+    }
+    // the kept roots of the warp's chunks, gathered 32 at a time so that
+    // every lane stages a cluster
+    {
+        uint32_t cnt = 0;
+        for (uint32_t ch = wc0;; ++ch) {
+            const bool last = ch >= wc1;
+            if (!last) {
+                const uint32_t i = (ch << 5) + lane;
+                const bool kept = i < nruns && (A::template ld<1>(a.at(i)) & kRunKept);
+                const uint32_t bal = __ballot_sync(kFull, kept);
+                if (kept) wlist[cnt + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)i;
+                cnt += __popc(bal);
+                __syncwarp();
+            }
+            if (cnt >= 32 || (last && cnt > 0)) {
+                if (lane < cnt) {
+                    const uint32_t i = wlist[lane];
+                    const typename A::At r = a.at(i);
+                    const uint32_t p = A::template ld<1>(r);
+                    const int32_t Q = (int32_t)A::template ld<2>(r), np = (int32_t)A::pixels(r);
+                    long long mr, mc;
+                    if (heavy) {
+                        mr = (long long)exact[2 * (size_t)i];
+                        mc = (long long)exact[2 * (size_t)i + 1];
+                    } else {
+                        mr = (int32_t)A::template ld<4>(r) + (int32_t)(p & 0xFFu) * Q;
+                        mc = (int32_t)A::template ld<3>(r);
+                    }
+                    L.ws.staging.put(it.b + ord + lane, (int32_t)((p & 0xFFu) * C + ((p >> 8) & 0x1FFu)), Q, np,
+                                     centroid_abs(mr, Q), centroid_abs(mc, Q));
+                    if (it.label16_e) A::set_ordinal(r, i, ord + lane); // read back by the compact labels
                 }
-                it.label16_e[iv[u]] = v;
+                if (last) break;
+                __syncwarp();
+                const uint32_t v = wlist[32 + lane];
+                __syncwarp();
+                wlist[lane] = (uint16_t)v;
+                __syncwarp();
+                cnt -= 32;
+                ord += 32;
+            } else if (last) {
+                break;
             }
         }
+    }
+    if (it.label16_e) { // compact labels, once every kept root has its ordinal
+        gsync<GT, kWhole>(bar);
+        each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
+            uint32_t run[4], in[4], head[4];
+            if constexpr (kSingle) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) run[u] = x[u];
+            } else {
+                runs_of(x, run, in, head);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (j + u >= mine) break;
+                uint16_t v = kLab16Below;
+                if (run[u] != kNoSlot) {
+                    const typename A::At rx = a.at(a.parent(run[u]));
+                    v = A::template ld<1>(rx) & kRunKept ? (uint16_t)A::pixels(rx) : kLab16Dropped;
+                }
+                it.label16_e[index_of(k + u, j + u)] = v;
+            }
+        });
     }
     return K;
 }
 
-// Zero nw words at p (16-byte stores where p is 16-byte aligned).
-__device__ __forceinline__ void clear_words(uint32_t *p, uint32_t nw)
+// The run tier on run records in global scratch: items with more runs than
+// the shared memory holds (out of line: rare, and its registers are its own).
+template <int GT, bool kWhole>
+__device__ __noinline__ uint32_t run_clusters_big(const Launch &L, const ItemCtx it, uint32_t sb, uint32_t rp,
+                                                  unsigned char *base, uint32_t nruns, GroupShared &gs,
+                                                  uint16_t *wlist, uint32_t gt, uint32_t bar)
 {
-    uint32_t done = 0;
-    if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) {
-        uint4 *v = reinterpret_cast<uint4 *>(p);
-        for (uint32_t i = threadIdx.x; i < nw / 4; i += kCCThreads) v[i] = make_uint4(0, 0, 0, 0);
-        done = nw & ~3u;
+    Runs<true> a;
+    a.base = reinterpret_cast<uint32_t *>(base + (size_t)16 * nruns); // after the 64-bit moments
+    uint32_t w[kRunDigis];
+    return run_clusters<GT, kWhole, true, false>(L, it, sb, rp, a, reinterpret_cast<unsigned long long *>(base), nruns,
+                                                 w, gs, wlist, gt, bar);
+}
+
+// One item of the run tier (phases 1-3, then run_clusters): `mem` is the
+// shared address of the group's slice with room for `cap` runs, `exact` its
+// slice of the 64-bit moments, `part` of `parts` its part of the block's slab
+// of global scratch.  kSingle: the item has at most kRunDigis * GT digis,
+// which stay in registers.  Returns the number of kept clusters (uniform
+// over the group).  An item with an invalid or a duplicated digi flags its
+// event and keeps none.
+template <int GT, bool kWhole, bool kSingle>
+__device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it, uint32_t mem, uint32_t cap,
+                                             unsigned long long *exact, uint32_t part, uint32_t parts,
+                                             GroupShared &gs, uint16_t *wlist, uint32_t gt, uint32_t bar)
+{
+    const uint32_t R = L.g.R, C = L.g.C, W = (C + 31) >> 5, nw4 = run_words(R, C);
+    const int32_t thr = L.g.pixel_thr;
+    const uint32_t n = it.n, mine = n > gt ? (n - gt - 1) / GT + 1 : 0u;
+    const uint32_t *bw = L.ws.bucket_w + it.b + gt;
+    const int32_t gain = it.gain, ped = it.ped;
+    const uint32_t sb = mem, rp = sb + 4 * nw4;
+    const uint32_t ab = mem + (uint32_t)run_fixed_bytes(R, C); // the bitmap of all digis; then the run records
+
+    // 1
+    uint32_t w[kRunDigis];
+    if constexpr (kSingle) load_digis<GT>(w, bw, mine);
+    for (uint32_t i = gt; i < nw4 / 4; i += GT) {
+        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(sb + 16 * i), "r"(0) : "memory");
+        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(ab + 16 * i), "r"(0) : "memory");
     }
-    for (uint32_t i = done + threadIdx.x; i < nw; i += kCCThreads) p[i] = 0;
-}
+    if (gt == 0) {
+        gs.flag = 0;
+        gs.heavy = 0;
+        gs.pixels = 0;
+        gs.extras = 0;
+    }
+    gsync<GT, kWhole>(bar);
 
-// Slot of the first pixel of the horizontal run holding surviving pixel lin,
-// whose row starts at linear index row0; word = sbits[lin >> 5] and base =
-// spre[lin >> 5] are passed in (already loaded by the caller).  The run
-// starts one past the nearest non-surviving pixel to the left of lin, or at
-// the row start.
-__device__ __noinline__ uint32_t run_head_slot_far(const uint32_t *sbits, const uint32_t *spre, uint32_t wi,
-                                                   uint32_t row0);
-__device__ __forceinline__ uint32_t run_head_slot(const uint32_t *sbits, const uint32_t *spre, uint32_t lin,
-                                                  uint32_t row0, uint32_t word, uint32_t base)
-{
-    uint32_t wi = lin >> 5;
-    const uint32_t b = lin & 31;
-    uint32_t lo = row0 > (wi << 5) ? row0 - (wi << 5) : 0u; // first bit of the row in this word
-    uint32_t z = ~word & ((1u << b) - 1u) & ~((1u << lo) - 1u);
-    if (z) return base + __popc(word & ((1u << (32 - __clz(z))) - 1u));
-    if ((wi << 5) + lo == row0) return base + __popc(word & ((1u << lo) - 1u));
-    return run_head_slot_far(sbits, spre, wi, row0);
-}
-
-__device__ __noinline__ uint32_t run_head_slot_far(const uint32_t *sbits, const uint32_t *spre, uint32_t wi,
-                                                   uint32_t row0)
-{
-    uint32_t word, lo, z;
-    for (;;) { // the run continues into the previous word (rare)
-        --wi;
-        word = sbits[wi];
-        lo = row0 > (wi << 5) ? row0 - (wi << 5) : 0u;
-        z = ~word & ~((1u << lo) - 1u);
-        if (z) {
-            const uint32_t hb = 32 - __clz(z);
-            return hb == 32 ? spre[wi + 1] : spre[wi] + __popc(word & ((1u << hb) - 1u));
+    // 2
+    uint32_t valid = 0;
+    each_four<GT, kSingle>(w, bw, mine, [&](int, uint32_t, const uint32_t (&x)[4]) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { // (words past the last digi are invalid, and OR in nothing)
+            const uint32_t r = x[u] & 0xFFu, c = (x[u] >> 8) & 0x1FFu, adc = x[u] >> 17;
+            const bool ok = r < R && c < C && adc - 1u < 255u; // ADC not 0, bits 25-31 clear
+            const uint32_t o = ok ? 4 * (r * W + (c >> 5)) : 0u, bit = ok ? 1u << (c & 31) : 0u;
+            reds_or(ab + o, bit);
+            reds_or(sb + o, (int32_t)adc * gain - ped >= thr ? bit : 0u);
+            valid += ok ? 1u : 0u;
         }
-        if ((wi << 5) + lo == row0) return spre[wi] + __popc(word & ((1u << lo) - 1u));
+    });
+    if (__any_sync(kFull, valid != mine) && (gt & 31) == 0) gs.flag = 1;
+    gsync<GT, kWhole>(bar);
+
+    // 3: runs of a word, counted over contiguous groups of four words a thread
+    const uint32_t per = ((nw4 / 4 + GT - 1) / GT) * 4;
+    const uint32_t w0 = min(nw4, gt * per), w1 = min(nw4, w0 + per);
+    auto four = [](uint32_t addr) {
+        uint4 v;
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                     : "r"(addr)
+                     : "memory");
+        return v;
+    };
+    uint32_t local = 0, pixels = 0;
+    for (uint32_t i = w0; i < w1; i += 4) {
+        const uint4 s = four(sb + 4 * i), d = four(ab + 4 * i);
+        local += __popc(s.x & ~(s.x << 1)) + __popc(s.y & ~(s.y << 1)) + __popc(s.z & ~(s.z << 1)) +
+                 __popc(s.w & ~(s.w << 1));
+        pixels += __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
     }
+    pixels = __reduce_add_sync(kFull, pixels);
+    if ((gt & 31) == 0 && pixels) atomicAdd(&gs.pixels, pixels);
+    uint32_t nruns;
+    uint32_t run = group_exclusive_scan<GT, kWhole>(local, gs.tmp, gt, bar, &nruns);
+    if (gs.flag || gs.pixels != n) { // (uniform: both are settled by the scan's barrier)
+        if (gt == 0) atomicOr(it.err_e, gs.flag ? kErrBadDigi : kErrDup);
+        gsync<GT, kWhole>(bar);
+        return 0;
+    }
+    for (uint32_t i = w0; i < w1; i += 4) {
+        const uint4 s = four(sb + 4 * i);
+        const uint32_t p0 = run, p1 = p0 + __popc(s.x & ~(s.x << 1)), p2 = p1 + __popc(s.y & ~(s.y << 1)),
+                       p3 = p2 + __popc(s.z & ~(s.z << 1));
+        asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(rp + 2 * i), "r"(p0 | (p1 << 16)), "r"(p2 | (p3 << 16))
+                     : "memory");
+        run = p3 + __popc(s.w & ~(s.w << 1));
+    }
+    uint32_t K;
+    if (nruns <= cap) {
+        Runs<false> a;
+        a.base = ab;
+        K = run_clusters<GT, kWhole, false, kSingle>(L, it, sb, rp, a, exact, nruns, w, gs, wlist, gt, bar);
+    } else {
+        uint64_t first, room;
+        if (L.ws.big_arena) { // a slot a run, bump-allocated
+            if (gt == 0) gs.pack_end = atomicAdd(&L.ws.ctl[2], nruns);
+            gsync<GT, kWhole>(bar);
+            first = gs.pack_end;
+            room = first < L.ws.big_slots ? L.ws.big_slots - first : 0;
+        } else { // the group's part of the block's slab
+            room = L.ws.big_slots / parts;
+            first = (uint64_t)blockIdx.x * L.ws.big_slots + part * room;
+        }
+        if (nruns <= room) {
+            K = run_clusters_big<GT, kWhole>(L, it, sb, rp, L.ws.big + first * kBigSlotBytes, nruns, gs, wlist, gt,
+                                             bar);
+        } else {
+            if (gt == 0) atomicOr(&L.ws.ctl[1], kErrCapacity);
+            K = 0;
+        }
+    }
+    gsync<GT, kWhole>(bar); // the slice is free for the next item
+    return K;
 }
 
-// Lock-free union of the trees of a and b by one thread: the larger root is
-// linked under the smaller with atomicMin; a link that finds its root already
-// linked elsewhere retries from the new parent.
-__device__ __noinline__ void uf_union(uint32_t *parent, uint32_t a, uint32_t b)
+// ---- packed tier
+//
+// The small items of a ticket together: up to 1,023 digis of up to 16 items
+// by a group of GT threads, each digi one entry of a hash table keyed by
+// (item, linear pixel index) with four slots a digi.  Entries are packed
+// words, (item << 17 | index) << 11 | surviving << 10 | digi, so that the
+// same word is the table's entry, the digi's union-find key (smaller key =
+// smaller index of the same item, so a root is its cluster's id) and the
+// sort key of the kept clusters.  Phases, one group barrier between them:
+//   0 the digis' items and words; table emptied
+//   1 every valid digi inserted (its pixel already there: a duplicate)
+//   2 survivors linked with their neighbours before them in row-major order:
+//     left and up; without up, upper-left unless the left one survives (it
+//     reaches it) and upper-right.  The first link is one atomicMin on the
+//     digi's own entry, the second a find and link.
+//   3 roots; charge, size and moments per root
+//   4 labels; kept roots appended to their item's list
+//   5 each kept root's ordinal = kept roots of its item with smaller keys;
+//     staging; compact labels
+// What bounds it: latency (a chain of dependent shared-memory accesses a
+// phase), so all the items of a ticket share each phase; the warp-per-item
+// tier this replaced walked all pairs of an item's digis by shuffles.  A table
+// of four slots a digi: with two, a probe of a warp went on for about ten
+// slots.  16 events of 1,856 items (32 digis each): 344 -> 166 us.
+constexpr uint32_t kPackDigis = 1023; // 10 index bits, and the all-ones word stays free for "empty"
+constexpr uint32_t kPackIdx = 1023u;
+constexpr uint32_t kPackEmpty = 0xFFFFFFFFu;
+
+// Home slot of a key in a table of H slots (multiplicative hashing: the high
+// bits of key times the 32-bit golden ratio, scaled to [0, H)).
+__device__ __forceinline__ uint32_t hash_home(uint32_t key, uint32_t H) { return __umulhi(key * 0x9E3779B1u, H); }
+
+// Entry of `key` if it is there and survives the pixel threshold, else
+// kPackEmpty.  The table holds at most H / 4 entries, so a probe always ends.
+__device__ __forceinline__ uint32_t pack_survivor(const uint32_t *table, uint32_t H, uint32_t key)
+{
+    uint32_t s = hash_home(key, H);
+    for (uint32_t i = 0; i < H; ++i) {
+        const uint32_t e = table[s];
+        if (e == kPackEmpty) return kPackEmpty;
+        if ((e >> 11) == key) return (e >> 10) & 1u ? e : kPackEmpty;
+        s = s + 1 == H ? 0u : s + 1;
+    }
+    return kPackEmpty;
+}
+
+// Find on packed keys with path halving (the index of a key is its low
+// bits); parents only ever decrease, as in uf_find_halving.
+template <uint32_t kIdx>
+__device__ __forceinline__ uint32_t key_find(uint32_t *par, uint32_t x)
+{
+    volatile uint32_t *p = par;
+    uint32_t y = p[x & kIdx];
+    while (y != x) {
+        const uint32_t z = p[y & kIdx];
+        if (z != y) p[x & kIdx] = z;
+        x = y;
+        y = z;
+    }
+    return x;
+}
+
+// Lock-free union of the trees of packed keys a and b (the root with the
+// larger key is linked under the smaller with atomicMin; a lost race retries
+// from the new parent), as uf_union on slots.
+template <uint32_t kIdx>
+__device__ __forceinline__ void key_union(uint32_t *par, uint32_t a, uint32_t b)
 {
     for (;;) {
-        a = uf_find_halving(parent, a);
-        b = uf_find_halving(parent, b);
+        a = key_find<kIdx>(par, a);
+        b = key_find<kIdx>(par, b);
         if (a == b) return;
         if (a < b) {
             const uint32_t t = a;
             a = b;
             b = t;
         }
-        const uint32_t old = atomicMin(&parent[a], b);
+        const uint32_t old = atomicMin(&par[a & kIdx], b);
         if (old == a) return;
         a = old;
     }
 }
 
-// Root reached from slot y (its parent not yet known to be the root).
-__device__ __noinline__ uint32_t root_walk_far(const uint32_t *parent, uint32_t y)
+// One warp (lane = its lane): the pack that starts at item i0 of the ticket,
+// as many of the next items of at most pmax digis as pcap holds (larger ones
+// are passed over).  Writes gs.pack (first packed digi of each item from i0
+// on, the total from the pack's end on) and returns the end.
+__device__ __forceinline__ uint32_t plan_pack(GroupShared &gs, uint32_t i0, uint32_t pmax, uint32_t pcap,
+                                              uint32_t lane, uint32_t n_lane)
 {
-    const volatile uint32_t *vp = parent;
-    uint32_t p = vp[y];
-    while (p != y && !(p & kMark)) {
-        y = p;
-        p = vp[y];
+    const uint32_t pn = n_lane <= pmax ? n_lane : 0u;
+    uint32_t incl = pn;
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if ((int)lane >= o) incl += y;
     }
-    return y;
+    const uint32_t fits = __ballot_sync(kFull, lane < (uint32_t)kGroup - i0 && incl <= pcap);
+    const uint32_t cnt = __ffs(~fits) - 1; // leading items that fit (kGroup < 32, so ~fits != 0)
+    const uint32_t total = __shfl_sync(kFull, incl, cnt ? cnt - 1 : 0);
+    if (lane <= (uint32_t)kGroup) gs.pack[lane] = (uint16_t)(lane < cnt ? incl - pn : total);
+    return i0 + cnt;
 }
 
-// Write kept cluster s (a root of tile t) to the item's staging slot ord.
-__device__ __forceinline__ void stage_cluster(const Launch &L, const ItemCtx &it, const Tile &t, bool heavy,
-                                              uint32_t s, uint32_t ord)
+template <int GT, bool kWhole>
+__device__ __forceinline__ void pack_items(const Launch &L, unsigned char *mem, unsigned long long *exact,
+                                           uint32_t i0, uint32_t total, GroupShared &gs, uint32_t gt, uint32_t bar)
 {
-    const int32_t Q = t.q[s];
-    long long mr, mc;
-    if (heavy) {
-        mr = (long long)t.exact[2 * s];
-        mc = (long long)t.exact[2 * s + 1];
-    } else {
-        const int2 mm = t.m[s];
-        mr = mm.x;
-        mc = mm.y;
-    }
-    L.ws.staging.put(it.b + ord, (int32_t)(t.parent[s] & ~kMark), Q, (int32_t)t.np[s], centroid_abs(mr, Q),
-                     centroid_abs(mc, Q));
-    if (it.label16_e) t.np[s] = ord; // read back by the compact labels
-}
-
-// Register tier of the block: items of at most kD * kCCThreads digis (and at
-// most the shared-memory tile).  Thread t holds digis t, t + kCCThreads, ...
-// of the item in registers from the first load to the labels, with its
-// slot (then its root) beside each word, so the bucket is read once per
-// digi (words) plus once (in-event indices, for the labels).
-//
-// Union-find runs on run heads only: every surviving pixel points at the
-// first pixel of its horizontal run (found from the survivor bitmap word by
-// a leading-zero count), and only heads are linked across rows, so finds
-// never visit another run's inner pixels.  Phases, one barrier each:
-//   1 occupancy + survivor bits (duplicates and invalid words flagged)
-//   2 prefix popcount -> slots; parent[s] = s; occupancy bitmap cleared
-//   3 slot and run head of every survivor; accumulators cleared at heads;
-//     one union per stretch of contact with the row above
-//   4 root of every survivor (roots marked with their linear index);
-//     charge, size and moments accumulated per root; survivor bitmap cleared
-//   5 labels; kept roots balloted per 32-slot chunk
-//   6 kept roots compacted in slot (= id) order, then staged
-// Both bitmaps are left zeroed for the next item.
-template <int kD, bool kCompact>
-__device__ uint32_t block_item_reg(const Launch &L, const ItemCtx &it, uint32_t *abits, uint32_t *sbits,
-                                   uint32_t *spre, const Tile &t, BlockShared &bs)
-{
-    const uint32_t R = L.g.R, C = L.g.C, nwords = (R * C + 31) >> 5;
+    const uint32_t pcap = L.cc.pack_digis;
+    constexpr int kP = (kPackDigis + GT) / GT; // digis a thread holds
+    const uint32_t R = L.g.R, C = L.g.C, H = 4 * total;
     const int32_t thr = L.g.pixel_thr, cthr = L.g.cluster_thr;
-    const uint32_t tid = threadIdx.x, n = it.n, lane = tid & 31, warp = tid >> 5;
-    const uint32_t *bw = L.ws.bucket_w + it.b;
-    const int32_t gain = it.gain, ped = it.ped;
+    int2 *m = reinterpret_cast<int2 *>(mem);
+    int32_t *q = reinterpret_cast<int32_t *>(m + pcap);
+    uint32_t *np = reinterpret_cast<uint32_t *>(q + pcap);
+    uint32_t *par = np + pcap;
+    uint32_t *table = par + pcap; // [4 * pcap]; then the kept roots' lists
 
-    // 1: the thread's words, then their bits
-    uint32_t w[kD], s[kD];
+    // 0
+    uint32_t w[kP], ent[kP], idx[kP], li[kP];
 #pragma unroll
-    for (int k = 0; k < kD; ++k) {
-        const uint32_t j = tid + k * kCCThreads;
-        w[k] = j < n ? __ldg(bw + j) : 0u;
+    for (int k = 0; k < kP; ++k) {
+        const uint32_t t = gt + k * GT;
+        w[k] = idx[k] = li[k] = 0;
+        ent[k] = kPackEmpty;
+        if (t < total) {
+            uint32_t i = 0; // the last item whose first digi is at or before t
+#pragma unroll
+            for (uint32_t step = kGroup / 2; step; step >>= 1)
+                if (gs.pack[i + step] <= t) i += step;
+            const uint32_t at = gs.b[i0 + i] + (t - gs.pack[i]);
+            li[k] = i;
+            w[k] = __ldg(L.ws.bucket_w + at);
+            idx[k] = __ldg(L.ws.bucket_i + at);
+        }
     }
-    uint32_t err = 0;
+    for (uint32_t i = gt; i < H; i += GT) table[i] = kPackEmpty;
+    if (gt < (uint32_t)kGroup) gs.tmp[gt] = 0;
+    if (gt == 0) gs.heavy = 0;
+    gsync<GT, kWhole>(bar);
+
+    // 1
 #pragma unroll
-    for (int k = 0; k < kD; ++k) {
-        s[k] = kNoSlot;
-        if (tid + k * kCCThreads < n) {
-            const uint32_t x = w[k], r = x & 0xFFu, c = (x >> 8) & 0x1FFu, adc = (x >> 17) & 0xFFu;
-            if (r >= R || c >= C || adc == 0 || (x >> 25) != 0) {
-                err |= kErrBadDigi;
-            } else {
-                const uint32_t lin = r * C + c, bit = 1u << (lin & 31);
-                if (atomicOr(&abits[lin >> 5], bit) & bit) err |= kErrDup;
-                if ((int32_t)adc * gain - ped >= thr) {
-                    atomicOr(&sbits[lin >> 5], bit);
-                    s[k] = 0;
+    for (int k = 0; k < kP; ++k) {
+        const uint32_t t = gt + k * GT;
+        if (t >= total) continue;
+        const ItemRec &rec = gs.rec[i0 + li[k]];
+        const uint32_t x = w[k], r = x & 0xFFu, c = (x >> 8) & 0x1FFu, adc = x >> 17;
+        if (r >= R || c >= C || adc - 1u >= 255u) { // ADC 0, or any of the bits 25-31
+            atomicOr(L.ws.event_err + rec.e, kErrBadDigi);
+            continue;
+        }
+        const bool surv = (int32_t)adc * rec.gain - rec.ped >= thr;
+        const uint32_t key = (li[k] << 17) | (r * C + c), e = (key << 11) | ((uint32_t)surv << 10) | t;
+        uint32_t s = hash_home(key, H);
+        bool dup = false;
+        for (uint32_t i = 0; i < H; ++i) {
+            const uint32_t old = atomicCAS(&table[s], kPackEmpty, e);
+            if (old == kPackEmpty) break;
+            if ((old >> 11) == key) {
+                dup = true;
+                break;
+            }
+            s = s + 1 == H ? 0u : s + 1;
+        }
+        if (dup) {
+            atomicOr(L.ws.event_err + rec.e, kErrDup);
+        } else if (surv) {
+            par[t] = e;
+            q[t] = 0;
+            np[t] = 0;
+            m[t] = make_int2(0, 0);
+            ent[k] = e;
+        }
+    }
+    gsync<GT, kWhole>(bar);
+
+    // 2
+#pragma unroll
+    for (int k = 0; k < kP; ++k) {
+        if (ent[k] == kPackEmpty) continue;
+        const uint32_t t = gt + k * GT, e = ent[k], key = e >> 11, r = w[k] & 0xFFu, c = (w[k] >> 8) & 0x1FFu;
+        uint32_t e1 = c > 0 ? pack_survivor(table, H, key - 1) : kPackEmpty, e2 = kPackEmpty;
+        if (r > 0) {
+            e2 = pack_survivor(table, H, key - C);
+            if (e2 == kPackEmpty) {
+                if (e1 == kPackEmpty && c > 0) e1 = pack_survivor(table, H, key - C - 1);
+                if (c + 1 < C) e2 = pack_survivor(table, H, key - C + 1);
+            } else if (e1 != kPackEmpty && pack_survivor(table, H, key - C - 1) != kPackEmpty) {
+                e2 = kPackEmpty; // the upper-left pixel already joins left and up
+            }
+        }
+        if (e1 == kPackEmpty) {
+            e1 = e2;
+            e2 = kPackEmpty;
+        }
+        if (e1 != kPackEmpty) {
+            const uint32_t old = atomicMin(&par[t], e1);
+            uint32_t a = e1, b = old; // another digi linked this one first: both trees are one
+            bool more = old != e;
+            for (;;) {
+                if (!more) {
+                    if (e2 == kPackEmpty) break;
+                    a = e;
+                    b = e2;
+                    e2 = kPackEmpty;
                 }
+                more = false;
+                key_union<kPackIdx>(par, a, b);
             }
         }
     }
-    err = __reduce_or_sync(kFull, err);
-    if (err && lane == 0) atomicOr(&bs.flag, err);
-    __syncthreads();
-    const uint32_t flag = bs.flag;
-    if (flag) {
-        if (tid == 0) atomicOr(it.err_e, flag);
-        clear_words(abits, nwords);
-        clear_words(sbits, nwords);
-        __syncthreads();
-        if (tid == 0) bs.flag = 0;
-        return 0;
-    }
+    gsync<GT, kWhole>(bar);
 
-    // 2: exclusive prefix popcount of the survivor bitmap -> dense slots
-    const uint32_t per = (nwords + kCCThreads - 1) / kCCThreads;
-    const uint32_t w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
-    uint32_t local = 0;
-    for (uint32_t i = w0; i < w1; ++i) local += __popc(sbits[i]);
-    uint32_t S;
-    uint32_t run = block_exclusive_scan<kCCThreads>(local, bs.scan_tmp, &S);
-    for (uint32_t i = w0; i < w1; ++i) {
-        spre[i] = run;
-        run += __popc(sbits[i]);
-    }
-    for (uint32_t i = tid; i < S; i += kCCThreads) t.parent[i] = i;
-    __syncthreads();
-
-    // 3: slots, run heads, and the unions with the row above.  For a pixel p
-    // whose upper neighbour U survives, one union per maximal stretch of such
-    // pixels (at the run head, or where the upper-left pixel does not
-    // survive) joins p's run to U's run; a run head whose U is empty checks
-    // its upper-left pixel, a run tail whose U is empty its upper-right one.
-    // Every 8-adjacency between two runs passes through one of these.
-    // union pairs (head slot | target head slot << 16) go to a per-warp list in
-    // the occupancy bitmap (free since phase 2); a full list unions in place
-    const uint32_t seg = nwords / (kCCThreads / 32);
-    uint32_t *plist = abits + warp * seg;
-    uint32_t pcount = 0;
-    const uint32_t lt = (1u << lane) - 1u;
+    // 3
+    bool heavy_here = false;
 #pragma unroll
-    for (int k = 0; k < kD; ++k) {
-        if (k * kCCThreads >= n) break;
-        uint32_t h = 0, th1 = kNoSlot, th2 = kNoSlot;
-        if (s[k] != kNoSlot) {
-            const uint32_t x = w[k], r = x & 0xFFu, c = (x >> 8) & 0x1FFu, lin = r * C + c;
-            const uint32_t wi = lin >> 5, b = lin & 31;
-            const uint32_t word = sbits[wi], base = spre[wi];
-            const uint32_t slot = base + __popc(word & ((1u << b) - 1u));
-            h = run_head_slot(sbits, spre, lin, r * C, word, base);
-            s[k] = slot;
-            if (h != slot) {
-                t.parent[slot] = h;
-            } else {
-                t.q[slot] = 0;
-                t.np[slot] = 0;
-                t.m[slot] = make_int2(0, 0);
-            }
-            if (r > 0) {
-                const uint32_t up = lin - C, wu = up >> 5, bu = up & 31;
-                const uint32_t uword = sbits[wu];
-                const bool U = (uword >> bu) & 1u;
-                const bool UL = c > 0 && (bu > 0 ? ((uword >> (bu - 1)) & 1u) : (sbits[wu - 1] >> 31));
-                const bool UR = c + 1 < C && (bu < 31 ? ((uword >> (bu + 1)) & 1u) : (sbits[wu + 1] & 1u));
-                const bool head = h == slot;
-                const bool tail = c + 1 == C || !(b < 31 ? ((word >> (b + 1)) & 1u) : (sbits[wi + 1] & 1u));
-                uint32_t t1 = kNoSlot, t2 = kNoSlot;
-                if (U) {
-                    if (head || !UL) t1 = up;
-                } else {
-                    if (head && UL) t1 = up - 1;
-                    if (tail && UR) t2 = up + 1;
-                }
-                const uint32_t row0u = (r - 1) * C;
-                if (t1 != kNoSlot) {
-                    const uint32_t tw = t1 >> 5;
-                    th1 = run_head_slot(sbits, spre, t1, row0u, sbits[tw], spre[tw]);
-                }
-                if (t2 != kNoSlot) {
-                    const uint32_t tw = t2 >> 5;
-                    th2 = run_head_slot(sbits, spre, t2, row0u, sbits[tw], spre[tw]);
-                }
+    for (int k = 0; k < kP; ++k) {
+        if (ent[k] == kPackEmpty) continue;
+        const ItemRec &rec = gs.rec[i0 + li[k]];
+        const uint32_t x = w[k], root = key_find<kPackIdx>(par, ent[k]), y = root & kPackIdx;
+        const int32_t qx = (int32_t)((x >> 17) & 0xFFu) * rec.gain - rec.ped;
+        if (atomicAdd(&q[y], qx) + qx > kQSafe32) heavy_here = true;
+        atomicAdd(&np[y], 1u);
+        atomicAdd(&m[y].x, qx * (int32_t)(x & 0xFFu));
+        atomicAdd(&m[y].y, qx * (int32_t)((x >> 8) & 0x1FFu));
+        ent[k] = root;
+    }
+    if (heavy_here) gs.heavy = 1;
+    gsync<GT, kWhole>(bar);
+    const bool heavy = gs.heavy != 0;
+    if (heavy) { // both moments again, in 64 bits
+        for (uint32_t i = gt; i < 2 * total; i += GT) exact[i] = 0;
+        gsync<GT, kWhole>(bar);
+#pragma unroll
+        for (int k = 0; k < kP; ++k) {
+            if (ent[k] == kPackEmpty) continue;
+            const ItemRec &rec = gs.rec[i0 + li[k]];
+            const uint32_t x = w[k], y = ent[k] & kPackIdx;
+            const long long qx = (long long)((int32_t)((x >> 17) & 0xFFu) * rec.gain - rec.ped);
+            atomicAdd(&exact[2 * y], (unsigned long long)(qx * (long long)(x & 0xFFu)));
+            atomicAdd(&exact[2 * y + 1], (unsigned long long)(qx * (long long)((x >> 8) & 0x1FFu)));
+        }
+        gsync<GT, kWhole>(bar);
+    }
+
+    // 4
+    uint32_t kr = 0; // bit k: digi k of this thread is a kept root
+#pragma unroll
+    for (int k = 0; k < kP; ++k) {
+        const uint32_t t = gt + k * GT;
+        if (t >= total) continue;
+        int32_t lab = -1;
+        if (ent[k] != kPackEmpty) {
+            const uint32_t y = ent[k] & kPackIdx;
+            const bool kept = q[y] >= cthr;
+            lab = kept ? (int32_t)((ent[k] >> 11) & 0x1FFFFu) : -2;
+            if (kept && y == t) {
+                table[gs.pack[li[k]] + atomicAdd(&gs.tmp[li[k]], 1u)] = ent[k];
+                kr |= 1u << k;
             }
         }
-        const uint32_t m1 = __ballot_sync(kFull, th1 != kNoSlot), m2 = __ballot_sync(kFull, th2 != kNoSlot);
-        const uint32_t p1 = pcount + __popc(m1 & lt), p2 = pcount + __popc(m1) + __popc(m2 & lt);
-        if (th1 != kNoSlot) {
-            if (p1 < seg) plist[p1] = h | (th1 << 16);
-            else uf_union(t.parent, h, th1);
-        }
-        if (th2 != kNoSlot) {
-            if (p2 < seg) plist[p2] = h | (th2 << 16);
-            else uf_union(t.parent, h, th2);
-        }
-        pcount += __popc(m1) + __popc(m2);
+        if (L.out.label) L.out.label[gs.rec[i0 + li[k]].label_off + idx[k]] = lab;
     }
-    __syncwarp();
-    for (uint32_t i = lane; i < min(pcount, seg); i += 32) {
-        const uint32_t pr = plist[i];
-        uf_union(t.parent, pr & 0xFFFFu, pr >> 16);
-    }
-    __syncthreads();
+    gsync<GT, kWhole>(bar);
 
-    // 4: roots and per-root sums.  Each pixel walks to its root (the smallest
-    // slot); a root's own pixel marks it with kMark | its linear index (the
-    // cluster id), the others point straight at it.  Moments accumulate in
-    // 32 bits; a cluster heavier than kQSafe32 sends the item through the
-    // exact 64-bit pass.
-    clear_words(sbits, nwords);
-    clear_words(abits, nwords);
+    // 5
+    if (gt < (uint32_t)kGroup && gs.pack[gt + 1] > gs.pack[gt])
+        L.ws.cursor[gs.ticket * L.cc.ticket_items + i0 + gt] = gs.tmp[gt];
 #pragma unroll
-    for (int k = 0; k < kD; ++k) {
-        if (s[k] == kNoSlot) continue;
-        const uint32_t slot = s[k];
-        const volatile uint32_t *vp = t.parent;
-        uint32_t y = slot, p = vp[slot];
-        if (p != y && !(p & kMark)) {
-            y = p;
-            p = vp[y];
-            if (p != y && !(p & kMark)) y = root_walk_far(t.parent, p);
+    for (int k = 0; k < kP; ++k) {
+        if (!((kr >> k) & 1u)) continue;
+        const uint32_t t = gt + k * GT, e = ent[k], *list = table + gs.pack[li[k]], nk = gs.tmp[li[k]];
+        uint32_t ord = 0;
+        for (uint32_t i = 0; i < nk; ++i) ord += list[i] < e ? 1u : 0u;
+        const int32_t Q = q[t];
+        long long mr, mc;
+        if (heavy) {
+            mr = (long long)exact[2 * t];
+            mc = (long long)exact[2 * t + 1];
+        } else {
+            const int2 mm = m[t];
+            mr = mm.x;
+            mc = mm.y;
         }
-        const uint32_t x = w[k], r = x & 0xFFu, c = (x >> 8) & 0x1FFu;
-        t.parent[slot] = y == slot ? (kMark | (r * C + c)) : y;
-        s[k] = y;
-        const int32_t q = (int32_t)((x >> 17) & 0xFFu) * gain - ped;
-        const int32_t old = atomicAdd(&t.q[y], q);
-        if (old + q > kQSafe32) bs.heavy = 1;
-        atomicAdd(&t.np[y], 1u);
-        atomicAdd(&t.m[y].x, q * (int32_t)r);
-        atomicAdd(&t.m[y].y, q * (int32_t)c);
+        L.ws.staging.put(gs.b[i0 + li[k]] + ord, (int32_t)((e >> 11) & 0x1FFFFu), Q, (int32_t)np[t],
+                         centroid_abs(mr, Q), centroid_abs(mc, Q));
+        if (L.out.label16) np[t] = ord; // read back by the compact labels
     }
-    __syncthreads();
-    const bool heavy = bs.heavy != 0;
-    if (heavy) {
-        for (uint32_t i = tid; i < S; i += kCCThreads) {
-            t.exact[2 * i] = 0;
-            t.exact[2 * i + 1] = 0;
-        }
-        __syncthreads();
+    if (L.out.label16) {
+        gsync<GT, kWhole>(bar);
 #pragma unroll
-        for (int k = 0; k < kD; ++k) {
-            if (s[k] == kNoSlot) continue;
-            const uint32_t x = w[k], y = s[k];
-            const long long q = (long long)((int32_t)((x >> 17) & 0xFFu) * gain - ped);
-            atomicAdd(&t.exact[2 * y], (unsigned long long)(q * (long long)(x & 0xFFu)));
-            atomicAdd(&t.exact[2 * y + 1], (unsigned long long)(q * (long long)((x >> 8) & 0x1FFu)));
-        }
-        __syncthreads();
-    }
-
-    // 5: labels, and the kept roots of every 32-slot chunk (a warp ballots a
-    // contiguous range of chunks into spre, free since phase 3)
-    if (it.label_e) {
-        const uint32_t *bi = L.ws.bucket_i + it.b;
-        uint32_t iv[kD];
-#pragma unroll
-        for (int k = 0; k < kD; ++k) {
-            const uint32_t j = tid + k * kCCThreads;
-            iv[k] = j < n ? __ldg(bi + j) : 0u;
-        }
-#pragma unroll
-        for (int k = 0; k < kD; ++k) {
-            if (tid + k * kCCThreads >= n) continue;
-            int32_t lab = -1;
-            if (s[k] != kNoSlot) {
-                const uint32_t y = s[k];
-                lab = t.q[y] >= cthr ? (int32_t)(t.parent[y] & ~kMark) : -2;
-            }
-            it.label_e[iv[k]] = lab;
-        }
-    }
-    constexpr uint32_t kWarps = kCCThreads / 32;
-    const uint32_t chunks = (S + 31) >> 5;
-    const uint32_t cpw = (chunks + kWarps - 1) / kWarps;
-    const uint32_t wc0 = min(chunks, warp * cpw), wc1 = min(chunks, wc0 + cpw);
-    uint32_t *ball = spre;
-    uint32_t wrun = 0;
-    for (uint32_t ch = wc0; ch < wc1; ++ch) {
-        const uint32_t sl = (ch << 5) + lane;
-        const bool kept = sl < S && (t.parent[sl] & kMark) && t.q[sl] >= cthr;
-        const uint32_t bal = __ballot_sync(kFull, kept);
-        if (lane == 0) ball[ch] = bal;
-        wrun += __popc(bal);
-    }
-    if (lane == 0) bs.scan_tmp[warp] = wrun;
-    __syncthreads();
-
-    // 6: ordinals of the kept roots, compaction, staging
-    uint32_t K, woff;
-    {
-        const uint32_t wt = lane < kWarps ? bs.scan_tmp[lane] : 0u;
-        uint32_t ws = wt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFull, ws, o);
-            if ((int)lane >= o) ws += y;
-        }
-        K = __shfl_sync(kFull, ws, kWarps - 1);
-        woff = __shfl_sync(kFull, ws - wt, warp);
-    }
-    if (tid == 0) bs.heavy = 0;
-    const uint32_t kslot_off = (chunks + 1) & ~1u; // words of ballots, rounded to keep kslot 4-byte aligned
-    if (K <= 2 * (nwords - min(nwords, kslot_off))) {
-        // compact the kept roots (their slots, by ordinal, after the ballot
-        // words) so that every lane stages a cluster
-        uint16_t *kslot = reinterpret_cast<uint16_t *>(spre + kslot_off);
-        uint32_t o = woff;
-        for (uint32_t ch = wc0; ch < wc1; ++ch) {
-            const uint32_t bal = ball[ch];
-            if ((bal >> lane) & 1u) kslot[o + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)((ch << 5) + lane);
-            o += __popc(bal);
-        }
-        __syncthreads();
-        for (uint32_t i = tid; i < K; i += kCCThreads) stage_cluster(L, it, t, heavy, kslot[i], i);
-    } else {
-        uint32_t o = woff;
-        for (uint32_t ch = wc0; ch < wc1; ++ch) {
-            const uint32_t bal = ball[ch];
-            if ((bal >> lane) & 1u) stage_cluster(L, it, t, heavy, (ch << 5) + lane, o + __popc(bal & ((1u << lane) - 1u)));
-            o += __popc(bal);
-        }
-    }
-    // 7: compact labels, once every kept root's ordinal is in t.np
-    if (kCompact) {
-        __syncthreads();
-        const uint32_t *bi = L.ws.bucket_i + it.b;
-#pragma unroll
-        for (int k = 0; k < kD; ++k) {
-            const uint32_t j = tid + k * kCCThreads;
-            if (j >= n) continue;
+        for (int k = 0; k < kP; ++k) {
+            const uint32_t t = gt + k * GT;
+            if (t >= total) continue;
             uint16_t v = kLab16Below;
-            if (s[k] != kNoSlot) v = t.q[s[k]] >= cthr ? (uint16_t)t.np[s[k]] : kLab16Dropped;
-            it.label16_e[__ldg(bi + j)] = v;
+            if (ent[k] != kPackEmpty) {
+                const uint32_t y = ent[k] & kPackIdx;
+                v = q[y] >= cthr ? (uint16_t)np[y] : kLab16Dropped;
+            }
+            L.out.label16[gs.rec[i0 + li[k]].label_off + idx[k]] = v;
         }
     }
-    return K;
+    gsync<GT, kWhole>(bar); // the slice and the plan are free
 }
 
 // ---------------------------------------------------------------- hash label store
@@ -1597,7 +1714,7 @@ __device__ uint32_t block_item_reg(const Launch &L, const ItemCtx &it, uint32_t 
 // counted per row, the row counts scanned, and each root ranked by column
 // among the kept roots of its own row.
 struct HashMem {
-    int2 *m;           // [cap] root: sum q*row, sum q*col (32-bit, as in the block tiers)
+    int2 *m;           // [cap] root: sum q*row, sum q*col (32-bit, as in the run tier)
     int32_t *q;        // [cap] root: charge
     uint32_t *np;      // [cap] root: pixel count; then its ordinal (compact labels)
     uint32_t *par;     // [cap] packed parent key; then a kept root's row base
@@ -1621,20 +1738,6 @@ __device__ __forceinline__ HashMem hash_mem(unsigned char *dsm, size_t smem, uin
     return h;
 }
 
-// Barrier of the `threads` threads of one group (named barrier `id` >= 1;
-// barrier 0 is the block's __syncthreads).  The compiler's own builtin, not
-// inline assembly: like __syncthreads it is convergent, so the compiler
-// never duplicates it into paths that a warp's threads take apart.
-__device__ __forceinline__ void group_sync(uint32_t id, uint32_t threads)
-{
-    __syncwarp();
-    __barrier_sync_count(id, threads);
-}
-
-// Home slot of pixel `lin` in a table of H slots (multiplicative hashing:
-// the high bits of lin times the 32-bit golden ratio, scaled to [0, H)).
-__device__ __forceinline__ uint32_t hash_home(uint32_t lin, uint32_t H) { return __umulhi(lin * 0x9E3779B1u, H); }
-
 // Table entry of pixel `lin` if it is there and survives the pixel
 // threshold, else 0.  The table holds at most H / 2 entries, so a probe
 // always ends at an empty slot.
@@ -1656,42 +1759,6 @@ __device__ __forceinline__ uint32_t hash_key(uint32_t e)
     return (((e >> 13) - 1u) << kHashIdxBits) | (e & ((1u << kHashIdxBits) - 1u));
 }
 
-// Find on packed keys with path halving (the index of a key is its low
-// kHashIdxBits bits); parents only ever decrease, as in uf_find_halving.
-__device__ __forceinline__ uint32_t hash_find(uint32_t *par, uint32_t x)
-{
-    constexpr uint32_t kIdx = (1u << kHashIdxBits) - 1u;
-    volatile uint32_t *p = par;
-    uint32_t y = p[x & kIdx];
-    while (y != x) {
-        const uint32_t z = p[y & kIdx];
-        if (z != y) p[x & kIdx] = z;
-        x = y;
-        y = z;
-    }
-    return x;
-}
-
-// Lock-free union of the trees of packed keys a and b (the root with the
-// larger key is linked under the smaller with atomicMin; a lost race retries
-// from the new parent), as uf_union on slots.
-__device__ __noinline__ void hash_union(uint32_t *par, uint32_t a, uint32_t b)
-{
-    for (;;) {
-        a = hash_find(par, a);
-        b = hash_find(par, b);
-        if (a == b) return;
-        if (a < b) {
-            const uint32_t t = a;
-            a = b;
-            b = t;
-        }
-        const uint32_t old = atomicMin(&par[a & ((1u << kHashIdxBits) - 1u)], b);
-        if (old == a) return;
-        a = old;
-    }
-}
-
 // One item of at most hash_capacity digis clustered by the calling group
 // (gt = thread index in the group, GT = its size, bar = its barrier id);
 // gflag and gheavy are the group's shared flag words (zero on entry, left
@@ -1707,7 +1774,7 @@ __device__ __noinline__ void hash_union(uint32_t *par, uint32_t a, uint32_t b)
 //     covered with at most two unions a pixel.
 //   3 roots, and charge, size and moments per root (32-bit shared atomics;
 //     a cluster heavier than kQSafe32 sends the item through the exact
-//     64-bit pass, as in the block tiers)
+//     64-bit pass, as in the run tier)
 //   4 labels; kept roots counted per row
 //   5 row bases by a scan of the row counts (each warp scans all 256, eight
 //     a lane); every kept root's column into its row's list
@@ -1802,8 +1869,8 @@ __device__ uint32_t hash_item(const Launch &L, const ItemCtx &it, const HashMem 
                 if (c + 1 < C) e2 = hash_survivor(h.table, H, lin - C + 1);
             }
         }
-        if (e1) hash_union(h.par, rt[k], hash_key(e1));
-        if (e2) hash_union(h.par, rt[k], hash_key(e2));
+        if (e1) key_union<kIdx>(h.par, rt[k], hash_key(e1));
+        if (e2) key_union<kIdx>(h.par, rt[k], hash_key(e2));
     }
     group_sync(bar, GT);
 
@@ -1812,7 +1879,7 @@ __device__ uint32_t hash_item(const Launch &L, const ItemCtx &it, const HashMem 
 #pragma unroll
     for (int k = 0; k < kD; ++k) {
         if (rt[k] == kNoSlot) continue;
-        const uint32_t root = hash_find(h.par, rt[k]), y = root & kIdx;
+        const uint32_t root = key_find<kIdx>(h.par, rt[k]), y = root & kIdx;
         const uint32_t x = w[k];
         const int32_t q = (int32_t)((x >> 17) & 0xFFu) * gain - ped;
         const int32_t old = atomicAdd(&h.q[y], q);
@@ -2023,170 +2090,217 @@ __device__ bool chain_resolve(unsigned long long *chain, uint32_t *frontier, uin
     }
 }
 
-template <int kMinBlocks, bool kHash>
-__global__ void __launch_bounds__(kCCThreads, kMinBlocks) cc_kernel(const Launch L)
+// ---------------------------------------------------------------- clustering kernels
+
+// The next ticket of a group (the first is its own, `first`, dealt over the
+// blocks before the groups of one, the others come from a counter): its items' counts, bucket starts and records,
+// and the plan of its first pack (returned); false when the tickets are out.
+template <int GT, bool kWhole>
+__device__ __forceinline__ bool take_ticket(const Launch &L, GroupShared &gs, uint32_t gt, uint32_t bar,
+                                            uint32_t first)
 {
+    const uint32_t G = L.cc.ticket_items, EM = L.cc.items;
+    if (gt < 32) { // one warp takes the ticket and loads its items
+        uint32_t g32 = 0;
+        if (first != kNoSlot) {
+            g32 = first;
+        } else {
+            if (gt == 0) g32 = L.cc.workers + atomicAdd(&L.ws.ctl[0], 1u);
+            g32 = __shfl_sync(kFull, g32, 0);
+        }
+        if (g32 < L.cc.tickets) {
+            const uint32_t item = g32 * G + gt;
+            const bool ok = gt < G && item < EM;
+            const uint32_t n = ok ? L.ws.count[item] : 0u;
+            if (gt < (uint32_t)kGroup) {
+                gs.n[gt] = n;
+                const uint32_t b = ok ? L.ws.boff[item] : 0u;
+                gs.b[gt] = b;
+                if (ok) {
+                    gs.rec[gt] = make_rec(L, item);
+                    if (n == 0) L.ws.cursor[item] = 0;
+                    if (gt == G - 1 || item == EM - 1) gs.bucket_end = b + n;
+                }
+            }
+            const uint32_t end = plan_pack(gs, 0, L.cc.pack_item, L.cc.pack_digis, gt, n);
+            if (gt == 0) gs.pack_end = end;
+        }
+        if (gt == 0) gs.ticket = g32;
+    }
+    gsync<GT, kWhole>(bar);
+    return gs.ticket < L.cc.tickets;
+}
+
+// Pull the ticket's buckets (words and digi indices, contiguous over its
+// items) into L2, one 128-byte line per thread, so that the items after the
+// first do not wait on DRAM.
+template <int GT>
+__device__ __forceinline__ void prefetch_ticket(const Launch &L, const GroupShared &gs, uint32_t gt)
+{
+    const uint32_t b0 = gs.b[0], digis = gs.bucket_end - b0;
+    for (uint32_t at = 32 * gt; at < digis; at += 32 * GT) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.ws.bucket_w + b0 + at));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.ws.bucket_i + b0 + at));
+    }
+}
+
+// All packs of a ticket (the first is planned by take_ticket).
+template <int GT, bool kWhole>
+__device__ __forceinline__ void pack_ticket(const Launch &L, unsigned char *mem, unsigned long long *exact,
+                                            GroupShared &gs, uint32_t gt, uint32_t bar)
+{
+    for (uint32_t i0 = 0;;) {
+        const uint32_t total = gs.pack[kGroup], end = gs.pack_end;
+        if (total) pack_items<GT, kWhole>(L, mem, exact, i0, total, gs, gt, bar);
+        i0 = end;
+        if (i0 >= L.cc.ticket_items) break;
+        gsync<GT, kWhole>(bar); // the last pack's plan is read
+        if (gt < 32) {
+            const uint32_t e = plan_pack(gs, i0, L.cc.pack_item, L.cc.pack_digis, gt,
+                                         i0 + gt < (uint32_t)kGroup ? gs.n[i0 + gt] : 0u);
+            if (gt == 0) gs.pack_end = e;
+        }
+        gsync<GT, kWhole>(bar);
+    }
+}
+
+// The clustering kernel, persistent: kGroups groups of kThreads / kGroups
+// threads a block, each with its own slice of the block's shared memory, its
+// own named barrier and its own tickets of consecutive items, so that one
+// group's barriers and loads overlap the others' work.  Items of at most
+// cc.pack_item digis go through the packed tier, a ticket's worth at a time,
+// the others through the run tier one by one.  (A bitmap costs its clearing
+// and scan whatever it holds, a hash probe costs each digi: the two break
+// even at a few hundred digis; 256 is the better line for items of 1,600 on
+// average, 256 and 512 the same for items of 32.)  Items of more than
+// cc.large_digis digis (scan_kernel lists them), whose runs would not fit a
+// slice, come first: the whole block takes them one at a time, on all of its
+// shared memory.
+template <int kThreads, int kGroups, int kMinBlocks>
+__global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_constant__ Launch L)
+{
+    constexpr int GT = kThreads / kGroups;
+    constexpr bool kWhole = kGroups == 1;
     extern __shared__ __align__(16) unsigned char dsm[];
-    __shared__ BlockShared bs;
+    __shared__ GroupShared s_gs[kGroups];
+    __shared__ uint16_t s_wlist[kThreads / 32][64];
     pdl_wait();
     pdl_trigger();
-    __shared__ uint32_t s_n[kGroup], s_b[kGroup];
-    __shared__ ItemRec s_rec[kGroup];
-    __shared__ uint32_t s_ticket;
+    if (L.ws.ctl[1] & kErrBadOffsets) return;
 
-    const uint32_t R = L.g.R, C = L.g.C, M = L.g.M;
-    const uint32_t nwords = (R * C + 31) >> 5;
     const uint32_t tid = threadIdx.x;
-    const uint32_t T = L.tune.tile_slots, warp_max = L.tune.warp_max;
-    Tile sm;
-    sm.q = reinterpret_cast<int32_t *>(dsm);
-    sm.np = reinterpret_cast<uint32_t *>(sm.q + T);
-    sm.m = reinterpret_cast<int2 *>(sm.np + T);
-    sm.parent = reinterpret_cast<uint32_t *>(sm.m + T);
-    sm.exact = L.ws.exact + (size_t)blockIdx.x * 2 * T;
-    uint32_t *abits = sm.parent + T;
-    uint32_t *sbits = abits + nwords;
-    uint32_t *spre = sbits + nwords;
+    uint16_t *wlist = s_wlist[tid >> 5];
+    unsigned long long *exact = L.ws.exact + (size_t)blockIdx.x * 2 * L.cc.exact_slots;
+    uint32_t *kcount = L.ws.cursor; // each item's count of kept clusters
 
-    const uint64_t EM = (uint64_t)L.E * M;
-    const uint32_t G = ticket_items(EM, gridDim.x, L.tune.ticket_max, L.N);
-    const uint64_t ngroups = (EM + G - 1) / G;
-    // items of the register tier and the hash store: kD digis a thread
-    constexpr int kD = cc_digis_per_thread(kMinBlocks);
-    // hash store: items of warp_max < n <= hash_max go to groups of GT
-    // threads (0 with the bitmap store)
-    const uint32_t GT = L.tune.item_threads, hgroups = (uint32_t)kCCThreads / GT;
-    const uint32_t hash_max = kHash ? hash_capacity(cc_smem_bytes(R, C, T), T, GT, (uint32_t)kD) : 0u;
-    const uint32_t gid = tid / GT, gtid = tid - gid * GT;
-    const HashMem hm = hash_mem(dsm, cc_smem_bytes(R, C, T), hgroups, gid, hash_max, sm.exact);
+    if constexpr (!kWhole) {
+        const uint32_t nlarge = L.ws.ctl[5];
+        if (nlarge) {
+            GroupShared &gs = s_gs[0];
+            for (;;) {
+                if (tid == 0) {
+                    const uint32_t t = atomicAdd(&L.ws.ctl[7], 1u);
+                    gs.ticket = t;
+                    if (t < nlarge) {
+                        const uint32_t item = L.ws.large[t];
+                        gs.pack_end = item;
+                        gs.n[0] = L.ws.count[item];
+                        gs.b[0] = L.ws.boff[item];
+                        gs.rec[0] = make_rec(L, item);
+                    }
+                }
+                __syncthreads();
+                if (gs.ticket >= nlarge) break;
+                const ItemCtx it = make_item(L, gs.rec[0], gs.b[0], gs.n[0]);
+                const uint32_t item = gs.pack_end;
+                const uint32_t K = run_item<kThreads, true, false>(L, it, smem_addr(dsm), L.cc.whole_runs, exact, 0, 1,
+                                                                     gs, wlist, tid, 0);
+                if (tid == 0) kcount[item] = K;
+                __syncthreads();
+            }
+        }
+        __syncthreads();
+    }
+
+    const uint32_t gid = tid / GT, gt = tid - gid * GT, bar = 1 + gid;
+    unsigned char *mem = dsm + L.cc.slice * gid;
+    exact += (size_t)2 * L.cc.runs * gid;
+    GroupShared &gs = s_gs[gid];
+    for (uint32_t first = gid * gridDim.x + blockIdx.x; take_ticket<GT, kWhole>(L, gs, gt, bar, first);
+         first = kNoSlot) {
+        prefetch_ticket<GT>(L, gs, gt);
+        pack_ticket<GT, kWhole>(L, mem, exact, gs, gt, bar);
+        for (uint32_t i = 0; i < L.cc.ticket_items; ++i) {
+            const uint32_t n = gs.n[i];
+            if (n <= L.cc.pack_item || (!kWhole && n > L.cc.large_digis)) continue;
+            const ItemCtx it = make_item(L, gs.rec[i], gs.b[i], n);
+            const uint32_t K = n <= (uint32_t)(kRunDigis * GT)
+                                   ? run_item<GT, kWhole, true>(L, it, smem_addr(mem), L.cc.runs, exact, gid, kGroups,
+                                                                gs, wlist, gt, bar)
+                                   : run_item<GT, kWhole, false>(L, it, smem_addr(mem), L.cc.runs, exact, gid, kGroups,
+                                                                 gs, wlist, gt, bar);
+            if (gt == 0) kcount[gs.ticket * L.cc.ticket_items + i] = K;
+        }
+        gsync<GT, kWhole>(bar); // the ticket's record is free
+    }
+}
+
+// The clustering kernel with the hash label store (tuning label_store =
+// kStoreHash): one ticket a block at a time; items of more than warp_max digis
+// and within the store's capacity go to groups of item_threads threads,
+// smaller ones through the packed tier and larger ones through the run tier,
+// both by the whole block.
+template <int kMinBlocks>
+__global__ void __launch_bounds__(kCCThreads, kMinBlocks) cc_hash_kernel(const __grid_constant__ Launch L)
+{
+    constexpr int GT0 = kCCThreads;
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ GroupShared gs;
     __shared__ uint32_t s_gflag[kCCThreads / 128], s_gheavy[kCCThreads / 128];
-    if (kHash && tid < (uint32_t)(kCCThreads / 128)) {
+    pdl_wait();
+    pdl_trigger();
+    if (L.ws.ctl[1] & kErrBadOffsets) return;
+
+    const uint32_t T = L.tune.tile_slots, tid = threadIdx.x;
+    constexpr int kD = cc_digis_per_thread(kMinBlocks);
+    const size_t smem = L.cc.slice;
+    // the run tier's warp lists, at the end of the dynamic shared memory
+    uint16_t *wlist = reinterpret_cast<uint16_t *>(dsm + (smem & ~(size_t)1) - kHashListBytes) + 64 * (tid >> 5);
+    unsigned long long *exact = L.ws.exact + (size_t)blockIdx.x * 2 * L.cc.exact_slots;
+    const uint32_t GT = L.tune.item_threads, hgroups = (uint32_t)kCCThreads / GT;
+    const uint32_t hash_max = hash_capacity(smem, T, GT, (uint32_t)kD);
+    const uint32_t gid = tid / GT, gtid = tid - gid * GT;
+    const HashMem hm = hash_mem(dsm, smem, hgroups, gid, hash_max, exact);
+    if (tid < (uint32_t)(kCCThreads / 128)) {
         s_gflag[tid] = 0;
         s_gheavy[tid] = 0;
     }
-    if (tid == 0) {
-        bs.flag = 0;
-        bs.heavy = 0;
-    }
-    // block-tier items start from zeroed bitmaps and leave them zeroed
-    clear_words(abits, nwords);
-    clear_words(sbits, nwords);
-    if (L.ws.ctl[1] & kErrBadOffsets) return;
-    // each item's count of kept clusters goes to kcount[item]; the ordered
-    // output is written by offsets_kernel and copy_kernel
     uint32_t *kcount = L.ws.cursor;
-    for (;;) {
-        {
-            if (tid == 0) s_ticket = atomicAdd(&L.ws.ctl[0], 1u);
-            __syncthreads();
-            const uint64_t g = s_ticket;
-            if (g >= ngroups) break;
-            {
-                const uint64_t item0 = g * G;
-                if (tid < (uint32_t)kGroup) {
-                    const uint64_t item = item0 + tid;
-                    const bool ok = tid < G && item < EM;
-                    s_n[tid] = ok ? L.ws.count[item] : 0u;
-                    s_b[tid] = ok ? L.ws.boff[item] : 0u;
-                    if (ok) {
-                        s_rec[tid] = make_rec(L, item);
-                        if (s_n[tid] == 0) kcount[item] = 0;
-                    }
-                }
-                __syncthreads();
-                {   // pull the ticket's buckets (words and digi indices, contiguous
-                    // over its items) into L2, one 128-byte line per thread, so
-                    // that the items after the first do not wait on DRAM
-                    uint32_t last = 0;
-                    for (uint32_t i = 0; i < G; ++i)
-                        if (s_n[i]) last = i;
-                    const uint64_t b0 = s_b[0], b1 = (uint64_t)s_b[last] + s_n[last];
-                    const uint32_t lines = b1 > b0 ? (uint32_t)(((b1 - b0) * 4 + 127) / 128) : 0u;
-                    for (uint32_t li = tid; li < 2 * lines; li += kCCThreads) {
-                        const bool second = li >= lines;
-                        const uint32_t *base = second ? L.ws.bucket_i : L.ws.bucket_w;
-                        const uint64_t off = b0 * 4 + (uint64_t)(second ? li - lines : li) * 128; // inside the array
-                        if (off < b1 * 4)
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const char *>(base) + off));
-                    }
-                }
-                {   // warp tier: one warp per small item
-                    const uint32_t wi = tid >> 5;
-                    const uint32_t n = s_n[wi];
-                    if (n > 0 && n <= warp_max) {
-                        const ItemCtx it = make_item(L, s_rec[wi], s_b[wi], n);
-                        const uint32_t K = n <= 32 ? warp_item<1>(L, it) : warp_item<2>(L, it);
-                        if ((tid & 31) == 0) kcount[item0 + wi] = K;
-                    }
-                }
-                __syncthreads();
-                if (kHash && hash_max > warp_max) {
-                    // hash store: the items above the warp tier and within
-                    // its capacity, dealt round-robin to the block's groups
-                    uint32_t nh = 0;
-                    for (int i = 0; i < kGroup; ++i) {
-                        const uint32_t n = s_n[i];
-                        if (n <= warp_max || n > hash_max) continue;
-                        if (nh++ % hgroups != gid) continue;
-                        const ItemCtx it = make_item(L, s_rec[i], s_b[i], n);
-                        const uint32_t K = hash_item<kD>(L, it, hm, gtid, GT, 1 + gid, &s_gflag[gid], &s_gheavy[gid]);
-                        if (gtid == 0) kcount[item0 + i] = K;
-                    }
-                    if (nh) { // block-uniform: the slices covered the bitmaps, which the block tier wants zeroed
-                        __syncthreads();
-                        clear_words(abits, nwords);
-                        clear_words(sbits, nwords);
-                        __syncthreads();
-                    }
-                }
-                for (int i = 0; i < kGroup; ++i) { // block tier: larger items one at a time
-                    const uint32_t n = s_n[i];
-                    if (n <= warp_max || n <= hash_max) continue;
-                    const ItemCtx it = make_item(L, s_rec[i], s_b[i], n);
-                    uint32_t K;
-                    if (n <= (uint32_t)kD * kCCThreads && n <= T) {
-                        // (compact labels keep each digi's root slot live through the
-                        // staging: a separate instance, so the other keeps its registers)
-                        K = it.label16_e ? block_item_reg<kD, true>(L, it, abits, sbits, spre, sm, bs)
-                                         : block_item_reg<kD, false>(L, it, abits, sbits, spre, sm, bs);
-                    } else if (n <= T) {
-                        K = block_item<false>(L, it, abits, sbits, spre, sm, bs);
-                    } else {
-                        if (tid == 0) {
-                            bs.big_off = 0;
-                            if (L.ws.big_arena) bs.big_off = atomicAdd(&L.ws.ctl[2], n);
-                        }
-                        __syncthreads();
-                        const uint64_t cap = L.ws.big_arena ? (uint64_t)n : L.ws.big_slots;
-                        unsigned char *base =
-                            L.ws.big + (L.ws.big_arena ? (uint64_t)bs.big_off : (uint64_t)blockIdx.x * L.ws.big_slots) *
-                                           kBigSlotBytes;
-                        const bool fits = L.ws.big_arena ? (uint64_t)bs.big_off + n <= L.ws.big_slots
-                                                         : (uint64_t)min(n, R * C) <= L.ws.big_slots;
-                        Tile gt;
-                        gt.q = reinterpret_cast<int32_t *>(base);
-                        gt.np = reinterpret_cast<uint32_t *>(gt.q + cap);
-                        gt.exact = reinterpret_cast<unsigned long long *>(gt.np + cap);
-                        gt.m = reinterpret_cast<int2 *>(gt.exact + 2 * cap);
-                        gt.parent = reinterpret_cast<uint32_t *>(gt.m + cap);
-                        K = fits ? block_item<true>(L, it, abits, sbits, spre, gt, bs) : 0u;
-                        if (!fits && tid == 0) atomicOr(&L.ws.ctl[1], kErrCapacity);
-                    }
-                    if (n > (uint32_t)kD * kCCThreads || n > T) {
-                        // the general tier leaves its bitmaps (and scratch in them) behind
-                        __syncthreads();
-                        clear_words(abits, nwords);
-                        clear_words(sbits, nwords);
-                        if (tid == 0) {
-                            bs.flag = 0;
-                            bs.heavy = 0;
-                        }
-                    }
-                    if (tid == 0) kcount[item0 + i] = K;
-                    __syncthreads();
-                }
-            }
+    for (uint32_t first = blockIdx.x; take_ticket<GT0, true>(L, gs, tid, 0, first); first = kNoSlot) {
+        prefetch_ticket<GT0>(L, gs, tid);
+        pack_ticket<GT0, true>(L, dsm, exact, gs, tid, 0);
+        const uint32_t item0 = gs.ticket * L.cc.ticket_items;
+        // the items above the packed tier and within the store's capacity,
+        // dealt round-robin to the block's groups
+        uint32_t nh = 0;
+        for (uint32_t i = 0; i < L.cc.ticket_items; ++i) {
+            const uint32_t n = gs.n[i];
+            if (n <= L.cc.pack_item || n > hash_max) continue;
+            if (nh++ % hgroups != gid) continue;
+            const ItemCtx it = make_item(L, gs.rec[i], gs.b[i], n);
+            const uint32_t K = hash_item<kD>(L, it, hm, gtid, GT, 1 + gid, &s_gflag[gid], &s_gheavy[gid]);
+            if (gtid == 0) kcount[item0 + i] = K;
         }
+        __syncthreads();
+        for (uint32_t i = 0; i < L.cc.ticket_items; ++i) {
+            const uint32_t n = gs.n[i];
+            if (n <= L.cc.pack_item || n <= hash_max) continue;
+            const ItemCtx it = make_item(L, gs.rec[i], gs.b[i], n);
+            const uint32_t K = run_item<GT0, true, false>(L, it, smem_addr(dsm), L.cc.runs, exact, 0, 1, gs,
+                                                          wlist, tid, 0);
+            if (tid == 0) kcount[item0 + i] = K;
+        }
+        __syncthreads(); // the ticket's record is free
     }
 }
 
@@ -2447,8 +2561,19 @@ size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t 
     w.staging.npix = reinterpret_cast<int32_t *>(take(4ull * N));
     w.staging.x = reinterpret_cast<float *>(take(4ull * N));
     w.staging.y = reinterpret_cast<float *>(take(4ull * N));
-    w.exact = reinterpret_cast<unsigned long long *>(take(16ull * tune.tile_slots * (cc_grid > 0 ? cc_grid : 1)));
-    const uint64_t slab_slots = std::min<uint64_t>((uint64_t)R * C, N);
+    w.large = reinterpret_cast<uint32_t *>(take(4ull * EM));
+    const bool hash = tune.label_store == kStoreHash;
+    const uint32_t groups = hash ? 1u : run_groups(tune.blocks_per_sm);
+    w.exact = reinterpret_cast<unsigned long long *>(
+        take(16ull * (hash ? tune.tile_slots : run_exact_slots(R, C, tune.tile_slots, groups)) *
+             (cc_grid > 0 ? cc_grid : 1)));
+    // a slab holds any item, and an item of each group at once (a group's
+    // part holds the largest item it takes: see large_digis)
+    const uint64_t slab_slots =
+        std::max<uint64_t>(std::min<uint64_t>((uint64_t)R * C, N),
+                 groups > 1 ? groups * std::min<uint64_t>(std::min<uint64_t>((uint64_t)R * C, N),
+                                                          large_digis(R, C, tune))
+                            : 0ull);
     const uint64_t slab_total = slab_slots * (uint64_t)(cc_grid > 0 ? cc_grid : 1);
     w.big_arena = N <= slab_total ? 1 : 0;
     w.big_slots = w.big_arena ? N : slab_slots;
@@ -2461,10 +2586,11 @@ size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t 
 namespace {
 
 // Largest tile (a multiple of 256 slots, at most max_slots) with which
-// `blocks` blocks of `kern` stay resident on one SM; 0 if none does.  Also
-// raises the kernel's dynamic shared memory limit to what that tile needs.
-template <class K>
-cudaError_t fit_tile(K kern, int device, int blocks, uint32_t R, uint32_t C, uint32_t max_slots, uint32_t *tile)
+// `blocks` blocks of `kern` (`threads` threads, bytes(tile) of dynamic shared
+// memory) stay resident on one SM; 0 if none does.  Also raises the kernel's
+// dynamic shared memory limit to what that tile needs.
+template <class K, class F>
+cudaError_t fit_tile(K kern, int device, int blocks, int threads, F bytes, uint32_t max_slots, uint32_t *tile)
 {
     *tile = 0;
     int optin = 0;
@@ -2475,13 +2601,13 @@ cudaError_t fit_tile(K kern, int device, int blocks, uint32_t R, uint32_t C, uin
     if (err != cudaSuccess) return err;
     const size_t limit = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
     uint32_t t = max_slots;
-    while (t >= 256 && cc_smem_bytes(R, C, t) > limit) t -= 256;
+    while (t >= 256 && bytes(t) > limit) t -= 256;
     if (t < 256) return cudaSuccess;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cc_smem_bytes(R, C, t));
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(t));
     if (err != cudaSuccess) return err;
     for (; t >= 256; t -= 256) {
         int nb = 0;
-        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, kCCThreads, cc_smem_bytes(R, C, t));
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, threads, bytes(t));
         if (err != cudaSuccess) return err;
         if (nb >= blocks) {
             *tile = t;
@@ -2500,18 +2626,54 @@ cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4
     err = cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
     if (err != cudaSuccess) return err;
     max_tile[0] = hash_tile[0] = 0;
-    // the bitmap and hash label stores are separate instances of the kernel
-    err = fit_tile(cc_kernel<1, false>, device, 1, R, C, kMaxTileSlots, &max_tile[1]);
-    if (err == cudaSuccess) err = fit_tile(cc_kernel<1, true>, device, 1, R, C, kMaxTileSlots, &hash_tile[1]);
-    if (err == cudaSuccess) err = fit_tile(cc_kernel<2, false>, device, 2, R, C, kSmemSlots, &max_tile[2]);
-    if (err == cudaSuccess) err = fit_tile(cc_kernel<2, true>, device, 2, R, C, kSmemSlots, &hash_tile[2]);
-    if (err == cudaSuccess) err = fit_tile(cc_kernel<3, false>, device, 3, R, C, kSmemSlots, &max_tile[3]);
-    if (err == cudaSuccess) err = fit_tile(cc_kernel<3, true>, device, 3, R, C, kSmemSlots, &hash_tile[3]);
+    auto run_bytes = [&](uint32_t groups) { return [=](uint32_t t) { return run_smem_bytes(R, C, t, groups); }; };
+    auto hash_bytes = [&](uint32_t t) { return hash_smem_bytes(R, C, t); };
+    err = fit_tile(cc_kernel<kRunThreads1, kRunGroups1, 1>, device, 1, kRunThreads1, run_bytes(kRunGroups1),
+                   kMaxTileSlots, &max_tile[1]);
+    if (err == cudaSuccess)
+        err = fit_tile(cc_kernel<kRunThreads2, kRunGroups2, 2>, device, 2, kRunThreads2, run_bytes(kRunGroups2),
+                       kSmemSlots, &max_tile[2]);
+    if (err == cudaSuccess)
+        err = fit_tile(cc_kernel<kRunThreads3, kRunGroups3, 3>, device, 3, kRunThreads3, run_bytes(kRunGroups3),
+                       kSmemSlots, &max_tile[3]);
+    if (err == cudaSuccess)
+        err = fit_tile(cc_hash_kernel<1>, device, 1, kCCThreads, hash_bytes, kMaxTileSlots, &hash_tile[1]);
+    if (err == cudaSuccess)
+        err = fit_tile(cc_hash_kernel<2>, device, 2, kCCThreads, hash_bytes, kSmemSlots, &hash_tile[2]);
+    if (err == cudaSuccess)
+        err = fit_tile(cc_hash_kernel<3>, device, 3, kCCThreads, hash_bytes, kSmemSlots, &hash_tile[3]);
+    // one tile for both label stores, so that a setting's store can be changed alone
+    for (int b = 1; b <= 3; ++b)
+        if (hash_tile[b] && hash_tile[b] < max_tile[b]) max_tile[b] = hash_tile[b];
     return err;
 }
 
 const char *const kKernelNames[kNumKernels] = {"hist_kernel", "scan_kernel",    "scatter_kernel",
                                                 "cc_kernel",   "offsets_kernel", "copy_kernel"};
+
+// Sizes of a launch's clustering kernel: its tickets, and what a group's
+// slice of the shared memory (and the whole of it) holds.
+static ClusterPlan cluster_plan(const Launch &L)
+{
+    const uint32_t R = L.g.R, C = L.g.C, T = L.tune.tile_slots;
+    const bool hash = L.tune.label_store == kStoreHash;
+    const uint32_t groups = hash ? 1u : run_groups(L.tune.blocks_per_sm);
+    ClusterPlan p;
+    p.items = (uint32_t)((uint64_t)L.E * L.g.M); // at most 2^31 (checked by the callers)
+    p.ticket_items = ticket_items(p.items, (unsigned)L.cc_grid * groups, L.tune.ticket_max, L.N);
+    p.workers = (uint32_t)L.cc_grid * groups;
+    p.tickets = (p.items + p.ticket_items - 1) / p.ticket_items;
+    p.smem = (uint32_t)(hash ? hash_smem_bytes(R, C, T) : run_smem_bytes(R, C, T, groups));
+    p.slice = (p.smem / groups) & ~15u;
+    p.whole_runs = run_capacity(p.smem, R, C);
+    p.runs = run_capacity(p.slice, R, C);
+    p.exact_slots = hash ? T : run_exact_slots(R, C, T, groups);
+    if (hash) p.runs = std::min(run_capacity(p.slice - kHashListBytes, R, C), T);
+    p.pack_digis = pack_capacity(p.slice, p.runs);
+    p.pack_item = std::min(hash ? L.tune.warp_max : pack_max(L.tune.warp_max), p.pack_digis);
+    p.large_digis = large_digis(R, C, L.tune);
+    return p;
+}
 
 // Launch `kern` on `stream` as a programmatic dependent of the kernel before it.
 template <typename K>
@@ -2530,16 +2692,17 @@ cudaError_t launch_dependent(K kern, unsigned grid, unsigned block, size_t smem,
     return cudaLaunchKernelEx(&cfg, kern, L);
 }
 
-cudaError_t launch_reconstruct(const Launch &L, cudaStream_t stream, uint64_t *kernel_count, cudaEvent_t *marks)
+cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *kernel_count, cudaEvent_t *marks)
 {
     NvtxRange range("hp_launch_reconstruct");
+    Launch L = in;
+    L.cc = cluster_plan(L);
     cudaError_t err = cudaMemsetAsync(L.ws.ctl, 0, L.ws.zero_bytes, stream);
     if (err != cudaSuccess) return err;
     auto mark = [&](int i) {
         if (marks && err == cudaSuccess) err = cudaEventRecord(marks[i], stream);
     };
     uint64_t nk = 0;
-    const uint64_t nchunks = (L.N + kChunk - 1) / kChunk;
     // persistent histogram and scatter over the same contiguous ranges
     const unsigned hist_grid = bucket_grid(L.N, L.sm_count), scat_grid = hist_grid; // the same ranges
     mark(0);
@@ -2556,18 +2719,20 @@ cudaError_t launch_reconstruct(const Launch &L, cudaStream_t stream, uint64_t *k
         ++nk;
     }
     mark(3);
-    const size_t cc_smem = cc_smem_bytes(L.g.R, L.g.C, L.tune.tile_slots);
     if (err == cudaSuccess) {
-        const bool hash = L.tune.label_store == kStoreHash;
-        if (L.tune.blocks_per_sm >= 3)
-            err = launch_dependent(hash ? cc_kernel<3, true> : cc_kernel<3, false>, L.cc_grid, kCCThreads, cc_smem,
-                                   stream, L);
-        else if (L.tune.blocks_per_sm == 1)
-            err = launch_dependent(hash ? cc_kernel<1, true> : cc_kernel<1, false>, L.cc_grid, kCCThreads, cc_smem,
-                                   stream, L);
+        const uint32_t b = L.tune.blocks_per_sm;
+        if (L.tune.label_store == kStoreHash)
+            err = launch_dependent(b >= 3 ? cc_hash_kernel<3> : b == 2 ? cc_hash_kernel<2> : cc_hash_kernel<1>,
+                                   L.cc_grid, kCCThreads, L.cc.smem, stream, L);
+        else if (b >= 3)
+            err = launch_dependent(cc_kernel<kRunThreads3, kRunGroups3, 3>, L.cc_grid, kRunThreads3,
+                                   L.cc.smem, stream, L);
+        else if (b == 2)
+            err = launch_dependent(cc_kernel<kRunThreads2, kRunGroups2, 2>, L.cc_grid, kRunThreads2,
+                                   L.cc.smem, stream, L);
         else
-            err = launch_dependent(hash ? cc_kernel<2, true> : cc_kernel<2, false>, L.cc_grid, kCCThreads, cc_smem,
-                                   stream, L);
+            err = launch_dependent(cc_kernel<kRunThreads1, kRunGroups1, 1>, L.cc_grid, kRunThreads1,
+                                   L.cc.smem, stream, L);
     }
     ++nk;
     mark(4);

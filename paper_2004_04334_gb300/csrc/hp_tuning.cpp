@@ -21,8 +21,7 @@ Shape shape_with(const hp_ctx *ctx, uint32_t E, uint64_t N, const hp::Tuning &t)
 {
     Shape sh;
     sh.tune = t;
-    // enough blocks for tickets of the smallest size (see ticket_items): one
-    // item for block-tier items, four for warp-tier ones
+    // enough blocks for tickets of the smallest size (see ticket_items)
     const uint64_t EM = (uint64_t)E * ctx->cfg.n_modules;
     const uint64_t groups = hp::large_items(N, EM) ? EM : (EM + 3) / 4;
     const uint64_t resident = (uint64_t)ctx->sm_count * t.blocks_per_sm;
