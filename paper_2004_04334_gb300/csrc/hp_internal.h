@@ -230,7 +230,7 @@ constexpr size_t kBigSlotBytes = 8 + 16 + 8 + 4 + 4;
 
 // Dynamic shared memory of a clustering block of the hash label store: 20
 // bytes a slot and three words per 32 pixels of a module.
-__host__ __device__ inline size_t hash_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots)
+__host__ __device__ inline size_t cc_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots)
 {
     const size_t nwords = ((size_t)R * C + 31) / 32;
     return (size_t)tile_slots * (8 + 8 + 4) + nwords * 4 * 3;
@@ -270,14 +270,17 @@ __host__ __device__ inline uint32_t run_exact_slots(uint32_t R, uint32_t C, uint
 {
     return run_capacity(run_smem_bytes(R, C, tile_slots, groups), R, C);
 }
-// Digis of a pack of the packed tier (36 bytes each) in a slice of `bytes`
-// with moment scratch for `cap` runs; and the largest item it takes.
-__host__ __device__ inline uint32_t pack_capacity(size_t bytes, uint32_t cap)
+// Digis of a pack of the packed tier (two bitmap words, two counts and a run
+// record each, beside kGroup items' tables of touched words) in a slice of
+// `bytes` with moment scratch for `cap` runs; and the largest item it takes.
+__host__ __device__ inline uint32_t pack_capacity(size_t bytes, uint32_t R, uint32_t cap)
 {
-    uint32_t p = bytes / 36 < 1023 ? (uint32_t)(bytes / 36) : 1023u;
+    const size_t fixed = 6 * (size_t)kGroup * ((R + 1) / 2) + 64;
+    const size_t fit = bytes > fixed ? (bytes - fixed) / (kRunBytes + 10) : 0;
+    const uint32_t p = fit < 1023 ? (uint32_t)fit : 1023u;
     return p < cap ? p : cap;
 }
-__host__ __device__ inline uint32_t pack_max(uint32_t warp_max) { return 8 * warp_max; }
+__host__ __device__ inline uint32_t pack_max(uint32_t warp_max) { return 12 * warp_max; }
 
 // Threads and groups of a clustering block for 1, 2 and 3 resident blocks per SM.
 constexpr int kRunThreads1 = 1024, kRunGroups1 = 4;

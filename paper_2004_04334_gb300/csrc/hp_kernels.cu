@@ -616,15 +616,27 @@ __device__ __forceinline__ void group_sync(uint32_t id, uint32_t threads)
 // Centroid coordinate sum / Q from an exact, non-negative moment: one float
 // division when both are exact in float (the correctly rounded quotient),
 // else integer quotient plus the remainder fraction, so the float result is
-// within a few ulps whatever the magnitude.
+// within a few ulps whatever the magnitude.  The integer quotient (below 512:
+// a row or a column) comes from a float estimate and the remainder's sign.
+__device__ __forceinline__ float centroid_abs(uint32_t sum, uint32_t Q)
+{
+    uint32_t qt = 0, rem = sum;
+    if (sum >= 16777216u || Q >= 16777216u) {
+        qt = (uint32_t)__fdividef((float)sum, (float)Q);
+        rem = sum - qt * Q;
+        if ((int32_t)rem < 0) {
+            --qt;
+            rem += Q;
+        } else if (rem >= Q) {
+            ++qt;
+            rem -= Q;
+        }
+    }
+    return (float)qt + (float)rem / (float)Q;
+}
 __device__ __forceinline__ float centroid_abs(long long sum, int32_t Q)
 {
-    if (sum < 16777216LL && Q < 16777216) return (float)sum / (float)Q;
-    if (sum < 0x80000000LL) {
-        const uint32_t su = (uint32_t)sum, qu = (uint32_t)Q;
-        const uint32_t qt = su / qu;
-        return (float)qt + (float)(su - qt * qu) / (float)Q;
-    }
+    if (sum < 0x80000000LL) return centroid_abs((uint32_t)sum, (uint32_t)Q);
     const long long qt = sum / Q;
     return (float)qt + (float)(sum - qt * Q) / (float)Q;
 }
@@ -705,11 +717,14 @@ __device__ __forceinline__ void reds_add(uint32_t a, uint32_t v)
 {
     asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(a), "n"(kOff), "r"(v) : "memory");
 }
-template <int kOff = 0>
-__device__ __forceinline__ uint32_t atoms_add(uint32_t a, uint32_t v)
+__device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
+{
+    asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
+}
+__device__ __forceinline__ uint32_t atoms_or(uint32_t a, uint32_t v)
 {
     uint32_t old;
-    asm volatile("atom.shared.add.u32 %0, [%1+%2], %3;" : "=r"(old) : "r"(a), "n"(kOff), "r"(v) : "memory");
+    asm volatile("atom.shared.or.b32 %0, [%1], %2;" : "=r"(old) : "r"(a), "r"(v) : "memory");
     return old;
 }
 __device__ __forceinline__ void reds_or(uint32_t a, uint32_t v)
@@ -732,14 +747,17 @@ __device__ __forceinline__ uint32_t atoms_min(uint32_t a, uint32_t v)
 // order, so the smallest run of a cluster holds its smallest linear index
 // (the id), and the runs of the row above that touch a run are consecutive.
 // Phases, one group barrier between them:
-//   1 the item's words; both bitmaps (all digis, survivors) cleared
-//   2 a bit per digi and per survivor; a digi whose bit is taken is found by
-//     counting: the set bits must be as many as the digis
+//   1 the item's words; both bitmaps cleared
+//   2 a bit per digi, in one of two bitmaps (survivors, the others); a digi
+//     whose pixel is taken is found by counting: the pixels set in either must
+//     be as many as the digis
 //   3 runs per word by a scan over the words; run records initialised (they
-//     lie over the bitmap of all digis, free from here on)
-//   4 every survivor adds its charge and q * col to its run; a run's first
-//     pixel stores the run's position
-//   5 a run links itself, by a plain store, under the first run above that
+//     lie over the bitmap of the dropped digis, free from here on)
+//   4 every survivor adds its ADC and ADC * bit to its run, both in one word
+//     (at most 32 pixels of 255: 13 and 17 bits); a run's first pixel stores
+//     the run's position
+//   5 a run works its charge and sum q * col out from these (its pixels'
+//     calibration and columns are its own), and links itself, by a plain store, under the first run above that
 //     it touches (or the run that ends the word to its left); runs with
 //     further contacts (one in ten or so) go to a list
 //   6 the listed runs are united with those, by find and link
@@ -762,14 +780,17 @@ __device__ __forceinline__ uint32_t atoms_min(uint32_t a, uint32_t v)
 //
 // Run records, in shared memory or (kBig) global scratch:
 //   word 0  union-find parent << kRunShift | (roots) pixels of the cluster
-//   word 1  row | col << 8 of the first pixel (the digi word's layout), and
-//           length << 17; from phase 8 on the root's position and a flag
-//   word 2  charge, word 3 sum q * col: of the run, then (roots) the cluster
+//   word 1  row | col << 8 of the first pixel (the digi word's layout), its
+//           length << 17, and in the packed tier its item << 23; from phase 8
+//           on the root's position and item, and a flag
+//   word 2  the sum of phase 4; then the charge, and word 3 sum q * col: of
+//           the run, then (roots) the cluster
 //   word 4  the list of phase 5; then (roots) sum q * (row - root's row)
 //   word 5  (kBig only, whose word 0 is the parent alone) pixels
 constexpr int kRunDigis = 8; // digis a thread holds at once
 constexpr uint32_t kRunShift = 18, kRunPixels = (1u << kRunShift) - 1u;
 constexpr uint32_t kRunKept = 1u << 31, kRunDropped = 1u << 30, kRunPos = 0x1FFFFu;
+constexpr uint32_t kRunItem = 15u << 23; // packed tier: the run's item
 
 template <bool kBig>
 struct Runs;
@@ -784,27 +805,23 @@ struct Runs<false> {
     __device__ __forceinline__ static void st(At a, uint32_t v) { sts<4 * f>(a, v); }
     template <int f>
     __device__ __forceinline__ static void red(At a, uint32_t v) { reds_add<4 * f>(a, v); }
-    template <int f>
-    __device__ __forceinline__ static uint32_t add(At a, uint32_t v) { return atoms_add<4 * f>(a, v); }
     __device__ __forceinline__ uint32_t parent(uint32_t i) const { return ld<0>(at(i)) >> kRunShift; }
     __device__ __forceinline__ void set_parent(uint32_t i, uint32_t p) const { st<0>(at(i), p << kRunShift); }
     __device__ __forceinline__ uint32_t min_parent(uint32_t i, uint32_t p) const
     {
         return atoms_min(at(i), p << kRunShift) >> kRunShift;
     }
-    // a pixel's charge and charge * column into its run, if in != 0; the
-    // run's position, if head != 0 (predicated: no branch among the lanes)
-    __device__ __forceinline__ static void add_pixel(At a, uint32_t q, uint32_t qc, uint32_t in, uint32_t head,
-                                                     uint32_t pos)
+    // the packed sum v into the pixel's run, if in != 0; the run's position,
+    // if head != 0 (predicated: no branch among the lanes)
+    __device__ __forceinline__ static void add_pixel(At a, uint32_t v, uint32_t in, uint32_t head, uint32_t pos)
     {
         asm volatile("{\n\t"
                      ".reg .pred p, h;\n\t"
-                     "setp.ne.u32 p, %3, 0;\n\t"
-                     "setp.ne.u32 h, %4, 0;\n\t"
+                     "setp.ne.u32 p, %2, 0;\n\t"
+                     "setp.ne.u32 h, %3, 0;\n\t"
                      "@p red.shared.add.u32 [%0+8], %1;\n\t"
-                     "@p red.shared.add.u32 [%0+12], %2;\n\t"
-                     "@h st.shared.u32 [%0+4], %5;\n\t"
-                     "}" ::"r"(a), "r"(q), "r"(qc), "r"(in), "r"(head), "r"(pos) : "memory");
+                     "@h st.shared.u32 [%0+4], %4;\n\t"
+                     "}" ::"r"(a), "r"(v), "r"(in), "r"(head), "r"(pos) : "memory");
     }
     __device__ __forceinline__ static void add_pixels(At a, uint32_t v) { red<0>(a, v); }
     __device__ __forceinline__ static uint32_t pixels(At a) { return ld<0>(a) & kRunPixels; }
@@ -813,7 +830,6 @@ struct Runs<false> {
     {
         st<0>(a, i << kRunShift);
         st<2>(a, 0);
-        st<3>(a, 0);
         st<4>(a, 0);
     }
 };
@@ -828,17 +844,13 @@ struct Runs<true> {
     __device__ __forceinline__ static void st(At a, uint32_t v) { *(volatile uint32_t *)(a + f) = v; }
     template <int f>
     __device__ __forceinline__ static void red(At a, uint32_t v) { atomicAdd(a + f, v); }
-    template <int f>
-    __device__ __forceinline__ static uint32_t add(At a, uint32_t v) { return atomicAdd(a + f, v); }
     __device__ __forceinline__ uint32_t parent(uint32_t i) const { return ld<0>(at(i)); }
     __device__ __forceinline__ void set_parent(uint32_t i, uint32_t p) const { st<0>(at(i), p); }
     __device__ __forceinline__ uint32_t min_parent(uint32_t i, uint32_t p) const { return atomicMin(at(i), p); }
-    __device__ __forceinline__ static void add_pixel(At a, uint32_t q, uint32_t qc, uint32_t in, uint32_t head,
-                                                     uint32_t pos)
+    __device__ __forceinline__ static void add_pixel(At a, uint32_t v, uint32_t in, uint32_t head, uint32_t pos)
     {
         if (in) {
-            atomicAdd(a + 2, q);
-            atomicAdd(a + 3, qc);
+            atomicAdd(a + 2, v);
             if (head) st<1>(a, pos);
         }
     }
@@ -849,7 +861,6 @@ struct Runs<true> {
     {
         st<0>(a, i);
         st<2>(a, 0);
-        st<3>(a, 0);
         st<4>(a, 0);
         st<5>(a, 0);
     }
@@ -889,27 +900,13 @@ __device__ __forceinline__ void run_union(const A &a, uint32_t x, uint32_t y)
     }
 }
 
-// What a run at position p sees of the bitmap: its word, the word above and
-// that word's first run, the words beside both (those left of the row's
-// first word read as themselves and are not used), and the first run of the
-// word after the one above.  All loads are independent of each other.
+// What a run sees of the bitmap: its word, the word above, the words beside
+// both (up_left and left are only used past a row's first word, up_right
+// before its last), the first run of the word above (or, if that word is
+// empty, of the next one) and of the word after it.
 struct RunView {
     uint32_t word, left, up, up_left, up_right, pre, next;
 };
-__device__ __forceinline__ RunView run_view(uint32_t sb, uint32_t rp, uint32_t W, uint32_t p)
-{
-    const uint32_t r = p & 0xFFu, cw = (p >> 13) & 0xFu, wi = r * W + cw, wu = r ? wi - W : wi;
-    const uint32_t a = sb + 4 * wi, u = sb + 4 * wu, ra = rp + 2 * wu, back = cw ? 4u : 0u;
-    RunView v;
-    v.word = lds(a);
-    v.up = lds(u);
-    v.pre = lds_u16(ra);
-    v.left = lds(a - back);
-    v.up_left = lds(u - back);
-    v.up_right = lds<4>(u); // (past the last word lies the table of first runs)
-    v.next = lds_u16(ra + 2);
-    return v;
-}
 // Runs that touch run i (position p) before it: [*k, *end) of the row above,
 // and *left, the run that ends the word to its left (kNoSlot: none).
 // Returns its length.
@@ -974,6 +971,219 @@ __device__ __forceinline__ void each_four(uint32_t (&w)[kRunDigis], const uint32
     }
 }
 
+// Packed sum of a surviving digi with word x: ADC, and ADC * bit << kSumShift.
+constexpr uint32_t kSumShift = 13, kSumMask = (1u << kSumShift) - 1u;
+__device__ __forceinline__ uint32_t pixel_sum(uint32_t x)
+{
+    const uint32_t adc = (x >> 17) & 0xFFu;
+    return adc * (1u | (((x >> 8) & 31u) << kSumShift));
+}
+
+// Phases 5 and 6 for the runs of a; view(p) is what the run at position p
+// sees (its loads independent of each other: two runs a thread at a time),
+// calib(p) its module's gain (x) and pedestal (y).
+template <int GT, bool kWhole, class A, class V, class B>
+__device__ __forceinline__ void link_runs(const A &a, const V &view, const B &calib, uint32_t W, uint32_t nruns,
+                                          GroupShared &gs, uint32_t gt, uint32_t bar)
+{
+    for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
+        uint32_t i[2] = {i0, i0 + GT}, p[2], sum[2];
+        RunView v[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const typename A::At r = a.at(i[u] < nruns ? i[u] : i0);
+            p[u] = A::template ld<1>(r);
+            sum[u] = A::template ld<2>(r);
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) v[u] = view(p[u]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (i[u] >= nruns) break;
+            uint32_t k, end, left;
+            const uint32_t len = run_contacts(v[u], W, i[u], p[u], &k, &end, &left);
+            const typename A::At r = a.at(i[u]);
+            A::template st<1>(r, p[u] | (len << 17));
+            // q = gain * ADC - ped over the run's pixels, columns c0 ..
+            const int2 cal = calib(p[u]);
+            const uint32_t c0 = (p[u] >> 8) & 0x1FFu, adc = sum[u] & kSumMask, base = c0 & ~31u;
+            A::template st<2>(r, cal.x * adc - cal.y * len);
+            A::template st<3>(r, cal.x * ((sum[u] >> kSumShift) + base * adc) -
+                                     cal.y * (len * c0 + ((len * (len - 1u)) >> 1)));
+            if (k < end)
+                a.set_parent(i[u], k);
+            else if (left != kNoSlot)
+                a.set_parent(i[u], left);
+            if (end > k + 1 || (k < end && left != kNoSlot))
+                A::template st<4>(a.at(atomicAdd(&gs.extras, 1u)), i[u]);
+        }
+    }
+    gsync<GT, kWhole>(bar);
+    for (uint32_t e = gt, ne = gs.extras; e < ne; e += GT) {
+        const typename A::At re = a.at(e);
+        const uint32_t i = A::template ld<4>(re);
+        A::template st<4>(re, 0);
+        const uint32_t p = A::template ld<1>(a.at(i));
+        uint32_t k, end, left;
+        run_contacts(view(p), W, i, p, &k, &end, &left);
+        for (++k;; ++k) { // the first contact is linked already
+            uint32_t y = k;
+            if (k >= end) {
+                if (left == kNoSlot) break;
+                y = left;
+                left = kNoSlot;
+            }
+            run_union(a, i, y);
+        }
+    }
+}
+
+// Phase 7: only roots receive sums, so a run's own are still its own; two
+// runs a thread at a time.
+template <int GT, class A>
+__device__ __forceinline__ void sum_runs(const A &a, uint32_t nruns, uint32_t gt)
+{
+    for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
+        const uint32_t i1 = i0 + GT < nruns ? i0 + GT : i0;
+        uint32_t x0 = i0, x1 = i1, y0 = a.parent(i0), y1 = a.parent(i1);
+        while (y0 != x0 || y1 != x1) {
+            x0 = y0;
+            x1 = y1;
+            y0 = a.parent(x0);
+            y1 = a.parent(x1);
+        }
+        const uint32_t i[2] = {i0, i1}, x[2] = {x0, x1};
+        uint32_t p[2], q[2], mc[2], px[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const typename A::At r = a.at(i[u]);
+            p[u] = A::template ld<1>(r);
+            q[u] = A::template ld<2>(r);
+            mc[u] = A::template ld<3>(r);
+            px[u] = A::template ld<1>(a.at(x[u]));
+        }
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            if (u == 1 && i1 == i0) break;
+            const typename A::At rx = a.at(x[u]);
+            if (x[u] != i[u]) {
+                a.set_parent(i[u], x[u]);
+                A::template red<2>(rx, q[u]);
+                A::template red<3>(rx, mc[u]);
+                A::template red<4>(rx, q[u] * ((p[u] & 0xFFu) - (px[u] & 0xFFu)));
+            }
+            A::add_pixels(rx, (p[u] >> 17) & 63u);
+        }
+    }
+}
+
+// The 32-run chunks [c0, c1) of a warp of the group (phases 8 and 9).
+template <int GT>
+__device__ __forceinline__ void warp_chunks(uint32_t nruns, uint32_t warp, uint32_t *c0, uint32_t *c1)
+{
+    const uint32_t chunks = (nruns + 31) >> 5, cpw = (chunks + GT / 32 - 1) / (GT / 32);
+    *c0 = min(chunks, warp * cpw);
+    *c1 = min(chunks, *c0 + cpw);
+}
+
+// Phase 8: the root's position (and item) into every run, with kRunKept on a
+// kept root and kRunDropped on the runs of a cluster below threshold; gs.heavy
+// set if a cluster's moments may have overflowed 32 bits.  With
+// kItems the kept roots of each item are counted in gs.tmp[16 ..].  One
+// barrier; returns the kept roots of all runs, and in *ord those before the
+// warp's chunks.
+template <int GT, bool kWhole, bool kItems, class A>
+__device__ __forceinline__ uint32_t mark_runs(const A &a, uint32_t nruns, int32_t cthr, GroupShared &gs, uint32_t gt,
+                                              uint32_t bar, uint32_t *ord)
+{
+    constexpr int kWarps = GT / 32;
+    const uint32_t lane = gt & 31, warp = gt >> 5;
+    uint32_t c0, c1, wrun = 0;
+    warp_chunks<GT>(nruns, warp, &c0, &c1);
+    for (uint32_t ch = c0; ch < c1; ++ch) {
+        const uint32_t i = (ch << 5) + lane;
+        bool lead = false;
+        if (i < nruns) {
+            const uint32_t x = a.parent(i);
+            const typename A::At rx = a.at(x);
+            const uint32_t px = A::template ld<1>(rx);
+            const int32_t Q = (int32_t)A::template ld<2>(rx);
+            const bool kept = Q >= cthr;
+            lead = kept && x == i;
+            if (Q > kQSafe32) gs.heavy = 1;
+            A::template st<1>(a.at(i), (px & (kItems ? kRunPos | kRunItem : kRunPos)) |
+                                           (lead ? kRunKept : kept ? 0u : kRunDropped));
+            if (kItems && lead) atomicAdd(&gs.tmp[16 + ((px & kRunItem) >> 23)], 1u);
+        }
+        wrun += __popc(__ballot_sync(kFull, lead));
+    }
+    if (lane == 0) gs.tmp[warp] = wrun;
+    gsync<GT, kWhole>(bar);
+    const uint32_t wt = lane < kWarps ? gs.tmp[lane] : 0u;
+    uint32_t ws = wt;
+#pragma unroll
+    for (int o = 1; o < kWarps; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, ws, o);
+        if ((int)lane >= o) ws += y;
+    }
+    *ord = __shfl_sync(kFull, ws - wt, warp);
+    return __shfl_sync(kFull, ws, kWarps - 1);
+}
+
+// Phase 9: put(run, ordinal) for every kept root, in run order, gathered 32
+// at a time so that every lane stages a cluster.
+template <int GT, class A, class P>
+__device__ __forceinline__ void stage_runs(const A &a, uint32_t nruns, uint32_t ord, uint16_t *wlist, uint32_t gt,
+                                           const P &put)
+{
+    const uint32_t lane = gt & 31;
+    uint32_t c0, c1, cnt = 0;
+    warp_chunks<GT>(nruns, gt >> 5, &c0, &c1);
+    for (uint32_t ch = c0;; ++ch) {
+        const bool last = ch >= c1;
+        if (!last) {
+            const uint32_t i = (ch << 5) + lane;
+            const bool kept = i < nruns && (A::template ld<1>(a.at(i)) & kRunKept);
+            const uint32_t bal = __ballot_sync(kFull, kept);
+            if (kept) wlist[cnt + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)i;
+            cnt += __popc(bal);
+            __syncwarp();
+        }
+        if (cnt >= 32 || (last && cnt > 0)) {
+            if (lane < cnt) put((uint32_t)wlist[lane], ord + lane);
+            if (last) break;
+            __syncwarp();
+            const uint32_t v = wlist[32 + lane];
+            __syncwarp();
+            wlist[lane] = (uint16_t)v;
+            __syncwarp();
+            cnt -= 32;
+            ord += 32;
+        } else if (last) {
+            break;
+        }
+    }
+}
+
+// The sums of root i as a staged cluster at position `at`.
+template <class A>
+__device__ __forceinline__ void stage_root(const Launch &L, const A &a, uint32_t i, uint64_t at, bool heavy,
+                                           const unsigned long long *exact)
+{
+    const typename A::At r = a.at(i);
+    const uint32_t p = A::template ld<1>(r);
+    const int32_t Q = (int32_t)A::template ld<2>(r), np = (int32_t)A::pixels(r);
+    float x, y;
+    if (heavy) {
+        x = centroid_abs((long long)exact[2 * (size_t)i], Q);
+        y = centroid_abs((long long)exact[2 * (size_t)i + 1], Q);
+    } else {
+        x = centroid_abs(A::template ld<4>(r) + (p & 0xFFu) * (uint32_t)Q, (uint32_t)Q);
+        y = centroid_abs(A::template ld<3>(r), (uint32_t)Q);
+    }
+    L.ws.staging.put(at, (int32_t)((p & 0xFFu) * L.g.C + ((p >> 8) & 0x1FFu)), Q, np, x, y);
+}
+
 template <int GT, bool kWhole, bool kBig, bool kSingle>
 __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx &it, uint32_t sb, uint32_t rp,
                                                  const Runs<kBig> a, unsigned long long *exact, uint32_t nruns,
@@ -982,8 +1192,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
 {
     using A = Runs<kBig>;
     const uint32_t C = L.g.C, W = (C + 31) >> 5;
-    const int32_t cthr = L.g.cluster_thr;
-    const uint32_t n = it.n, lane = gt & 31, warp = gt >> 5;
+    const uint32_t n = it.n;
     const uint32_t mine = n > gt ? (n - gt - 1) / GT + 1 : 0u;
     const uint32_t *bw = L.ws.bucket_w + it.b + gt;
     const uint32_t *bi = L.ws.bucket_i + it.b + gt;
@@ -1016,95 +1225,31 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
         runs_of(x, run, in, head);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const uint32_t q = ((x[u] >> 17) & 0xFFu) * (uint32_t)gain - (uint32_t)ped;
-            A::add_pixel(a.at(in[u] ? run[u] : 0u), q, q * ((x[u] >> 8) & 0x1FFu), in[u], head[u], x[u] & kRunPos);
+            A::add_pixel(a.at(in[u] ? run[u] : 0u), pixel_sum(x[u]), in[u], head[u], x[u] & kRunPos);
             if constexpr (kSingle) w[k + u] = run[u];
         }
     });
     gsync<GT, kWhole>(bar);
 
-    // 5: two runs a thread at a time
-    for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
-        uint32_t i[2] = {i0, i0 + GT}, p[2];
-        RunView v[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) p[u] = i[u] < nruns ? A::template ld<1>(a.at(i[u])) : 0u;
-#pragma unroll
-        for (int u = 0; u < 2; ++u) v[u] = run_view(sb, rp, W, p[u]);
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (i[u] >= nruns) break;
-            uint32_t k, end, left;
-            const uint32_t len = run_contacts(v[u], W, i[u], p[u], &k, &end, &left);
-            const typename A::At r = a.at(i[u]);
-            A::template st<1>(r, p[u] | (len << 17));
-            if (k < end)
-                a.set_parent(i[u], k);
-            else if (left != kNoSlot)
-                a.set_parent(i[u], left);
-            if (end > k + 1 || (k < end && left != kNoSlot))
-                A::template st<4>(a.at(atomicAdd(&gs.extras, 1u)), i[u]);
-        }
-    }
+    // 5, 6
+    auto view = [&](uint32_t p) {
+        const uint32_t r = p & 0xFFu, cw = (p >> 13) & 0xFu, wi = r * W + cw, wu = r ? wi - W : wi;
+        const uint32_t own = sb + 4 * wi, u = sb + 4 * wu, ra = rp + 2 * wu, back = cw ? 4u : 0u;
+        RunView v;
+        v.word = lds(own);
+        v.up = lds(u);
+        v.pre = lds_u16(ra);
+        v.left = lds(own - back);
+        v.up_left = lds(u - back);
+        v.up_right = lds<4>(u); // (past the last word lies the table of first runs)
+        v.next = lds_u16(ra + 2);
+        return v;
+    };
+    link_runs<GT, kWhole>(a, view, [&](uint32_t) { return make_int2(gain, ped); }, W, nruns, gs, gt, bar);
     gsync<GT, kWhole>(bar);
 
-    // 6
-    for (uint32_t e = gt, ne = gs.extras; e < ne; e += GT) {
-        const typename A::At re = a.at(e);
-        const uint32_t i = A::template ld<4>(re);
-        A::template st<4>(re, 0);
-        const uint32_t p = A::template ld<1>(a.at(i)) & kRunPos;
-        const RunView v = run_view(sb, rp, W, p);
-        uint32_t k, end, left;
-        run_contacts(v, W, i, p, &k, &end, &left);
-        for (++k;; ++k) { // the first contact is linked already
-            uint32_t y = k;
-            if (k >= end) {
-                if (left == kNoSlot) break;
-                y = left;
-                left = kNoSlot;
-            }
-            run_union(a, i, y);
-        }
-    }
-    gsync<GT, kWhole>(bar);
-
-    // 7: only roots receive sums, so a run's own are still its own; two runs
-    // a thread at a time
-    for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
-        const uint32_t i1 = i0 + GT < nruns ? i0 + GT : i0;
-        uint32_t x0 = i0, x1 = i1, y0 = a.parent(i0), y1 = a.parent(i1);
-        while (y0 != x0 || y1 != x1) {
-            x0 = y0;
-            x1 = y1;
-            y0 = a.parent(x0);
-            y1 = a.parent(x1);
-        }
-        const uint32_t i[2] = {i0, i1}, x[2] = {x0, x1};
-        uint32_t p[2], q[2], mc[2], px[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            const typename A::At r = a.at(i[u]);
-            p[u] = A::template ld<1>(r);
-            q[u] = A::template ld<2>(r);
-            mc[u] = A::template ld<3>(r);
-            px[u] = A::template ld<1>(a.at(x[u]));
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-            if (u == 1 && i1 == i0) break;
-            const typename A::At rx = a.at(x[u]);
-            if (x[u] != i[u]) {
-                a.set_parent(i[u], x[u]);
-                if ((int32_t)(A::template add<2>(rx, q[u]) + q[u]) > kQSafe32) gs.heavy = 1;
-                A::template red<3>(rx, mc[u]);
-                A::template red<4>(rx, q[u] * ((p[u] & 0xFFu) - (px[u] & 0xFFu)));
-            } else if ((int32_t)q[u] > kQSafe32) {
-                gs.heavy = 1;
-            }
-            A::add_pixels(rx, p[u] >> 17);
-        }
-    }
+    // 7
+    sum_runs<GT>(a, nruns, gt);
     uint32_t iv[kSingle ? kRunDigis : 1] = {}; // in-event indices for the labels
     auto index_of = [&](int k, uint32_t j) {
         if constexpr (kSingle)
@@ -1120,6 +1265,9 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
         }
     }
     gsync<GT, kWhole>(bar);
+    // 8
+    uint32_t ord;
+    const uint32_t K = mark_runs<GT, kWhole, false>(a, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
     const bool heavy = gs.heavy != 0;
     if (heavy) { // both moments of every root again, in 64 bits
         for (uint32_t i = gt; i < nruns; i += GT) {
@@ -1138,38 +1286,6 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
             atomicAdd(&exact[2 * y + 1], (unsigned long long)(q * (long long)((x[0] >> 8) & 0x1FFu)));
         }
         gsync<GT, kWhole>(bar);
-    }
-
-    // 8: a warp takes a contiguous range of 32-run chunks
-    constexpr uint32_t kWarps = GT / 32;
-    const uint32_t chunks = (nruns + 31) >> 5, cpw = (chunks + kWarps - 1) / kWarps;
-    const uint32_t wc0 = min(chunks, warp * cpw), wc1 = min(chunks, wc0 + cpw);
-    uint32_t wrun = 0;
-    for (uint32_t ch = wc0; ch < wc1; ++ch) {
-        const uint32_t i = (ch << 5) + lane;
-        bool lead = false;
-        if (i < nruns) {
-            const uint32_t x = a.parent(i);
-            const typename A::At rx = a.at(x);
-            const bool kept = (int32_t)A::template ld<2>(rx) >= cthr;
-            lead = kept && x == i;
-            A::template st<1>(a.at(i), (A::template ld<1>(rx) & kRunPos) | (lead ? kRunKept : kept ? 0u : kRunDropped));
-        }
-        wrun += __popc(__ballot_sync(kFull, lead));
-    }
-    if (lane == 0) gs.tmp[warp] = wrun;
-    gsync<GT, kWhole>(bar);
-    uint32_t K, ord;
-    {
-        const uint32_t wt = lane < kWarps ? gs.tmp[lane] : 0u;
-        uint32_t ws = wt;
-#pragma unroll
-        for (int o = 1; o < (int)kWarps; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(kFull, ws, o);
-            if ((int)lane >= o) ws += y;
-        }
-        K = __shfl_sync(kFull, ws, kWarps - 1);
-        ord = __shfl_sync(kFull, ws - wt, warp);
     }
 
     // 9: labels (the stores drain behind the staging)
@@ -1194,51 +1310,10 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
             }
         });
     }
-    // the kept roots of the warp's chunks, gathered 32 at a time so that
-    // every lane stages a cluster
-    {
-        uint32_t cnt = 0;
-        for (uint32_t ch = wc0;; ++ch) {
-            const bool last = ch >= wc1;
-            if (!last) {
-                const uint32_t i = (ch << 5) + lane;
-                const bool kept = i < nruns && (A::template ld<1>(a.at(i)) & kRunKept);
-                const uint32_t bal = __ballot_sync(kFull, kept);
-                if (kept) wlist[cnt + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)i;
-                cnt += __popc(bal);
-                __syncwarp();
-            }
-            if (cnt >= 32 || (last && cnt > 0)) {
-                if (lane < cnt) {
-                    const uint32_t i = wlist[lane];
-                    const typename A::At r = a.at(i);
-                    const uint32_t p = A::template ld<1>(r);
-                    const int32_t Q = (int32_t)A::template ld<2>(r), np = (int32_t)A::pixels(r);
-                    long long mr, mc;
-                    if (heavy) {
-                        mr = (long long)exact[2 * (size_t)i];
-                        mc = (long long)exact[2 * (size_t)i + 1];
-                    } else {
-                        mr = (int32_t)A::template ld<4>(r) + (int32_t)(p & 0xFFu) * Q;
-                        mc = (int32_t)A::template ld<3>(r);
-                    }
-                    L.ws.staging.put(it.b + ord + lane, (int32_t)((p & 0xFFu) * C + ((p >> 8) & 0x1FFu)), Q, np,
-                                     centroid_abs(mr, Q), centroid_abs(mc, Q));
-                    if (it.label16_e) A::set_ordinal(r, i, ord + lane); // read back by the compact labels
-                }
-                if (last) break;
-                __syncwarp();
-                const uint32_t v = wlist[32 + lane];
-                __syncwarp();
-                wlist[lane] = (uint16_t)v;
-                __syncwarp();
-                cnt -= 32;
-                ord += 32;
-            } else if (last) {
-                break;
-            }
-        }
-    }
+    stage_runs<GT>(a, nruns, ord, wlist, gt, [&](uint32_t i, uint32_t o) {
+        stage_root(L, a, i, it.b + o, heavy, exact);
+        if (it.label16_e) A::set_ordinal(a.at(i), i, o); // read back by the compact labels
+    });
     if (it.label16_e) { // compact labels, once every kept root has its ordinal
         gsync<GT, kWhole>(bar);
         each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
@@ -1296,7 +1371,7 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
     const uint32_t *bw = L.ws.bucket_w + it.b + gt;
     const int32_t gain = it.gain, ped = it.ped;
     const uint32_t sb = mem, rp = sb + 4 * nw4;
-    const uint32_t ab = mem + (uint32_t)run_fixed_bytes(R, C); // the bitmap of all digis; then the run records
+    const uint32_t ab = mem + (uint32_t)run_fixed_bytes(R, C); // the bitmap of the dropped digis; then the run records
 
     // 1
     uint32_t w[kRunDigis];
@@ -1321,8 +1396,7 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
             const uint32_t r = x[u] & 0xFFu, c = (x[u] >> 8) & 0x1FFu, adc = x[u] >> 17;
             const bool ok = r < R && c < C && adc - 1u < 255u; // ADC not 0, bits 25-31 clear
             const uint32_t o = ok ? 4 * (r * W + (c >> 5)) : 0u, bit = ok ? 1u << (c & 31) : 0u;
-            reds_or(ab + o, bit);
-            reds_or(sb + o, (int32_t)adc * gain - ped >= thr ? bit : 0u);
+            reds_or(((int32_t)adc * gain - ped >= thr ? sb : ab) + o, bit);
             valid += ok ? 1u : 0u;
         }
     });
@@ -1345,7 +1419,7 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
         const uint4 s = four(sb + 4 * i), d = four(ab + 4 * i);
         local += __popc(s.x & ~(s.x << 1)) + __popc(s.y & ~(s.y << 1)) + __popc(s.z & ~(s.z << 1)) +
                  __popc(s.w & ~(s.w << 1));
-        pixels += __popc(d.x) + __popc(d.y) + __popc(d.z) + __popc(d.w);
+        pixels += __popc(s.x | d.x) + __popc(s.y | d.y) + __popc(s.z | d.z) + __popc(s.w | d.w);
     }
     pixels = __reduce_add_sync(kFull, pixels);
     if ((gt & 31) == 0 && pixels) atomicAdd(&gs.pixels, pixels);
@@ -1395,48 +1469,276 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 // ---- packed tier
 //
 // The small items of a ticket together: up to 1,023 digis of up to 16 items
-// by a group of GT threads, each digi one entry of a hash table keyed by
-// (item, linear pixel index) with four slots a digi.  Entries are packed
-// words, (item << 17 | index) << 11 | surviving << 10 | digi, so that the
-// same word is the table's entry, the digi's union-find key (smaller key =
-// smaller index of the same item, so a root is its cluster's id) and the
-// sort key of the kept clusters.  Phases, one group barrier between them:
-//   0 the digis' items and words; table emptied
-//   1 every valid digi inserted (its pixel already there: a duplicate)
-//   2 survivors linked with their neighbours before them in row-major order:
-//     left and up; without up, upper-left unless the left one survives (it
-//     reaches it) and upper-right.  The first link is one atomicMin on the
-//     digi's own entry, the second a find and link.
-//   3 roots; charge, size and moments per root
-//   4 labels; kept roots appended to their item's list
-//   5 each kept root's ordinal = kept roots of its item with smaller keys;
-//     staging; compact labels
-// What bounds it: latency (a chain of dependent shared-memory accesses a
-// phase), so all the items of a ticket share each phase; the warp-per-item
-// tier this replaced walked all pairs of an item's digis by shuffles.  A table
-// of four slots a digi: with two, a probe of a warp went on for about ten
-// slots.  16 events of 1,856 items (32 digis each): 344 -> 166 us.
-constexpr uint32_t kPackDigis = 1023; // 10 index bits, and the all-ones word stays free for "empty"
-constexpr uint32_t kPackIdx = 1023u;
-constexpr uint32_t kPackEmpty = 0xFFFFFFFFu;
+// by a group of GT threads, through the run tier's phases on a sparse bitmap.
+// Of each item's bitmap words only the touched ones are stored, in (item,
+// row, word) order: a bit per word of the module says which are (16 bits a
+// row, so that a word's neighbours in its row lie in the same field), and the
+// set bits before a word are its place.  So the runs are numbered in (item,
+// row-major) order as in the run tier, with no hashing and nothing to probe,
+// and the kept roots come out item by item in id order.  Phases, one group
+// barrier between them:
+//   a the digis' items and words; tables cleared
+//   b a bit per touched word
+//   c touched words before each field, by a scan
+//   d a bit per digi, among the survivors or the dropped (set already, or in
+//     both: a duplicate)
+//   e runs before each touched word, by a scan; run records initialised
+//   f charge and position into the runs, then 5 to 9 of the run tier
+// What bounds it: the latency of the phases, which all items of a ticket
+// share; the work is the digis', not the modules'.
+constexpr uint32_t kPackDigis = 1023;
+
+// One warp (lane = its lane): the pack that starts at item i0 of the ticket,
+// as many of the next items of at most pmax digis as pcap holds (larger ones
+// are passed over).  Writes gs.pack (first packed digi of each item from i0
+// on, the total from the pack's end on) and returns the end.
+__device__ __forceinline__ uint32_t plan_pack(GroupShared &gs, uint32_t i0, uint32_t pmax, uint32_t pcap,
+                                              uint32_t lane, uint32_t n_lane)
+{
+    const uint32_t pn = n_lane <= pmax ? n_lane : 0u;
+    uint32_t incl = pn;
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, incl, o);
+        if ((int)lane >= o) incl += y;
+    }
+    const uint32_t fits = __ballot_sync(kFull, lane < (uint32_t)kGroup - i0 && incl <= pcap);
+    const uint32_t cnt = __ffs(~fits) - 1; // leading items that fit (kGroup < 32, so ~fits != 0)
+    const uint32_t total = __shfl_sync(kFull, incl, cnt ? cnt - 1 : 0);
+    if (lane <= (uint32_t)kGroup) gs.pack[lane] = (uint16_t)(lane < cnt ? incl - pn : total);
+    return i0 + cnt;
+}
+
+template <int GT, bool kWhole>
+__device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsigned long long *exact, uint32_t i0,
+                                           uint32_t items, uint32_t total, GroupShared &gs, uint16_t *wlist,
+                                           uint32_t gt, uint32_t bar)
+{
+    using A = Runs<false>;
+    static_assert(kPackDigis < 4 * GT, "four digis a thread at most");
+    const uint32_t R = L.g.R, C = L.g.C, W = (C + 31) >> 5, RH = (R + 1) >> 1, pcap = L.cc.pack_digis;
+    const int32_t thr = L.g.pixel_thr;
+    // fields: RH words of two rows an item; and the touched words before each
+    const uint32_t nf = items * RH, fields = mem, before = fields + 4 * kGroup * RH;
+    const uint32_t drop = (before + 2 * kGroup * RH + 15) & ~15u, surv = drop + 4 * (pcap + 1);
+    const uint32_t rpre = surv + 4 * (pcap + 1);
+    A a;
+    a.base = (rpre + 2 * (pcap + 2) + 3) & ~3u;
+
+    // a
+    uint32_t w[4], idx[4], li[4], at[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const uint32_t t = gt + k * GT;
+        w[k] = kNoDigi;
+        idx[k] = li[k] = at[k] = 0;
+        if (t < total) {
+            uint32_t i = 0; // the last item whose first digi is at or before t
+#pragma unroll
+            for (uint32_t step = kGroup / 2; step; step >>= 1)
+                if (gs.pack[i + step] <= t) i += step;
+            const uint32_t pos = gs.b[i0 + i] + (t - gs.pack[i]);
+            li[k] = i;
+            w[k] = __ldg(L.ws.bucket_w + pos);
+            idx[k] = __ldg(L.ws.bucket_i + pos);
+        }
+    }
+    for (uint32_t i = gt; i < nf; i += GT) sts(fields + 4 * i, 0);
+    for (uint32_t i = gt; i <= total; i += GT) {
+        sts(drop + 4 * i, 0);
+        sts(surv + 4 * i, 0);
+    }
+    if (gt < (uint32_t)kGroup) gs.tmp[16 + gt] = 0;
+    if (gt == 0) {
+        gs.heavy = 0;
+        gs.extras = 0;
+    }
+    gsync<GT, kWhole>(bar);
+
+    // b
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (gt + k * GT >= total) break;
+        const uint32_t r = w[k] & 0xFFu, c = (w[k] >> 8) & 0x1FFu, adc = w[k] >> 17;
+        if (r >= R || c >= C || adc - 1u >= 255u) { // ADC 0, or any of the bits 25-31
+            atomicOr(L.ws.event_err + gs.rec[i0 + li[k]].e, kErrBadDigi);
+            w[k] = kNoDigi;
+        } else {
+            reds_or(fields + 4 * (li[k] * RH + (r >> 1)), 1u << (((r & 1u) << 4) + (c >> 5)));
+        }
+    }
+    gsync<GT, kWhole>(bar);
+
+    // c
+    uint32_t touched;
+    {
+        const uint32_t per = (nf + GT - 1) / GT, f0 = min(nf, gt * per), f1 = min(nf, f0 + per);
+        uint32_t local = 0;
+        for (uint32_t i = f0; i < f1; ++i) local += __popc(lds(fields + 4 * i));
+        uint32_t run = group_exclusive_scan<GT, kWhole>(local, gs.tmp, gt, bar, &touched);
+        for (uint32_t i = f0; i < f1; ++i) {
+            sts_u16(before + 2 * i, run);
+            run += __popc(lds(fields + 4 * i));
+        }
+    }
+    gsync<GT, kWhole>(bar);
+    // place of word cw of row r of item i (of the next touched one if it is
+    // not), and whether it and the words beside it in the row are touched
+    // (bits 1, 0 and 2 of *near)
+    auto place = [&](uint32_t i, uint32_t r, uint32_t cw, uint32_t *near) {
+        const uint32_t f = i * RH + (r >> 1), field = lds(fields + 4 * f), sh = ((r & 1u) << 4) + cw;
+        const uint32_t row = ((field >> ((r & 1u) << 4)) & 0xFFFFu) << 1; // bit cw + 1: word cw
+        *near = (row >> cw) & 7u;
+        return lds_u16(before + 2 * f) + __popc(field & ((1u << sh) - 1u));
+    };
+
+    // d
+    uint32_t dropped = 0; // bit k: digi k is below threshold
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (gt + k * GT >= total) break;
+        if (w[k] == kNoDigi) continue;
+        const ItemRec &rec = gs.rec[i0 + li[k]];
+        const uint32_t r = w[k] & 0xFFu, c = (w[k] >> 8) & 0x1FFu, bit = 1u << (c & 31);
+        uint32_t near;
+        at[k] = place(li[k], r, c >> 5, &near);
+        const bool keep = (int32_t)((w[k] >> 17) & 0xFFu) * rec.gain - rec.ped >= thr;
+        if (atoms_or((keep ? surv : drop) + 4 * at[k], bit) & bit) atomicOr(L.ws.event_err + rec.e, kErrDup);
+        dropped |= keep ? 0u : 1u << k;
+    }
+    gsync<GT, kWhole>(bar);
+
+    // e
+    uint32_t nruns;
+    {
+        const uint32_t per = (touched + GT - 1) / GT, f0 = min(touched, gt * per), f1 = min(touched, f0 + per);
+        uint32_t local = 0;
+        for (uint32_t i = f0; i < f1; ++i) {
+            const uint32_t x = lds(surv + 4 * i);
+            local += __popc(x & ~(x << 1));
+        }
+        uint32_t run = group_exclusive_scan<GT, kWhole>(local, gs.tmp, gt, bar, &nruns);
+        for (uint32_t i = f0; i < f1; ++i) {
+            const uint32_t x = lds(surv + 4 * i);
+            sts_u16(rpre + 2 * i, run);
+            run += __popc(x & ~(x << 1));
+        }
+        if (gt == 0) sts_u16(rpre + 2 * touched, nruns);
+        for (uint32_t i = gt; i < nruns; i += GT) A::init(a.at(i), i);
+    }
+    gsync<GT, kWhole>(bar);
+
+    // f
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (gt + k * GT >= total) break;
+        const uint32_t x = w[k];
+        w[k] = kNoSlot;
+        if (x == kNoDigi) continue;
+        const ItemRec &rec = gs.rec[i0 + li[k]];
+        const uint32_t word = lds(surv + 4 * at[k]), b = 1u << ((x >> 8) & 31u), h = word & ~(word << 1);
+        if ((dropped >> k) & 1u) { // (a survivor at its pixel is a duplicate too)
+            if (word & b) atomicOr(L.ws.event_err + rec.e, kErrDup);
+            continue;
+        }
+        const uint32_t run = lds_u16(rpre + 2 * at[k]) + __popc(h & (b | (b - 1u))) - 1u;
+        A::add_pixel(a.at(run), pixel_sum(x), 1u, h & b, (x & kRunPos) | (li[k] << 23));
+        w[k] = run;
+    }
+    gsync<GT, kWhole>(bar);
+    auto view = [&](uint32_t p) {
+        const uint32_t r = p & 0xFFu, cw = (p >> 13) & 0xFu, i = (p & kRunItem) >> 23;
+        uint32_t near, above;
+        const uint32_t own = surv + 4 * place(i, r, cw, &near);
+        const uint32_t up = place(i, r ? r - 1u : 0u, cw, &above), here = (above >> 1) & 1u;
+        RunView v;
+        v.word = lds(own);
+        v.left = near & 1u ? lds<-4>(own) : 0u;
+        v.up = here ? lds(surv + 4 * up) : 0u;
+        v.up_left = above & 1u ? lds<-4>(surv + 4 * up) : 0u;
+        v.up_right = above & 4u ? lds(surv + 4 * (up + here)) : 0u;
+        v.pre = lds_u16(rpre + 2 * up);
+        v.next = lds_u16(rpre + 2 * (up + here));
+        return v;
+    };
+    auto calib = [&](uint32_t p) {
+        const ItemRec &rec = gs.rec[i0 + ((p & kRunItem) >> 23)];
+        return make_int2(rec.gain, rec.ped);
+    };
+    link_runs<GT, kWhole>(a, view, calib, W, nruns, gs, gt, bar);
+    gsync<GT, kWhole>(bar);
+    sum_runs<GT>(a, nruns, gt);
+    gsync<GT, kWhole>(bar);
+    uint32_t ord;
+    mark_runs<GT, kWhole, true>(a, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
+    const bool heavy = gs.heavy != 0;
+    if (heavy) { // both moments again, in 64 bits
+        for (uint32_t i = gt; i < 2 * nruns; i += GT) exact[i] = 0;
+        gsync<GT, kWhole>(bar);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (gt + k * GT >= total || w[k] == kNoSlot) continue;
+            const ItemRec &rec = gs.rec[i0 + li[k]];
+            const uint32_t x = __ldg(L.ws.bucket_w + gs.b[i0 + li[k]] + (gt + k * GT - gs.pack[li[k]]));
+            const uint32_t y = a.parent(w[k]);
+            const long long q = (long long)((int32_t)((x >> 17) & 0xFFu) * rec.gain - rec.ped);
+            atomicAdd(&exact[2 * y], (unsigned long long)(q * (long long)(x & 0xFFu)));
+            atomicAdd(&exact[2 * y + 1], (unsigned long long)(q * (long long)((x >> 8) & 0x1FFu)));
+        }
+        gsync<GT, kWhole>(bar);
+    }
+    // each item's kept clusters, and those of the items before it
+    const uint32_t lane = gt & 31, kept = lane < (uint32_t)kGroup ? gs.tmp[16 + lane] : 0u;
+    uint32_t first = kept;
+#pragma unroll
+    for (int o = 1; o < kGroup; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(kFull, first, o);
+        if ((int)lane >= o) first += y;
+    }
+    first -= kept;
+    if (gt < (uint32_t)kGroup && gs.pack[gt + 1] > gs.pack[gt]) {
+        L.ws.cursor[gs.ticket * L.cc.ticket_items + i0 + gt] = kept;
+        gs.rec[i0 + gt].gain = (int32_t)first; // (a packed item's calibration is not needed any more)
+    }
+    if (L.out.label) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (gt + k * GT >= total) break;
+            int32_t lab = -1;
+            if (w[k] != kNoSlot) {
+                const uint32_t p = A::ld<1>(a.at(w[k]));
+                lab = p & kRunDropped ? -2 : (int32_t)((p & 0xFFu) * C + ((p >> 8) & 0x1FFu));
+            }
+            L.out.label[gs.rec[i0 + li[k]].label_off + idx[k]] = lab;
+        }
+    }
+    gsync<GT, kWhole>(bar);
+    stage_runs<GT>(a, nruns, ord, wlist, gt, [&](uint32_t i, uint32_t o) {
+        const uint32_t item = (A::ld<1>(a.at(i)) & kRunItem) >> 23, k = o - (uint32_t)gs.rec[i0 + item].gain;
+        stage_root(L, a, i, gs.b[i0 + item] + k, heavy, exact);
+        if (L.out.label16) A::set_ordinal(a.at(i), i, k); // read back by the compact labels
+    });
+    if (L.out.label16) {
+        gsync<GT, kWhole>(bar);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (gt + k * GT >= total) break;
+            uint16_t v = kLab16Below;
+            if (w[k] != kNoSlot) {
+                const A::At rx = a.at(a.parent(w[k]));
+                v = A::ld<1>(rx) & kRunKept ? (uint16_t)A::pixels(rx) : kLab16Dropped;
+            }
+            L.out.label16[gs.rec[i0 + li[k]].label_off + idx[k]] = v;
+        }
+    }
+    gsync<GT, kWhole>(bar); // the slice and the plan are free
+}
+
+// ---------------------------------------------------------------- hash label store
 
 // Home slot of a key in a table of H slots (multiplicative hashing: the high
 // bits of key times the 32-bit golden ratio, scaled to [0, H)).
 __device__ __forceinline__ uint32_t hash_home(uint32_t key, uint32_t H) { return __umulhi(key * 0x9E3779B1u, H); }
-
-// Entry of `key` if it is there and survives the pixel threshold, else
-// kPackEmpty.  The table holds at most H / 4 entries, so a probe always ends.
-__device__ __forceinline__ uint32_t pack_survivor(const uint32_t *table, uint32_t H, uint32_t key)
-{
-    uint32_t s = hash_home(key, H);
-    for (uint32_t i = 0; i < H; ++i) {
-        const uint32_t e = table[s];
-        if (e == kPackEmpty) return kPackEmpty;
-        if ((e >> 11) == key) return (e >> 10) & 1u ? e : kPackEmpty;
-        s = s + 1 == H ? 0u : s + 1;
-    }
-    return kPackEmpty;
-}
 
 // Find on packed keys with path halving (the index of a key is its low
 // bits); parents only ever decrease, as in uf_find_halving.
@@ -1474,231 +1776,6 @@ __device__ __forceinline__ void key_union(uint32_t *par, uint32_t a, uint32_t b)
         a = old;
     }
 }
-
-// One warp (lane = its lane): the pack that starts at item i0 of the ticket,
-// as many of the next items of at most pmax digis as pcap holds (larger ones
-// are passed over).  Writes gs.pack (first packed digi of each item from i0
-// on, the total from the pack's end on) and returns the end.
-__device__ __forceinline__ uint32_t plan_pack(GroupShared &gs, uint32_t i0, uint32_t pmax, uint32_t pcap,
-                                              uint32_t lane, uint32_t n_lane)
-{
-    const uint32_t pn = n_lane <= pmax ? n_lane : 0u;
-    uint32_t incl = pn;
-#pragma unroll
-    for (int o = 1; o < kGroup; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, incl, o);
-        if ((int)lane >= o) incl += y;
-    }
-    const uint32_t fits = __ballot_sync(kFull, lane < (uint32_t)kGroup - i0 && incl <= pcap);
-    const uint32_t cnt = __ffs(~fits) - 1; // leading items that fit (kGroup < 32, so ~fits != 0)
-    const uint32_t total = __shfl_sync(kFull, incl, cnt ? cnt - 1 : 0);
-    if (lane <= (uint32_t)kGroup) gs.pack[lane] = (uint16_t)(lane < cnt ? incl - pn : total);
-    return i0 + cnt;
-}
-
-template <int GT, bool kWhole>
-__device__ __forceinline__ void pack_items(const Launch &L, unsigned char *mem, unsigned long long *exact,
-                                           uint32_t i0, uint32_t total, GroupShared &gs, uint32_t gt, uint32_t bar)
-{
-    const uint32_t pcap = L.cc.pack_digis;
-    constexpr int kP = (kPackDigis + GT) / GT; // digis a thread holds
-    const uint32_t R = L.g.R, C = L.g.C, H = 4 * total;
-    const int32_t thr = L.g.pixel_thr, cthr = L.g.cluster_thr;
-    int2 *m = reinterpret_cast<int2 *>(mem);
-    int32_t *q = reinterpret_cast<int32_t *>(m + pcap);
-    uint32_t *np = reinterpret_cast<uint32_t *>(q + pcap);
-    uint32_t *par = np + pcap;
-    uint32_t *table = par + pcap; // [4 * pcap]; then the kept roots' lists
-
-    // 0
-    uint32_t w[kP], ent[kP], idx[kP], li[kP];
-#pragma unroll
-    for (int k = 0; k < kP; ++k) {
-        const uint32_t t = gt + k * GT;
-        w[k] = idx[k] = li[k] = 0;
-        ent[k] = kPackEmpty;
-        if (t < total) {
-            uint32_t i = 0; // the last item whose first digi is at or before t
-#pragma unroll
-            for (uint32_t step = kGroup / 2; step; step >>= 1)
-                if (gs.pack[i + step] <= t) i += step;
-            const uint32_t at = gs.b[i0 + i] + (t - gs.pack[i]);
-            li[k] = i;
-            w[k] = __ldg(L.ws.bucket_w + at);
-            idx[k] = __ldg(L.ws.bucket_i + at);
-        }
-    }
-    for (uint32_t i = gt; i < H; i += GT) table[i] = kPackEmpty;
-    if (gt < (uint32_t)kGroup) gs.tmp[gt] = 0;
-    if (gt == 0) gs.heavy = 0;
-    gsync<GT, kWhole>(bar);
-
-    // 1
-#pragma unroll
-    for (int k = 0; k < kP; ++k) {
-        const uint32_t t = gt + k * GT;
-        if (t >= total) continue;
-        const ItemRec &rec = gs.rec[i0 + li[k]];
-        const uint32_t x = w[k], r = x & 0xFFu, c = (x >> 8) & 0x1FFu, adc = x >> 17;
-        if (r >= R || c >= C || adc - 1u >= 255u) { // ADC 0, or any of the bits 25-31
-            atomicOr(L.ws.event_err + rec.e, kErrBadDigi);
-            continue;
-        }
-        const bool surv = (int32_t)adc * rec.gain - rec.ped >= thr;
-        const uint32_t key = (li[k] << 17) | (r * C + c), e = (key << 11) | ((uint32_t)surv << 10) | t;
-        uint32_t s = hash_home(key, H);
-        bool dup = false;
-        for (uint32_t i = 0; i < H; ++i) {
-            const uint32_t old = atomicCAS(&table[s], kPackEmpty, e);
-            if (old == kPackEmpty) break;
-            if ((old >> 11) == key) {
-                dup = true;
-                break;
-            }
-            s = s + 1 == H ? 0u : s + 1;
-        }
-        if (dup) {
-            atomicOr(L.ws.event_err + rec.e, kErrDup);
-        } else if (surv) {
-            par[t] = e;
-            q[t] = 0;
-            np[t] = 0;
-            m[t] = make_int2(0, 0);
-            ent[k] = e;
-        }
-    }
-    gsync<GT, kWhole>(bar);
-
-    // 2
-#pragma unroll
-    for (int k = 0; k < kP; ++k) {
-        if (ent[k] == kPackEmpty) continue;
-        const uint32_t t = gt + k * GT, e = ent[k], key = e >> 11, r = w[k] & 0xFFu, c = (w[k] >> 8) & 0x1FFu;
-        uint32_t e1 = c > 0 ? pack_survivor(table, H, key - 1) : kPackEmpty, e2 = kPackEmpty;
-        if (r > 0) {
-            e2 = pack_survivor(table, H, key - C);
-            if (e2 == kPackEmpty) {
-                if (e1 == kPackEmpty && c > 0) e1 = pack_survivor(table, H, key - C - 1);
-                if (c + 1 < C) e2 = pack_survivor(table, H, key - C + 1);
-            } else if (e1 != kPackEmpty && pack_survivor(table, H, key - C - 1) != kPackEmpty) {
-                e2 = kPackEmpty; // the upper-left pixel already joins left and up
-            }
-        }
-        if (e1 == kPackEmpty) {
-            e1 = e2;
-            e2 = kPackEmpty;
-        }
-        if (e1 != kPackEmpty) {
-            const uint32_t old = atomicMin(&par[t], e1);
-            uint32_t a = e1, b = old; // another digi linked this one first: both trees are one
-            bool more = old != e;
-            for (;;) {
-                if (!more) {
-                    if (e2 == kPackEmpty) break;
-                    a = e;
-                    b = e2;
-                    e2 = kPackEmpty;
-                }
-                more = false;
-                key_union<kPackIdx>(par, a, b);
-            }
-        }
-    }
-    gsync<GT, kWhole>(bar);
-
-    // 3
-    bool heavy_here = false;
-#pragma unroll
-    for (int k = 0; k < kP; ++k) {
-        if (ent[k] == kPackEmpty) continue;
-        const ItemRec &rec = gs.rec[i0 + li[k]];
-        const uint32_t x = w[k], root = key_find<kPackIdx>(par, ent[k]), y = root & kPackIdx;
-        const int32_t qx = (int32_t)((x >> 17) & 0xFFu) * rec.gain - rec.ped;
-        if (atomicAdd(&q[y], qx) + qx > kQSafe32) heavy_here = true;
-        atomicAdd(&np[y], 1u);
-        atomicAdd(&m[y].x, qx * (int32_t)(x & 0xFFu));
-        atomicAdd(&m[y].y, qx * (int32_t)((x >> 8) & 0x1FFu));
-        ent[k] = root;
-    }
-    if (heavy_here) gs.heavy = 1;
-    gsync<GT, kWhole>(bar);
-    const bool heavy = gs.heavy != 0;
-    if (heavy) { // both moments again, in 64 bits
-        for (uint32_t i = gt; i < 2 * total; i += GT) exact[i] = 0;
-        gsync<GT, kWhole>(bar);
-#pragma unroll
-        for (int k = 0; k < kP; ++k) {
-            if (ent[k] == kPackEmpty) continue;
-            const ItemRec &rec = gs.rec[i0 + li[k]];
-            const uint32_t x = w[k], y = ent[k] & kPackIdx;
-            const long long qx = (long long)((int32_t)((x >> 17) & 0xFFu) * rec.gain - rec.ped);
-            atomicAdd(&exact[2 * y], (unsigned long long)(qx * (long long)(x & 0xFFu)));
-            atomicAdd(&exact[2 * y + 1], (unsigned long long)(qx * (long long)((x >> 8) & 0x1FFu)));
-        }
-        gsync<GT, kWhole>(bar);
-    }
-
-    // 4
-    uint32_t kr = 0; // bit k: digi k of this thread is a kept root
-#pragma unroll
-    for (int k = 0; k < kP; ++k) {
-        const uint32_t t = gt + k * GT;
-        if (t >= total) continue;
-        int32_t lab = -1;
-        if (ent[k] != kPackEmpty) {
-            const uint32_t y = ent[k] & kPackIdx;
-            const bool kept = q[y] >= cthr;
-            lab = kept ? (int32_t)((ent[k] >> 11) & 0x1FFFFu) : -2;
-            if (kept && y == t) {
-                table[gs.pack[li[k]] + atomicAdd(&gs.tmp[li[k]], 1u)] = ent[k];
-                kr |= 1u << k;
-            }
-        }
-        if (L.out.label) L.out.label[gs.rec[i0 + li[k]].label_off + idx[k]] = lab;
-    }
-    gsync<GT, kWhole>(bar);
-
-    // 5
-    if (gt < (uint32_t)kGroup && gs.pack[gt + 1] > gs.pack[gt])
-        L.ws.cursor[gs.ticket * L.cc.ticket_items + i0 + gt] = gs.tmp[gt];
-#pragma unroll
-    for (int k = 0; k < kP; ++k) {
-        if (!((kr >> k) & 1u)) continue;
-        const uint32_t t = gt + k * GT, e = ent[k], *list = table + gs.pack[li[k]], nk = gs.tmp[li[k]];
-        uint32_t ord = 0;
-        for (uint32_t i = 0; i < nk; ++i) ord += list[i] < e ? 1u : 0u;
-        const int32_t Q = q[t];
-        long long mr, mc;
-        if (heavy) {
-            mr = (long long)exact[2 * t];
-            mc = (long long)exact[2 * t + 1];
-        } else {
-            const int2 mm = m[t];
-            mr = mm.x;
-            mc = mm.y;
-        }
-        L.ws.staging.put(gs.b[i0 + li[k]] + ord, (int32_t)((e >> 11) & 0x1FFFFu), Q, (int32_t)np[t],
-                         centroid_abs(mr, Q), centroid_abs(mc, Q));
-        if (L.out.label16) np[t] = ord; // read back by the compact labels
-    }
-    if (L.out.label16) {
-        gsync<GT, kWhole>(bar);
-#pragma unroll
-        for (int k = 0; k < kP; ++k) {
-            const uint32_t t = gt + k * GT;
-            if (t >= total) continue;
-            uint16_t v = kLab16Below;
-            if (ent[k] != kPackEmpty) {
-                const uint32_t y = ent[k] & kPackIdx;
-                v = q[y] >= cthr ? (uint16_t)np[y] : kLab16Dropped;
-            }
-            L.out.label16[gs.rec[i0 + li[k]].label_off + idx[k]] = v;
-        }
-    }
-    gsync<GT, kWhole>(bar); // the slice and the plan are free
-}
-
-// ---------------------------------------------------------------- hash label store
 
 // The hash store (tuning label_store = kStoreHash) clusters an item with a
 // group of item_threads threads, one of the block's kCCThreads / item_threads
@@ -2146,12 +2223,12 @@ __device__ __forceinline__ void prefetch_ticket(const Launch &L, const GroupShar
 
 // All packs of a ticket (the first is planned by take_ticket).
 template <int GT, bool kWhole>
-__device__ __forceinline__ void pack_ticket(const Launch &L, unsigned char *mem, unsigned long long *exact,
-                                            GroupShared &gs, uint32_t gt, uint32_t bar)
+__device__ __forceinline__ void pack_ticket(const Launch &L, uint32_t mem, unsigned long long *exact,
+                                            GroupShared &gs, uint16_t *wlist, uint32_t gt, uint32_t bar)
 {
     for (uint32_t i0 = 0;;) {
         const uint32_t total = gs.pack[kGroup], end = gs.pack_end;
-        if (total) pack_items<GT, kWhole>(L, mem, exact, i0, total, gs, gt, bar);
+        if (total) pack_items<GT, kWhole>(L, mem, exact, i0, end - i0, total, gs, wlist, gt, bar);
         i0 = end;
         if (i0 >= L.cc.ticket_items) break;
         gsync<GT, kWhole>(bar); // the last pack's plan is read
@@ -2223,21 +2300,21 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
     }
 
     const uint32_t gid = tid / GT, gt = tid - gid * GT, bar = 1 + gid;
-    unsigned char *mem = dsm + L.cc.slice * gid;
+    const uint32_t mem = smem_addr(dsm) + L.cc.slice * gid;
     exact += (size_t)2 * L.cc.runs * gid;
     GroupShared &gs = s_gs[gid];
     for (uint32_t first = gid * gridDim.x + blockIdx.x; take_ticket<GT, kWhole>(L, gs, gt, bar, first);
          first = kNoSlot) {
         prefetch_ticket<GT>(L, gs, gt);
-        pack_ticket<GT, kWhole>(L, mem, exact, gs, gt, bar);
+        pack_ticket<GT, kWhole>(L, mem, exact, gs, wlist, gt, bar);
         for (uint32_t i = 0; i < L.cc.ticket_items; ++i) {
             const uint32_t n = gs.n[i];
             if (n <= L.cc.pack_item || (!kWhole && n > L.cc.large_digis)) continue;
             const ItemCtx it = make_item(L, gs.rec[i], gs.b[i], n);
             const uint32_t K = n <= (uint32_t)(kRunDigis * GT)
-                                   ? run_item<GT, kWhole, true>(L, it, smem_addr(mem), L.cc.runs, exact, gid, kGroups,
+                                   ? run_item<GT, kWhole, true>(L, it, mem, L.cc.runs, exact, gid, kGroups,
                                                                 gs, wlist, gt, bar)
-                                   : run_item<GT, kWhole, false>(L, it, smem_addr(mem), L.cc.runs, exact, gid, kGroups,
+                                   : run_item<GT, kWhole, false>(L, it, mem, L.cc.runs, exact, gid, kGroups,
                                                                  gs, wlist, gt, bar);
             if (gt == 0) kcount[gs.ticket * L.cc.ticket_items + i] = K;
         }
@@ -2278,7 +2355,7 @@ __global__ void __launch_bounds__(kCCThreads, kMinBlocks) cc_hash_kernel(const _
     uint32_t *kcount = L.ws.cursor;
     for (uint32_t first = blockIdx.x; take_ticket<GT0, true>(L, gs, tid, 0, first); first = kNoSlot) {
         prefetch_ticket<GT0>(L, gs, tid);
-        pack_ticket<GT0, true>(L, dsm, exact, gs, tid, 0);
+        pack_ticket<GT0, true>(L, smem_addr(dsm), exact, gs, wlist, tid, 0);
         const uint32_t item0 = gs.ticket * L.cc.ticket_items;
         // the items above the packed tier and within the store's capacity,
         // dealt round-robin to the block's groups
@@ -2627,7 +2704,7 @@ cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4
     if (err != cudaSuccess) return err;
     max_tile[0] = hash_tile[0] = 0;
     auto run_bytes = [&](uint32_t groups) { return [=](uint32_t t) { return run_smem_bytes(R, C, t, groups); }; };
-    auto hash_bytes = [&](uint32_t t) { return hash_smem_bytes(R, C, t); };
+    auto hash_bytes = [&](uint32_t t) { return cc_smem_bytes(R, C, t); };
     err = fit_tile(cc_kernel<kRunThreads1, kRunGroups1, 1>, device, 1, kRunThreads1, run_bytes(kRunGroups1),
                    kMaxTileSlots, &max_tile[1]);
     if (err == cudaSuccess)
@@ -2663,15 +2740,20 @@ static ClusterPlan cluster_plan(const Launch &L)
     p.ticket_items = ticket_items(p.items, (unsigned)L.cc_grid * groups, L.tune.ticket_max, L.N);
     p.workers = (uint32_t)L.cc_grid * groups;
     p.tickets = (p.items + p.ticket_items - 1) / p.ticket_items;
-    p.smem = (uint32_t)(hash ? hash_smem_bytes(R, C, T) : run_smem_bytes(R, C, T, groups));
+    p.smem = (uint32_t)(hash ? cc_smem_bytes(R, C, T) : run_smem_bytes(R, C, T, groups));
     p.slice = (p.smem / groups) & ~15u;
     p.whole_runs = run_capacity(p.smem, R, C);
     p.runs = run_capacity(p.slice, R, C);
     p.exact_slots = hash ? T : run_exact_slots(R, C, T, groups);
     if (hash) p.runs = std::min(run_capacity(p.slice - kHashListBytes, R, C), T);
-    p.pack_digis = pack_capacity(p.slice, p.runs);
+    p.pack_digis = pack_capacity(hash ? p.slice - kHashListBytes : p.slice, R, p.runs);
     p.pack_item = std::min(hash ? L.tune.warp_max : pack_max(L.tune.warp_max), p.pack_digis);
     p.large_digis = large_digis(R, C, L.tune);
+    // with no more items than blocks a group's neighbours are idle: items past
+    // what a group holds in registers take the whole block (64 items of 3,125
+    // digis: 61 -> 45 us; of 1,562, which it does hold: 41 us either way)
+    if (groups > 1 && p.items <= (uint32_t)L.cc_grid)
+        p.large_digis = std::min<uint32_t>(p.large_digis, kRunDigis * (kRunThreads1 / kRunGroups1));
     return p;
 }
 
