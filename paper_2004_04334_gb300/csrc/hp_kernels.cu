@@ -29,6 +29,9 @@
 //   copy_kernel     staged clusters to their ordered output positions; per-event
 //                   status codes
 //
+// Launches of few digis run three kernels instead: bucket_kernel (the first
+// three in one), the clustering kernel and finish_kernel (the last two).
+//
 // Labels are unique and the order of clusters fixed, so every tier gives the
 // same result: the id of a cluster is its smallest linear pixel index, the
 // root of its tree in every union-find here; charge, pixel count and the two
@@ -564,8 +567,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
             for (uint32_t p = threadIdx.x; p < total; p += kHistThreads) {
                 const uint32_t key = stage_k[p];
                 const uint32_t g = gb[key] + (p - lk[key]);
-                L.ws.bucket_w[g] = stage_w[p];
-                L.ws.bucket_i[g] = stage_i[p];
+                L.ws.bucket[g] = make_uint2(stage_w[p], stage_i[p]);
             }
             __syncthreads();
             if (threadIdx.x < ci.nkeys) gb[threadIdx.x] = kg + tot; // the key's cursor after this step
@@ -580,8 +582,7 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
                 if (m[j] == 0xFFFFFFFFu) continue;
                 const uint64_t key = (uint64_t)e_of[j] * M + m[j];
                 const uint32_t p = ci.use_sh ? bas[key - ci.keybase] + rank[j] : rank[j];
-                L.ws.bucket_w[p] = w[j];
-                L.ws.bucket_i[p] = (uint32_t)(k0 + j - event_start(e_of[j]));
+                L.ws.bucket[p] = make_uint2(w[j], (uint32_t)(k0 + j - event_start(e_of[j])));
             }
         }
         __syncthreads();
@@ -593,6 +594,209 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
             load_words(L, k0 + kChunk, c1, w);
         }
     }
+}
+
+// ---------------------------------------------------------------- bucketing of small launches
+
+// bucket_kernel: histogram, scan and scatter in one, for launches of few
+// digis: a thread-block cluster an event, each of its blocks a contiguous
+// slice of the event.  Every block counts its slice by module in shared
+// memory; after a cluster barrier each reads the others' counts (distributed
+// shared memory, four modules a load) and so knows, for every module, the
+// bucket's start and its own offset inside it; then it sorts its digis by
+// module in shared memory, kBucketStep at a time, and writes each module's run
+// with consecutive threads.  With one event the kernel also clears the
+// launch's control words, so that nothing precedes it.  Bound by launch and
+// global-memory latency: one launch in place of a memset and three kernels.
+constexpr int kBucketThreads = 1024;
+constexpr int kBucketCluster = 8;                             // portable cluster size
+constexpr int kBucketPer = 2 * kPerThread;                    // digis a thread holds
+constexpr uint32_t kBucketStep = kBucketThreads * kBucketPer; // digis a block sorts at a time
+
+// Lines of the small launches (bucket_fits, finish_fits).
+constexpr uint64_t kSmallDigis = 1u << 21;   // digis of the launch
+constexpr uint32_t kBucketModules = 2048;    // modules (four counters each in shared memory)
+constexpr uint64_t kBucketDigis = kBucketCluster * kBucketStep; // mean digis of an event (a step a block)
+constexpr uint32_t kFinishItems = 16384;     // (event, module) items every block scans
+
+__host__ __device__ constexpr uint32_t bucket_keys(uint32_t M) { return (M + 3) & ~3u; }
+__host__ __device__ constexpr size_t bucket_smem(uint32_t M)
+{
+    return (size_t)kBucketStep * (8 + 2) + (size_t)bucket_keys(M) * 4 * 4;
+}
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// Four words at this block's shared address a, in block r of the cluster.
+__device__ __forceinline__ uint4 lds_cluster4(uint32_t a, uint32_t r)
+{
+    uint4 v;
+    asm volatile("{\n\t"
+                 ".reg .u32 ra;\n\t"
+                 "mapa.shared::cluster.u32 ra, %4, %5;\n\t"
+                 "ld.shared::cluster.v4.u32 {%0, %1, %2, %3}, [ra];\n\t"
+                 "}" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a), "r"(r) : "memory");
+    return v;
+}
+
+__global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_constant__ Launch L)
+{
+    extern __shared__ __align__(16) uint32_t sh[];
+    __shared__ uint32_t tmp[2][kBucketThreads / 32 + 1];
+    __shared__ uint32_t s_bad;
+    pdl_trigger();
+    const uint32_t tid = threadIdx.x, M = L.g.M, MK = bucket_keys(M), rank = cluster_rank();
+    const uint32_t e = blockIdx.x / kBucketCluster;
+    uint2 *stage = reinterpret_cast<uint2 *>(sh);                       // [kBucketStep] sorted by module
+    uint16_t *skey = reinterpret_cast<uint16_t *>(stage + kBucketStep); // [kBucketStep]
+    uint32_t *hist = reinterpret_cast<uint32_t *>(skey + kBucketStep);  // [MK] digis of the slice
+    uint32_t *cnt = hist + MK;                                          // [MK] of a step
+    uint32_t *lk = cnt + MK;                                            // [MK] their start in the stage
+    uint32_t *gb = lk + MK;                                             // [MK] next bucket position
+    for (uint32_t k = tid; k < MK; k += kBucketThreads) hist[k] = 0;
+    if (tid == 0) s_bad = 0;
+    const uint64_t o0 = L.offsets[e], o1 = L.offsets[e + 1];
+    const bool bad_offsets = o0 > o1 || o1 > L.N || (e == 0 && o0 != 0) || (e == L.E - 1 && o1 != L.N);
+    if (L.E == 1 && rank == 0) { // otherwise cleared before the launch
+        if (tid < 16) L.ws.ctl[tid] = tid == 1 && bad_offsets ? kErrBadOffsets : 0u;
+        if (tid == 16) L.ws.event_err[0] = 0;
+    }
+    if (bad_offsets) { // uniform over the cluster
+        if (L.E > 1 && rank == 0 && tid == 0) atomicOr(&L.ws.ctl[1], kErrBadOffsets);
+        return;
+    }
+    // the slice [c0, c1), cut at multiples of kPerThread digis of the launch
+    // (so that every thread's groups of digis are 16-byte aligned)
+    const uint64_t g0 = o0 / kPerThread, ng = (o1 + kPerThread - 1) / kPerThread - g0;
+    const uint64_t a0 = (g0 + ng * rank / kBucketCluster) * kPerThread;
+    const uint64_t c0 = max(o0, a0), c1 = min(o1, (g0 + ng * (rank + 1) / kBucketCluster) * kPerThread);
+    const bool one_step = c1 <= a0 + kBucketStep;
+    // a thread's digis of the step at s0: group h at s0 + (h * threads + tid) * kPerThread;
+    // km: module, and (from the count of its step on) rank << 16; 0xFFFF: none
+    uint32_t km[kBucketPer], w[kBucketPer];
+    auto first = [&](uint64_t s0, int h) { return s0 + ((uint64_t)h * kBucketThreads + tid) * kPerThread; };
+    auto load_step = [&](uint64_t s0, bool words) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t k0 = first(s0, h);
+            uint32_t m8[kPerThread], w8[kPerThread];
+            load_modules(L, k0, c1, m8);
+            if (words) load_words(L, k0, c1, w8);
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) {
+                const bool in = k0 + j >= c0 && k0 + j < c1;
+                km[h * kPerThread + j] = in ? m8[j] : 0xFFFFFFFFu;
+                if (words) w[h * kPerThread + j] = w8[j];
+            }
+        }
+    };
+    bool bad = false;
+    auto count_step = [&](uint32_t *counts) {
+#pragma unroll
+        for (int j = 0; j < kBucketPer; ++j) {
+            if (km[j] < M)
+                km[j] |= atomicAdd(&counts[km[j]], 1u) << 16;
+            else {
+                bad |= km[j] != 0xFFFFFFFFu;
+                km[j] = 0xFFFFu;
+            }
+        }
+    };
+    load_step(a0, true);
+    __syncthreads();
+    count_step(hist); // (with a slice of one step these are its ranks)
+    for (uint64_t s0 = a0 + kBucketStep; s0 < c1; s0 += kBucketStep) {
+        load_step(s0, false);
+        count_step(hist);
+    }
+    if (!one_step) load_step(a0, false);
+    if (bad) s_bad = 1;
+    cluster_arrive();
+    cluster_wait();
+    if (tid == 0 && s_bad) atomicOr(&L.ws.event_err[e], kErrBadDigi);
+    // every module's bucket, and this block's offset inside it: four modules a thread
+    static_assert(kBucketModules <= 4 * kBucketThreads, "four modules a thread");
+    uint32_t total; // digis in the stage
+    {
+        const uint32_t k = 4 * tid;
+        uint4 t = make_uint4(0, 0, 0, 0), before = t, own = t;
+        if (k < MK) {
+            const uint32_t ha = (uint32_t)__cvta_generic_to_shared(hist + k);
+            uint4 v[kBucketCluster];
+#pragma unroll
+            for (uint32_t r = 0; r < kBucketCluster; ++r) v[r] = lds_cluster4(ha, r);
+#pragma unroll
+            for (uint32_t r = 0; r < kBucketCluster; ++r) {
+                t.x += v[r].x, t.y += v[r].y, t.z += v[r].z, t.w += v[r].w;
+                if (r < rank) before.x += v[r].x, before.y += v[r].y, before.z += v[r].z, before.w += v[r].w;
+                if (r == rank) own = v[r];
+            }
+        }
+        cluster_arrive(); // the others' counts are read
+        uint32_t unused;
+        uint32_t run = block_exclusive_scan<kBucketThreads>(t.x + t.y + t.z + t.w, tmp[0], &unused) + (uint32_t)o0;
+        const uint32_t mine = block_exclusive_scan<kBucketThreads>(own.x + own.y + own.z + own.w, tmp[1], &total);
+        if (k < MK) {
+            const uint4 b = make_uint4(run, run + t.x, run + t.x + t.y, run + t.x + t.y + t.z);
+            *reinterpret_cast<uint4 *>(gb + k) =
+                make_uint4(b.x + before.x, b.y + before.y, b.z + before.z, b.w + before.w);
+            *reinterpret_cast<uint4 *>(lk + k) =
+                make_uint4(mine, mine + own.x, mine + own.x + own.y, mine + own.x + own.y + own.z);
+            if (rank == 0) {
+                const uint32_t bs[4] = {b.x, b.y, b.z, b.w}, ts[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+                for (uint32_t i = 0; i < 4; ++i) {
+                    if (k + i >= M) break;
+                    const uint64_t item = (uint64_t)e * M + k + i;
+                    L.ws.count[item] = ts[i];
+                    L.ws.boff[item] = bs[i];
+                    if (ts[i] > L.cc.large_digis) L.ws.large[atomicAdd(&L.ws.ctl[5], 1u)] = (uint32_t)item;
+                }
+            }
+        }
+    }
+    for (uint64_t s0 = a0; s0 < c1; s0 += kBucketStep) {
+        __syncthreads();
+        if (!one_step) { // this step's counts, ranks and starts
+            for (uint32_t k = tid; k < MK; k += kBucketThreads) cnt[k] = 0;
+            __syncthreads();
+            count_step(cnt);
+            __syncthreads();
+            const uint32_t k = 4 * tid;
+            const uint4 c = k < MK ? *reinterpret_cast<const uint4 *>(cnt + k) : make_uint4(0, 0, 0, 0);
+            const uint32_t mine = block_exclusive_scan<kBucketThreads>(c.x + c.y + c.z + c.w, tmp[0], &total);
+            if (k < MK)
+                *reinterpret_cast<uint4 *>(lk + k) = make_uint4(mine, mine + c.x, mine + c.x + c.y, mine + c.x + c.y + c.z);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int j = 0; j < kBucketPer; ++j) {
+            const uint32_t key = km[j] & 0xFFFFu;
+            if (key == 0xFFFFu) continue;
+            const uint32_t p = lk[key] + (km[j] >> 16);
+            const uint64_t at = first(s0, j / kPerThread) + j % kPerThread;
+            stage[p] = make_uint2(w[j], (uint32_t)(at - o0));
+            skey[p] = (uint16_t)key;
+        }
+        __syncthreads();
+        // (the next step's digis load while this one is written out)
+        if (s0 + kBucketStep < c1) load_step(s0 + kBucketStep, true);
+        for (uint32_t p = tid; p < total; p += kBucketThreads) {
+            const uint32_t key = skey[p], g = gb[key] + (p - lk[key]);
+            L.ws.bucket[g] = stage[p];
+        }
+        if (!one_step) {
+            __syncthreads();
+            for (uint32_t k = tid; k < M; k += kBucketThreads) gb[k] += cnt[k];
+        }
+    }
+    cluster_wait(); // the others have read this block's counts
 }
 
 // ---------------------------------------------------------------- clustering
@@ -943,15 +1147,15 @@ __device__ __forceinline__ uint32_t run_contacts(const RunView &v, uint32_t W, u
 // loaded by load_digis), else loaded here.
 constexpr uint32_t kNoDigi = 0xFFFFFFFFu; // an invalid word (row 255, column 511)
 template <int GT>
-__device__ __forceinline__ void load_digis(uint32_t (&w)[kRunDigis], const uint32_t *bw, uint32_t mine)
+__device__ __forceinline__ void load_digis(uint32_t (&w)[kRunDigis], const uint2 *digis, uint32_t mine)
 {
 #pragma unroll
-    for (int k = 0; k < kRunDigis; ++k) w[k] = (uint32_t)k < mine ? __ldg(bw + k * GT) : kNoDigi;
+    for (int k = 0; k < kRunDigis; ++k) w[k] = (uint32_t)k < mine ? __ldg(&digis[k * GT].x) : kNoDigi;
 }
 template <int GT, bool kSingle, class F>
-__device__ __forceinline__ void each_four(uint32_t (&w)[kRunDigis], const uint32_t *bw, uint32_t mine, F &&f)
+__device__ __forceinline__ void each_four(uint32_t (&w)[kRunDigis], const uint2 *digis, uint32_t mine, F &&f)
 {
-    // bw points at the thread's first digi, mine = how many it has
+    // digis: the thread's first, GT from one to the next, mine of them
     if constexpr (kSingle) {
 #pragma unroll
         for (int k = 0; k < kRunDigis; k += 4) {
@@ -965,7 +1169,7 @@ __device__ __forceinline__ void each_four(uint32_t (&w)[kRunDigis], const uint32
         for (uint32_t base = 0; base < mine; base += 4) {
             uint32_t x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = base + u < mine ? __ldg(bw + (size_t)(base + u) * GT) : kNoDigi;
+            for (int u = 0; u < 4; ++u) x[u] = base + u < mine ? __ldg(&digis[(size_t)(base + u) * GT].x) : kNoDigi;
             f(0, base, x);
         }
     }
@@ -1194,8 +1398,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
     const uint32_t C = L.g.C, W = (C + 31) >> 5;
     const uint32_t n = it.n;
     const uint32_t mine = n > gt ? (n - gt - 1) / GT + 1 : 0u;
-    const uint32_t *bw = L.ws.bucket_w + it.b + gt;
-    const uint32_t *bi = L.ws.bucket_i + it.b + gt;
+    const uint2 *digis = L.ws.bucket + it.b + gt;
     const int32_t gain = it.gain, ped = it.ped;
     // runs of four digis, kNoSlot for those below threshold and past the last
     auto runs_of = [&](const uint32_t (&x)[4], uint32_t (&run)[4], uint32_t (&in)[4], uint32_t (&head)[4]) {
@@ -1220,7 +1423,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
     gsync<GT, kWhole>(bar);
 
     // 4
-    each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t, const uint32_t (&x)[4]) {
+    each_four<GT, kSingle>(w, digis, mine, [&](int k, uint32_t, const uint32_t (&x)[4]) {
         uint32_t run[4], in[4], head[4];
         runs_of(x, run, in, head);
 #pragma unroll
@@ -1255,13 +1458,13 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
         if constexpr (kSingle)
             return iv[k];
         else
-            return __ldg(bi + (size_t)j * GT);
+            return __ldg(&digis[(size_t)j * GT].y);
     };
     if constexpr (kSingle) {
         if (it.label_e || it.label16_e) {
 #pragma unroll
             for (int k = 0; k < kRunDigis; ++k)
-                if ((uint32_t)k < mine) iv[k] = __ldg(bi + k * GT);
+                if ((uint32_t)k < mine) iv[k] = __ldg(&digis[k * GT].y);
         }
     }
     gsync<GT, kWhole>(bar);
@@ -1276,7 +1479,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
         }
         gsync<GT, kWhole>(bar);
         for (uint32_t j = 0; j < mine; ++j) {
-            const uint32_t x[4] = {__ldg(bw + (size_t)j * GT), kNoDigi, kNoDigi, kNoDigi};
+            const uint32_t x[4] = {__ldg(&digis[(size_t)j * GT].x), kNoDigi, kNoDigi, kNoDigi};
             uint32_t run[4], in[4], head[4];
             runs_of(x, run, in, head);
             if (!in[0]) continue;
@@ -1290,7 +1493,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
 
     // 9: labels (the stores drain behind the staging)
     if (it.label_e) {
-        each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
+        each_four<GT, kSingle>(w, digis, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
             uint32_t run[4], in[4], head[4], at[4], p[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) at[u] = j + u < mine ? index_of(k + u, j + u) : 0u;
@@ -1316,7 +1519,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
     });
     if (it.label16_e) { // compact labels, once every kept root has its ordinal
         gsync<GT, kWhole>(bar);
-        each_four<GT, kSingle>(w, bw, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
+        each_four<GT, kSingle>(w, digis, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
             uint32_t run[4], in[4], head[4];
             if constexpr (kSingle) {
 #pragma unroll
@@ -1368,14 +1571,14 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
     const uint32_t R = L.g.R, C = L.g.C, W = (C + 31) >> 5, nw4 = run_words(R, C);
     const int32_t thr = L.g.pixel_thr;
     const uint32_t n = it.n, mine = n > gt ? (n - gt - 1) / GT + 1 : 0u;
-    const uint32_t *bw = L.ws.bucket_w + it.b + gt;
+    const uint2 *digis = L.ws.bucket + it.b + gt;
     const int32_t gain = it.gain, ped = it.ped;
     const uint32_t sb = mem, rp = sb + 4 * nw4;
     const uint32_t ab = mem + (uint32_t)run_fixed_bytes(R, C); // the bitmap of the dropped digis; then the run records
 
     // 1
     uint32_t w[kRunDigis];
-    if constexpr (kSingle) load_digis<GT>(w, bw, mine);
+    if constexpr (kSingle) load_digis<GT>(w, digis, mine);
     for (uint32_t i = gt; i < nw4 / 4; i += GT) {
         asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(sb + 16 * i), "r"(0) : "memory");
         asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(ab + 16 * i), "r"(0) : "memory");
@@ -1390,7 +1593,7 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 
     // 2
     uint32_t valid = 0;
-    each_four<GT, kSingle>(w, bw, mine, [&](int, uint32_t, const uint32_t (&x)[4]) {
+    each_four<GT, kSingle>(w, digis, mine, [&](int, uint32_t, const uint32_t (&x)[4]) {
 #pragma unroll
         for (int u = 0; u < 4; ++u) { // (words past the last digi are invalid, and OR in nothing)
             const uint32_t r = x[u] & 0xFFu, c = (x[u] >> 8) & 0x1FFu, adc = x[u] >> 17;
@@ -1537,10 +1740,10 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
 #pragma unroll
             for (uint32_t step = kGroup / 2; step; step >>= 1)
                 if (gs.pack[i + step] <= t) i += step;
-            const uint32_t pos = gs.b[i0 + i] + (t - gs.pack[i]);
+            const uint2 d = __ldg(L.ws.bucket + gs.b[i0 + i] + (t - gs.pack[i]));
             li[k] = i;
-            w[k] = __ldg(L.ws.bucket_w + pos);
-            idx[k] = __ldg(L.ws.bucket_i + pos);
+            w[k] = d.x;
+            idx[k] = d.y;
         }
     }
     for (uint32_t i = gt; i < nf; i += GT) sts(fields + 4 * i, 0);
@@ -1679,7 +1882,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
         for (int k = 0; k < 4; ++k) {
             if (gt + k * GT >= total || w[k] == kNoSlot) continue;
             const ItemRec &rec = gs.rec[i0 + li[k]];
-            const uint32_t x = __ldg(L.ws.bucket_w + gs.b[i0 + li[k]] + (gt + k * GT - gs.pack[li[k]]));
+            const uint32_t x = __ldg(&L.ws.bucket[gs.b[i0 + li[k]] + (gt + k * GT - gs.pack[li[k]])].x);
             const uint32_t y = a.parent(w[k]);
             const long long q = (long long)((int32_t)((x >> 17) & 0xFFu) * rec.gain - rec.ped);
             atomicAdd(&exact[2 * y], (unsigned long long)(q * (long long)(x & 0xFFu)));
@@ -1866,8 +2069,7 @@ __device__ uint32_t hash_item(const Launch &L, const ItemCtx &it, const HashMem 
     const uint32_t R = L.g.R, C = L.g.C;
     const int32_t thr = L.g.pixel_thr, cthr = L.g.cluster_thr;
     const uint32_t n = it.n, lane = threadIdx.x & 31, H = 2 * n;
-    const uint32_t *bw = L.ws.bucket_w + it.b;
-    const uint32_t *bi = L.ws.bucket_i + it.b;
+    const uint2 *digis = L.ws.bucket + it.b;
     const int32_t gain = it.gain, ped = it.ped;
 
     // 0
@@ -1877,7 +2079,7 @@ __device__ uint32_t hash_item(const Launch &L, const ItemCtx &it, const HashMem 
 #pragma unroll
     for (int k = 0; k < kD; ++k) {
         const uint32_t j = gt + k * GT;
-        w[k] = j < n ? __ldg(bw + j) : 0u;
+        w[k] = j < n ? __ldg(&digis[j].x) : 0u;
     }
     group_sync(bar, GT);
 
@@ -1999,7 +2201,7 @@ __device__ uint32_t hash_item(const Launch &L, const ItemCtx &it, const HashMem 
                 kr |= 1u << k;
             }
         }
-        if (it.label_e) it.label_e[__ldg(bi + j)] = lab;
+        if (it.label_e) it.label_e[__ldg(&digis[j].y)] = lab;
     }
     group_sync(bar, GT);
     if (gt == 0) *gheavy = 0; // read by every thread before the barrier above
@@ -2066,7 +2268,7 @@ __device__ uint32_t hash_item(const Launch &L, const ItemCtx &it, const HashMem 
                 const uint32_t y = rt[k] & kIdx;
                 v = h.q[y] >= cthr ? (uint16_t)h.np[y] : kLab16Dropped;
             }
-            it.label16_e[__ldg(bi + j)] = v;
+            it.label16_e[__ldg(&digis[j].y)] = v;
         }
     }
     group_sync(bar, GT); // the slice is free for the group's next item
@@ -2188,18 +2390,26 @@ __device__ __forceinline__ bool take_ticket(const Launch &L, GroupShared &gs, ui
         if (g32 < L.cc.tickets) {
             const uint32_t item = g32 * G + gt;
             const bool ok = gt < G && item < EM;
-            const uint32_t n = ok ? L.ws.count[item] : 0u;
+            // (every load before the first store, so that their latencies overlap)
+            const uint32_t at = ok ? item : g32 * G;
+            const uint32_t e = L.E == 1 ? 0u : at / L.g.M, m = at - e * L.g.M;
+            const uint32_t count = L.ws.count[at], b = L.ws.boff[at];
+            ItemRec rec;
+            rec.e = e;
+            rec.gain = L.g.gain[m];
+            rec.ped = L.g.ped[m];
+            rec.label_off = (uint32_t)L.offsets[e];
+            const uint32_t n = ok ? count : 0u;
             if (gt < (uint32_t)kGroup) {
                 gs.n[gt] = n;
-                const uint32_t b = ok ? L.ws.boff[item] : 0u;
                 gs.b[gt] = b;
+                gs.rec[gt] = rec;
                 if (ok) {
-                    gs.rec[gt] = make_rec(L, item);
                     if (n == 0) L.ws.cursor[item] = 0;
                     if (gt == G - 1 || item == EM - 1) gs.bucket_end = b + n;
                 }
             }
-            const uint32_t end = plan_pack(gs, 0, L.cc.pack_item, L.cc.pack_digis, gt, n);
+            const uint32_t end = min(plan_pack(gs, 0, L.cc.pack_item, L.cc.pack_digis, gt, n), G);
             if (gt == 0) gs.pack_end = end;
         }
         if (gt == 0) gs.ticket = g32;
@@ -2215,10 +2425,8 @@ template <int GT>
 __device__ __forceinline__ void prefetch_ticket(const Launch &L, const GroupShared &gs, uint32_t gt)
 {
     const uint32_t b0 = gs.b[0], digis = gs.bucket_end - b0;
-    for (uint32_t at = 32 * gt; at < digis; at += 32 * GT) {
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.ws.bucket_w + b0 + at));
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.ws.bucket_i + b0 + at));
-    }
+    for (uint32_t at = 16 * gt; at < digis; at += 16 * GT)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.ws.bucket + b0 + at));
 }
 
 // All packs of a ticket (the first is planned by take_ticket).
@@ -2233,8 +2441,9 @@ __device__ __forceinline__ void pack_ticket(const Launch &L, uint32_t mem, unsig
         if (i0 >= L.cc.ticket_items) break;
         gsync<GT, kWhole>(bar); // the last pack's plan is read
         if (gt < 32) {
-            const uint32_t e = plan_pack(gs, i0, L.cc.pack_item, L.cc.pack_digis, gt,
-                                         i0 + gt < (uint32_t)kGroup ? gs.n[i0 + gt] : 0u);
+            const uint32_t e = min(plan_pack(gs, i0, L.cc.pack_item, L.cc.pack_digis, gt,
+                                             i0 + gt < (uint32_t)kGroup ? gs.n[i0 + gt] : 0u),
+                                   L.cc.ticket_items);
             if (gt == 0) gs.pack_end = e;
         }
         gsync<GT, kWhole>(bar);
@@ -2263,7 +2472,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
     __shared__ uint16_t s_wlist[kThreads / 32][64];
     pdl_wait();
     pdl_trigger();
-    if (L.ws.ctl[1] & kErrBadOffsets) return;
+    const uint32_t launch_err = L.ws.ctl[1], nlarge = kWhole ? 0u : L.ws.ctl[5];
+    if (launch_err & kErrBadOffsets) return;
 
     const uint32_t tid = threadIdx.x;
     uint16_t *wlist = s_wlist[tid >> 5];
@@ -2271,7 +2481,6 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
     uint32_t *kcount = L.ws.cursor; // each item's count of kept clusters
 
     if constexpr (!kWhole) {
-        const uint32_t nlarge = L.ws.ctl[5];
         if (nlarge) {
             GroupShared &gs = s_gs[0];
             for (;;) {
@@ -2446,6 +2655,84 @@ __global__ void __launch_bounds__(kOffThreads) offsets_kernel(const Launch L)
     if (tid == 0 && P + total > L.out.capacity) atomicOr(&L.ws.ctl[1], kErrCapacity);
 }
 
+// Output positions p0 .. p0 + 3 (those below T) of one thread: `it` is the
+// item of p0, its clusters the positions [start, start + K); next(i, &start,
+// &K) gives those of item i.
+template <class F>
+__device__ __forceinline__ void copy_positions(const Launch &L, uint32_t p0, uint32_t T, bool vec, uint32_t it,
+                                               uint32_t start, uint32_t K, F &&next)
+{
+    const Staging sg = L.ws.staging;
+    const uint32_t M = L.g.M;
+    const uint32_t nv = min(4u, T - p0);
+    uint32_t mo[4];
+    int32_t id[4], q[4], np[4];
+    float x[4], y[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        mo[j] = 0;
+        id[j] = q[j] = np[j] = 0;
+        x[j] = y[j] = 0.f;
+        if ((uint32_t)j >= nv) continue;
+        const uint32_t p = p0 + j;
+        while (p - start >= K) { // on to the item holding p (count[it + 1] = start + K)
+            ++it;
+            next(it, &start, &K);
+        }
+        const uint64_t a = (uint64_t)L.ws.boff[it] + (p - start);
+        uint32_t e, m;
+        item_coords(it, M, &e, &m);
+        mo[j] = m;
+        id[j] = sg.id[a];
+        q[j] = sg.charge[a];
+        np[j] = sg.npix[a];
+        x[j] = sg.x[a];
+        y[j] = sg.y[a];
+    }
+    const ClusterCols host = {L.out.module, L.out.id, L.out.charge, L.out.npix, L.out.x, L.out.y};
+    const bool in_head = p0 + nv <= L.out.head_n, past_head = p0 >= L.out.head_n;
+    if (nv == 4 && (in_head || (past_head && vec))) {
+        const ClusterCols &d = in_head ? L.out.head : host;
+        *reinterpret_cast<uint4 *>(d.module + p0) = make_uint4(mo[0], mo[1], mo[2], mo[3]);
+        *reinterpret_cast<int4 *>(d.id + p0) = make_int4(id[0], id[1], id[2], id[3]);
+        *reinterpret_cast<int4 *>(d.charge + p0) = make_int4(q[0], q[1], q[2], q[3]);
+        *reinterpret_cast<int4 *>(d.npix + p0) = make_int4(np[0], np[1], np[2], np[3]);
+        *reinterpret_cast<float4 *>(d.x + p0) = make_float4(x[0], x[1], x[2], x[3]);
+        *reinterpret_cast<float4 *>(d.y + p0) = make_float4(y[0], y[1], y[2], y[3]);
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if ((uint32_t)j >= nv) continue;
+            const ClusterCols &d = p0 + j < L.out.head_n ? L.out.head : host;
+            d.module[p0 + j] = mo[j];
+            d.id[p0 + j] = id[j];
+            d.charge[p0 + j] = q[j];
+            d.npix[p0 + j] = np[j];
+            d.x[p0 + j] = x[j];
+            d.y[p0 + j] = y[j];
+        }
+    }
+}
+
+// 16-byte stores into the output columns are possible.
+__device__ __forceinline__ bool columns_aligned(const Outputs &o)
+{
+    return ((reinterpret_cast<uintptr_t>(o.module) | reinterpret_cast<uintptr_t>(o.id) |
+             reinterpret_cast<uintptr_t>(o.charge) | reinterpret_cast<uintptr_t>(o.npix) |
+             reinterpret_cast<uintptr_t>(o.x) | reinterpret_cast<uintptr_t>(o.y)) & 15) == 0;
+}
+
+// Status code of an event with these error bits (its own and the launch's).
+__device__ __forceinline__ int32_t event_status(uint32_t bits)
+{
+    if (bits & kErrBadOffsets) return 3; // HP_EINVAL
+    if (bits & kErrTimeout) return 8;    // HP_ETIMEOUT
+    if (bits & kErrCapacity) return 6;   // HP_ECAPACITY
+    if (bits & kErrBadDigi) return 4;    // HP_EBADDIGI
+    if (bits & kErrDup) return 5;        // HP_EDUP
+    return 0;                            // HP_OK
+}
+
 // copy_kernel: the staged clusters (SoA, at each item's bucket start) to
 // their ordered output positions, driven by the output: a warp takes a chunk
 // of kOutChunk consecutive positions, four a lane, finds the item of its
@@ -2465,24 +2752,14 @@ __global__ void __launch_bounds__(kCopyThreads) copy_kernel(const Launch L)
     const bool bad_offsets = (L.ws.ctl[1] & kErrBadOffsets) != 0;
     if (bad_offsets && gt <= L.E) L.out.cluster_offsets[gt] = 0; // no clusters
     if (gt < L.E) {
-        const uint32_t bits = L.ws.event_err[gt] | L.ws.ctl[1];
-        int32_t st = 0;                          // HP_OK
-        if (bits & kErrBadOffsets) st = 3;       // HP_EINVAL
-        else if (bits & kErrTimeout) st = 8;     // HP_ETIMEOUT
-        else if (bits & kErrCapacity) st = 6;    // HP_ECAPACITY
-        else if (bits & kErrBadDigi) st = 4;     // HP_EBADDIGI
-        else if (bits & kErrDup) st = 5;         // HP_EDUP
-        L.out.event_status[gt] = st;
+        L.out.event_status[gt] = event_status(L.ws.event_err[gt] | L.ws.ctl[1]);
     }
     if (bad_offsets) return;
-    const Staging sg = L.ws.staging;
     const uint32_t total = L.ws.ctl[6];
     const uint32_t T = (uint32_t)min((unsigned long long)total, (unsigned long long)L.out.capacity);
     const uint32_t nchunks = (uint32_t)(((uint64_t)total + kOutChunk - 1) / kOutChunk);
     const uint32_t last_item = (uint32_t)((uint64_t)L.E * M - 1);
-    const bool vec = ((reinterpret_cast<uintptr_t>(L.out.module) | reinterpret_cast<uintptr_t>(L.out.id) |
-                       reinterpret_cast<uintptr_t>(L.out.charge) | reinterpret_cast<uintptr_t>(L.out.npix) |
-                       reinterpret_cast<uintptr_t>(L.out.x) | reinterpret_cast<uintptr_t>(L.out.y)) & 15) == 0;
+    const bool vec = columns_aligned(L.out);
     const uint64_t warps = (uint64_t)gridDim.x * (kCopyThreads / 32);
     for (uint64_t ch = gt >> 5; ch < nchunks; ch += warps) {
         const uint32_t p0 = (uint32_t)ch * kOutChunk + 4 * lane;
@@ -2497,55 +2774,10 @@ __global__ void __launch_bounds__(kCopyThreads) copy_kernel(const Launch L)
             else hi = mid - 1;
         }
         uint32_t it = lo, start = L.ws.count[it], K = L.ws.cursor[it];
-        const uint32_t nv = min(4u, T - p0);
-        uint32_t mo[4];
-        int32_t id[4], q[4], np[4];
-        float x[4], y[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            mo[j] = 0;
-            id[j] = q[j] = np[j] = 0;
-            x[j] = y[j] = 0.f;
-            if ((uint32_t)j >= nv) continue;
-            const uint32_t p = p0 + j;
-            while (p - start >= K) { // on to the item holding p (count[it + 1] = start + K)
-                ++it;
-                start = L.ws.count[it];
-                K = L.ws.cursor[it];
-            }
-            const uint64_t a = (uint64_t)L.ws.boff[it] + (p - start);
-            uint32_t e, m;
-            item_coords(it, M, &e, &m);
-            mo[j] = m;
-            id[j] = sg.id[a];
-            q[j] = sg.charge[a];
-            np[j] = sg.npix[a];
-            x[j] = sg.x[a];
-            y[j] = sg.y[a];
-        }
-        const ClusterCols host = {L.out.module, L.out.id, L.out.charge, L.out.npix, L.out.x, L.out.y};
-        const bool in_head = p0 + nv <= L.out.head_n, past_head = p0 >= L.out.head_n;
-        if (nv == 4 && (in_head || (past_head && vec))) {
-            const ClusterCols &d = in_head ? L.out.head : host;
-            *reinterpret_cast<uint4 *>(d.module + p0) = make_uint4(mo[0], mo[1], mo[2], mo[3]);
-            *reinterpret_cast<int4 *>(d.id + p0) = make_int4(id[0], id[1], id[2], id[3]);
-            *reinterpret_cast<int4 *>(d.charge + p0) = make_int4(q[0], q[1], q[2], q[3]);
-            *reinterpret_cast<int4 *>(d.npix + p0) = make_int4(np[0], np[1], np[2], np[3]);
-            *reinterpret_cast<float4 *>(d.x + p0) = make_float4(x[0], x[1], x[2], x[3]);
-            *reinterpret_cast<float4 *>(d.y + p0) = make_float4(y[0], y[1], y[2], y[3]);
-        } else {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if ((uint32_t)j >= nv) continue;
-                const ClusterCols &d = p0 + j < L.out.head_n ? L.out.head : host;
-                d.module[p0 + j] = mo[j];
-                d.id[p0 + j] = id[j];
-                d.charge[p0 + j] = q[j];
-                d.npix[p0 + j] = np[j];
-                d.x[p0 + j] = x[j];
-                d.y[p0 + j] = y[j];
-            }
-        }
+        copy_positions(L, p0, T, vec, it, start, K, [&](uint32_t i, uint32_t *start_, uint32_t *k_) {
+            *start_ = L.ws.count[i];
+            *k_ = L.ws.cursor[i];
+        });
     }
     // with compact labels: every item's first cluster counted from its event's first
     if (L.out.item_first) {
@@ -2553,6 +2785,75 @@ __global__ void __launch_bounds__(kCopyThreads) copy_kernel(const Launch L)
         for (uint64_t item = gt; item < EM; item += (uint64_t)gridDim.x * kCopyThreads)
             L.out.item_first[item] = L.ws.count[item] - L.ws.count[item - item % M];
     }
+}
+
+// finish_kernel: offsets_kernel and copy_kernel in one, for launches of few
+// items (finish_fits): every block scans all items' counts for itself (in
+// shared memory, so no block waits for another), then copies its share of the
+// output positions, one a thread (whole lines a warp, and one chain of loads a
+// thread), finding its item by a binary search there.  Bound by launch latency
+// and a handful of L2 round trips.
+constexpr int kFinishThreads = 1024;
+
+__global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_constant__ Launch L)
+{
+    extern __shared__ uint32_t offs[]; // [EM + 1] first output position of each item
+    __shared__ uint32_t tmp[kFinishThreads / 32 + 1];
+    pdl_wait();
+    const uint32_t tid = threadIdx.x, M = L.g.M, EM = L.cc.items;
+    const uint64_t gt = (uint64_t)blockIdx.x * kFinishThreads + tid;
+    const uint32_t launch_bits = L.ws.ctl[1];
+    if (launch_bits & kErrBadOffsets) {
+        for (uint64_t e = gt; e <= L.E; e += (uint64_t)gridDim.x * kFinishThreads) {
+            L.out.cluster_offsets[e] = 0; // no clusters
+            if (e < L.E) L.out.event_status[e] = event_status(launch_bits);
+        }
+        return;
+    }
+    for (uint32_t i = tid; i < EM; i += kFinishThreads) offs[i] = L.ws.cursor[i];
+    __syncthreads();
+    const uint32_t per = ((EM + kFinishThreads - 1) / kFinishThreads) | 1u; // odd: no bank conflicts
+    const uint32_t i0 = min(EM, tid * per), i1 = min(EM, i0 + per);
+    uint32_t sum = 0, total;
+    for (uint32_t i = i0; i < i1; ++i) sum += offs[i];
+    uint32_t run = block_exclusive_scan<kFinishThreads>(sum, tmp, &total);
+    for (uint32_t i = i0; i < i1; ++i) {
+        const uint32_t k = offs[i];
+        offs[i] = run;
+        run += k;
+    }
+    if (tid == 0) offs[EM] = total;
+    __syncthreads();
+    const uint32_t bits = launch_bits | (total > L.out.capacity ? kErrCapacity : 0u);
+    for (uint64_t e = gt; e <= L.E; e += (uint64_t)gridDim.x * kFinishThreads) {
+        L.out.cluster_offsets[e] = offs[e * M];
+        if (e < L.E) L.out.event_status[e] = event_status(L.ws.event_err[e] | bits);
+    }
+    const uint32_t T = (uint32_t)min((unsigned long long)total, (unsigned long long)L.out.capacity);
+    const Staging sg = L.ws.staging;
+    const ClusterCols host = {L.out.module, L.out.id, L.out.charge, L.out.npix, L.out.x, L.out.y};
+    for (uint64_t at = gt; at < T; at += (uint64_t)gridDim.x * kFinishThreads) {
+        const uint32_t p = (uint32_t)at;
+        uint32_t lo = 0, hi = EM - 1; // the last item that starts at or before p
+        while (lo < hi) {
+            const uint32_t mid = (lo + hi + 1) >> 1;
+            if (offs[mid] <= p) lo = mid;
+            else hi = mid - 1;
+        }
+        const uint64_t a = (uint64_t)L.ws.boff[lo] + (p - offs[lo]);
+        const ClusterCols &d = p < L.out.head_n ? L.out.head : host;
+        d.module[p] = L.E == 1 ? lo : lo % M;
+        const int32_t id = sg.id[a], q = sg.charge[a], np = sg.npix[a];
+        const float x = sg.x[a], y = sg.y[a];
+        d.id[p] = id;
+        d.charge[p] = q;
+        d.npix[p] = np;
+        d.x[p] = x;
+        d.y[p] = y;
+    }
+    if (L.out.item_first)
+        for (uint64_t item = gt; item < EM; item += (uint64_t)gridDim.x * kFinishThreads)
+            L.out.item_first[item] = offs[item] - offs[item - item % M];
 }
 
 // Serving batches: block (x, e) copies a slice of request e's digis.
@@ -2630,8 +2931,7 @@ size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t 
     w.boff = reinterpret_cast<uint32_t *>(take(4ull * EM));
     w.blk_off = reinterpret_cast<uint32_t *>(take(4ull * kHistCap * bucket_grid(N, sm_count)));
     w.cursor = reinterpret_cast<uint32_t *>(take(4ull * EM));
-    w.bucket_w = reinterpret_cast<uint32_t *>(take(4ull * N));
-    w.bucket_i = reinterpret_cast<uint32_t *>(take(4ull * N));
+    w.bucket = reinterpret_cast<uint2 *>(take(8ull * N));
     w.chunk_item = reinterpret_cast<uint32_t *>(take(4ull * (N / kOutChunk + 2)));
     w.staging.id = reinterpret_cast<int32_t *>(take(4ull * N));
     w.staging.charge = reinterpret_cast<int32_t *>(take(4ull * N));
@@ -2701,6 +3001,12 @@ cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4
     cudaError_t err = cudaSetDevice(device);
     if (err != cudaSuccess) return err;
     err = cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kScatterSmem);
+    if (err != cudaSuccess) return err;
+    err = cudaFuncSetAttribute(bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)bucket_smem(kBucketModules));
+    if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)((kFinishItems + 1) * 4));
     if (err != cudaSuccess) return err;
     max_tile[0] = hash_tile[0] = 0;
     auto run_bytes = [&](uint32_t groups) { return [=](uint32_t t) { return run_smem_bytes(R, C, t, groups); }; };
@@ -2774,12 +3080,49 @@ cudaError_t launch_dependent(K kern, unsigned grid, unsigned block, size_t smem,
     return cudaLaunchKernelEx(&cfg, kern, L);
 }
 
+// Whether the launch's digis are bucketed by bucket_kernel (one launch, a
+// cluster an event) and its clusters ordered by finish_kernel, instead of by
+// three kernels and two: small launches, whose time is that of the kernel
+// boundaries (one event of 1,300 digis 36 -> 23 us, of 60,000 on 1,856 modules
+// 49 -> 33 us).  Events past a step a block are counted twice, by eight blocks
+// only, and the three kernels' grid is faster (200,000 digis: 51 us against
+// 43); past kSmallDigis the boundaries no longer count.
+static bool bucket_fits(const Launch &L)
+{
+    return L.N > 0 && L.N <= kSmallDigis && L.g.M <= kBucketModules && L.N / L.E <= kBucketDigis;
+}
+static bool finish_fits(const Launch &L)
+{
+    return L.N <= kSmallDigis && L.cc.items <= kFinishItems && !L.debug;
+}
+static cudaError_t launch_bucket(const Launch &L, cudaStream_t stream)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(L.E * kBucketCluster);
+    cfg.blockDim = dim3(kBucketThreads);
+    cfg.dynamicSmemBytes = bucket_smem(L.g.M);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kBucketCluster;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, bucket_kernel, L);
+}
+
 cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *kernel_count, cudaEvent_t *marks)
 {
     NvtxRange range("hp_launch_reconstruct");
     Launch L = in;
     L.cc = cluster_plan(L);
-    cudaError_t err = cudaMemsetAsync(L.ws.ctl, 0, L.ws.zero_bytes, stream);
+    const bool finish = finish_fits(L), fused = finish && bucket_fits(L); // (the order chain is cleared for neither)
+    cudaError_t err = cudaSuccess;
+    if (!fused)
+        err = cudaMemsetAsync(L.ws.ctl, 0, L.ws.zero_bytes, stream);
+    else if (L.E > 1) // (with one event the bucket kernel clears them)
+        err = cudaMemsetAsync(L.ws.ctl, 0, (size_t)((unsigned char *)L.ws.count - (unsigned char *)L.ws.ctl), stream);
     if (err != cudaSuccess) return err;
     auto mark = [&](int i) {
         if (marks && err == cudaSuccess) err = cudaEventRecord(marks[i], stream);
@@ -2788,15 +3131,23 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
     // persistent histogram and scatter over the same contiguous ranges
     const unsigned hist_grid = bucket_grid(L.N, L.sm_count), scat_grid = hist_grid; // the same ranges
     mark(0);
-    if (L.N > 0) {
+    if (fused) { // (counted as the scatter)
+        mark(1);
+        mark(2);
+        if (err == cudaSuccess) err = launch_bucket(L, stream);
+        ++nk;
+    }
+    if (!fused && L.N > 0) {
         hist_kernel<<<hist_grid, kHistThreads, kHistCap * sizeof(uint32_t), stream>>>(L);
         ++nk;
     }
-    mark(1);
-    if (err == cudaSuccess) err = launch_dependent(scan_kernel, L.E, 256, 0, stream, L);
-    ++nk;
-    mark(2);
-    if (L.N > 0) {
+    if (!fused) {
+        mark(1);
+        if (err == cudaSuccess) err = launch_dependent(scan_kernel, L.E, 256, 0, stream, L);
+        ++nk;
+        mark(2);
+    }
+    if (!fused && L.N > 0) {
         if (err == cudaSuccess) err = launch_dependent(scatter_kernel, scat_grid, kHistThreads, kScatterSmem, stream, L);
         ++nk;
     }
@@ -2819,11 +3170,20 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
     ++nk;
     mark(4);
     const uint64_t EM = (uint64_t)L.E * L.g.M;
-    if (err == cudaSuccess)
-        err = launch_dependent(offsets_kernel, (unsigned)((EM + kOffItems - 1) / kOffItems), kOffThreads, 0, stream, L);
-    ++nk;
+    if (!finish) {
+        if (err == cudaSuccess)
+            err = launch_dependent(offsets_kernel, (unsigned)((EM + kOffItems - 1) / kOffItems), kOffThreads, 0, stream,
+                                   L);
+        ++nk;
+    }
     mark(5);
-    {   // a warp per output chunk (at most copy_grid blocks, looping), and a thread per event status and offset
+    if (finish) { // a thread per expected cluster (one in eight digis; at most the copy's threads, looping)
+        const uint64_t by_items = (L.N / 8 + kFinishThreads) / kFinishThreads;
+        const uint64_t most = std::max<uint64_t>(1, (uint64_t)L.copy_grid * kCopyThreads / kFinishThreads);
+        if (err == cudaSuccess)
+            err = launch_dependent(finish_kernel, (unsigned)std::min(by_items, most), kFinishThreads,
+                                   ((size_t)L.cc.items + 1) * 4, stream, L);
+    } else { // a warp per output chunk (at most copy_grid blocks, looping), and a thread per event status and offset
         const uint64_t by_items = (L.N / kOutChunk + 1 + kCopyThreads / 32 - 1) / (kCopyThreads / 32);
         const uint64_t by_events = ((uint64_t)L.E + kCopyThreads) / kCopyThreads; // E + 1 offsets
         const uint64_t blocks =
