@@ -1137,24 +1137,31 @@ __device__ __forceinline__ uint32_t atoms_min(uint32_t a, uint32_t v)
 // 13,000-digi ones among them: 1,374 -> 614 us (its records are 20 bytes, so
 // these fit a block's shared memory now).
 //
-// Run records, in shared memory or (kBig) global scratch:
-//   word 0  union-find parent << kRunShift | (roots) pixels of the cluster
+// Run records:
+//   word 0  union-find parent
 //   word 1  row | col << 8 of the first pixel (the digi word's layout), its
 //           length << 17, and in the packed tier its item << 23; from phase 8
 //           on the root's position and item, and a flag
-//   word 2  the sum of phase 4; then the charge, and word 3 sum q * col: of
-//           the run, then (roots) the cluster
-//   word 4  the list of phase 5; then (roots) sum q * (row - root's row)
-//   word 5  (kBig only, whose word 0 is the parent alone) pixels
+//   word 2  the sum of phase 4; then the ADC sum and << 20 the pixels, of the
+//           run, then (roots) of the cluster: Q = gain * ADC - ped * pixels
+//   word 3  sum q * col, the same way
+//   word 4  the list of phase 5; then (roots) sum q * (row - root's row);
+//           with compact labels at last the ordinal
+// Items of up to kNarrowDigis digis, whose sums fit word 2, in shared memory
+// (kNarrow).  Larger ones keep the charge in word 2 and the pixels below the
+// parent in word 0, or with records in global scratch (kGlobal) in a word of
+// their own.
 constexpr int kRunDigis = 8; // digis a thread holds at once
-constexpr uint32_t kRunShift = 18, kRunPixels = (1u << kRunShift) - 1u;
+constexpr uint32_t kRunShift = 18, kRunPixels = (1u << kRunShift) - 1u; // kWide: parent << 18 | pixels
+constexpr uint32_t kAdcBits = 20, kAdcMask = (1u << kAdcBits) - 1u;       // kNarrow: ADC sum | pixels << 20
+constexpr uint32_t kNarrowDigis = 4095;
+static_assert(kNarrowDigis * 255u <= kAdcMask && kNarrowDigis < 1u << (32 - kAdcBits), "word 2 of kNarrow");
+enum RunKind { kNarrow, kWide, kGlobal };
 constexpr uint32_t kRunKept = 1u << 31, kRunDropped = 1u << 30, kRunPos = 0x1FFFFu;
 constexpr uint32_t kRunItem = 15u << 23; // packed tier: the run's item
 
-template <bool kBig>
-struct Runs;
-template <>
-struct Runs<false> {
+template <RunKind kKind>
+struct Runs { // kNarrow and kWide: shared memory
     uint32_t base;
     using At = uint32_t;
     __device__ __forceinline__ At at(uint32_t i) const { return base + i * (uint32_t)kRunBytes; }
@@ -1164,11 +1171,17 @@ struct Runs<false> {
     __device__ __forceinline__ static void st(At a, uint32_t v) { sts<4 * f>(a, v); }
     template <int f>
     __device__ __forceinline__ static void red(At a, uint32_t v) { reds_add<4 * f>(a, v); }
-    __device__ __forceinline__ uint32_t parent(uint32_t i) const { return ld<0>(at(i)) >> kRunShift; }
-    __device__ __forceinline__ void set_parent(uint32_t i, uint32_t p) const { st<0>(at(i), p << kRunShift); }
+    __device__ __forceinline__ uint32_t parent(uint32_t i) const
+    {
+        return kKind == kWide ? ld<0>(at(i)) >> kRunShift : ld<0>(at(i));
+    }
+    __device__ __forceinline__ void set_parent(uint32_t i, uint32_t p) const
+    {
+        st<0>(at(i), kKind == kWide ? p << kRunShift : p);
+    }
     __device__ __forceinline__ uint32_t min_parent(uint32_t i, uint32_t p) const
     {
-        return atoms_min(at(i), p << kRunShift) >> kRunShift;
+        return kKind == kWide ? atoms_min(at(i), p << kRunShift) >> kRunShift : atoms_min(at(i), p);
     }
     // the packed sum v into the pixel's run, if in != 0; the run's position,
     // if head != 0 (predicated: no branch among the lanes)
@@ -1182,18 +1195,35 @@ struct Runs<false> {
                      "@h st.shared.u32 [%0+4], %4;\n\t"
                      "}" ::"r"(a), "r"(v), "r"(in), "r"(head), "r"(pos) : "memory");
     }
-    __device__ __forceinline__ static void add_pixels(At a, uint32_t v) { red<0>(a, v); }
-    __device__ __forceinline__ static uint32_t pixels(At a) { return ld<0>(a) & kRunPixels; }
-    __device__ __forceinline__ static void set_ordinal(At a, uint32_t i, uint32_t v) { st<0>(a, (i << kRunShift) | v); }
+    // a run's ADC sum and length, or its charge, into word 2
+    __device__ __forceinline__ static void set_sum(At a, uint32_t adc, uint32_t len, uint32_t q)
+    {
+        st<2>(a, kKind == kWide ? q : adc | (len << kAdcBits));
+    }
+    __device__ __forceinline__ static uint32_t charge(uint32_t word2, int2 cal)
+    {
+        return kKind == kWide ? word2 : (uint32_t)cal.x * (word2 & kAdcMask) - (uint32_t)cal.y * (word2 >> kAdcBits);
+    }
+    // pixels of a run into its root's (its own if it is one)
+    __device__ __forceinline__ static void add_pixels(At a, uint32_t v)
+    {
+        if (kKind == kWide) red<0>(a, v);
+    }
+    __device__ __forceinline__ static uint32_t pixels(At a)
+    {
+        return kKind == kWide ? ld<0>(a) & kRunPixels : ld<2>(a) >> kAdcBits;
+    }
+    __device__ __forceinline__ static void set_ordinal(At a, uint32_t v) { st<4>(a, v); }
+    __device__ __forceinline__ static uint32_t ordinal(At a) { return ld<4>(a); }
     __device__ __forceinline__ static void init(At a, uint32_t i)
     {
-        st<0>(a, i << kRunShift);
+        st<0>(a, kKind == kWide ? i << kRunShift : i);
         st<2>(a, 0);
         st<4>(a, 0);
     }
 };
 template <>
-struct Runs<true> {
+struct Runs<kGlobal> {
     uint32_t *base;
     using At = uint32_t *;
     __device__ __forceinline__ At at(uint32_t i) const { return base + (size_t)i * (kBigRunBytes / 4); }
@@ -1213,9 +1243,12 @@ struct Runs<true> {
             if (head) st<1>(a, pos);
         }
     }
+    __device__ __forceinline__ static void set_sum(At a, uint32_t, uint32_t, uint32_t q) { st<2>(a, q); }
+    __device__ __forceinline__ static uint32_t charge(uint32_t word2, int2) { return word2; }
     __device__ __forceinline__ static void add_pixels(At a, uint32_t v) { atomicAdd(a + 5, v); }
     __device__ __forceinline__ static uint32_t pixels(At a) { return ld<5>(a); }
-    __device__ __forceinline__ static void set_ordinal(At a, uint32_t, uint32_t v) { st<5>(a, v); }
+    __device__ __forceinline__ static void set_ordinal(At a, uint32_t v) { st<4>(a, v); }
+    __device__ __forceinline__ static uint32_t ordinal(At a) { return ld<4>(a); }
     __device__ __forceinline__ static void init(At a, uint32_t i)
     {
         st<0>(a, i);
@@ -1297,9 +1330,10 @@ __device__ __forceinline__ uint32_t run_contacts(const RunView &v, uint32_t W, u
 }
 
 // The item's digis, four at a time so that their loads overlap:
-// f(k, j, x) for the thread's digis j .. j + 3 with words x[4] (kNoDigi for
+// f(k, j, x) for the thread's digis j .. j + 3 with words x[kBatch] (kNoDigi for
 // those past the last), held in w[k] .. w[k + 3] with kSingle (all of them
 // loaded by load_digis), else loaded here.
+constexpr int kBatch = 2; // (4: more slots past a thread's last digi; 27.7M digis 530 us, 2: 519, 1: 526)
 constexpr uint32_t kNoDigi = 0xFFFFFFFFu; // an invalid word (row 255, column 511)
 template <int GT>
 __device__ __forceinline__ void load_digis(uint32_t (&w)[kRunDigis], const uint2 *digis, uint32_t mine)
@@ -1308,23 +1342,25 @@ __device__ __forceinline__ void load_digis(uint32_t (&w)[kRunDigis], const uint2
     for (int k = 0; k < kRunDigis; ++k) w[k] = (uint32_t)k < mine ? __ldg(&digis[k * GT].x) : kNoDigi;
 }
 template <int GT, bool kSingle, class F>
-__device__ __forceinline__ void each_four(uint32_t (&w)[kRunDigis], const uint2 *digis, uint32_t mine, F &&f)
+__device__ __forceinline__ void each_batch(uint32_t (&w)[kRunDigis], const uint2 *digis, uint32_t mine, F &&f)
 {
     // digis: the thread's first, GT from one to the next, mine of them
     if constexpr (kSingle) {
 #pragma unroll
-        for (int k = 0; k < kRunDigis; k += 4) {
+        for (int k = 0; k < kRunDigis; k += kBatch) {
             if ((uint32_t)k < mine) {
-                uint32_t x[4] = {w[k], w[k + 1], w[k + 2], w[k + 3]};
+                uint32_t x[kBatch];
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) x[u] = w[k + u];
                 f(k, (uint32_t)k, x);
             }
         }
     } else {
 #pragma unroll 1
-        for (uint32_t base = 0; base < mine; base += 4) {
-            uint32_t x[4];
+        for (uint32_t base = 0; base < mine; base += kBatch) {
+            uint32_t x[kBatch];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = base + u < mine ? __ldg(&digis[(size_t)(base + u) * GT].x) : kNoDigi;
+            for (int u = 0; u < kBatch; ++u) x[u] = base + u < mine ? __ldg(&digis[(size_t)(base + u) * GT].x) : kNoDigi;
             f(0, base, x);
         }
     }
@@ -1366,7 +1402,7 @@ __device__ __forceinline__ void link_runs(const A &a, const V &view, const B &ca
             // q = gain * ADC - ped over the run's pixels, columns c0 ..
             const int2 cal = calib(p[u]);
             const uint32_t c0 = (p[u] >> 8) & 0x1FFu, adc = sum[u] & kSumMask, base = c0 & ~31u;
-            A::template st<2>(r, cal.x * adc - cal.y * len);
+            A::set_sum(r, adc, len, cal.x * adc - cal.y * len);
             A::template st<3>(r, cal.x * ((sum[u] >> kSumShift) + base * adc) -
                                      cal.y * (len * c0 + ((len * (len - 1u)) >> 1)));
             if (k < end)
@@ -1399,8 +1435,8 @@ __device__ __forceinline__ void link_runs(const A &a, const V &view, const B &ca
 
 // Phase 7: only roots receive sums, so a run's own are still its own; two
 // runs a thread at a time.
-template <int GT, class A>
-__device__ __forceinline__ void sum_runs(const A &a, uint32_t nruns, uint32_t gt)
+template <int GT, class A, class B>
+__device__ __forceinline__ void sum_runs(const A &a, const B &calib, uint32_t nruns, uint32_t gt)
 {
     for (uint32_t i0 = gt; i0 < nruns; i0 += 2 * GT) {
         const uint32_t i1 = i0 + GT < nruns ? i0 + GT : i0;
@@ -1429,7 +1465,7 @@ __device__ __forceinline__ void sum_runs(const A &a, uint32_t nruns, uint32_t gt
                 a.set_parent(i[u], x[u]);
                 A::template red<2>(rx, q[u]);
                 A::template red<3>(rx, mc[u]);
-                A::template red<4>(rx, q[u] * ((p[u] & 0xFFu) - (px[u] & 0xFFu)));
+                A::template red<4>(rx, A::charge(q[u], calib(p[u])) * ((p[u] & 0xFFu) - (px[u] & 0xFFu)));
             }
             A::add_pixels(rx, (p[u] >> 17) & 63u);
         }
@@ -1447,13 +1483,14 @@ __device__ __forceinline__ void warp_chunks(uint32_t nruns, uint32_t warp, uint3
 
 // Phase 8: the root's position (and item) into every run, with kRunKept on a
 // kept root and kRunDropped on the runs of a cluster below threshold; gs.heavy
-// set if a cluster's moments may have overflowed 32 bits.  With
+// set if a cluster's moments may have overflowed 32 bits; also(run, root's
+// position, kept) for every run.  With
 // kItems the kept roots of each item are counted in gs.tmp[16 ..].  One
 // barrier; returns the kept roots of all runs, and in *ord those before the
 // warp's chunks.
-template <int GT, bool kWhole, bool kItems, class A>
-__device__ __forceinline__ uint32_t mark_runs(const A &a, uint32_t nruns, int32_t cthr, GroupShared &gs, uint32_t gt,
-                                              uint32_t bar, uint32_t *ord)
+template <int GT, bool kWhole, bool kItems, class A, class B, class T>
+__device__ __forceinline__ uint32_t mark_runs(const A &a, const B &calib, const T &also, uint32_t nruns, int32_t cthr,
+                                              GroupShared &gs, uint32_t gt, uint32_t bar, uint32_t *ord)
 {
     constexpr int kWarps = GT / 32;
     const uint32_t lane = gt & 31, warp = gt >> 5;
@@ -1466,10 +1503,11 @@ __device__ __forceinline__ uint32_t mark_runs(const A &a, uint32_t nruns, int32_
             const uint32_t x = a.parent(i);
             const typename A::At rx = a.at(x);
             const uint32_t px = A::template ld<1>(rx);
-            const int32_t Q = (int32_t)A::template ld<2>(rx);
+            const int32_t Q = (int32_t)A::charge(A::template ld<2>(rx), calib(px));
             const bool kept = Q >= cthr;
             lead = kept && x == i;
             if (Q > kQSafe32) gs.heavy = 1;
+            also(a.at(i), px, kept);
             A::template st<1>(a.at(i), (px & (kItems ? kRunPos | kRunItem : kRunPos)) |
                                            (lead ? kRunKept : kept ? 0u : kRunDropped));
             if (kItems && lead) atomicAdd(&gs.tmp[16 + ((px & kRunItem) >> 23)], 1u);
@@ -1526,12 +1564,12 @@ __device__ __forceinline__ void stage_runs(const A &a, uint32_t nruns, uint32_t 
 
 // The sums of root i as a staged cluster at position `at`.
 template <class A>
-__device__ __forceinline__ void stage_root(const Launch &L, const A &a, uint32_t i, uint64_t at, bool heavy,
+__device__ __forceinline__ void stage_root(const Launch &L, const A &a, uint32_t i, uint64_t at, int2 cal, bool heavy,
                                            const unsigned long long *exact)
 {
     const typename A::At r = a.at(i);
     const uint32_t p = A::template ld<1>(r);
-    const int32_t Q = (int32_t)A::template ld<2>(r), np = (int32_t)A::pixels(r);
+    const int32_t Q = (int32_t)A::charge(A::template ld<2>(r), cal), np = (int32_t)A::pixels(r);
     float x, y;
     if (heavy) {
         x = centroid_abs((long long)exact[2 * (size_t)i], Q);
@@ -1543,29 +1581,29 @@ __device__ __forceinline__ void stage_root(const Launch &L, const A &a, uint32_t
     L.ws.staging.put(at, (int32_t)((p & 0xFFu) * L.g.C + ((p >> 8) & 0x1FFu)), Q, np, x, y);
 }
 
-template <int GT, bool kWhole, bool kBig, bool kSingle>
+template <int GT, bool kWhole, RunKind kKind, bool kSingle>
 __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx &it, uint32_t sb, uint32_t rp,
-                                                 const Runs<kBig> a, unsigned long long *exact, uint32_t nruns,
+                                                 const Runs<kKind> a, unsigned long long *exact, uint32_t nruns,
                                                  uint32_t (&w)[kRunDigis], GroupShared &gs, uint16_t *wlist,
                                                  uint32_t gt, uint32_t bar)
 {
-    using A = Runs<kBig>;
+    using A = Runs<kKind>;
     const uint32_t C = L.g.C, W = (C + 31) >> 5;
     const uint32_t n = it.n;
     const uint32_t mine = n > gt ? (n - gt - 1) / GT + 1 : 0u;
     const uint2 *digis = L.ws.bucket + it.b + gt;
     const int32_t gain = it.gain, ped = it.ped;
-    // runs of four digis, kNoSlot for those below threshold and past the last
-    auto runs_of = [&](const uint32_t (&x)[4], uint32_t (&run)[4], uint32_t (&in)[4], uint32_t (&head)[4]) {
-        uint32_t word[4], pre[4];
+    // runs of a batch of digis, kNoSlot for those below threshold and past the last
+    auto runs_of = [&](const uint32_t (&x)[kBatch], uint32_t (&run)[kBatch], uint32_t (&in)[kBatch], uint32_t (&head)[kBatch]) {
+        uint32_t word[kBatch], pre[kBatch];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kBatch; ++u) {
             const uint32_t wi = x[u] == kNoDigi ? 0u : (x[u] & 0xFFu) * W + ((x[u] >> 13) & 0xFu);
             word[u] = lds(sb + 4 * wi);
             pre[u] = lds_u16(rp + 2 * wi);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kBatch; ++u) {
             const uint32_t b = x[u] == kNoDigi ? 0u : 1u << ((x[u] >> 8) & 31u), h = word[u] & ~(word[u] << 1);
             in[u] = word[u] & b;
             head[u] = h & b;
@@ -1578,11 +1616,11 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
     gsync<GT, kWhole>(bar);
 
     // 4
-    each_four<GT, kSingle>(w, digis, mine, [&](int k, uint32_t, const uint32_t (&x)[4]) {
-        uint32_t run[4], in[4], head[4];
+    each_batch<GT, kSingle>(w, digis, mine, [&](int k, uint32_t, const uint32_t (&x)[kBatch]) {
+        uint32_t run[kBatch], in[kBatch], head[kBatch];
         runs_of(x, run, in, head);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kBatch; ++u) {
             A::add_pixel(a.at(in[u] ? run[u] : 0u), pixel_sum(x[u]), in[u], head[u], x[u] & kRunPos);
             if constexpr (kSingle) w[k + u] = run[u];
         }
@@ -1603,11 +1641,12 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
         v.next = lds_u16(ra + 2);
         return v;
     };
-    link_runs<GT, kWhole>(a, view, [&](uint32_t) { return make_int2(gain, ped); }, W, nruns, gs, gt, bar);
+    auto calib = [&](uint32_t) { return make_int2(gain, ped); };
+    link_runs<GT, kWhole>(a, view, calib, W, nruns, gs, gt, bar);
     gsync<GT, kWhole>(bar);
 
     // 7
-    sum_runs<GT>(a, nruns, gt);
+    sum_runs<GT>(a, calib, nruns, gt);
     uint32_t iv[kSingle ? kRunDigis : 1] = {}; // in-event indices for the labels
     auto index_of = [&](int k, uint32_t j) {
         if constexpr (kSingle)
@@ -1625,7 +1664,13 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
     gsync<GT, kWhole>(bar);
     // 8
     uint32_t ord;
-    const uint32_t K = mark_runs<GT, kWhole, false>(a, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
+    // (kNarrow: the label itself into word 0, whose parent is used up, so that
+    // a digi's label is one load)
+    const bool label0 = kKind == kNarrow && it.label_e;
+    auto label_run = [&](typename A::At r, uint32_t px, bool kept) {
+        if (label0) A::template st<0>(r, kept ? (px & 0xFFu) * C + ((px >> 8) & 0x1FFu) : (uint32_t)-2);
+    };
+    const uint32_t K = mark_runs<GT, kWhole, false>(a, calib, label_run, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
     const bool heavy = gs.heavy != 0;
     if (heavy) { // both moments of every root again, in 64 bits
         for (uint32_t i = gt; i < nruns; i += GT) {
@@ -1634,61 +1679,79 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
         }
         gsync<GT, kWhole>(bar);
         for (uint32_t j = 0; j < mine; ++j) {
-            const uint32_t x[4] = {__ldg(&digis[(size_t)j * GT].x), kNoDigi, kNoDigi, kNoDigi};
-            uint32_t run[4], in[4], head[4];
+            const uint32_t digi = __ldg(&digis[(size_t)j * GT].x);
+            uint32_t x[kBatch];
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) x[u] = u ? kNoDigi : digi;
+            uint32_t run[kBatch], in[kBatch], head[kBatch];
             runs_of(x, run, in, head);
             if (!in[0]) continue;
-            const size_t y = a.parent(run[0]);
-            const long long q = (long long)((int32_t)((x[0] >> 17) & 0xFFu) * gain - ped);
-            atomicAdd(&exact[2 * y], (unsigned long long)(q * (long long)(x[0] & 0xFFu)));
-            atomicAdd(&exact[2 * y + 1], (unsigned long long)(q * (long long)((x[0] >> 8) & 0x1FFu)));
+            uint32_t root;
+            if (label0) { // the run of the label's pixel
+                const uint32_t id = A::template ld<0>(a.at(run[0]));
+                if ((int32_t)id < 0) continue;
+                x[0] = id / C;
+                x[0] |= (id - x[0] * C) << 8;
+                runs_of(x, run, in, head);
+                root = run[0];
+            } else {
+                root = a.parent(run[0]);
+            }
+            const size_t y = root;
+            const long long q = (long long)((int32_t)((digi >> 17) & 0xFFu) * gain - ped);
+            atomicAdd(&exact[2 * y], (unsigned long long)(q * (long long)(digi & 0xFFu)));
+            atomicAdd(&exact[2 * y + 1], (unsigned long long)(q * (long long)((digi >> 8) & 0x1FFu)));
         }
         gsync<GT, kWhole>(bar);
     }
 
     // 9: labels (the stores drain behind the staging)
     if (it.label_e) {
-        each_four<GT, kSingle>(w, digis, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
-            uint32_t run[4], in[4], head[4], at[4], p[4];
+        each_batch<GT, kSingle>(w, digis, mine, [&](int k, uint32_t j, const uint32_t (&x)[kBatch]) {
+            uint32_t run[kBatch], in[kBatch], head[kBatch], at[kBatch], p[kBatch];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) at[u] = j + u < mine ? index_of(k + u, j + u) : 0u;
+            for (int u = 0; u < kBatch; ++u) at[u] = j + u < mine ? index_of(k + u, j + u) : 0u;
             if constexpr (kSingle) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) run[u] = x[u];
+                for (int u = 0; u < kBatch; ++u) run[u] = x[u];
             } else {
                 runs_of(x, run, in, head);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) p[u] = A::template ld<1>(a.at(run[u] == kNoSlot ? 0u : run[u]));
+            for (int u = 0; u < kBatch; ++u) {
+                const typename A::At r = a.at(run[u] == kNoSlot ? 0u : run[u]);
+                p[u] = kKind == kNarrow ? A::template ld<0>(r) : A::template ld<1>(r);
+            }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t id = (p[u] & 0xFFu) * C + ((p[u] >> 8) & 0x1FFu);
-                const int32_t lab = run[u] == kNoSlot ? -1 : p[u] & kRunDropped ? -2 : (int32_t)id;
-                if (j + u < mine) it.label_e[at[u]] = lab;
+            for (int u = 0; u < kBatch; ++u) {
+                int32_t lab = (int32_t)p[u];
+                if (kKind != kNarrow)
+                    lab = p[u] & kRunDropped ? -2 : (int32_t)((p[u] & 0xFFu) * C + ((p[u] >> 8) & 0x1FFu));
+                if (j + u < mine) it.label_e[at[u]] = run[u] == kNoSlot ? -1 : lab;
             }
         });
     }
     stage_runs<GT>(a, nruns, ord, wlist, gt, [&](uint32_t i, uint32_t o) {
-        stage_root(L, a, i, it.b + o, heavy, exact);
-        if (it.label16_e) A::set_ordinal(a.at(i), i, o); // read back by the compact labels
+        stage_root(L, a, i, it.b + o, make_int2(gain, ped), heavy, exact);
+        if (it.label16_e) A::set_ordinal(a.at(i), o); // read back by the compact labels
     });
     if (it.label16_e) { // compact labels, once every kept root has its ordinal
         gsync<GT, kWhole>(bar);
-        each_four<GT, kSingle>(w, digis, mine, [&](int k, uint32_t j, const uint32_t (&x)[4]) {
-            uint32_t run[4], in[4], head[4];
+        each_batch<GT, kSingle>(w, digis, mine, [&](int k, uint32_t j, const uint32_t (&x)[kBatch]) {
+            uint32_t run[kBatch], in[kBatch], head[kBatch];
             if constexpr (kSingle) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) run[u] = x[u];
+                for (int u = 0; u < kBatch; ++u) run[u] = x[u];
             } else {
                 runs_of(x, run, in, head);
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < kBatch; ++u) {
                 if (j + u >= mine) break;
                 uint16_t v = kLab16Below;
                 if (run[u] != kNoSlot) {
                     const typename A::At rx = a.at(a.parent(run[u]));
-                    v = A::template ld<1>(rx) & kRunKept ? (uint16_t)A::pixels(rx) : kLab16Dropped;
+                    v = A::template ld<1>(rx) & kRunKept ? (uint16_t)A::ordinal(rx) : kLab16Dropped;
                 }
                 it.label16_e[index_of(k + u, j + u)] = v;
             }
@@ -1704,21 +1767,21 @@ __device__ __noinline__ uint32_t run_clusters_big(const Launch &L, const ItemCtx
                                                   unsigned char *base, uint32_t nruns, GroupShared &gs,
                                                   uint16_t *wlist, uint32_t gt, uint32_t bar)
 {
-    Runs<true> a;
+    Runs<kGlobal> a;
     a.base = reinterpret_cast<uint32_t *>(base + (size_t)16 * nruns); // after the 64-bit moments
     uint32_t w[kRunDigis];
-    return run_clusters<GT, kWhole, true, false>(L, it, sb, rp, a, reinterpret_cast<unsigned long long *>(base), nruns,
+    return run_clusters<GT, kWhole, kGlobal, false>(L, it, sb, rp, a, reinterpret_cast<unsigned long long *>(base), nruns,
                                                  w, gs, wlist, gt, bar);
 }
 
 // One item of the run tier (phases 1-3, then run_clusters): `mem` is the
 // shared address of the group's slice with room for `cap` runs, `exact` its
 // slice of the 64-bit moments, `part` of `parts` its part of the block's slab
-// of global scratch.  kSingle: the item has at most kRunDigis * GT digis,
-// which stay in registers.  Returns the number of kept clusters (uniform
+// of global scratch.  kKind kNarrow: the item has at most kNarrowDigis digis;
+// kSingle: at most kRunDigis * GT, which stay in registers.  Returns the number of kept clusters (uniform
 // over the group).  An item with an invalid or a duplicated digi flags its
 // event and keeps none.
-template <int GT, bool kWhole, bool kSingle>
+template <int GT, bool kWhole, RunKind kKind, bool kSingle>
 __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it, uint32_t mem, uint32_t cap,
                                              unsigned long long *exact, uint32_t part, uint32_t parts,
                                              GroupShared &gs, uint16_t *wlist, uint32_t gt, uint32_t bar)
@@ -1748,9 +1811,9 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 
     // 2
     uint32_t valid = 0;
-    each_four<GT, kSingle>(w, digis, mine, [&](int, uint32_t, const uint32_t (&x)[4]) {
+    each_batch<GT, kSingle>(w, digis, mine, [&](int, uint32_t, const uint32_t (&x)[kBatch]) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) { // (words past the last digi are invalid, and OR in nothing)
+        for (int u = 0; u < kBatch; ++u) { // (words past the last digi are invalid, and OR in nothing)
             const uint32_t r = x[u] & 0xFFu, c = (x[u] >> 8) & 0x1FFu, adc = x[u] >> 17;
             const bool ok = r < R && c < C && adc - 1u < 255u; // ADC not 0, bits 25-31 clear
             const uint32_t o = ok ? 4 * (r * W + (c >> 5)) : 0u, bit = ok ? 1u << (c & 31) : 0u;
@@ -1798,9 +1861,9 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
     }
     uint32_t K;
     if (nruns <= cap) {
-        Runs<false> a;
+        Runs<kKind> a;
         a.base = ab;
-        K = run_clusters<GT, kWhole, false, kSingle>(L, it, sb, rp, a, exact, nruns, w, gs, wlist, gt, bar);
+        K = run_clusters<GT, kWhole, kKind, kSingle>(L, it, sb, rp, a, exact, nruns, w, gs, wlist, gt, bar);
     } else {
         uint64_t first, room;
         if (L.ws.big_arena) { // a slot a run, bump-allocated
@@ -1872,7 +1935,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
                                            uint32_t items, uint32_t total, GroupShared &gs, uint16_t *wlist,
                                            uint32_t gt, uint32_t bar)
 {
-    using A = Runs<false>;
+    using A = Runs<kNarrow>;
     static_assert(kPackDigis < 4 * GT, "four digis a thread at most");
     const uint32_t R = L.g.R, C = L.g.C, W = (C + 31) >> 5, RH = (R + 1) >> 1, pcap = L.cc.pack_digis;
     const int32_t thr = L.g.pixel_thr;
@@ -2025,10 +2088,10 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     };
     link_runs<GT, kWhole>(a, view, calib, W, nruns, gs, gt, bar);
     gsync<GT, kWhole>(bar);
-    sum_runs<GT>(a, nruns, gt);
+    sum_runs<GT>(a, calib, nruns, gt);
     gsync<GT, kWhole>(bar);
     uint32_t ord;
-    mark_runs<GT, kWhole, true>(a, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
+    mark_runs<GT, kWhole, true>(a, calib, [](A::At, uint32_t, bool) {}, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
     const bool heavy = gs.heavy != 0;
     if (heavy) { // both moments again, in 64 bits
         for (uint32_t i = gt; i < 2 * nruns; i += GT) exact[i] = 0;
@@ -2056,7 +2119,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     first -= kept;
     if (gt < (uint32_t)kGroup && gs.pack[gt + 1] > gs.pack[gt]) {
         L.ws.cursor[gs.ticket * L.cc.ticket_items + i0 + gt] = kept;
-        gs.rec[i0 + gt].gain = (int32_t)first; // (a packed item's calibration is not needed any more)
+        gs.rec[i0 + gt].e = first; // (a packed item's event is not needed any more)
     }
     if (L.out.label) {
 #pragma unroll
@@ -2072,9 +2135,11 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     }
     gsync<GT, kWhole>(bar);
     stage_runs<GT>(a, nruns, ord, wlist, gt, [&](uint32_t i, uint32_t o) {
-        const uint32_t item = (A::ld<1>(a.at(i)) & kRunItem) >> 23, k = o - (uint32_t)gs.rec[i0 + item].gain;
-        stage_root(L, a, i, gs.b[i0 + item] + k, heavy, exact);
-        if (L.out.label16) A::set_ordinal(a.at(i), i, k); // read back by the compact labels
+        const uint32_t item = (A::ld<1>(a.at(i)) & kRunItem) >> 23;
+        const ItemRec &rec = gs.rec[i0 + item];
+        const uint32_t k = o - rec.e;
+        stage_root(L, a, i, gs.b[i0 + item] + k, make_int2(rec.gain, rec.ped), heavy, exact);
+        if (L.out.label16) A::set_ordinal(a.at(i), k); // read back by the compact labels
     });
     if (L.out.label16) {
         gsync<GT, kWhole>(bar);
@@ -2084,7 +2149,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
             uint16_t v = kLab16Below;
             if (w[k] != kNoSlot) {
                 const A::At rx = a.at(a.parent(w[k]));
-                v = A::ld<1>(rx) & kRunKept ? (uint16_t)A::pixels(rx) : kLab16Dropped;
+                v = A::ld<1>(rx) & kRunKept ? (uint16_t)A::ordinal(rx) : kLab16Dropped;
             }
             L.out.label16[gs.rec[i0 + li[k]].label_off + idx[k]] = v;
         }
@@ -2654,7 +2719,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
                 if (gs.ticket >= nlarge) break;
                 const ItemCtx it = make_item(L, gs.rec[0], gs.b[0], gs.n[0]);
                 const uint32_t item = gs.pack_end;
-                const uint32_t K = run_item<kThreads, true, false>(L, it, smem_addr(dsm), L.cc.whole_runs, exact, 0, 1,
+                const uint32_t K = run_item<kThreads, true, kWide, false>(L, it, smem_addr(dsm), L.cc.whole_runs, exact, 0, 1,
                                                                      gs, wlist, tid, 0);
                 if (tid == 0) kcount[item] = K;
                 __syncthreads();
@@ -2675,10 +2740,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
             const uint32_t n = gs.n[i];
             if (n <= L.cc.pack_item || (!kWhole && n > L.cc.large_digis)) continue;
             const ItemCtx it = make_item(L, gs.rec[i], gs.b[i], n);
+            constexpr RunKind kMulti = kWhole ? kWide : kNarrow; // (of groups: at most cc.large_digis digis)
+            static_assert(kRunDigis * GT <= kNarrowDigis, "items held in registers");
             const uint32_t K = n <= (uint32_t)(kRunDigis * GT)
-                                   ? run_item<GT, kWhole, true>(L, it, mem, L.cc.runs, exact, gid, kGroups,
+                                   ? run_item<GT, kWhole, kNarrow, true>(L, it, mem, L.cc.runs, exact, gid, kGroups,
                                                                 gs, wlist, gt, bar)
-                                   : run_item<GT, kWhole, false>(L, it, mem, L.cc.runs, exact, gid, kGroups,
+                                   : run_item<GT, kWhole, kMulti, false>(L, it, mem, L.cc.runs, exact, gid, kGroups,
                                                                  gs, wlist, gt, bar);
             if (gt == 0) kcount[gs.ticket * L.cc.ticket_items + i] = K;
         }
@@ -2737,7 +2804,7 @@ __global__ void __launch_bounds__(kCCThreads, kMinBlocks) cc_hash_kernel(const _
             const uint32_t n = gs.n[i];
             if (n <= L.cc.pack_item || n <= hash_max) continue;
             const ItemCtx it = make_item(L, gs.rec[i], gs.b[i], n);
-            const uint32_t K = run_item<GT0, true, false>(L, it, smem_addr(dsm), L.cc.runs, exact, 0, 1, gs,
+            const uint32_t K = run_item<GT0, true, kWide, false>(L, it, smem_addr(dsm), L.cc.runs, exact, 0, 1, gs,
                                                           wlist, tid, 0);
             if (tid == 0) kcount[item0 + i] = K;
         }
@@ -3211,7 +3278,7 @@ static ClusterPlan cluster_plan(const Launch &L)
     if (hash) p.runs = std::min(run_capacity(p.slice - kHashListBytes, R, C), T);
     p.pack_digis = pack_capacity(hash ? p.slice - kHashListBytes : p.slice, R, p.runs);
     p.pack_item = std::min(hash ? L.tune.warp_max : pack_max(L.tune.warp_max), p.pack_digis);
-    p.large_digis = large_digis(R, C, L.tune);
+    p.large_digis = std::min(large_digis(R, C, L.tune), groups > 1 ? kNarrowDigis : 0xFFFFFFFFu);
     // with no more items than blocks a group's neighbours are idle: items past
     // what a group holds in registers take the whole block (64 items of 3,125
     // digis: 61 -> 45 us; of 1,562, which it does hold: 41 us either way)
