@@ -188,7 +188,7 @@ struct Workspace {
 // Sizes of the clustering kernel of one launch, worked out on the host.
 struct ClusterPlan {
     uint32_t items, ticket_items, tickets; // (event, module) items, items a ticket, tickets
-    uint32_t workers;                      // groups of all blocks
+    uint32_t threads, workers;             // threads of a block; groups of all blocks
     uint32_t smem, slice;                  // dynamic shared memory of a block, and of each of its groups
     uint32_t runs, whole_runs;             // run records in a group's slice, and in the whole block's
     uint32_t exact_slots;                  // 64-bit moment slots of a block
@@ -260,12 +260,16 @@ __host__ __device__ inline uint32_t run_capacity(size_t bytes, uint32_t R, uint3
     return bytes > fixed ? (uint32_t)((bytes - fixed) / kRunBytes) : 0u;
 }
 // Dynamic shared memory of a block of `groups` groups whose whole holds
-// tile_slots runs: at least slices of 256 runs, and of the bitmaps.
+// tile_slots runs: at least slices of kSliceRuns runs where those leave two
+// blocks an SM, of 256 where not, and of the bitmaps.
+constexpr size_t kSliceRuns = 1200, kSliceBytes = 112000;
 __host__ __device__ inline size_t run_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots, uint32_t groups)
 {
     const size_t fixed = run_fixed_bytes(R, C), bits = (size_t)run_words(R, C) * 4;
     auto at_least = [&](size_t runs) { return fixed + (kRunBytes * runs > bits ? kRunBytes * runs : bits); };
-    const size_t whole = at_least(tile_slots), parts = groups * ((at_least(256) + 15) & ~(size_t)15);
+    const size_t whole = at_least(tile_slots);
+    size_t parts = groups * ((at_least(kSliceRuns) + 15) & ~(size_t)15);
+    if (parts > kSliceBytes) parts = groups * ((at_least(256) + 15) & ~(size_t)15);
     return whole > parts ? whole : parts;
 }
 // 64-bit moment slots of a block (its groups' slices hold no more runs together).
@@ -285,22 +289,42 @@ __host__ __device__ inline uint32_t pack_capacity(size_t bytes, uint32_t R, uint
 }
 __host__ __device__ inline uint32_t pack_max(uint32_t warp_max) { return 12 * warp_max; }
 
-// Threads and groups of a clustering block for 1, 2 and 3 resident blocks per SM.
+// Threads and groups of a clustering block for 1, 2 and 3 resident blocks per
+// SM.  Two blocks an SM come as two groups of 256 threads each or as three of
+// 160 (2n): an item is a chain of phases, and six groups an SM hide more of it
+// than four, but a pack then holds 640 digis instead of 1,023 and a lone item
+// has fewer threads.  Clustering kernel, 256 against 160 threads a group, in
+// us: 16,384 items of 20 digis 39 / 31, of 80 73 / 55, of 150 88 / 91, of 300
+// 164 / 161, of 500 238 / 258, of 781 347 / 270, of 1,000 357 / 317; 5,568
+// items of 796 133 / 115; one event's 400 items of 796 20 / 24, its 64 of 469
+// 14 / 20.
 constexpr int kRunThreads1 = 1024, kRunGroups1 = 4;
 constexpr int kRunThreads2 = 512, kRunGroups2 = 2;
+constexpr int kRunThreads2n = 480, kRunGroups2n = 3;
 constexpr int kRunThreads3 = 256, kRunGroups3 = 1;
-__host__ __device__ inline uint32_t run_groups(uint32_t blocks_per_sm)
+struct RunShape {
+    uint32_t threads, groups;
+};
+inline RunShape run_shape(const Tuning &t, uint64_t items, uint64_t N, int cc_grid)
 {
-    return blocks_per_sm >= 3 ? kRunGroups3 : blocks_per_sm == 2 ? kRunGroups2 : kRunGroups1;
+    if (t.label_store == kStoreHash) return {(uint32_t)kCCThreads, 1u};
+    if (t.blocks_per_sm >= 3) return {(uint32_t)kRunThreads3, (uint32_t)kRunGroups3};
+    if (t.blocks_per_sm == 1) return {(uint32_t)kRunThreads1, (uint32_t)kRunGroups1};
+    // three groups: more than one round of tickets, and items that leave most
+    // of a pack, or of a group's registers, empty at 256 threads
+    const unsigned workers = (unsigned)(cc_grid > 0 ? cc_grid : 1) * kRunGroups2;
+    const bool rounds = items > (uint64_t)workers * ticket_items(items, workers, t.ticket_max, N);
+    const bool size = N < 128 * items || N >= 640 * items;
+    if (rounds && size) return {(uint32_t)kRunThreads2n, (uint32_t)kRunGroups2n};
+    return {(uint32_t)kRunThreads2, (uint32_t)kRunGroups2};
 }
 // Digis above which an item is a whole block's: one and a half times the
 // runs of a group's slice (0.6 runs a digi are usual; an item with more runs
 // than the slice holds is finished in global scratch).
-inline uint32_t large_digis(uint32_t R, uint32_t C, const Tuning &t)
+inline uint32_t large_digis(uint32_t R, uint32_t C, uint32_t tile_slots, RunShape sh)
 {
-    const uint32_t groups = run_groups(t.blocks_per_sm);
-    if (t.label_store == kStoreHash || groups == 1) return 0xFFFFFFFFu;
-    return run_capacity((run_smem_bytes(R, C, t.tile_slots, groups) / groups) & ~(size_t)15, R, C) / 2 * 3;
+    if (sh.groups == 1) return 0xFFFFFFFFu;
+    return run_capacity((run_smem_bytes(R, C, tile_slots, sh.groups) / sh.groups) & ~(size_t)15, R, C) / 2 * 3;
 }
 // Lay out the workspace for (E, M, N) in `base` (nullptr: only compute size).
 size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t R, uint32_t C, int cc_grid,

@@ -1889,7 +1889,8 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 
 // ---- packed tier
 //
-// The small items of a ticket together: up to 1,023 digis of up to 16 items
+// The small items of a ticket together: up to four digis a thread (at most
+// 1,023) of up to 16 items
 // by a group of GT threads, through the run tier's phases on a sparse bitmap.
 // Of each item's bitmap words only the touched ones are stored, in (item,
 // row, word) order: a bit per word of the module says which are (16 bits a
@@ -1907,7 +1908,7 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 //   f charge and position into the runs, then 5 to 9 of the run tier
 // What bounds it: the latency of the phases, which all items of a ticket
 // share; the work is the digis', not the modules'.
-constexpr uint32_t kPackDigis = 1023;
+constexpr int kPackPer = 4; // digis a thread holds
 
 // One warp (lane = its lane): the pack that starts at item i0 of the ticket,
 // as many of the next items of at most pmax digis as pcap holds (larger ones
@@ -1936,7 +1937,6 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
                                            uint32_t gt, uint32_t bar)
 {
     using A = Runs<kNarrow>;
-    static_assert(kPackDigis < 4 * GT, "four digis a thread at most");
     const uint32_t R = L.g.R, C = L.g.C, W = (C + 31) >> 5, RH = (R + 1) >> 1, pcap = L.cc.pack_digis;
     const int32_t thr = L.g.pixel_thr;
     // fields: RH words of two rows an item; and the touched words before each
@@ -1947,9 +1947,9 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     a.base = (rpre + 2 * (pcap + 2) + 3) & ~3u;
 
     // a
-    uint32_t w[4], idx[4], li[4], at[4];
+    uint32_t w[kPackPer], idx[kPackPer], li[kPackPer], at[kPackPer];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kPackPer; ++k) {
         const uint32_t t = gt + k * GT;
         w[k] = kNoDigi;
         idx[k] = li[k] = at[k] = 0;
@@ -1978,7 +1978,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
 
     // b
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kPackPer; ++k) {
         if (gt + k * GT >= total) break;
         const uint32_t r = w[k] & 0xFFu, c = (w[k] >> 8) & 0x1FFu, adc = w[k] >> 17;
         if (r >= R || c >= C || adc - 1u >= 255u) { // ADC 0, or any of the bits 25-31
@@ -2016,7 +2016,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     // d
     uint32_t dropped = 0; // bit k: digi k is below threshold
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kPackPer; ++k) {
         if (gt + k * GT >= total) break;
         if (w[k] == kNoDigi) continue;
         const ItemRec &rec = gs.rec[i0 + li[k]];
@@ -2051,7 +2051,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
 
     // f
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < kPackPer; ++k) {
         if (gt + k * GT >= total) break;
         const uint32_t x = w[k];
         w[k] = kNoSlot;
@@ -2097,7 +2097,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
         for (uint32_t i = gt; i < 2 * nruns; i += GT) exact[i] = 0;
         gsync<GT, kWhole>(bar);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < kPackPer; ++k) {
             if (gt + k * GT >= total || w[k] == kNoSlot) continue;
             const ItemRec &rec = gs.rec[i0 + li[k]];
             const uint32_t x = __ldg(&L.ws.bucket[gs.b[i0 + li[k]] + (gt + k * GT - gs.pack[li[k]])].x);
@@ -2123,7 +2123,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     }
     if (L.out.label) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < kPackPer; ++k) {
             if (gt + k * GT >= total) break;
             int32_t lab = -1;
             if (w[k] != kNoSlot) {
@@ -2144,7 +2144,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     if (L.out.label16) {
         gsync<GT, kWhole>(bar);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < kPackPer; ++k) {
             if (gt + k * GT >= total) break;
             uint16_t v = kLab16Below;
             if (w[k] != kNoSlot) {
@@ -3162,17 +3162,15 @@ size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t 
     w.staging.y = reinterpret_cast<float *>(take(4ull * N));
     w.large = reinterpret_cast<uint32_t *>(take(4ull * EM));
     const bool hash = tune.label_store == kStoreHash;
-    const uint32_t groups = hash ? 1u : run_groups(tune.blocks_per_sm);
+    const RunShape sh = run_shape(tune, EM, N, cc_grid);
     w.exact = reinterpret_cast<unsigned long long *>(
-        take(16ull * (hash ? tune.tile_slots : run_exact_slots(R, C, tune.tile_slots, groups)) *
+        take(16ull * (hash ? tune.tile_slots : run_exact_slots(R, C, tune.tile_slots, sh.groups)) *
              (cc_grid > 0 ? cc_grid : 1)));
     // a slab holds any item, and an item of each group at once (a group's
     // part holds the largest item it takes: see large_digis)
+    const uint64_t any = std::min<uint64_t>((uint64_t)R * C, N);
     const uint64_t slab_slots =
-        std::max<uint64_t>(std::min<uint64_t>((uint64_t)R * C, N),
-                 groups > 1 ? groups * std::min<uint64_t>(std::min<uint64_t>((uint64_t)R * C, N),
-                                                          large_digis(R, C, tune))
-                            : 0ull);
+        sh.groups > 1 ? std::max(any, sh.groups * std::min<uint64_t>(any, large_digis(R, C, tune.tile_slots, sh))) : any;
     const uint64_t slab_total = slab_slots * (uint64_t)(cc_grid > 0 ? cc_grid : 1);
     w.big_arena = N <= slab_total ? 1 : 0;
     w.big_slots = w.big_arena ? N : slab_slots;
@@ -3240,6 +3238,11 @@ cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4
     if (err == cudaSuccess)
         err = fit_tile(cc_kernel<kRunThreads2, kRunGroups2, 2>, device, 2, kRunThreads2, run_bytes(kRunGroups2),
                        kSmemSlots, &max_tile[2]);
+    uint32_t narrow = 0; // (the two-block kernel with more groups: the same tiles)
+    if (err == cudaSuccess)
+        err = fit_tile(cc_kernel<kRunThreads2n, kRunGroups2n, 2>, device, 2, kRunThreads2n, run_bytes(kRunGroups2n),
+                       kSmemSlots, &narrow);
+    max_tile[2] = std::min(max_tile[2], narrow);
     if (err == cudaSuccess)
         err = fit_tile(cc_kernel<kRunThreads3, kRunGroups3, 3>, device, 3, kRunThreads3, run_bytes(kRunGroups3),
                        kSmemSlots, &max_tile[3]);
@@ -3264,11 +3267,19 @@ static ClusterPlan cluster_plan(const Launch &L)
 {
     const uint32_t R = L.g.R, C = L.g.C, T = L.tune.tile_slots;
     const bool hash = L.tune.label_store == kStoreHash;
-    const uint32_t groups = hash ? 1u : run_groups(L.tune.blocks_per_sm);
     ClusterPlan p;
     p.items = (uint32_t)((uint64_t)L.E * L.g.M); // at most 2^31 (checked by the callers)
-    p.ticket_items = ticket_items(p.items, (unsigned)L.cc_grid * groups, L.tune.ticket_max, L.N);
+    const RunShape sh = run_shape(L.tune, p.items, L.N, L.cc_grid);
+    const uint32_t groups = sh.groups;
+    p.threads = sh.threads;
     p.workers = (uint32_t)L.cc_grid * groups;
+    p.ticket_items = ticket_items(p.items, p.workers, L.tune.ticket_max, L.N);
+    // small items: no more a ticket than fill the last round of tickets
+    if (!large_items(L.N, p.items)) {
+        const uint64_t per = (uint64_t)p.workers * p.ticket_items, rounds = (p.items + per - 1) / per;
+        const uint64_t fill = (p.items + p.workers * rounds - 1) / (p.workers * rounds);
+        p.ticket_items = (uint32_t)std::min<uint64_t>(p.ticket_items, std::max<uint64_t>(4, fill));
+    }
     p.tickets = (p.items + p.ticket_items - 1) / p.ticket_items;
     p.smem = (uint32_t)(hash ? cc_smem_bytes(R, C, T) : run_smem_bytes(R, C, T, groups));
     p.slice = (p.smem / groups) & ~15u;
@@ -3276,14 +3287,15 @@ static ClusterPlan cluster_plan(const Launch &L)
     p.runs = run_capacity(p.slice, R, C);
     p.exact_slots = hash ? T : run_exact_slots(R, C, T, groups);
     if (hash) p.runs = std::min(run_capacity(p.slice - kHashListBytes, R, C), T);
-    p.pack_digis = pack_capacity(hash ? p.slice - kHashListBytes : p.slice, R, p.runs);
+    p.pack_digis = std::min(pack_capacity(hash ? p.slice - kHashListBytes : p.slice, R, p.runs),
+                            (uint32_t)kPackPer * sh.threads / groups);
     p.pack_item = std::min(hash ? L.tune.warp_max : pack_max(L.tune.warp_max), p.pack_digis);
-    p.large_digis = std::min(large_digis(R, C, L.tune), groups > 1 ? kNarrowDigis : 0xFFFFFFFFu);
+    p.large_digis = std::min(large_digis(R, C, T, sh), groups > 1 ? kNarrowDigis : 0xFFFFFFFFu);
     // with no more items than blocks a group's neighbours are idle: items past
     // what a group holds in registers take the whole block (64 items of 3,125
     // digis: 61 -> 45 us; of 1,562, which it does hold: 41 us either way)
     if (groups > 1 && p.items <= (uint32_t)L.cc_grid)
-        p.large_digis = std::min<uint32_t>(p.large_digis, kRunDigis * (kRunThreads1 / kRunGroups1));
+        p.large_digis = std::min(p.large_digis, (uint32_t)kRunDigis * sh.threads / groups);
     return p;
 }
 
@@ -3313,7 +3325,8 @@ cudaError_t launch_dependent(K kern, unsigned grid, unsigned block, size_t smem,
 // 43); past kSmallDigis the boundaries no longer count.
 static bool bucket_fits(const Launch &L)
 {
-    return L.N > 0 && L.N <= kSmallDigis && L.g.M <= kBucketModules && L.N / L.E <= kBucketDigis;
+    return L.N > 0 && L.N <= kSmallDigis && L.g.M <= kBucketModules && L.N / L.E <= kBucketDigis &&
+           (uint64_t)L.E * kBucketCluster <= (uint64_t)L.sm_count;
 }
 static bool finish_fits(const Launch &L)
 {
@@ -3392,6 +3405,9 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
                                    L.cc_grid, kCCThreads, L.cc.smem, stream, L);
         else if (b >= 3)
             err = launch_dependent(cc_kernel<kRunThreads3, kRunGroups3, 3>, L.cc_grid, kRunThreads3,
+                                   L.cc.smem, stream, L);
+        else if (b == 2 && L.cc.threads == (uint32_t)kRunThreads2n)
+            err = launch_dependent(cc_kernel<kRunThreads2n, kRunGroups2n, 2>, L.cc_grid, kRunThreads2n,
                                    L.cc.smem, stream, L);
         else if (b == 2)
             err = launch_dependent(cc_kernel<kRunThreads2, kRunGroups2, 2>, L.cc_grid, kRunThreads2,
