@@ -804,7 +804,7 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
 {
     extern __shared__ __align__(16) uint32_t sh[];
     __shared__ uint32_t tmp[2][kBucketThreads / 32 + 1];
-    __shared__ uint32_t s_bad;
+    __shared__ uint32_t s_bad, s_none[32];
     pdl_trigger();
     const uint32_t tid = threadIdx.x, M = L.g.M, MK = bucket_keys(M), rank = cluster_rank();
     const uint32_t e = blockIdx.x / kBucketCluster;
@@ -832,6 +832,9 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
     const uint64_t a0 = (g0 + ng * rank / kBucketCluster) * kPerThread;
     const uint64_t c0 = max(o0, a0), c1 = min(o1, (g0 + ng * (rank + 1) / kBucketCluster) * kPerThread);
     const bool one_step = c1 <= a0 + kBucketStep;
+    // whether the second group of a thread's digis holds any: an event of at
+    // most half a step a block does without it (30,000 digis: 30.9 -> 25.4 us)
+    const bool both = c1 > a0 + kBucketStep / 2;
     // a thread's digis of the step at s0: group h at s0 + (h * threads + tid) * kPerThread;
     // km: module, and (from the count of its step on) rank << 16; 0xFFFF: none
     uint32_t km[kBucketPer], w[kBucketPer];
@@ -840,9 +843,11 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint64_t k0 = first(s0, h);
-            uint32_t m8[kPerThread], w8[kPerThread];
-            load_modules(L, k0, c1, m8);
-            if (words) load_words(L, k0, c1, w8);
+            uint32_t m8[kPerThread] = {}, w8[kPerThread] = {};
+            if (h == 0 || both) {
+                load_modules(L, k0, c1, m8);
+                if (words) load_words(L, k0, c1, w8);
+            }
 #pragma unroll
             for (int j = 0; j < kPerThread; ++j) {
                 const bool in = k0 + j >= c0 && k0 + j < c1;
@@ -852,14 +857,25 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
         }
     };
     bool bad = false;
-    auto count_step = [&](uint32_t *counts) {
+    auto count_step = [&](uint32_t *counts) { // (no branches: the latencies overlap; 60,000 digis: 32.9 -> 30.9 us)
 #pragma unroll
-        for (int j = 0; j < kBucketPer; ++j) {
-            if (km[j] < M)
-                km[j] |= atomicAdd(&counts[km[j]], 1u) << 16;
-            else {
-                bad |= km[j] != 0xFFFFFFFFu;
-                km[j] = 0xFFFFu;
+        for (int h = 0; h < 2; ++h) {
+            if (h && !both) {
+#pragma unroll
+                for (int j = 0; j < kPerThread; ++j) km[kPerThread + j] = 0xFFFFu;
+                continue;
+            }
+            uint32_t r[kPerThread];
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) {
+                const uint32_t k = km[h * kPerThread + j];
+                r[j] = atomicAdd(k < M ? counts + k : s_none + (tid & 31), 1u);
+            }
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) {
+                uint32_t &k = km[h * kPerThread + j];
+                bad |= k >= M && k != 0xFFFFFFFFu;
+                k = k < M ? k | (r[j] << 16) : 0xFFFFu;
             }
         }
     };
@@ -2591,48 +2607,71 @@ __device__ bool chain_resolve(unsigned long long *chain, uint32_t *frontier, uin
 
 // ---------------------------------------------------------------- clustering kernels
 
-// The next ticket of a group (the first is its own, `first`, dealt over the
-// blocks before the groups of one, the others come from a counter): its items' counts, bucket starts and records,
-// and the plan of its first pack (returned); false when the tickets are out.
-template <int GT, bool kWhole>
-__device__ __forceinline__ bool take_ticket(const Launch &L, GroupShared &gs, uint32_t gt, uint32_t bar,
-                                            uint32_t first)
+// What lane gt of a group's first warp loads of ticket g: its item's record
+// (calibration and event start: inputs, so these can be read before the
+// previous kernel is done) and then its count and bucket start.  Lanes past
+// the ticket read its first item and drop it.
+struct TicketLane {
+    ItemRec rec;
+    uint32_t count, b;
+};
+__device__ __forceinline__ uint32_t ticket_item(const Launch &L, uint32_t g, uint32_t lane, bool *ok)
 {
-    const uint32_t G = L.cc.ticket_items, EM = L.cc.items;
+    const uint32_t item = g * L.cc.ticket_items + lane;
+    *ok = lane < L.cc.ticket_items && item < L.cc.items;
+    return *ok ? item : g * L.cc.ticket_items;
+}
+__device__ __forceinline__ void load_record(const Launch &L, uint32_t g, uint32_t lane, TicketLane *t)
+{
+    bool ok;
+    const uint32_t at = ticket_item(L, g, lane, &ok), e = L.E == 1 ? 0u : at / L.g.M, m = at - e * L.g.M;
+    t->rec.e = e;
+    t->rec.gain = L.g.gain[m];
+    t->rec.ped = L.g.ped[m];
+    t->rec.label_off = (uint32_t)L.offsets[e];
+}
+__device__ __forceinline__ void load_counts(const Launch &L, uint32_t g, uint32_t lane, TicketLane *t)
+{
+    bool ok;
+    const uint32_t at = ticket_item(L, g, lane, &ok);
+    t->count = L.ws.count[at];
+    t->b = L.ws.boff[at];
+}
+
+// Ticket g of a group: its items' counts, bucket starts and records, and the
+// plan of its first pack; false when the tickets are out.  first: t is
+// loaded, and g is the group's own first ticket (dealt over the blocks before
+// the groups of one); else the next one comes from a counter.
+template <int GT, bool kWhole>
+__device__ __forceinline__ bool take_ticket(const Launch &L, GroupShared &gs, uint32_t gt, uint32_t bar, bool first,
+                                            uint32_t g, TicketLane &t)
+{
+    const uint32_t G = L.cc.ticket_items;
     if (gt < 32) { // one warp takes the ticket and loads its items
-        uint32_t g32 = 0;
-        if (first != kNoSlot) {
-            g32 = first;
-        } else {
-            if (gt == 0) g32 = L.cc.workers + atomicAdd(&L.ws.ctl[0], 1u);
-            g32 = __shfl_sync(kFull, g32, 0);
+        if (!first) {
+            if (gt == 0) g = L.cc.workers + atomicAdd(&L.ws.ctl[0], 1u);
+            g = __shfl_sync(kFull, g, 0);
+            if (g < L.cc.tickets) { // (every load before the first store, so that their latencies overlap)
+                load_record(L, g, gt, &t);
+                load_counts(L, g, gt, &t);
+            }
         }
-        if (g32 < L.cc.tickets) {
-            const uint32_t item = g32 * G + gt;
-            const bool ok = gt < G && item < EM;
-            // (every load before the first store, so that their latencies overlap)
-            const uint32_t at = ok ? item : g32 * G;
-            const uint32_t e = L.E == 1 ? 0u : at / L.g.M, m = at - e * L.g.M;
-            const uint32_t count = L.ws.count[at], b = L.ws.boff[at];
-            ItemRec rec;
-            rec.e = e;
-            rec.gain = L.g.gain[m];
-            rec.ped = L.g.ped[m];
-            rec.label_off = (uint32_t)L.offsets[e];
-            const uint32_t n = ok ? count : 0u;
+        if (g < L.cc.tickets) {
+            bool ok;
+            const uint32_t item = ticket_item(L, g, gt, &ok), n = ok ? t.count : 0u;
             if (gt < (uint32_t)kGroup) {
                 gs.n[gt] = n;
-                gs.b[gt] = b;
-                gs.rec[gt] = rec;
+                gs.b[gt] = t.b;
+                gs.rec[gt] = t.rec;
                 if (ok) {
                     if (n == 0) L.ws.cursor[item] = 0;
-                    if (gt == G - 1 || item == EM - 1) gs.bucket_end = b + n;
+                    if (gt == G - 1 || item == L.cc.items - 1) gs.bucket_end = t.b + n;
                 }
             }
             const uint32_t end = min(plan_pack(gs, 0, L.cc.pack_item, L.cc.pack_digis, gt, n), G);
             if (gt == 0) gs.pack_end = end;
         }
-        if (gt == 0) gs.ticket = g32;
+        if (gt == 0) gs.ticket = g;
     }
     gsync<GT, kWhole>(bar);
     return gs.ticket < L.cc.tickets;
@@ -2690,12 +2729,19 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ GroupShared s_gs[kGroups];
     __shared__ uint16_t s_wlist[kThreads / 32][64];
+    const uint32_t tid = threadIdx.x, gid = tid / GT, gt = tid - gid * GT, bar = 1 + gid;
+    // the group's first ticket: its records before the previous kernel is done
+    // (the launch's first kernel is an ordinary launch, so that the call's
+    // inputs are in place when this one starts; 760 -> 751 us for 256 events)
+    const uint32_t ticket0 = gid * gridDim.x + blockIdx.x;
+    TicketLane lane_of;
+    if (gt < 32 && ticket0 < L.cc.tickets) load_record(L, ticket0, gt, &lane_of);
     pdl_wait();
     pdl_trigger();
     const uint32_t launch_err = L.ws.ctl[1], nlarge = kWhole ? 0u : L.ws.ctl[5];
+    if (gt < 32 && ticket0 < L.cc.tickets) load_counts(L, ticket0, gt, &lane_of);
     if (launch_err & kErrBadOffsets) return;
 
-    const uint32_t tid = threadIdx.x;
     uint16_t *wlist = s_wlist[tid >> 5];
     unsigned long long *exact = L.ws.exact + (size_t)blockIdx.x * 2 * L.cc.exact_slots;
     uint32_t *kcount = L.ws.cursor; // each item's count of kept clusters
@@ -2728,12 +2774,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
         __syncthreads();
     }
 
-    const uint32_t gid = tid / GT, gt = tid - gid * GT, bar = 1 + gid;
     const uint32_t mem = smem_addr(dsm) + L.cc.slice * gid;
     exact += (size_t)2 * L.cc.runs * gid;
     GroupShared &gs = s_gs[gid];
-    for (uint32_t first = gid * gridDim.x + blockIdx.x; take_ticket<GT, kWhole>(L, gs, gt, bar, first);
-         first = kNoSlot) {
+    for (bool first = true; take_ticket<GT, kWhole>(L, gs, gt, bar, first, ticket0, lane_of); first = false) {
         prefetch_ticket<GT>(L, gs, gt);
         pack_ticket<GT, kWhole>(L, mem, exact, gs, wlist, gt, bar);
         for (uint32_t i = 0; i < L.cc.ticket_items; ++i) {
@@ -2784,7 +2828,12 @@ __global__ void __launch_bounds__(kCCThreads, kMinBlocks) cc_hash_kernel(const _
         s_gheavy[tid] = 0;
     }
     uint32_t *kcount = L.ws.cursor;
-    for (uint32_t first = blockIdx.x; take_ticket<GT0, true>(L, gs, tid, 0, first); first = kNoSlot) {
+    TicketLane lane_of;
+    if (tid < 32 && blockIdx.x < L.cc.tickets) {
+        load_record(L, blockIdx.x, tid, &lane_of);
+        load_counts(L, blockIdx.x, tid, &lane_of);
+    }
+    for (bool first = true; take_ticket<GT0, true>(L, gs, tid, 0, first, blockIdx.x, lane_of); first = false) {
         prefetch_ticket<GT0>(L, gs, tid);
         pack_ticket<GT0, true>(L, smem_addr(dsm), exact, gs, wlist, tid, 0);
         const uint32_t item0 = gs.ticket * L.cc.ticket_items;
@@ -3024,7 +3073,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_con
     pdl_wait();
     const uint32_t tid = threadIdx.x, M = L.g.M, EM = L.cc.items;
     const uint64_t gt = (uint64_t)blockIdx.x * kFinishThreads + tid;
-    const uint32_t launch_bits = L.ws.ctl[1];
+    const uint32_t launch_bits = L.ws.ctl[1], err0 = gt < L.E ? L.ws.event_err[gt] : 0u;
     if (launch_bits & kErrBadOffsets) {
         for (uint64_t e = gt; e <= L.E; e += (uint64_t)gridDim.x * kFinishThreads) {
             L.out.cluster_offsets[e] = 0; // no clusters
@@ -3049,7 +3098,7 @@ __global__ void __launch_bounds__(kFinishThreads) finish_kernel(const __grid_con
     const uint32_t bits = launch_bits | (total > L.out.capacity ? kErrCapacity : 0u);
     for (uint64_t e = gt; e <= L.E; e += (uint64_t)gridDim.x * kFinishThreads) {
         L.out.cluster_offsets[e] = offs[e * M];
-        if (e < L.E) L.out.event_status[e] = event_status(L.ws.event_err[e] | bits);
+        if (e < L.E) L.out.event_status[e] = event_status((e == gt ? err0 : L.ws.event_err[e]) | bits);
     }
     const uint32_t T = (uint32_t)min((unsigned long long)total, (unsigned long long)L.out.capacity);
     const Staging sg = L.ws.staging;
@@ -3320,7 +3369,7 @@ cudaError_t launch_dependent(K kern, unsigned grid, unsigned block, size_t smem,
 // cluster an event) and its clusters ordered by finish_kernel, instead of by
 // three kernels and two: small launches, whose time is that of the kernel
 // boundaries (one event of 1,300 digis 36 -> 23 us, of 60,000 on 1,856 modules
-// 49 -> 33 us).  Events past a step a block are counted twice, by eight blocks
+// 49 -> 31 us).  Events past a step a block are counted twice, by eight blocks
 // only, and the three kernels' grid is faster (200,000 digis: 51 us against
 // 43); past kSmallDigis the boundaries no longer count.
 static bool bucket_fits(const Launch &L)
