@@ -353,19 +353,31 @@ __device__ __forceinline__ ChunkInfo chunk_info(const Launch &L, uint64_t c0, ui
 constexpr uint32_t kHistWarps = kHistThreads / 32;
 constexpr uint32_t kSubKeys = kHistCap / kHistWarps; // keys per warp sub-histogram
 
+// The thread's group of module ids at k0, packed (absent ones 0).
+__device__ __forceinline__ uint4 load_packed(const Launch &L, uint64_t k0, uint64_t c1)
+{
+    if (((reinterpret_cast<uintptr_t>(L.modules) & 15) == 0) && k0 + kPerThread <= c1)
+        return *reinterpret_cast<const uint4 *>(L.modules + k0);
+    uint32_t m[kPerThread];
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j) m[j] = k0 + j < c1 ? (uint32_t)L.modules[k0 + j] : 0u;
+    return make_uint4(m[0] | m[1] << 16, m[2] | m[3] << 16, m[4] | m[5] << 16, m[6] | m[7] << 16);
+}
+
 // Histogram, persistent: block b counts the digis of its contiguous range
 // (one event search a block), 8 module ids a thread per step with the next
-// step's ids loaded ahead (cp.async), into a shared histogram over the
-// range's keys, flushed once with one global atomic per non-empty key; the
+// two steps' ids loaded ahead, into a shared histogram over the range's keys, flushed once with one global atomic per non-empty key; the
 // atomic's return value (the block's offset inside the key's bucket) is
-// kept in blk_off for the scatter kernel.
-__global__ void __launch_bounds__(kHistThreads, 3) hist_kernel(const Launch L)
+// kept in blk_off for the scatter kernel.  A group of digis of a step that
+// lies in one event (most do), all valid, is counted without a look at its
+// digis' events: three instructions a digi, which bound this kernel, instead of
+// a dozen (27.7M digis in 256 events: 45.7 -> 29.7 us, 1.9 TB/s).
+__global__ void __launch_bounds__(kHistThreads, 3) hist_kernel(const __grid_constant__ Launch L)
 {
     extern __shared__ uint32_t sh[];
     __shared__ uint32_t s_ev[2];
     pdl_trigger();
     __shared__ uint64_t s_off[kChunkEvents + 1];
-    __shared__ __align__(16) uint16_t pf_m[kChunk];
     // the event offsets must run 0 = o[0] <= o[1] <= ... <= o[E] = N (the
     // device entry points take them from the caller); each block checks a
     // slice, and a violation makes every later kernel skip its writes and
@@ -382,9 +394,8 @@ __global__ void __launch_bounds__(kHistThreads, 3) hist_kernel(const Launch L)
     if (c0 >= c1) return;
     // the first module ids are loaded before the event search, so that the
     // two latencies overlap
-    uint64_t k0 = c0 + (uint64_t)threadIdx.x * kPerThread;
-    uint32_t m[kPerThread], e_of[kPerThread];
-    load_modules(L, k0, c1, m);
+    const uint64_t mine = (uint64_t)threadIdx.x * kPerThread;
+    uint4 cur = load_packed(L, c0 + mine, c1), next = load_packed(L, c0 + kChunk + mine, c1);
     const ChunkInfo ci = chunk_info<>(L, c0, c1, s_ev, s_off);
     const uint32_t M = L.g.M, warp = threadIdx.x >> 5;
     const bool sub = ci.use_sh && ci.nkeys <= kSubKeys;
@@ -392,25 +403,41 @@ __global__ void __launch_bounds__(kHistThreads, 3) hist_kernel(const Launch L)
     for (uint32_t i = threadIdx.x; i < nbins; i += kHistThreads) sh[i] = 0;
     __syncthreads();
     uint32_t *bins = sub ? sh + warp * ci.nkeys : sh;
-    for (; k0 < c1; k0 += kChunk) {
-        const bool pf = prefetch_digis(L, k0 + kChunk, c1, pf_m, nullptr);
+    const bool off_sh = ci.el - ci.ef + 1 < kChunkEvents;
+    uint32_t es = ci.ef; // event of the step's first digi
+    for (uint64_t s0 = c0; s0 < c1; s0 += kChunk) {
+        const uint64_t k0 = s0 + mine;
+        const uint32_t a[4] = {cur.x, cur.y, cur.z, cur.w};
+        cur = next;
+        next = load_packed(L, k0 + 2 * kChunk, c1);
+        if (k0 >= c1) continue; // (no barriers below)
+        if (off_sh)
+            while (es < ci.el && s_off[es + 1 - ci.ef] <= s0) ++es;
+        const bool one = ci.use_sh && off_sh && (es == ci.el || s_off[es + 1 - ci.ef] >= min(c1, s0 + kChunk));
+        const uint32_t top = __vmaxu2(__vmaxu2(a[0], a[1]), __vmaxu2(a[2], a[3]));
+        // all present, valid and of the step's event: most groups
+        if (one && k0 + kPerThread <= c1 && max(top & 0xFFFFu, top >> 16) < M) {
+            uint32_t *eb = bins + (es - ci.ef) * M;
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) atomicAdd(eb + (j & 1 ? a[j / 2] >> 16 : a[j / 2] & 0xFFFFu), 1u);
+            continue;
+        }
+        uint32_t e_of[kPerThread];
         digi_events(L, s_off, ci.ef, ci.el, k0, e_of);
 #pragma unroll
         for (int j = 0; j < kPerThread; ++j) {
-            const bool present = k0 + j < c1;
-            const bool ok = present && m[j] < M;
-            if (present && !ok) atomicOr(&L.ws.event_err[e_of[j]], kErrBadDigi);
-            if (!ok) continue;
-            const uint64_t key = (uint64_t)e_of[j] * M + m[j];
+            const uint32_t m = j & 1 ? a[j / 2] >> 16 : a[j / 2] & 0xFFFFu;
+            if (k0 + j >= c1) continue;
+            if (m >= M) {
+                atomicOr(&L.ws.event_err[e_of[j]], kErrBadDigi);
+                continue;
+            }
+            const uint64_t key = (uint64_t)e_of[j] * M + m;
             if (ci.use_sh)
                 atomicAdd(&bins[key - ci.keybase], 1u);
             else
                 atomicAdd(&L.ws.count2[key], 1u);
         }
-        if (pf)
-            take_prefetched(pf_m, nullptr, m, nullptr);
-        else if (k0 + kChunk < c1)
-            load_modules(L, k0 + kChunk, c1, m);
     }
     __syncthreads();
     // With few keys (long runs per key) the flush's atomic returns this
@@ -462,37 +489,138 @@ __global__ void __launch_bounds__(256) scan_kernel(const Launch L)
     }
 }
 
-// Shared memory of the scatter kernel (bytes).
-constexpr size_t kScatterSmem = kHistCap * 4 + kChunk * (4 + 4 + 2) + (2 * kSubKeys + 2) * 4 + 16 + kChunk * (2 + 4);
-static_assert(kChunk * (4 + 4 + 2) >= kHistCap * 4, "the staging area also holds the single-histogram bases");
+// Digis a thread of the scatter kernel holds where a range has few keys, the
+// step of a block there, and the kernel's shared memory (bytes): the staged
+// digis with their keys and three words a key, or (many keys) a count and a
+// base a key and the next step's digis.
+constexpr int kScatPer = 2 * kPerThread;
+constexpr uint32_t kScatStep = kHistThreads * kScatPer;
+constexpr size_t kScatSort = (size_t)kScatStep * (8 + 2) + 3 * 4 * (kSubKeys + 32);
+constexpr size_t kScatDirect = (size_t)kHistCap * 8 + kChunk * (2 + 4);
+constexpr size_t kScatterSmem = kScatSort > kScatDirect ? kScatSort : kScatDirect;
+static_assert(kSubKeys + 32 <= (uint32_t)kHistThreads && kSubKeys < kChunkEvents, "a key a thread, every offset kept");
+
+// A thread's modules (~0: absent) and words of the step at s0.
+__device__ __forceinline__ void load_scatter(const Launch &L, uint64_t s0, uint64_t c1, uint32_t (&m)[kScatPer],
+                                             uint32_t (&w)[kScatPer])
+{
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint64_t k0 = s0 + ((uint64_t)h * kHistThreads + threadIdx.x) * kPerThread;
+        uint32_t m8[kPerThread], w8[kPerThread];
+        load_modules(L, k0, c1, m8);
+        load_words(L, k0, c1, w8);
+#pragma unroll
+        for (int j = 0; j < kPerThread; ++j) {
+            m[h * kPerThread + j] = m8[j];
+            w[h * kPerThread + j] = w8[j];
+        }
+    }
+}
+
+// The scatter of a block's range [c0, c1) with at most kSubKeys keys: every
+// step of kScatStep digis is ranked by key with one shared-memory atomic a
+// digi, sorted by key in shared memory, and each key's run is written with
+// consecutive threads from the block's offset inside the bucket (reserved by
+// the histogram's flush), so no step needs a global atomic.  Bound by
+// shared-memory wavefronts (69% of the LSU pipe: rank, place and read back
+// each digi, the last two with the bank conflicts of a random order).  Against
+// steps of half the size with a histogram a warp and the event looked up for
+// every digi: 27.7M digis on 64 modules 153 -> 127 us.  Leaving the keys out
+// of the stage, a warp finding the runs of its share, was 124 us there but
+// 35 us instead of 30 for 5.8M digis in 48 events.  km and w: the
+// first step's modules (then key | rank << 16; 0xFFFF: none) and words, two
+// groups of kPerThread a thread.
+__device__ __forceinline__ void scatter_few(const Launch &L, uint32_t *sh, const ChunkInfo &ci, const uint64_t *s_off,
+                                            uint32_t *s_scan, uint32_t (&km)[kScatPer], uint32_t (&w)[kScatPer])
+{
+    const uint32_t tid = threadIdx.x, M = L.g.M, nkeys = ci.nkeys;
+    uint2 *stage = reinterpret_cast<uint2 *>(sh);                     // [kScatStep] sorted by key
+    uint16_t *skey = reinterpret_cast<uint16_t *>(stage + kScatStep); // [kScatStep]
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(skey + kScatStep);   // [kSubKeys + 32] digis of a key (and of none)
+    uint32_t *lk = cnt + kSubKeys + 32;                               // their start in the stage
+    uint32_t *to = lk + kSubKeys + 32;                                // from the stage to the buckets
+    uint32_t kg = 0; // thread t: where the next digis of key t go
+    if (tid < nkeys) kg = L.ws.boff[ci.keybase + tid] + L.ws.blk_off[(size_t)blockIdx.x * kHistCap + tid];
+    if (tid < kSubKeys + 32) cnt[tid] = 0;
+    __syncthreads();
+    uint32_t es = ci.ef; // event of the step's first digi
+    for (uint64_t s0 = ci.c0; s0 < ci.c1; s0 += kScatStep) {
+        while (es < ci.el && s_off[es + 1 - ci.ef] <= s0) ++es;
+        const bool one = es == ci.el || s_off[es + 1 - ci.ef] >= min(ci.c1, s0 + kScatStep);
+        const bool both = s0 + kScatStep / 2 < ci.c1; // the second groups hold digis
+        const uint32_t ekey = (es - ci.ef) * M;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (h && !both) continue;
+            uint32_t *x = km + h * kPerThread, rank[kPerThread];
+            uint32_t e_of[kPerThread];
+            if (!one) digi_events(L, s_off, ci.ef, ci.el, s0 + ((uint64_t)h * kHistThreads + tid) * kPerThread, e_of);
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) // (an absent digi's module is ~0)
+                x[j] = x[j] < M ? (one ? ekey : (e_of[j] - ci.ef) * M) + x[j] : 0xFFFFu;
+            // (no branches, so that the atomics' latencies overlap)
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j)
+                rank[j] = atomicAdd(&cnt[x[j] == 0xFFFFu ? kSubKeys + (tid & 31) : x[j]], 1u);
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) x[j] |= x[j] == 0xFFFFu ? 0u : rank[j] << 16;
+        }
+        __syncthreads();
+        const uint32_t tot = tid < nkeys ? cnt[tid] : 0u;
+        uint32_t total;
+        const uint32_t start = block_exclusive_scan<kHistThreads>(tot, s_scan, &total);
+        if (tid < kSubKeys + 32) {
+            lk[tid] = start;
+            to[tid] = kg - start;
+            cnt[tid] = 0;
+            kg += tot;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t k0 = s0 + ((uint64_t)h * kHistThreads + tid) * kPerThread;
+            if (h && !both) continue;
+            const uint32_t *x = km + h * kPerThread;
+            uint32_t e_of[kPerThread];
+            if (!one) digi_events(L, s_off, ci.ef, ci.el, k0, e_of);
+            const uint32_t i0 = (uint32_t)(k0 - s_off[es - ci.ef]);
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) {
+                const uint32_t key = x[j] & 0xFFFFu;
+                if (key == 0xFFFFu) continue;
+                const uint32_t p = lk[key] + (x[j] >> 16);
+                stage[p] = make_uint2(w[h * kPerThread + j],
+                                      one ? i0 + j : (uint32_t)(k0 + j - s_off[e_of[j] - ci.ef]));
+                skey[p] = (uint16_t)key;
+            }
+        }
+        __syncthreads();
+        if (s0 + kScatStep < ci.c1) load_scatter(L, s0 + kScatStep, ci.c1, km, w); // (in flight while this step is written out)
+#pragma unroll 4
+        for (uint32_t p = tid; p < total; p += kHistThreads) L.ws.bucket[to[skey[p]] + p] = stage[p];
+    }
+}
 
 // Scatter, persistent, over the histogram kernel's ranges: block b walks its
-// range in steps of kChunk digis (one event search a block; the next step's
-// words and module ids are loaded while the current step is written out,
-// cp.async).  Each step ranks its digis per key in shared memory.  With few
-// keys it sorts them by key in shared memory and writes each key's run with
-// consecutive threads, from the block's offset inside the bucket (reserved
-// by the histogram's flush), so no step needs a global atomic.  With many
-// keys one global atomic per key and step hands out the positions (after
-// the reserved runs), and each digi goes straight to its place; a range
-// with more keys than a shared histogram holds takes one atomic per digi.
-__global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L)
+// range (one event search a block).  With few keys scatter_few.  With many
+// keys, in steps of kChunk digis (the next step's words and module ids are
+// loaded while the current step is written out, cp.async), one global atomic
+// per key and step hands out the positions (after the reserved runs), and each
+// digi goes straight to its place; a range with more keys than a shared
+// histogram holds takes one atomic per digi.
+__global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const __grid_constant__ Launch L)
 {
     extern __shared__ __align__(16) uint32_t sh[];
     pdl_wait();
     pdl_trigger();
-    uint32_t *cnt = sh;             // counts: per warp sub-histograms, or one histogram
-    uint32_t *bas = sh + kHistCap;  // single-histogram mode: base of each key
-    uint32_t *stage_w = sh + kHistCap;                                      // sub mode: block-local sorted words
-    uint32_t *stage_i = stage_w + kChunk;                                   // and in-event indices
-    uint16_t *stage_k = reinterpret_cast<uint16_t *>(stage_i + kChunk);     // and local keys
-    uint32_t *lk = reinterpret_cast<uint32_t *>(stage_k + kChunk);          // block-local start of each key
-    uint32_t *gb = lk + kSubKeys + 1;                                       // bucket position of each key's run
+    uint32_t *cnt = sh;             // digis of each key
+    uint32_t *bas = sh + kHistCap;  // and its base
     __shared__ uint32_t s_ev[2];
     __shared__ uint64_t s_off[kChunkEvents + 1];
     __shared__ uint32_t s_scan[kHistThreads / 32 + 1];
     // next step's module ids and words (16-byte aligned for cp.async)
-    uint16_t *pf_m = reinterpret_cast<uint16_t *>((reinterpret_cast<uintptr_t>(gb + kSubKeys + 1) + 15) & ~(uintptr_t)15);
+    uint16_t *pf_m = reinterpret_cast<uint16_t *>(bas + kHistCap);
     uint32_t *pf_w = reinterpret_cast<uint32_t *>(pf_m + kChunk);
     if (L.ws.ctl[1] & kErrBadOffsets) return;
     uint64_t c0, c1;
@@ -500,26 +628,23 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
     if (c0 >= c1) return;
     // the first digis are loaded before the event search, so that the two
     // latencies overlap
+    uint32_t m0[kScatPer], w0[kScatPer];
+    load_scatter(L, c0, c1, m0, w0);
+    const ChunkInfo ci = chunk_info<>(L, c0, c1, s_ev, s_off);
+    const uint32_t M = L.g.M;
+    if (ci.use_sh && ci.nkeys <= kSubKeys) { // (uniform)
+        __syncthreads();                     // s_off
+        scatter_few(L, sh, ci, s_off, s_scan, m0, w0);
+        return;
+    }
     uint64_t k0 = c0 + (uint64_t)threadIdx.x * kPerThread;
     uint32_t m[kPerThread], e_of[kPerThread], w[kPerThread], rank[kPerThread];
-    load_modules(L, k0, c1, m);
-    load_words(L, k0, c1, w);
-    const ChunkInfo ci = chunk_info<>(L, c0, c1, s_ev, s_off);
-    const uint32_t M = L.g.M, warp = threadIdx.x >> 5;
-    const bool sub = ci.use_sh && ci.nkeys <= kSubKeys;
-    const uint32_t nbins = sub ? ci.nkeys * kHistWarps : ci.nkeys;
+#pragma unroll
+    for (int j = 0; j < kPerThread; ++j) m[j] = m0[j], w[j] = w0[j];
     const bool off_sh = ci.el - ci.ef + 1 < kChunkEvents;
     auto event_start = [&](uint32_t e) -> uint64_t { return off_sh ? s_off[e - ci.ef] : L.offsets[e]; };
-    uint32_t *bins = sub ? cnt + warp * ci.nkeys : cnt;
-    // each key's next bucket position for this block: the bucket start, plus
-    // the block's offset inside the bucket (from the histogram's flush),
-    // advanced step by step
-    if (sub) {
-        const uint32_t *boffs = L.ws.blk_off + (size_t)blockIdx.x * kHistCap;
-        for (uint32_t i = threadIdx.x; i < ci.nkeys; i += kHistThreads) gb[i] = L.ws.boff[ci.keybase + i] + boffs[i];
-    }
     for (uint64_t s0 = c0;; s0 += kChunk, k0 += kChunk) {
-        for (uint32_t i = threadIdx.x; i < nbins; i += kHistThreads) cnt[i] = 0;
+        for (uint32_t i = threadIdx.x; i < ci.nkeys; i += kHistThreads) cnt[i] = 0;
         __syncthreads();
         const bool more = s0 + kChunk < c1; // another step follows
         const bool pf = more && prefetch_digis(L, k0 + kChunk, c1, pf_m, pf_w);
@@ -532,59 +657,20 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
                 continue;
             }
             const uint64_t key = (uint64_t)e_of[j] * M + m[j];
-            rank[j] = ci.use_sh ? atomicAdd(&bins[key - ci.keybase], 1u) : atomicAdd(&L.ws.cursor[key], 1u);
+            rank[j] = ci.use_sh ? atomicAdd(&cnt[key - ci.keybase], 1u) : atomicAdd(&L.ws.cursor[key], 1u);
         }
         __syncthreads();
-        if (sub) {
-            // Per key: per-warp counts become offsets within the key, the
-            // key's block start comes from a scan over keys, and one atomic
-            // reserves its run in the bucket.
-            uint32_t tot = 0;
-            if (threadIdx.x < ci.nkeys) {
-                for (uint32_t wi = 0; wi < kHistWarps; ++wi) {
-                    const uint32_t c = cnt[wi * ci.nkeys + threadIdx.x];
-                    cnt[wi * ci.nkeys + threadIdx.x] = tot;
-                    tot += c;
-                }
-            }
-            uint32_t total;
-            const uint32_t start = block_exclusive_scan<kHistThreads>(tot, s_scan, &total);
-            uint32_t kg = 0;
-            if (threadIdx.x < ci.nkeys) {
-                lk[threadIdx.x] = start;
-                kg = gb[threadIdx.x];
-            }
-            __syncthreads();
+        for (uint32_t i = threadIdx.x; i < ci.nkeys; i += kHistThreads) {
+            const uint32_t v = cnt[i];
+            if (v) bas[i] = atomicAdd(&L.ws.cursor[ci.keybase + i], v);
+        }
+        __syncthreads();
 #pragma unroll
-            for (int j = 0; j < kPerThread; ++j) {
-                if (m[j] == 0xFFFFFFFFu) continue;
-                const uint32_t key = (uint32_t)((uint64_t)e_of[j] * M + m[j] - ci.keybase);
-                const uint32_t p = lk[key] + cnt[warp * ci.nkeys + key] + rank[j];
-                stage_w[p] = w[j];
-                stage_i[p] = (uint32_t)(k0 + j - event_start(e_of[j]));
-                stage_k[p] = (uint16_t)key;
-            }
-            __syncthreads();
-            for (uint32_t p = threadIdx.x; p < total; p += kHistThreads) {
-                const uint32_t key = stage_k[p];
-                const uint32_t g = gb[key] + (p - lk[key]);
-                L.ws.bucket[g] = make_uint2(stage_w[p], stage_i[p]);
-            }
-            __syncthreads();
-            if (threadIdx.x < ci.nkeys) gb[threadIdx.x] = kg + tot; // the key's cursor after this step
-        } else {
-            for (uint32_t i = threadIdx.x; i < ci.nkeys; i += kHistThreads) {
-                const uint32_t v = cnt[i];
-                if (v) bas[i] = atomicAdd(&L.ws.cursor[ci.keybase + i], v);
-            }
-            __syncthreads();
-#pragma unroll
-            for (int j = 0; j < kPerThread; ++j) {
-                if (m[j] == 0xFFFFFFFFu) continue;
-                const uint64_t key = (uint64_t)e_of[j] * M + m[j];
-                const uint32_t p = ci.use_sh ? bas[key - ci.keybase] + rank[j] : rank[j];
-                L.ws.bucket[p] = make_uint2(w[j], (uint32_t)(k0 + j - event_start(e_of[j])));
-            }
+        for (int j = 0; j < kPerThread; ++j) {
+            if (m[j] == 0xFFFFFFFFu) continue;
+            const uint64_t key = (uint64_t)e_of[j] * M + m[j];
+            const uint32_t p = ci.use_sh ? bas[key - ci.keybase] + rank[j] : rank[j];
+            L.ws.bucket[p] = make_uint2(w[j], (uint32_t)(k0 + j - event_start(e_of[j])));
         }
         __syncthreads();
         if (!more) break;
@@ -603,14 +689,15 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const Launch L
 // writes each key's run with consecutive threads.  Against scatter_kernel's
 // step of 4,096 digis, whose digis land nearly alone (2.2 a key for 1,856
 // modules), a run is 8.8 digis: a third of the sectors and a quarter of the
-// atomics (29.4M digis in 8 events: 281 -> 183 us).  Bound by shared-memory
+// atomics (29.4M digis in 8 events: 281 -> 183 us; 171 us with the digis'
+// events looked up only in steps over several).  Bound by shared-memory
 // wavefronts (rank, placing and reading back each digi; half of their peak,
 // one block an SM) and by L2 writes.  A step over more keys than the tables
 // hold takes one atomic a digi, as scatter_kernel does.
 constexpr int kWideThreads = 1024;
 constexpr int kWidePer = 2 * kPerThread;                // digis a thread holds
 constexpr uint32_t kWideStep = kWideThreads * kWidePer; // digis a block sorts at a time
-constexpr size_t kWideSmem = (size_t)kWideStep * (8 + 2) + 3 * 4 * (size_t)kHistCap;
+constexpr size_t kWideSmem = (size_t)kWideStep * (8 + 2) + 4 * (3 * (size_t)kHistCap + 32);
 
 __global__ void __launch_bounds__(kWideThreads, 1) scatter_wide_kernel(const __grid_constant__ Launch L)
 {
@@ -624,9 +711,9 @@ __global__ void __launch_bounds__(kWideThreads, 1) scatter_wide_kernel(const __g
     const uint32_t tid = threadIdx.x, M = L.g.M;
     uint2 *stage = reinterpret_cast<uint2 *>(sh);                     // [kWideStep] sorted by key
     uint16_t *skey = reinterpret_cast<uint16_t *>(stage + kWideStep); // [kWideStep]
-    uint32_t *cnt = reinterpret_cast<uint32_t *>(skey + kWideStep);   // [kHistCap] digis of a key
-    uint32_t *lk = cnt + kHistCap;                                    // [kHistCap] their start in the stage
-    uint32_t *gb = lk + kHistCap;                                     // [kHistCap] and in the buckets
+    uint32_t *cnt = reinterpret_cast<uint32_t *>(skey + kWideStep);   // [kHistCap + 32] digis of a key (and of none)
+    uint32_t *lk = cnt + kHistCap + 32;                               // [kHistCap] their start in the stage
+    uint32_t *to = lk + kHistCap;                                     // [kHistCap] from the stage to the buckets
     static_assert(kHistCap <= 4 * kWideThreads, "four keys a thread");
     // all event offsets in shared memory when they fit, else a step's
     const bool all_off = L.E < kChunkEvents;
@@ -694,22 +781,26 @@ __global__ void __launch_bounds__(kWideThreads, 1) scatter_wide_kernel(const __g
             __syncthreads();
             continue;
         }
-        // rank of each digi among its key's
+        // whether the step lies in one event, which then no digi looks for
+        const bool one = ci.ef == ci.el;
+        // rank of each digi among its key's (no branches, so that the atomics'
+        // latencies overlap)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const uint64_t k0 = s0 + ((uint64_t)h * kWideThreads + tid) * kPerThread;
-            uint32_t e_of[kPerThread];
-            digi_events(L, off, ci.ef, ci.el, k0, e_of);
+            uint32_t *x = km + h * kPerThread, rank[kPerThread];
+            if (!one) {
+                uint32_t e_of[kPerThread];
+                digi_events(L, off, ci.ef, ci.el, s0 + ((uint64_t)h * kWideThreads + tid) * kPerThread, e_of);
 #pragma unroll
-            for (int j = 0; j < kPerThread; ++j) {
-                uint32_t &x = km[h * kPerThread + j];
-                if (k0 + j < c1 && x < M) {
-                    const uint32_t key = (e_of[j] - ci.ef) * M + x;
-                    x = key | (atomicAdd(&cnt[key], 1u) << 16);
-                } else {
-                    x = 0xFFFFu;
-                }
+                for (int j = 0; j < kPerThread; ++j) x[j] = x[j] < M ? (e_of[j] - ci.ef) * M + x[j] : 0xFFFFu;
             }
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) { // (an absent digi's module is ~0)
+                x[j] = x[j] < (one ? M : 0xFFFFu) ? x[j] : 0xFFFFu;
+                rank[j] = atomicAdd(&cnt[x[j] == 0xFFFFu ? (uint32_t)kHistCap + (tid & 31) : x[j]], 1u);
+            }
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) x[j] |= x[j] == 0xFFFFu ? 0u : rank[j] << 16;
         }
         __syncthreads();
         uint32_t total;
@@ -722,31 +813,34 @@ __global__ void __launch_bounds__(kWideThreads, 1) scatter_wide_kernel(const __g
 #pragma unroll
             for (int i = 0; i < 4; ++i) g[i] = cs[i] ? atomicAdd(&L.ws.cursor[ci.keybase + k + i], cs[i]) : 0u;
             const uint32_t l0 = block_exclusive_scan<kWideThreads>(c.x + c.y + c.z + c.w, tmp, &total);
-            *reinterpret_cast<uint4 *>(lk + k) = make_uint4(l0, l0 + c.x, l0 + c.x + c.y, l0 + c.x + c.y + c.z);
-            *reinterpret_cast<uint4 *>(gb + k) = make_uint4(g[0], g[1], g[2], g[3]);
+            const uint32_t l1 = l0 + c.x, l2 = l1 + c.y, l3 = l2 + c.z;
+            *reinterpret_cast<uint4 *>(lk + k) = make_uint4(l0, l1, l2, l3);
+            *reinterpret_cast<uint4 *>(to + k) = make_uint4(g[0] - l0, g[1] - l1, g[2] - l2, g[3] - l3);
         }
         __syncthreads();
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint64_t k0 = s0 + ((uint64_t)h * kWideThreads + tid) * kPerThread;
+            const uint32_t *x = km + h * kPerThread;
             uint32_t e_of[kPerThread];
-            digi_events(L, off, ci.ef, ci.el, k0, e_of);
+            if (!one) digi_events(L, off, ci.ef, ci.el, k0, e_of);
+            const bool off_sh = all_off || ci.el - ci.ef + 1 < kChunkEvents;
+            const uint32_t i0 = (uint32_t)(k0 - off[0]);
 #pragma unroll
             for (int j = 0; j < kPerThread; ++j) {
-                const uint32_t x = km[h * kPerThread + j], key = x & 0xFFFFu;
+                const uint32_t key = x[j] & 0xFFFFu;
                 if (key == 0xFFFFu) continue;
-                const uint32_t p = lk[key] + (x >> 16);
-                const uint64_t start = ci.el - ci.ef + 1 < kChunkEvents ? off[e_of[j] - ci.ef] : L.offsets[e_of[j]];
-                stage[p] = make_uint2(w[h * kPerThread + j], (uint32_t)(k0 + j - start));
+                const uint32_t p = lk[key] + (x[j] >> 16);
+                uint32_t index = i0 + j;
+                if (!one) index = (uint32_t)(k0 + j - (off_sh ? off[e_of[j] - ci.ef] : L.offsets[e_of[j]]));
+                stage[p] = make_uint2(w[h * kPerThread + j], index);
                 skey[p] = (uint16_t)key;
             }
         }
         __syncthreads();
         if (s0 + stride < L.N) load_step(s0 + stride); // (in flight while this step is written out)
-        for (uint32_t p = tid; p < total; p += kWideThreads) {
-            const uint32_t key = skey[p];
-            L.ws.bucket[gb[key] + (p - lk[key])] = stage[p];
-        }
+#pragma unroll 4
+        for (uint32_t p = tid; p < total; p += kWideThreads) L.ws.bucket[to[skey[p]] + p] = stage[p];
         __syncthreads();
     }
 }
