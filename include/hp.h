@@ -390,7 +390,7 @@ hp_status hp_reconstruct_device_noalloc(hp_ctx *ctx, uint32_t n_events, uint64_t
  *                  or 2 (halved for launches too small to fill the GPU: down
  *                  to 4 for items of under 64 digis on average, to 1 for
  *                  larger ones);
- *   warp_max       32 or 64: items of up to eight times as many digis are
+ *   warp_max       32 or 64: items of up to twelve times as many digis are
  *                  clustered together, a ticket's worth at a time (with the
  *                  hash store, items of up to warp_max digis);
  *   label_store    how the items above these look up a pixel's neighbours:

@@ -40,9 +40,9 @@ constexpr int kMaxTileSlots = 16384; // largest tile considered (one block per S
 // autotuner (defaults: the values above, two resident blocks per SM).
 struct Tuning {
     uint32_t tile_slots = kSmemSlots; // runs in a block's shared memory; items with more use global scratch
-    uint32_t blocks_per_sm = 2;       // 1 (four groups a block, largest tile), 2 (two groups) or 3 (one group)
+    uint32_t blocks_per_sm = 2;       // 1 (four groups a block, largest tile), 2 (two or three groups) or 3 (one group)
     uint32_t ticket_max = kGroup;     // items per ticket before halving for small launches (<= kGroup)
-    uint32_t warp_max = kWarpMax;     // 32 or 64: an eighth of the packed tier's largest item (hash store: all of it)
+    uint32_t warp_max = kWarpMax;     // 32 or 64: a twelfth of the packed tier's largest item (hash store: all of it)
     uint32_t label_store = 0;         // kStoreBitmap or kStoreHash: pixel lookup of the items above the packed tier
     uint32_t item_threads = kCCThreads; // threads clustering one item of the hash store: 128, 256 or 512
 };
@@ -173,8 +173,8 @@ struct Workspace {
                           //       clusters (cc_kernel)
     // [N] digi word and index within its event, item after item.  Pairs, so
     // that a digi that lands alone writes one sector instead of two: the
-    // scatter of 29.4M digis over 1,856 modules an event 441 -> 281 us, over
-    // 64 modules 170 -> 154 us.
+    // scatter of 29.4M digis over 1,856 modules an event 441 -> 281 us (171
+    // since, sorted in wide steps), over 64 modules 170 -> 154 us (127 since).
     uint2 *bucket;
     Staging staging;      // [N] each array
     uint32_t *large;      // [E*M] items of more than cc.large_digis digis, ctl[5] of them (scan_kernel)
@@ -287,6 +287,8 @@ __host__ __device__ inline uint32_t pack_capacity(size_t bytes, uint32_t R, uint
     const uint32_t p = fit < 1023 ? (uint32_t)fit : 1023u;
     return p < cap ? p : cap;
 }
+// (384 or 768 digis: the best line for packs on sparse bitmaps; with hash
+// tables in their place it lay at half of that)
 __host__ __device__ inline uint32_t pack_max(uint32_t warp_max) { return 12 * warp_max; }
 
 // Threads and groups of a clustering block for 1, 2 and 3 resident blocks per

@@ -4,22 +4,25 @@
 // E = 1).  The unit of clustering work is an item = (event, module); there
 // are E * M items, in (event, module) order.
 //
-//   hist_kernel     module histogram: count[item] (shared-memory bins per
-//                   block of 4096 digis, flushed with global atomics);
+//   hist_kernel     module histogram: count[item] (shared-memory bins over a
+//                   block's range of digis, flushed with global atomics);
 //                   validates module ids
 //   scan_kernel     one block per event: exclusive prefix sum of the event's
 //                   M counts -> bucket start of every item (the event's digi
 //                   offset is the base, so events scan independently)
 //   scatter_kernel  bucket scatter: each digi's word and in-event index go to
 //                   its item's bucket (block-local ranks in shared memory,
-//                   one global atomic per non-empty bin to reserve a range)
+//                   positions reserved by the histogram or by one global
+//                   atomic per non-empty bin); scatter_wide_kernel for many
+//                   digis on many modules
 //   cc_kernel       persistent clustering: groups of threads take tickets of
 //                   up to kGroup consecutive items (the count is a tuning
 //                   parameter); a ticket's small items go together through
-//                   the packed tier (a hash table of their pixels), larger
+//                   the packed tier (bitmaps of the words they touch), larger
 //                   ones one by one through the run tier (bitmaps of the
 //                   module, union-find over horizontal runs), in shared
 //                   memory, or in global scratch if their runs do not fit;
+//                   items too large for a group's share by the whole block;
 //                   cc_hash_kernel (the hash label store, a tuning choice)
 //                   has groups of 128-512 threads cluster the items between
 //                   on a hash table each; kept clusters are staged per item
@@ -54,9 +57,10 @@ constexpr unsigned kFull = 0xFFFFFFFFu;
 // Programmatic dependent launch between the pass's kernels: each kernel lets
 // the next one launch as soon as all its own blocks are running (the next
 // kernel's blocks then take free SM slots and wait), and each dependent
-// kernel waits, before its first access to memory, until the previous grid
-// has completed and its writes are visible.  The waits are the hardware's,
-// not spins.
+// kernel waits, before it reads anything but the call's inputs, until the
+// previous grid has completed and its writes are visible.  (A launch's first
+// kernel is an ordinary launch, so the inputs are in place by then.)  The
+// waits are the hardware's, not spins.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 constexpr uint32_t kSpinLimit = 1u << 24;          // iterations of a blocking wait, at most
@@ -1251,9 +1255,13 @@ __device__ __forceinline__ uint32_t atoms_min(uint32_t a, uint32_t v)
 // data (0.5 to 0.8): against a node and four atomics a pixel (the tier this
 // replaced) a pixel needs no rank and two atomics, and a run looks at one word
 // above it instead of eight pixels.  27.7M digis in 16,384 items: 24 -> 14
-// warp instructions a digi, 934 -> 564 us; 29.4M digis in 14,848 items with
-// 13,000-digi ones among them: 1,374 -> 614 us (its records are 20 bytes, so
-// these fit a block's shared memory now).
+// warp instructions a digi, 934 -> 514 us; 29.4M digis in 14,848 items with
+// 13,000-digi ones among them: 1,374 -> 570 us (its records are 20 bytes, so
+// these fit a block's shared memory now).  Of 146 us for 7.0M digis (57% of
+// the issue slots and 60% of the LSU pipe in use): labels and root positions
+// 31, links and unions 26, sums over runs 13, staging 13, pixel sums 11, the
+// bits 8, first runs and records 6, their scan 3, clearing 2, tickets and packs
+// the rest.
 //
 // Run records:
 //   word 0  union-find parent
@@ -2008,8 +2016,8 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 // ---- packed tier
 //
 // The small items of a ticket together: up to four digis a thread (at most
-// 1,023) of up to 16 items
-// by a group of GT threads, through the run tier's phases on a sparse bitmap.
+// 1,023) of up to 16 items by a group of GT threads, through the run tier's
+// phases on a sparse bitmap.
 // Of each item's bitmap words only the touched ones are stored, in (item,
 // row, word) order: a bit per word of the module says which are (16 bits a
 // row, so that a word's neighbours in its row lie in the same field), and the
@@ -2025,7 +2033,8 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 //   e runs before each touched word, by a scan; run records initialised
 //   f charge and position into the runs, then 5 to 9 of the run tier
 // What bounds it: the latency of the phases, which all items of a ticket
-// share; the work is the digis', not the modules'.
+// share; the work is the digis', not the modules'.  29,696 items of 32 digis:
+// 343 us with a warp an item -> 57 us.
 constexpr int kPackPer = 4; // digis a thread holds
 
 // One warp (lane = its lane): the pack that starts at item i0 of the ticket,
