@@ -84,9 +84,9 @@ bool valid_tuning(const hp_ctx *ctx, const hp::Tuning &t)
 // The autotuner's search space on this device: the default tile at two
 // resident blocks per SM, the largest tile that keeps three resident, and
 // the largest tile of a single block, each with the bitmap label store
-// (tickets of 16, 8, 4 or 2 items, a warp tier up to 64 or 32 digis) and
+// (tickets of 16, 8, 4 or 2 items, warp_max 64 or 32) and
 // with the hash label store at 128, 256 or 512 threads an item (tickets of
-// 16 or 4 items, a warp tier up to 64 digis).
+// 16 or 4 items, warp_max 64).
 std::vector<hp::Tuning> tuning_candidates(const hp_ctx *ctx)
 {
     std::vector<hp::Tuning> c;

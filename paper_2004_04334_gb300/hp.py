@@ -255,11 +255,19 @@ class HitsResult:
         return len(self.x)
 
 
+# A writable view of memory at an address: 2 us a column.  (A ctypes array type
+# for every length costs 15 where the length is new, and numbers of clusters
+# hardly ever repeat: first fetch of a 60,000-digi event's product 29 us less.)
+_memory = ctypes.pythonapi.PyMemoryView_FromMemory
+_memory.argtypes = (ctypes.c_void_p, ctypes.c_ssize_t, ctypes.c_int)
+_memory.restype = ctypes.py_object
+_PYBUF_WRITE = 0x200
+
+
 def _arr(ptr, n, dtype, copy=True):
     if n == 0 or not ptr:
         return np.empty(0, dtype)
-    buf = (ctypes.c_char * (n * np.dtype(dtype).itemsize)).from_address(ptr)
-    a = np.frombuffer(buf, dtype=dtype, count=n)
+    a = np.frombuffer(_memory(ptr, n * np.dtype(dtype).itemsize, _PYBUF_WRITE), dtype)
     return a.copy() if copy else a
 
 
