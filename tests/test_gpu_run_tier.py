@@ -122,3 +122,16 @@ def test_invalid_and_duplicated_digis(torch_cuda):
     items.append(ok)
     expect.append(hp.HP_OK)
     _check(items, np.full(4, 70, np.int32), np.full(4, 50, np.int32), expect=expect)
+
+
+@pytest.mark.parametrize("threads", [480, 512, 1024])
+def test_items_a_whole_block_holds_in_registers(torch_cuda, threads):
+    """At and past eight digis a thread of a block, scattered and in one cluster that needs the 64-bit moments."""
+    rng = np.random.default_rng(threads)
+    line = 8 * threads
+    dense = synth.pack(*(x.ravel()[:line] for x in np.meshgrid(np.arange(120) + 20, np.arange(100) + 200, indexing="ij")),
+                       np.full(line, 250))
+    items = [[_random(line - 1, rng), _random(line, rng), _random(line + 1, rng)], [dense, dense[:line - 1], _random(9, rng)]]
+    gain = np.full(3, 126, np.int32)
+    assert line * 250 * 126 * 200 > 0x7FFFFFFF
+    _check(items, gain, np.zeros(3, np.int32))
