@@ -224,15 +224,12 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // issued) for a partial or unaligned group, which is then loaded directly.
 __device__ __forceinline__ bool prefetch_digis(const Launch &L, uint64_t k0, uint64_t c1, uint16_t *pf_m, uint32_t *pf_w)
 {
-    if (k0 + kPerThread > c1 || (reinterpret_cast<uintptr_t>(L.modules) & 15) ||
-        (pf_w && (reinterpret_cast<uintptr_t>(L.words) & 15)))
+    if (k0 + kPerThread > c1 || ((reinterpret_cast<uintptr_t>(L.modules) | reinterpret_cast<uintptr_t>(L.words)) & 15))
         return false;
     const uint32_t t = threadIdx.x * kPerThread;
     cp_async16(pf_m + t, L.modules + k0);
-    if (pf_w) {
-        cp_async16(pf_w + t, L.words + k0);
-        cp_async16(pf_w + t + 4, L.words + k0 + 4);
-    }
+    cp_async16(pf_w + t, L.words + k0);
+    cp_async16(pf_w + t + 4, L.words + k0 + 4);
     cp_async_commit();
     return true;
 }
@@ -245,11 +242,9 @@ __device__ __forceinline__ void take_prefetched(const uint16_t *pf_m, const uint
     const uint4 a = *reinterpret_cast<const uint4 *>(pf_m + t);
     m[0] = a.x & 0xFFFFu, m[1] = a.x >> 16, m[2] = a.y & 0xFFFFu, m[3] = a.y >> 16;
     m[4] = a.z & 0xFFFFu, m[5] = a.z >> 16, m[6] = a.w & 0xFFFFu, m[7] = a.w >> 16;
-    if (pf_w) {
-        const uint4 b = *reinterpret_cast<const uint4 *>(pf_w + t);
-        const uint4 c = *reinterpret_cast<const uint4 *>(pf_w + t + 4);
-        w[0] = b.x, w[1] = b.y, w[2] = b.z, w[3] = b.w, w[4] = c.x, w[5] = c.y, w[6] = c.z, w[7] = c.w;
-    }
+    const uint4 b = *reinterpret_cast<const uint4 *>(pf_w + t);
+    const uint4 c = *reinterpret_cast<const uint4 *>(pf_w + t + 4);
+    w[0] = b.x, w[1] = b.y, w[2] = b.z, w[3] = b.w, w[4] = c.x, w[5] = c.y, w[6] = c.z, w[7] = c.w;
 }
 
 // Event of each of the thread's digis: a binary search over the block's
