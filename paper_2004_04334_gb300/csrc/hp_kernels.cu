@@ -1121,7 +1121,8 @@ __device__ __forceinline__ float centroid_abs(long long sum, int32_t Q)
 // own (GT threads: its own named barrier, its own tickets).
 struct GroupShared {
     uint32_t ticket;
-    uint32_t flag, heavy, pixels, extras;
+    uint32_t flag;                 // run tier: an invalid digi; packed tier: bit i: the pack's item i is faulty
+    uint32_t heavy, pixels, extras;
     uint32_t bucket_end;           // end of the ticket's buckets
     uint32_t pack_end;             // packed tier: end of the planned pack (an item of the ticket); run tier: scratch slot
     uint32_t tmp[32];              // scans; packed tier: kept clusters of each item
@@ -1608,10 +1609,11 @@ __device__ __forceinline__ void warp_chunks(uint32_t nruns, uint32_t warp, uint3
 // position, kept) for every run.  With
 // kItems the kept roots of each item are counted in gs.tmp[16 ..].  One
 // barrier; returns the kept roots of all runs, and in *ord those before the
-// warp's chunks.
+// warp's chunks.  Roots of the items in `faulty` (bits; kItems) are not kept.
 template <int GT, bool kWhole, bool kItems, class A, class B, class T>
 __device__ __forceinline__ uint32_t mark_runs(const A &a, const B &calib, const T &also, uint32_t nruns, int32_t cthr,
-                                              GroupShared &gs, uint32_t gt, uint32_t bar, uint32_t *ord)
+                                              uint32_t faulty, GroupShared &gs, uint32_t gt, uint32_t bar,
+                                              uint32_t *ord)
 {
     constexpr int kWarps = GT / 32;
     const uint32_t lane = gt & 31, warp = gt >> 5;
@@ -1625,7 +1627,7 @@ __device__ __forceinline__ uint32_t mark_runs(const A &a, const B &calib, const 
             const typename A::At rx = a.at(x);
             const uint32_t px = A::template ld<1>(rx);
             const int32_t Q = (int32_t)A::charge(A::template ld<2>(rx), calib(px));
-            const bool kept = Q >= cthr;
+            const bool kept = Q >= cthr && !(kItems && (faulty >> ((px & kRunItem) >> 23)) & 1u);
             lead = kept && x == i;
             if (Q > kQSafe32) gs.heavy = 1;
             also(a.at(i), px, kept);
@@ -1791,7 +1793,7 @@ __device__ __forceinline__ uint32_t run_clusters(const Launch &L, const ItemCtx 
     auto label_run = [&](typename A::At r, uint32_t px, bool kept) {
         if (label0) A::template st<0>(r, kept ? (px & 0xFFu) * C + ((px >> 8) & 0x1FFu) : (uint32_t)-2);
     };
-    const uint32_t K = mark_runs<GT, kWhole, false>(a, calib, label_run, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
+    const uint32_t K = mark_runs<GT, kWhole, false>(a, calib, label_run, nruns, L.g.cluster_thr, 0u, gs, gt, bar, &ord);
     const bool heavy = gs.heavy != 0;
     if (heavy) { // both moments of every root again, in 64 bits
         for (uint32_t i = gt; i < nruns; i += GT) {
@@ -2027,6 +2029,9 @@ __device__ __forceinline__ uint32_t run_item(const Launch &L, const ItemCtx &it,
 //     both: a duplicate)
 //   e runs before each touched word, by a scan; run records initialised
 //   f charge and position into the runs, then 5 to 9 of the run tier
+// An item with an invalid or a duplicated digi flags its event, keeps no
+// cluster and gets no labels, as in the other tiers (its digis pass through
+// the phases all the same: their sums mean nothing, but stay in its own runs).
 // What bounds it: the latency of the phases, which all items of a ticket
 // share; the work is the digis', not the modules'.  29,696 items of 32 digis:
 // 343 us with a warp an item -> 57 us.
@@ -2095,8 +2100,14 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     if (gt == 0) {
         gs.heavy = 0;
         gs.extras = 0;
+        gs.flag = 0;
     }
     gsync<GT, kWhole>(bar);
+    // (phase f is the last to flag)
+    auto flag = [&](uint32_t i, uint32_t err) {
+        atomicOr(L.ws.event_err + gs.rec[i0 + i].e, err);
+        atomicOr(&gs.flag, 1u << i);
+    };
 
     // b
 #pragma unroll
@@ -2104,7 +2115,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
         if (gt + k * GT >= total) break;
         const uint32_t r = w[k] & 0xFFu, c = (w[k] >> 8) & 0x1FFu, adc = w[k] >> 17;
         if (r >= R || c >= C || adc - 1u >= 255u) { // ADC 0, or any of the bits 25-31
-            atomicOr(L.ws.event_err + gs.rec[i0 + li[k]].e, kErrBadDigi);
+            flag(li[k], kErrBadDigi);
             w[k] = kNoDigi;
         } else {
             reds_or(fields + 4 * (li[k] * RH + (r >> 1)), 1u << (((r & 1u) << 4) + (c >> 5)));
@@ -2146,7 +2157,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
         uint32_t near;
         at[k] = place(li[k], r, c >> 5, &near);
         const bool keep = (int32_t)((w[k] >> 17) & 0xFFu) * rec.gain - rec.ped >= thr;
-        if (atoms_or((keep ? surv : drop) + 4 * at[k], bit) & bit) atomicOr(L.ws.event_err + rec.e, kErrDup);
+        if (atoms_or((keep ? surv : drop) + 4 * at[k], bit) & bit) flag(li[k], kErrDup);
         dropped |= keep ? 0u : 1u << k;
     }
     gsync<GT, kWhole>(bar);
@@ -2178,10 +2189,9 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
         const uint32_t x = w[k];
         w[k] = kNoSlot;
         if (x == kNoDigi) continue;
-        const ItemRec &rec = gs.rec[i0 + li[k]];
         const uint32_t word = lds(surv + 4 * at[k]), b = 1u << ((x >> 8) & 31u), h = word & ~(word << 1);
         if ((dropped >> k) & 1u) { // (a survivor at its pixel is a duplicate too)
-            if (word & b) atomicOr(L.ws.event_err + rec.e, kErrDup);
+            if (word & b) flag(li[k], kErrDup);
             continue;
         }
         const uint32_t run = lds_u16(rpre + 2 * at[k]) + __popc(h & (b | (b - 1u))) - 1u;
@@ -2213,8 +2223,10 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
     sum_runs<GT>(a, calib, nruns, gt);
     gsync<GT, kWhole>(bar);
     uint32_t ord;
-    mark_runs<GT, kWhole, true>(a, calib, [](A::At, uint32_t, bool) {}, nruns, L.g.cluster_thr, gs, gt, bar, &ord);
+    mark_runs<GT, kWhole, true>(a, calib, [](A::At, uint32_t, bool) {}, nruns, L.g.cluster_thr, gs.flag, gs, gt, bar,
+                                &ord);
     const bool heavy = gs.heavy != 0;
+    const uint32_t faulty = gs.flag;
     if (heavy) { // both moments again, in 64 bits
         for (uint32_t i = gt; i < 2 * nruns; i += GT) exact[i] = 0;
         gsync<GT, kWhole>(bar);
@@ -2247,6 +2259,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
 #pragma unroll
         for (int k = 0; k < kPackPer; ++k) {
             if (gt + k * GT >= total) break;
+            if ((faulty >> li[k]) & 1u) continue;
             int32_t lab = -1;
             if (w[k] != kNoSlot) {
                 const uint32_t p = A::ld<1>(a.at(w[k]));
@@ -2268,6 +2281,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
 #pragma unroll
         for (int k = 0; k < kPackPer; ++k) {
             if (gt + k * GT >= total) break;
+            if ((faulty >> li[k]) & 1u) continue;
             uint16_t v = kLab16Below;
             if (w[k] != kNoSlot) {
                 const A::At rx = a.at(a.parent(w[k]));
