@@ -3359,7 +3359,10 @@ namespace {
 // Largest tile (a multiple of 256 slots, at most max_slots) with which
 // `blocks` blocks of `kern` (`threads` threads, bytes(tile) of dynamic shared
 // memory) stay resident on one SM; 0 if none does.  Also raises the kernel's
-// dynamic shared memory limit to what that tile needs.
+// dynamic shared memory limit to the most the device gives: the limit is the
+// process's, not the context's, and a context for other modules must not lower
+// it under one that lives (bytes() does not even grow with the module: slices
+// fall back to 256 runs where larger ones would not fit).
 template <class K, class F>
 cudaError_t fit_tile(K kern, int device, int blocks, int threads, F bytes, uint32_t max_slots, uint32_t *tile)
 {
@@ -3374,7 +3377,7 @@ cudaError_t fit_tile(K kern, int device, int blocks, int threads, F bytes, uint3
     uint32_t t = max_slots;
     while (t >= 256 && bytes(t) > limit) t -= 256;
     if (t < 256) return cudaSuccess;
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes(t));
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)limit);
     if (err != cudaSuccess) return err;
     for (; t >= 256; t -= 256) {
         int nb = 0;
