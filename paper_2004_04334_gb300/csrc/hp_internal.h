@@ -261,13 +261,16 @@ __host__ __device__ inline uint32_t run_capacity(size_t bytes, uint32_t R, uint3
 }
 // Dynamic shared memory of a block of `groups` groups whose whole holds
 // tile_slots runs: at least slices of kSliceRuns runs where those leave two
-// blocks an SM, of 256 where not, and of the bitmaps.
-constexpr size_t kSliceRuns = 1200, kSliceBytes = 112000;
+// blocks an SM, of 256 where not, and of the bitmaps; at most what a lone
+// block has besides its static memory (6,400 bytes for four groups), so that
+// the largest tiles of small modules, which the hash store's limit allows,
+// hold a few hundred runs less than they name.
+constexpr size_t kSliceRuns = 1200, kSliceBytes = 112000, kWholeBytes = 225792;
 __host__ __device__ inline size_t run_smem_bytes(uint32_t R, uint32_t C, uint32_t tile_slots, uint32_t groups)
 {
     const size_t fixed = run_fixed_bytes(R, C), bits = (size_t)run_words(R, C) * 4;
     auto at_least = [&](size_t runs) { return fixed + (kRunBytes * runs > bits ? kRunBytes * runs : bits); };
-    const size_t whole = at_least(tile_slots);
+    const size_t full = at_least(tile_slots), whole = full < kWholeBytes ? full : kWholeBytes;
     size_t parts = groups * ((at_least(kSliceRuns) + 15) & ~(size_t)15);
     if (parts > kSliceBytes) parts = groups * ((at_least(256) + 15) & ~(size_t)15);
     return whole > parts ? whole : parts;

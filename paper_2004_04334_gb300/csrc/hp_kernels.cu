@@ -1130,6 +1130,8 @@ struct GroupShared {
     ItemRec rec[kGroup];
     uint16_t pack[kGroup + 1];     // packed tier: first packed digi of each item, and the total
 };
+static_assert(kWholeBytes + sizeof(GroupShared) * kRunGroups1 + kRunThreads1 / 32 * 128 <= 227 * 1024,
+              "the largest tile beside a block's static memory");
 
 template <int GT, bool kWhole>
 __device__ __forceinline__ void gsync(uint32_t bar)
