@@ -860,25 +860,31 @@ __global__ void __launch_bounds__(kWideThreads, 1) scatter_wide_kernel(const __g
 // memory; after a cluster barrier each reads the others' counts (distributed
 // shared memory, four modules a load) and so knows, for every module, the
 // bucket's start and its own offset inside it; then it sorts its digis by
-// module in shared memory, kBucketStep at a time, and writes each module's run
-// with consecutive threads.  With one event the kernel also clears the
-// launch's control words, so that nothing precedes it.  Bound by launch and
-// global-memory latency: one launch in place of a memset and three kernels.
+// module in shared memory and writes each module's run with consecutive
+// threads.  A slice is at most kBucketStep digis, a step a block: no event of
+// the launch has more than kBucketDigis (bucket_fits).  With one event the
+// kernel also clears the launch's control words, so that nothing precedes it.
+// Bound by launch and global-memory latency: one launch in place of a memset
+// and three kernels.
 constexpr int kBucketThreads = 1024;
 constexpr int kBucketCluster = 8;                             // portable cluster size
 constexpr int kBucketPer = 2 * kPerThread;                    // digis a thread holds
-constexpr uint32_t kBucketStep = kBucketThreads * kBucketPer; // digis a block sorts at a time
+constexpr uint32_t kBucketStep = kBucketThreads * kBucketPer; // digis a block sorts
 
 // Lines of the small launches (bucket_fits, finish_fits).
-constexpr uint64_t kSmallDigis = 1u << 21;   // digis of the launch
-constexpr uint32_t kBucketModules = 2048;    // modules (four counters each in shared memory)
-constexpr uint64_t kBucketDigis = kBucketCluster * kBucketStep; // mean digis of an event (a step a block)
+constexpr uint64_t kSmallDigis = 1u << 21;   // digis of a launch that finish_kernel ends
+constexpr uint64_t kBucketTotal = 1u << 20;  // digis of a launch that bucket_kernel starts
+constexpr uint32_t kBucketModules = 2048;    // modules (three words each in shared memory)
+// largest event: a step a block, wherever the event starts (its groups of
+// kPerThread digis are up to two more than its digis fill)
+constexpr uint64_t kBucketDigis = kBucketCluster * (kBucketStep - kPerThread);
+static_assert(kBucketDigis / kPerThread + 2 <= kBucketCluster * (kBucketStep / kPerThread), "a step a block");
 constexpr uint32_t kFinishItems = 16384;     // (event, module) items every block scans
 
 __host__ __device__ constexpr uint32_t bucket_keys(uint32_t M) { return (M + 3) & ~3u; }
 __host__ __device__ constexpr size_t bucket_smem(uint32_t M)
 {
-    return (size_t)kBucketStep * (8 + 2) + (size_t)bucket_keys(M) * 4 * 4;
+    return (size_t)kBucketStep * (8 + 2) + (size_t)bucket_keys(M) * 3 * 4;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -912,9 +918,8 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
     uint2 *stage = reinterpret_cast<uint2 *>(sh);                       // [kBucketStep] sorted by module
     uint16_t *skey = reinterpret_cast<uint16_t *>(stage + kBucketStep); // [kBucketStep]
     uint32_t *hist = reinterpret_cast<uint32_t *>(skey + kBucketStep);  // [MK] digis of the slice
-    uint32_t *cnt = hist + MK;                                          // [MK] of a step
-    uint32_t *lk = cnt + MK;                                            // [MK] their start in the stage
-    uint32_t *gb = lk + MK;                                             // [MK] next bucket position
+    uint32_t *lk = hist + MK;                                           // [MK] their start in the stage
+    uint32_t *gb = lk + MK;                                             // [MK] their first bucket position
     for (uint32_t k = tid; k < MK; k += kBucketThreads) hist[k] = 0;
     if (tid == 0) s_bad = 0;
     const uint64_t o0 = L.offsets[e], o1 = L.offsets[e + 1];
@@ -932,62 +937,50 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
     const uint64_t g0 = o0 / kPerThread, ng = (o1 + kPerThread - 1) / kPerThread - g0;
     const uint64_t a0 = (g0 + ng * rank / kBucketCluster) * kPerThread;
     const uint64_t c0 = max(o0, a0), c1 = min(o1, (g0 + ng * (rank + 1) / kBucketCluster) * kPerThread);
-    const bool one_step = c1 <= a0 + kBucketStep;
     // whether the second group of a thread's digis holds any: an event of at
     // most half a step a block does without it (30,000 digis: 30.9 -> 25.4 us)
     const bool both = c1 > a0 + kBucketStep / 2;
-    // a thread's digis of the step at s0: group h at s0 + (h * threads + tid) * kPerThread;
-    // km: module, and (from the count of its step on) rank << 16; 0xFFFF: none
+    // a thread's digis: group h at a0 + (h * threads + tid) * kPerThread;
+    // km: module, then (counted) module | rank << 16; 0xFFFF: none
     uint32_t km[kBucketPer], w[kBucketPer];
-    auto first = [&](uint64_t s0, int h) { return s0 + ((uint64_t)h * kBucketThreads + tid) * kPerThread; };
-    auto load_step = [&](uint64_t s0, bool words) {
+    auto first = [&](int h) { return a0 + ((uint64_t)h * kBucketThreads + tid) * kPerThread; };
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint64_t k0 = first(s0, h);
-            uint32_t m8[kPerThread] = {}, w8[kPerThread] = {};
-            if (h == 0 || both) {
-                load_modules(L, k0, c1, m8);
-                if (words) load_words(L, k0, c1, w8);
-            }
-#pragma unroll
-            for (int j = 0; j < kPerThread; ++j) {
-                const bool in = k0 + j >= c0 && k0 + j < c1;
-                km[h * kPerThread + j] = in ? m8[j] : 0xFFFFFFFFu;
-                if (words) w[h * kPerThread + j] = w8[j];
-            }
+    for (int h = 0; h < 2; ++h) {
+        const uint64_t k0 = first(h);
+        uint32_t m8[kPerThread] = {}, w8[kPerThread] = {};
+        if (h == 0 || both) {
+            load_modules(L, k0, c1, m8);
+            load_words(L, k0, c1, w8);
         }
-    };
-    bool bad = false;
-    auto count_step = [&](uint32_t *counts) { // (no branches: the latencies overlap; 60,000 digis: 32.9 -> 30.9 us)
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (h && !both) {
-#pragma unroll
-                for (int j = 0; j < kPerThread; ++j) km[kPerThread + j] = 0xFFFFu;
-                continue;
-            }
-            uint32_t r[kPerThread];
-#pragma unroll
-            for (int j = 0; j < kPerThread; ++j) {
-                const uint32_t k = km[h * kPerThread + j];
-                r[j] = atomicAdd(k < M ? counts + k : s_none + (tid & 31), 1u);
-            }
-#pragma unroll
-            for (int j = 0; j < kPerThread; ++j) {
-                uint32_t &k = km[h * kPerThread + j];
-                bad |= k >= M && k != 0xFFFFFFFFu;
-                k = k < M ? k | (r[j] << 16) : 0xFFFFu;
-            }
+        for (int j = 0; j < kPerThread; ++j) {
+            const bool in = k0 + j >= c0 && k0 + j < c1;
+            km[h * kPerThread + j] = in ? m8[j] : 0xFFFFFFFFu;
+            w[h * kPerThread + j] = w8[j];
         }
-    };
-    load_step(a0, true);
-    __syncthreads();
-    count_step(hist); // (with a slice of one step these are its ranks)
-    for (uint64_t s0 = a0 + kBucketStep; s0 < c1; s0 += kBucketStep) {
-        load_step(s0, false);
-        count_step(hist);
     }
-    if (!one_step) load_step(a0, false);
+    __syncthreads();
+    bool bad = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) { // (no branches: the latencies overlap; 60,000 digis: 32.9 -> 30.9 us)
+        if (h && !both) {
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j) km[kPerThread + j] = 0xFFFFu;
+            continue;
+        }
+        uint32_t r[kPerThread];
+#pragma unroll
+        for (int j = 0; j < kPerThread; ++j) {
+            const uint32_t k = km[h * kPerThread + j];
+            r[j] = atomicAdd(k < M ? hist + k : s_none + (tid & 31), 1u);
+        }
+#pragma unroll
+        for (int j = 0; j < kPerThread; ++j) {
+            uint32_t &k = km[h * kPerThread + j];
+            bad |= k >= M && k != 0xFFFFFFFFu;
+            k = k < M ? k | (r[j] << 16) : 0xFFFFu;
+        }
+    }
     if (bad) s_bad = 1;
     cluster_arrive();
     cluster_wait();
@@ -1033,40 +1026,19 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
             }
         }
     }
-    for (uint64_t s0 = a0; s0 < c1; s0 += kBucketStep) {
-        __syncthreads();
-        if (!one_step) { // this step's counts, ranks and starts
-            for (uint32_t k = tid; k < MK; k += kBucketThreads) cnt[k] = 0;
-            __syncthreads();
-            count_step(cnt);
-            __syncthreads();
-            const uint32_t k = 4 * tid;
-            const uint4 c = k < MK ? *reinterpret_cast<const uint4 *>(cnt + k) : make_uint4(0, 0, 0, 0);
-            const uint32_t mine = block_exclusive_scan<kBucketThreads>(c.x + c.y + c.z + c.w, tmp[0], &total);
-            if (k < MK)
-                *reinterpret_cast<uint4 *>(lk + k) = make_uint4(mine, mine + c.x, mine + c.x + c.y, mine + c.x + c.y + c.z);
-            __syncthreads();
-        }
+    __syncthreads();
 #pragma unroll
-        for (int j = 0; j < kBucketPer; ++j) {
-            const uint32_t key = km[j] & 0xFFFFu;
-            if (key == 0xFFFFu) continue;
-            const uint32_t p = lk[key] + (km[j] >> 16);
-            const uint64_t at = first(s0, j / kPerThread) + j % kPerThread;
-            stage[p] = make_uint2(w[j], (uint32_t)(at - o0));
-            skey[p] = (uint16_t)key;
-        }
-        __syncthreads();
-        // (the next step's digis load while this one is written out)
-        if (s0 + kBucketStep < c1) load_step(s0 + kBucketStep, true);
-        for (uint32_t p = tid; p < total; p += kBucketThreads) {
-            const uint32_t key = skey[p], g = gb[key] + (p - lk[key]);
-            L.ws.bucket[g] = stage[p];
-        }
-        if (!one_step) {
-            __syncthreads();
-            for (uint32_t k = tid; k < M; k += kBucketThreads) gb[k] += cnt[k];
-        }
+    for (int j = 0; j < kBucketPer; ++j) {
+        const uint32_t key = km[j] & 0xFFFFu;
+        if (key == 0xFFFFu) continue;
+        const uint32_t p = lk[key] + (km[j] >> 16);
+        stage[p] = make_uint2(w[j], (uint32_t)(first(j / kPerThread) + j % kPerThread - o0));
+        skey[p] = (uint16_t)key;
+    }
+    __syncthreads();
+    for (uint32_t p = tid; p < total; p += kBucketThreads) {
+        const uint32_t key = skey[p];
+        L.ws.bucket[gb[key] + (p - lk[key])] = stage[p];
     }
     cluster_wait(); // the others have read this block's counts
 }
@@ -3499,12 +3471,17 @@ cudaError_t launch_dependent(K kern, unsigned grid, unsigned block, size_t smem,
 // cluster an event) and its clusters ordered by finish_kernel, instead of by
 // three kernels and two: small launches, whose time is that of the kernel
 // boundaries (one event of 1,300 digis 36 -> 23 us, of 60,000 on 1,856 modules
-// 49 -> 31 us).  Events past a step a block are counted twice, by eight blocks
-// only, and the three kernels' grid is faster (200,000 digis: 51 us against
-// 43); past kSmallDigis the boundaries no longer count.
+// 49 -> 31 us).  The largest event decides, for an event is bucketed by eight
+// blocks however many digis it has: in steps of 16,384 a block it lost against
+// the three kernels from the second step on (events of 400,000 and three times
+// 30,000 digis: 84 us against 55; of 1.9M and fifteen times 2,000: 754 against
+// 620).  Where the offsets are the device's the launch's digis bound it.
+// Launches past kBucketTotal digis gain nothing from it (8 events of 130,000:
+// 50 us against 56; 16, which take two rounds of clusters: 85 against 81).
 static bool bucket_fits(const Launch &L)
 {
-    return L.N > 0 && L.N <= kSmallDigis && L.g.M <= kBucketModules && L.N / L.E <= kBucketDigis &&
+    return L.N > 0 && L.N <= kBucketTotal && L.g.M <= kBucketModules &&
+           (L.max_event ? L.max_event : L.N) <= kBucketDigis &&
            (uint64_t)L.E * kBucketCluster <= (uint64_t)L.sm_count;
 }
 static bool finish_fits(const Launch &L)

@@ -269,11 +269,13 @@ hp_status enqueue_impl(hp_ctx *ctx, uint32_t E, const uint64_t *offsets, uint64_
     if (!ctx || !out) return HP_EINVAL;
     if (ctx->failed.load()) return HP_ECUDA;
     if (E < 1) return HP_EINVAL;
-    uint64_t N = n_single;
+    uint64_t N = n_single, max_event = n_single;
     if (offsets) {
         if (offsets[0] != 0) return HP_EINVAL;
-        for (uint32_t e = 0; e < E; ++e)
+        for (uint32_t e = 0; e < E; ++e) {
             if (offsets[e + 1] < offsets[e]) return HP_EINVAL;
+            max_event = std::max<uint64_t>(max_event, offsets[e + 1] - offsets[e]);
+        }
         N = offsets[E];
     }
     if (N >= 0xFFFFFFFFull) return HP_EINVAL;
@@ -445,6 +447,7 @@ hp_status enqueue_impl(hp_ctx *ctx, uint32_t E, const uint64_t *offsets, uint64_
     L.g = geometry(ctx);
     L.E = E;
     L.N = N;
+    L.max_event = max_event;
     L.offsets = reinterpret_cast<const uint64_t *>(db + d_offs);
     L.words = dev_input ? static_cast<const uint32_t *>(words) : reinterpret_cast<const uint32_t *>(db + d_words);
     L.modules = dev_input ? static_cast<const uint16_t *>(mods) : reinterpret_cast<const uint16_t *>(db + d_mods);
