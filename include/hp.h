@@ -605,9 +605,11 @@ hp_status hp_get_stats(hp_ctx *ctx, hp_stats *out);
  * kernels on the launching stream (asynchronous, no host wait); n = 0 stops
  * and clears.  hp_profile_read waits for the recorded events (a blocking
  * call: use it outside event processing) and returns, per kernel name, the
- * number of timed launches and their summed device time in milliseconds.
- * names[i] are static strings.  *n_kernels receives the number of kernels
- * (at most cap are written).
+ * number of timed launches of that kernel and their summed device time in
+ * milliseconds (0 and 0 for kernels that did not run: a launch runs six of
+ * them at most, three if it is small).  names[i] are static strings.
+ * *n_kernels receives the number of kernels the library has (at most cap are
+ * written).
  */
 /*
  * Serving trace (tracing of the loop of hp_serve_start).  After

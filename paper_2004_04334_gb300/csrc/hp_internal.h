@@ -341,13 +341,23 @@ size_t carve_workspace(void *base, uint32_t E, uint32_t M, uint64_t N, uint32_t 
 // kMaxTileSlots for one block, kSmemSlots otherwise); max_tile[0] unused.
 // hash_tile[b] receives the same for the kernel's hash-store instance.
 cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4], uint32_t hash_tile[4]);
-// Kernels of one launch, in order; marks[i] (if given) is recorded before
-// kernel i and marks[kNumKernels] after the last one.
-constexpr int kNumKernels = 6;
+// The stages of one launch, in order, and the kernels that can run in them.
+// Stage timers: ev[i] is recorded before stage i and ev[kNumStages] after the
+// last one; kernel[i] is the kernel that ran in stage i (an index of
+// kKernelNames), kNoKernel where none did (small launches fuse stages).
+constexpr int kNumStages = 6;
+enum Kernel : uint8_t {
+    kHist, kScan, kScatter, kCluster, kOffsets, kCopy, kBucket, kScatterWide, kClusterHash, kFinish, kNumKernels,
+    kNoKernel = 0xFF
+};
 extern const char *const kKernelNames[kNumKernels];
+struct StageMarks {
+    cudaEvent_t ev[kNumStages + 1];
+    uint8_t kernel[kNumStages];
+};
 // Queue the whole reconstruction of one launch on `stream` (memset + kernels).
 cudaError_t launch_reconstruct(const Launch &L, cudaStream_t stream, uint64_t *kernel_count,
-                               cudaEvent_t *marks = nullptr);
+                               StageMarks *marks = nullptr);
 
 // One request of a serving batch: its inputs in (mapped) pinned host memory
 // and where they go in the batch's device arrays.

@@ -3409,8 +3409,9 @@ cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4
     return err;
 }
 
-const char *const kKernelNames[kNumKernels] = {"hist_kernel", "scan_kernel",    "scatter_kernel",
-                                                "cc_kernel",   "offsets_kernel", "copy_kernel"};
+const char *const kKernelNames[kNumKernels] = {"hist_kernel",   "scan_kernel",         "scatter_kernel", "cc_kernel",
+                                                "offsets_kernel", "copy_kernel",         "bucket_kernel",
+                                                "scatter_wide_kernel", "cc_hash_kernel", "finish_kernel"};
 
 // Sizes of a launch's clustering kernel: its tickets, and what a group's
 // slice of the shared memory (and the whole of it) holds.
@@ -3505,7 +3506,7 @@ static cudaError_t launch_bucket(const Launch &L, cudaStream_t stream)
     return cudaLaunchKernelEx(&cfg, bucket_kernel, L);
 }
 
-cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *kernel_count, cudaEvent_t *marks)
+cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *kernel_count, StageMarks *marks)
 {
     NvtxRange range("hp_launch_reconstruct");
     Launch L = in;
@@ -3518,40 +3519,45 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
         err = cudaMemsetAsync(L.ws.ctl, 0, (size_t)((unsigned char *)L.ws.count - (unsigned char *)L.ws.ctl), stream);
     if (err != cudaSuccess) return err;
     auto mark = [&](int i) {
-        if (marks && err == cudaSuccess) err = cudaEventRecord(marks[i], stream);
+        if (marks && err == cudaSuccess) err = cudaEventRecord(marks->ev[i], stream);
     };
     uint64_t nk = 0;
+    auto ran = [&](int stage, Kernel k) {
+        if (marks) marks->kernel[stage] = k;
+        ++nk;
+    };
     // persistent histogram and scatter over the same contiguous ranges
     const unsigned hist_grid = bucket_grid(L.N, L.sm_count), scat_grid = hist_grid; // the same ranges
     mark(0);
-    if (fused) { // (counted as the scatter)
+    if (fused) {
         mark(1);
         mark(2);
         if (err == cudaSuccess) err = launch_bucket(L, stream);
-        ++nk;
+        ran(2, kBucket);
     }
     if (!fused && L.N > 0) {
         hist_kernel<<<hist_grid, kHistThreads, kHistCap * sizeof(uint32_t), stream>>>(L);
-        ++nk;
+        ran(0, kHist);
     }
     if (!fused) {
         mark(1);
         if (err == cudaSuccess) err = launch_dependent(scan_kernel, L.E, 256, 0, stream, L);
-        ++nk;
+        ran(1, kScan);
         mark(2);
     }
     if (!fused && L.N > 0) {
+        const uint64_t steps = (L.N + kWideStep - 1) / kWideStep;
+        // (the wide scatter wants a step a block, and steps over few events:
+        // below, scatter_kernel's more and smaller blocks are faster)
+        const bool wide = L.g.M > kSubKeys && steps >= (uint64_t)L.sm_count && L.N / L.E >= kWideStep;
         if (err == cudaSuccess) {
-            const uint64_t steps = (L.N + kWideStep - 1) / kWideStep;
-            // (the wide scatter wants a step a block, and steps over few events:
-            // below, scatter_kernel's more and smaller blocks are faster)
-            if (L.g.M > kSubKeys && steps >= (uint64_t)L.sm_count && L.N / L.E >= kWideStep)
+            if (wide)
                 err = launch_dependent(scatter_wide_kernel, (unsigned)std::min<uint64_t>(steps, L.sm_count),
                                        kWideThreads, kWideSmem, stream, L);
             else
                 err = launch_dependent(scatter_kernel, scat_grid, kHistThreads, kScatterSmem, stream, L);
         }
-        ++nk;
+        ran(2, wide ? kScatterWide : kScatter);
     }
     mark(3);
     if (err == cudaSuccess) {
@@ -3572,14 +3578,14 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
             err = launch_dependent(cc_kernel<kRunThreads1, kRunGroups1, 1>, L.cc_grid, kRunThreads1,
                                    L.cc.smem, stream, L);
     }
-    ++nk;
+    ran(3, L.tune.label_store == kStoreHash ? kClusterHash : kCluster);
     mark(4);
     const uint64_t EM = (uint64_t)L.E * L.g.M;
     if (!finish) {
         if (err == cudaSuccess)
             err = launch_dependent(offsets_kernel, (unsigned)((EM + kOffItems - 1) / kOffItems), kOffThreads, 0, stream,
                                    L);
-        ++nk;
+        ran(4, kOffsets);
     }
     mark(5);
     if (finish) { // a thread per expected cluster (one in eight digis; at most the copy's threads, looping)
@@ -3595,7 +3601,7 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
             std::max<uint64_t>(1, std::max<uint64_t>(by_events, std::min<uint64_t>(by_items, (uint64_t)L.copy_grid)));
         if (err == cudaSuccess) err = launch_dependent(copy_kernel, (unsigned)blocks, kCopyThreads, 0, stream, L);
     }
-    ++nk;
+    ran(5, finish ? kFinish : kCopy);
     mark(6);
     if (kernel_count) *kernel_count += nk;
     if (err != cudaSuccess) return err;

@@ -242,12 +242,13 @@ int copy_grid(const hp_ctx *ctx, bool host_outputs)
 }
 
 // Timing marks for the next launch, or null when stage timers are off.
-cudaEvent_t *profile_marks(hp_ctx *ctx)
+hp::StageMarks *profile_marks(hp_ctx *ctx)
 {
     std::lock_guard<std::mutex> g(ctx->prof_mu);
     if (ctx->prof_left == 0) return nullptr;
-    hp_ctx::ProfRec rec;
-    for (int i = 0; i <= hp::kNumKernels; ++i) {
+    hp::StageMarks rec;
+    std::fill(std::begin(rec.kernel), std::end(rec.kernel), (uint8_t)hp::kNoKernel);
+    for (int i = 0; i <= hp::kNumStages; ++i) {
         if (!ctx->prof_pool.empty()) {
             rec.ev[i] = ctx->prof_pool.back();
             ctx->prof_pool.pop_back();
@@ -259,7 +260,7 @@ cudaEvent_t *profile_marks(hp_ctx *ctx)
     }
     --ctx->prof_left;
     ctx->prof_used.push_back(rec);
-    return ctx->prof_used.back().ev;
+    return &ctx->prof_used.back();
 }
 
 hp_status enqueue_impl(hp_ctx *ctx, uint32_t E, const uint64_t *offsets, uint64_t n_single, const uint32_t *words,
@@ -648,7 +649,7 @@ hp_status check_device_args(hp_ctx *ctx, uint32_t n_events, uint64_t n_digis, co
 // Queue one device-resident pass with its scratch at `base`.
 cudaError_t device_pass(hp_ctx *ctx, uint32_t n_events, uint64_t n_digis, const uint64_t *d_offsets,
                         const uint32_t *d_words, const uint16_t *d_module_ids, const hp_device_clusters *out,
-                        const Shape &sh, void *base, cudaStream_t s, uint64_t *nk, cudaEvent_t *marks,
+                        const Shape &sh, void *base, cudaStream_t s, uint64_t *nk, hp::StageMarks *marks,
                         uint32_t debug)
 {
     hp::Launch L;
@@ -1395,12 +1396,14 @@ hp_status hp_profile_read(hp_ctx *ctx, uint32_t cap, const char **names, double 
     uint64_t cnt[hp::kNumKernels] = {0};
     std::lock_guard<std::mutex> g(ctx->prof_mu);
     for (auto &r : ctx->prof_used) {
-        if (cudaEventSynchronize(r.ev[hp::kNumKernels]) != cudaSuccess) return fail(ctx);
-        for (int i = 0; i < hp::kNumKernels; ++i) {
+        if (cudaEventSynchronize(r.ev[hp::kNumStages]) != cudaSuccess) return fail(ctx);
+        for (int i = 0; i < hp::kNumStages; ++i) {
+            const uint8_t k = r.kernel[i];
+            if (k == hp::kNoKernel) continue;
             float t = 0.f;
             if (cudaEventElapsedTime(&t, r.ev[i], r.ev[i + 1]) != cudaSuccess) return fail(ctx);
-            ms[i] += t;
-            cnt[i] += 1;
+            ms[k] += t;
+            cnt[k] += 1;
         }
     }
     *n_kernels = hp::kNumKernels;

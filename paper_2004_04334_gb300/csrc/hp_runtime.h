@@ -243,12 +243,9 @@ struct hp_ctx {
     std::mutex ws_mu;
     std::map<cudaStream_t, Block> stream_ws;
     // stage timers (hp_profile_enable / hp_profile_read)
-    struct ProfRec {
-        cudaEvent_t ev[hp::kNumKernels + 1];
-    };
     std::mutex prof_mu;
     uint32_t prof_left = 0;
-    std::vector<ProfRec> prof_used;
+    std::deque<hp::StageMarks> prof_used; // (a launch writes to its own, which stays where it is)
     std::vector<cudaEvent_t> prof_pool;
     // serving loop (hp_serve_start / hp_submit / hp_serve_stop)
     std::mutex serve_mu;
@@ -375,7 +372,7 @@ hp::Geometry geometry(const hp_ctx *ctx);
 bool pinned_host(const void *p);
 const void *device_view(const hp_ctx *ctx, const void *p);
 int copy_grid(const hp_ctx *ctx, bool host_outputs);
-cudaEvent_t *profile_marks(hp_ctx *ctx);
+hp::StageMarks *profile_marks(hp_ctx *ctx);
 hp_status cpu_create(hp_ctx *ctx, const hp_config *cfg);
 void cpu_destroy(hp_ctx *ctx);
 hp_status cpu_enqueue(hp_ctx *ctx, uint32_t E, const uint64_t *offsets, uint64_t N, const uint32_t *words,
@@ -384,7 +381,7 @@ hp_status check_device_args(hp_ctx *ctx, uint32_t n_events, uint64_t n_digis, co
                             const uint32_t *d_words, const uint16_t *d_module_ids, const hp_device_clusters *out);
 cudaError_t device_pass(hp_ctx *ctx, uint32_t n_events, uint64_t n_digis, const uint64_t *d_offsets,
                         const uint32_t *d_words, const uint16_t *d_module_ids, const hp_device_clusters *out,
-                        const Shape &sh, void *base, cudaStream_t s, uint64_t *nk, cudaEvent_t *marks,
+                        const Shape &sh, void *base, cudaStream_t s, uint64_t *nk, hp::StageMarks *marks,
                         uint32_t debug = 0);
 
 // hp_tuning.cpp
