@@ -193,7 +193,8 @@ struct ClusterPlan {
     uint32_t runs, whole_runs;             // run records in a group's slice, and in the whole block's
     uint32_t exact_slots;                  // 64-bit moment slots of a block
     uint32_t pack_digis, pack_item;        // packed tier: digis of a pack, and of its largest item
-    uint32_t large_digis;                  // items of more digis are clustered by a whole block
+    uint32_t large_digis;                  // items of more digis are clustered by a whole block,
+    uint32_t own;                          // and every block clusters its own (an item a block), not those of a list
 };
 
 struct Launch {

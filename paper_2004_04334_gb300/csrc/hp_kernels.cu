@@ -2811,8 +2811,9 @@ __device__ __forceinline__ void pack_ticket(const Launch &L, uint32_t mem, unsig
 // the others through the run tier one by one.  (A module's bitmap costs its
 // clearing and scan whatever it holds, a pack's list of touched words costs
 // each digi: the line is pack_max.)  Items of more than
-// cc.large_digis digis (scan_kernel lists them), whose runs would not fit a
-// slice, come first: the whole block takes them one at a time, on all of its
+// cc.large_digis digis (scan_kernel lists them; with cc.own a block looks at
+// its own item), whose runs would not fit a slice or which are few, come first:
+// the whole block takes them one at a time, on all of its
 // shared memory, held in registers up to kRunDigis a thread (items of 4,500
 // digis: 24.9 -> 22.2 us a million digis, of 8,000: 20.7 -> 19.3; four items
 // of 2,500 at once: 17.2, which is why the groups have the rest).
@@ -2846,10 +2847,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
             GroupShared &gs = s_gs[0];
             for (;;) {
                 if (tid == 0) {
-                    const uint32_t t = atomicAdd(&L.ws.ctl[7], 1u);
+                    uint32_t t, item = blockIdx.x;
+                    if (L.cc.own) {
+                        t = item < L.cc.items && L.ws.count[item] > L.cc.large_digis ? 0u : nlarge;
+                    } else {
+                        t = atomicAdd(&L.ws.ctl[7], 1u);
+                        if (t < nlarge) item = L.ws.large[t];
+                    }
                     gs.ticket = t;
                     if (t < nlarge) {
-                        const uint32_t item = L.ws.large[t];
                         gs.pack_end = item;
                         gs.n[0] = L.ws.count[item];
                         gs.b[0] = L.ws.boff[item];
@@ -2867,6 +2873,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
                         : run_item<kThreads, true, kWide, false>(L, it, smem_addr(dsm), L.cc.whole_runs, exact, 0, 1,
                                                                  gs, wlist, tid, 0);
                 if (tid == 0) kcount[item] = K;
+                if (L.cc.own) break;
                 __syncthreads();
             }
         }
@@ -3443,11 +3450,16 @@ static ClusterPlan cluster_plan(const Launch &L)
                             (uint32_t)kPackPer * sh.threads / groups);
     p.pack_item = std::min(hash ? L.tune.warp_max : pack_max(L.tune.warp_max), p.pack_digis);
     p.large_digis = std::min(large_digis(R, C, T, sh), groups > 1 ? kNarrowDigis : 0xFFFFFFFFu);
-    // with no more items than blocks a group's neighbours are idle: items past
-    // what a group holds in registers take the whole block (64 items of 3,125
-    // digis: 61 -> 45 us; of 1,562, which it does hold: 41 us either way)
+    // With no more items than blocks a group's neighbours are idle, and larger
+    // items take the whole block: with an item a ticket each block its own (with
+    // a list, a block that clustered another's item came to its own item after
+    // it: 128 items of 1,900-2,100 digis 51 us, 48 with a whole block for every
+    // item, 37 so).  The line is five digis a thread of a group; 64 to 300 items,
+    // a group / the whole block: of 1,200 digis 31-36 us either way, of 1,600
+    // 34-41 / 32-36, of 1,800 38-47 / 33-37.  Else what a group holds in registers.
+    p.own = groups > 1 && p.ticket_items == 1 && p.items <= (uint32_t)L.cc_grid;
     if (groups > 1 && p.items <= (uint32_t)L.cc_grid)
-        p.large_digis = std::min(p.large_digis, (uint32_t)kRunDigis * sh.threads / groups);
+        p.large_digis = std::min(p.large_digis, (uint32_t)(p.own ? 5 : kRunDigis) * (sh.threads / groups));
     return p;
 }
 
