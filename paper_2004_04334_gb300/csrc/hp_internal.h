@@ -202,6 +202,7 @@ struct Launch {
     uint32_t E;
     uint64_t N;
     uint64_t max_event = 0;  // digis of the largest event, 0 where the host does not know
+    bool host_out = false;   // the cluster columns are mapped host memory
     const uint64_t *offsets; // device [E+1]
     const uint32_t *words;   // device [N]
     const uint16_t *modules; // device [N]

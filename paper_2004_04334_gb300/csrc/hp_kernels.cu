@@ -873,6 +873,7 @@ constexpr uint32_t kBucketStep = kBucketThreads * kBucketPer; // digis a block s
 
 // Lines of the small launches (bucket_fits, finish_fits).
 constexpr uint64_t kSmallDigis = 1u << 21;   // digis of a launch that finish_kernel ends
+constexpr uint64_t kSmallHost = 1u << 19;    // the same with outputs in host memory, bucket_kernel not before it
 constexpr uint64_t kBucketTotal = 1u << 20;  // digis of a launch that bucket_kernel starts
 constexpr uint32_t kBucketModules = 2048;    // modules (three words each in shared memory)
 // largest event: a step a block, wherever the event starts (its groups of
@@ -3497,9 +3498,16 @@ static bool bucket_fits(const Launch &L)
            (L.max_event ? L.max_event : L.N) <= kBucketDigis &&
            (uint64_t)L.E * kBucketCluster <= (uint64_t)L.sm_count;
 }
+// (With outputs in mapped host memory the copy keeps to 76 blocks of 1,216,
+// and finish_kernel's one position a thread then takes longer than
+// copy_kernel's four: latency of a host batch with the one / the other, 64
+// events of 30,000 digis 289 / 273 us, in the mean over 32 and 64 events of
+// 0.5 to 2M digis in all 3% more, below within 1%.  Where bucket_kernel starts
+// the launch the pair is ahead by 2% up to kBucketTotal.)
 static bool finish_fits(const Launch &L)
 {
-    return L.N <= kSmallDigis && L.cc.items <= kFinishItems && !L.debug;
+    const uint64_t most = !L.host_out ? kSmallDigis : bucket_fits(L) ? kBucketTotal : kSmallHost;
+    return L.N <= most && L.cc.items <= kFinishItems && !L.debug;
 }
 static cudaError_t launch_bucket(const Launch &L, cudaStream_t stream)
 {

@@ -449,6 +449,7 @@ hp_status enqueue_impl(hp_ctx *ctx, uint32_t E, const uint64_t *offsets, uint64_
     L.E = E;
     L.N = N;
     L.max_event = max_event;
+    L.host_out = !keep;
     L.offsets = reinterpret_cast<const uint64_t *>(db + d_offs);
     L.words = dev_input ? static_cast<const uint32_t *>(words) : reinterpret_cast<const uint32_t *>(db + d_words);
     L.modules = dev_input ? static_cast<const uint16_t *>(mods) : reinterpret_cast<const uint16_t *>(db + d_mods);

@@ -289,6 +289,7 @@ void launch_batch(hp_ctx *ctx, Serve *sv, std::vector<hp_event *> &take)
     L.g = geometry(ctx);
     L.E = E;
     L.N = N;
+    L.host_out = true;
     for (const hp_event *r : take) L.max_event = std::max<uint64_t>(L.max_event, r->N);
     L.offsets = reinterpret_cast<const uint64_t *>(db + l.d_offs);
     L.words = reinterpret_cast<const uint32_t *>(db + l.d_words);
