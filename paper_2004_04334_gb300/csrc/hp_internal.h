@@ -160,7 +160,8 @@ constexpr uint32_t kOutChunk = 128;
 struct Workspace {
     uint32_t *ctl;        // [16]: 0 item ticket, 1 launch error bits, 2 arena bump, 3 prefix frontier,
                           //       4 offsets chunk ticket, 5 large items and 7 their ticket,
-                          //       6 clusters of the launch (offsets_kernel)
+                          //       6 clusters of the launch (offsets_kernel),
+                          //       8-15 a bit per SM whose block came for large items (cc_kernel)
     uint32_t *event_err;  // [E]
     uint32_t *count;      // [E*M] digis of each item (reserved part, then the total: scan_kernel);
                           //       then each item's first output position (offsets_kernel)

@@ -93,6 +93,13 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
+__device__ __forceinline__ uint32_t sm_id()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%smid;" : "=r"(r));
+    return r;
+}
+
 __device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long long v)
 {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
@@ -2846,7 +2853,21 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
     if constexpr (!kWhole) {
         if (nlarge) {
             GroupShared &gs = s_gs[0];
-            for (;;) {
+            bool come = true;
+            // where several blocks share an SM and the list is short, only the
+            // first of each SM comes for it: two at work on one SM take 1.6 times
+            // as long (ten items of 13,000 digis 210 -> 130 us)
+            if constexpr (kMinBlocks > 1) {
+                if (!L.cc.own && nlarge <= (uint32_t)L.sm_count) {
+                    if (tid == 0) {
+                        const uint32_t sm = sm_id() & 255u, bit = 1u << (sm & 31u);
+                        gs.flag = atomicOr(&L.ws.ctl[8 + (sm >> 5)], bit) & bit;
+                    }
+                    __syncthreads();
+                    come = gs.flag == 0;
+                }
+            }
+            while (come) {
                 if (tid == 0) {
                     uint32_t t, item = blockIdx.x;
                     if (L.cc.own) {
