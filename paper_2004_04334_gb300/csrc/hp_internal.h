@@ -204,6 +204,7 @@ struct Launch {
     uint64_t N;
     uint64_t max_event = 0;  // digis of the largest event, 0 where the host does not know
     bool host_out = false;   // the cluster columns are mapped host memory
+    uint32_t bucket_parts = 0; // clusters of bucket_kernel where large events are split, else 0
     const uint64_t *offsets; // device [E+1]
     const uint32_t *words;   // device [N]
     const uint16_t *modules; // device [N]

@@ -868,11 +868,15 @@ __global__ void __launch_bounds__(kWideThreads, 1) scatter_wide_kernel(const __g
 // shared memory, four modules a load) and so knows, for every module, the
 // bucket's start and its own offset inside it; then it sorts its digis by
 // module in shared memory and writes each module's run with consecutive
-// threads.  A slice is at most kBucketStep digis, a step a block: no event of
-// the launch has more than kBucketDigis (bucket_fits).  With one event the
-// kernel also clears the launch's control words, so that nothing precedes it.
-// Bound by launch and global-memory latency: one launch in place of a memset
-// and three kernels.
+// threads.  A slice is at most kBucketStep digis, a step a block.  Where no
+// event has more than kBucketDigis (the host knows the largest) a cluster has
+// an event.  Else (L.bucket_parts) a larger event is split evenly among
+// several, and each counts the others' parts as well, before its own and after
+// it, so that no cluster waits for another (17 us where no event is split, 21
+// with two parts, 25 with four; one cluster in two and four steps took 30 and
+// 49).  With one event the kernel also clears the launch's control words, so
+// that nothing precedes it.  Bound by launch and global-memory latency: one
+// launch in place of a memset and three kernels.
 constexpr int kBucketThreads = 1024;
 constexpr int kBucketCluster = 8;                             // portable cluster size
 constexpr int kBucketPer = 2 * kPerThread;                    // digis a thread holds
@@ -881,8 +885,9 @@ constexpr uint32_t kBucketStep = kBucketThreads * kBucketPer; // digis a block s
 // Lines of the small launches (bucket_fits, finish_fits).
 constexpr uint64_t kSmallDigis = 1u << 21;   // digis of a launch that finish_kernel ends
 constexpr uint64_t kSmallHost = 1u << 19;    // the same with outputs in host memory, bucket_kernel not before it
-constexpr uint64_t kBucketTotal = 1u << 20;  // digis of a launch that bucket_kernel starts
-constexpr uint32_t kBucketModules = 2048;    // modules (three words each in shared memory)
+constexpr uint64_t kBucketTotal = 1u << 20;  // digis of a launch of more events that bucket_kernel starts
+constexpr uint32_t kBucketAtOnce = 15;       // its clusters that run at once (of 19: eight blocks of a GPC each)
+constexpr uint32_t kBucketModules = 2048;    // modules (three or five words each in shared memory)
 // largest event: a step a block, wherever the event starts (its groups of
 // kPerThread digis are up to two more than its digis fill)
 constexpr uint64_t kBucketDigis = kBucketCluster * (kBucketStep - kPerThread);
@@ -890,9 +895,9 @@ static_assert(kBucketDigis / kPerThread + 2 <= kBucketCluster * (kBucketStep / k
 constexpr uint32_t kFinishItems = 16384;     // (event, module) items every block scans
 
 __host__ __device__ constexpr uint32_t bucket_keys(uint32_t M) { return (M + 3) & ~3u; }
-__host__ __device__ constexpr size_t bucket_smem(uint32_t M)
+__host__ __device__ constexpr size_t bucket_smem(uint32_t M, bool parts)
 {
-    return (size_t)kBucketStep * (8 + 2) + (size_t)bucket_keys(M) * 3 * 4;
+    return (size_t)kBucketStep * (8 + 2) + (size_t)bucket_keys(M) * (parts ? 5 : 3) * 4;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -915,6 +920,7 @@ __device__ __forceinline__ uint4 lds_cluster4(uint32_t a, uint32_t r)
     return v;
 }
 
+template <bool kParts>
 __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_constant__ Launch L)
 {
     extern __shared__ __align__(16) uint32_t sh[];
@@ -922,13 +928,42 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
     __shared__ uint32_t s_bad, s_none[32];
     pdl_trigger();
     const uint32_t tid = threadIdx.x, M = L.g.M, MK = bucket_keys(M), rank = cluster_rank();
-    const uint32_t e = blockIdx.x / kBucketCluster;
+    uint32_t e = blockIdx.x / kBucketCluster, part = 0, parts = 1; // the cluster's event, and which part of it
+    if constexpr (kParts) {
+        __shared__ uint32_t s_place[3];
+        if (tid < 32) { // (at most 32 events; offsets that do not fit are found below, by the first event they spoil)
+            const uint64_t a = tid < L.E ? L.offsets[tid] : 0, b = tid < L.E ? L.offsets[tid + 1] : 0;
+            const bool fit = a < b && b <= L.N;
+            const uint32_t n = tid >= L.E ? 0u : fit ? (uint32_t)((b - a + kBucketDigis - 1) / kBucketDigis) : 1u;
+            uint32_t incl = n;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, incl, o);
+                if ((int)tid >= o) incl += y;
+            }
+            const uint32_t past = __ballot_sync(kFull, incl > e), at = past ? __ffs(past) - 1 : 0u;
+            const uint32_t first = __shfl_sync(kFull, incl - n, at), of = __shfl_sync(kFull, n, at);
+            if (tid == 0) {
+                s_place[0] = past ? at : ~0u;
+                s_place[1] = e - first;
+                s_place[2] = of;
+            }
+        }
+        __syncthreads();
+        if (s_place[0] == ~0u) return; // (the whole cluster: every event has its clusters already)
+        e = s_place[0];
+        part = s_place[1];
+        parts = s_place[2];
+    }
     uint2 *stage = reinterpret_cast<uint2 *>(sh);                       // [kBucketStep] sorted by module
     uint16_t *skey = reinterpret_cast<uint16_t *>(stage + kBucketStep); // [kBucketStep]
     uint32_t *hist = reinterpret_cast<uint32_t *>(skey + kBucketStep);  // [MK] digis of the slice
     uint32_t *lk = hist + MK;                                           // [MK] their start in the stage
     uint32_t *gb = lk + MK;                                             // [MK] their first bucket position
+    uint32_t *rest = gb + MK; // [2 * MK] (with parts) digis of the parts before this one, and of those after
     for (uint32_t k = tid; k < MK; k += kBucketThreads) hist[k] = 0;
+    if (kParts && parts > 1)
+        for (uint32_t k = tid; k < 2 * MK; k += kBucketThreads) rest[k] = 0;
     if (tid == 0) s_bad = 0;
     const uint64_t o0 = L.offsets[e], o1 = L.offsets[e + 1];
     const bool bad_offsets = o0 > o1 || o1 > L.N || (e == 0 && o0 != 0) || (e == L.E - 1 && o1 != L.N);
@@ -943,8 +978,10 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
     // the slice [c0, c1), cut at multiples of kPerThread digis of the launch
     // (so that every thread's groups of digis are 16-byte aligned)
     const uint64_t g0 = o0 / kPerThread, ng = (o1 + kPerThread - 1) / kPerThread - g0;
-    const uint64_t a0 = (g0 + ng * rank / kBucketCluster) * kPerThread;
-    const uint64_t c0 = max(o0, a0), c1 = min(o1, (g0 + ng * (rank + 1) / kBucketCluster) * kPerThread);
+    const uint32_t slices = kParts ? parts * kBucketCluster : kBucketCluster;
+    auto cut = [&](uint32_t p) { return (g0 + ng * (p * kBucketCluster + rank) / slices) * kPerThread; };
+    auto end = [&](uint32_t p) { return (g0 + ng * (p * kBucketCluster + rank + 1) / slices) * kPerThread; };
+    const uint64_t a0 = cut(part), c0 = max(o0, a0), c1 = min(o1, end(part));
     // whether the second group of a thread's digis holds any: an event of at
     // most half a step a block does without it (30,000 digis: 30.9 -> 25.4 us)
     const bool both = c1 > a0 + kBucketStep / 2;
@@ -990,6 +1027,20 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
         }
     }
     if (bad) s_bad = 1;
+    for (uint32_t p = 0; kParts && p < parts; ++p) { // this block's slice of the event's other parts
+        if (p == part) continue;
+        const uint64_t b0 = cut(p), b1 = min(o1, end(p));
+        uint32_t *counts = p < part ? rest : rest + MK;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t k0 = b0 + ((uint64_t)h * kBucketThreads + tid) * kPerThread;
+            uint32_t m8[kPerThread];
+            load_modules(L, k0, b1, m8);
+#pragma unroll
+            for (int j = 0; j < kPerThread; ++j)
+                if (k0 + j >= o0 && k0 + j < b1 && m8[j] < M) atomicAdd(counts + m8[j], 1u);
+        }
+    }
     cluster_arrive();
     cluster_wait();
     if (tid == 0 && s_bad) atomicOr(&L.ws.event_err[e], kErrBadDigi);
@@ -1010,6 +1061,15 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
                 if (r < rank) before.x += v[r].x, before.y += v[r].y, before.z += v[r].z, before.w += v[r].w;
                 if (r == rank) own = v[r];
             }
+            if (kParts && parts > 1) {
+                const uint32_t ra = (uint32_t)__cvta_generic_to_shared(rest + k);
+#pragma unroll
+                for (uint32_t r = 0; r < kBucketCluster; ++r) {
+                    const uint4 b = lds_cluster4(ra, r), a = lds_cluster4(ra + 4 * MK, r);
+                    before.x += b.x, before.y += b.y, before.z += b.z, before.w += b.w;
+                    t.x += a.x + b.x, t.y += a.y + b.y, t.z += a.z + b.z, t.w += a.w + b.w;
+                }
+            }
         }
         cluster_arrive(); // the others' counts are read
         uint32_t unused;
@@ -1021,7 +1081,7 @@ __global__ void __launch_bounds__(kBucketThreads, 1) bucket_kernel(const __grid_
                 make_uint4(b.x + before.x, b.y + before.y, b.z + before.z, b.w + before.w);
             *reinterpret_cast<uint4 *>(lk + k) =
                 make_uint4(mine, mine + own.x, mine + own.x + own.y, mine + own.x + own.y + own.z);
-            if (rank == 0) {
+            if (rank == 0 && part == 0) {
                 const uint32_t bs[4] = {b.x, b.y, b.z, b.w}, ts[4] = {t.x, t.y, t.z, t.w};
 #pragma unroll
                 for (uint32_t i = 0; i < 4; ++i) {
@@ -3404,8 +3464,11 @@ cudaError_t init_kernels(int device, uint32_t R, uint32_t C, uint32_t max_tile[4
     if (err != cudaSuccess) return err;
     err = cudaFuncSetAttribute(scatter_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
     if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(bucket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)bucket_smem(kBucketModules));
+    err = cudaFuncSetAttribute(bucket_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)bucket_smem(kBucketModules, false));
+    if (err == cudaSuccess)
+        err = cudaFuncSetAttribute(bucket_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)bucket_smem(kBucketModules, true));
     if (err == cudaSuccess)
         err = cudaFuncSetAttribute(finish_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    (int)((kFinishItems + 1) * 4));
@@ -3502,22 +3565,32 @@ cudaError_t launch_dependent(K kern, unsigned grid, unsigned block, size_t smem,
     return cudaLaunchKernelEx(&cfg, kern, L);
 }
 
+// Clusters that bucket_kernel needs besides one an event, where any of the
+// events may hold most of the launch's digis.
+static uint64_t bucket_parts(const Launch &L)
+{
+    return L.max_event || L.N <= kBucketDigis ? 0 : L.N / kBucketDigis;
+}
+
 // Whether the launch's digis are bucketed by bucket_kernel (one launch, a
 // cluster an event) and its clusters ordered by finish_kernel, instead of by
 // three kernels and two: small launches, whose time is that of the kernel
 // boundaries (one event of 1,300 digis 36 -> 23 us, of 60,000 on 1,856 modules
 // 49 -> 31 us).  The largest event decides, for an event is bucketed by eight
-// blocks however many digis it has: in steps of 16,384 a block it lost against
-// the three kernels from the second step on (events of 400,000 and three times
-// 30,000 digis: 84 us against 55; of 1.9M and fifteen times 2,000: 754 against
-// 620).  Where the offsets are the device's the launch's digis bound it.
-// Launches past kBucketTotal digis gain nothing from it (8 events of 130,000:
-// 50 us against 56; 16, which take two rounds of clusters: 85 against 81).
+// blocks: in several steps it lost against the three kernels (events of 400,000
+// and three times 30,000 digis: 84 us against 55; of 1.9M and fifteen times
+// 2,000: 754 against 620).  Where the offsets are the device's, a launch of more
+// than kBucketDigis gets as many clusters as its events can have parts, which
+// costs even events 1 us and the others little or nothing (those of 400,000
+// and 30,000: 61 us; of 250,000 and 10,000: 44 against 46; 9 even events of 0.3
+// to 1M digis in all 13% less than with the three kernels).  8 events of
+// 130,000 digis: 50 us against 56; 16, which take two rounds of clusters, of
+// 60,000 2% less, of 130,000: 85 against 81.
 static bool bucket_fits(const Launch &L)
 {
-    return L.N > 0 && L.N <= kBucketTotal && L.g.M <= kBucketModules &&
-           (L.max_event ? L.max_event : L.N) <= kBucketDigis &&
-           (uint64_t)L.E * kBucketCluster <= (uint64_t)L.sm_count;
+    return L.N > 0 && L.N <= (L.E <= kBucketAtOnce ? kSmallDigis : kBucketTotal) && L.g.M <= kBucketModules &&
+           (L.max_event ? L.max_event <= kBucketDigis : L.N / L.E <= kBucketDigis && L.E <= 32) &&
+           (L.E + bucket_parts(L)) * kBucketCluster <= (uint64_t)L.sm_count;
 }
 // (With outputs in mapped host memory the copy keeps to 76 blocks of 1,216,
 // and finish_kernel's one position a thread then takes longer than
@@ -3533,9 +3606,9 @@ static bool finish_fits(const Launch &L)
 static cudaError_t launch_bucket(const Launch &L, cudaStream_t stream)
 {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(L.E * kBucketCluster);
+    cfg.gridDim = dim3((L.bucket_parts ? L.bucket_parts : L.E) * kBucketCluster);
     cfg.blockDim = dim3(kBucketThreads);
-    cfg.dynamicSmemBytes = bucket_smem(L.g.M);
+    cfg.dynamicSmemBytes = bucket_smem(L.g.M, L.bucket_parts != 0);
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -3544,7 +3617,7 @@ static cudaError_t launch_bucket(const Launch &L, cudaStream_t stream)
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, bucket_kernel, L);
+    return cudaLaunchKernelEx(&cfg, L.bucket_parts ? bucket_kernel<true> : bucket_kernel<false>, L);
 }
 
 cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *kernel_count, StageMarks *marks)
@@ -3553,6 +3626,7 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
     Launch L = in;
     L.cc = cluster_plan(L);
     const bool finish = finish_fits(L), fused = finish && bucket_fits(L); // (the order chain is cleared for neither)
+    L.bucket_parts = bucket_parts(L) ? L.E + (uint32_t)bucket_parts(L) : 0u;
     cudaError_t err = cudaSuccess;
     if (!fused)
         err = cudaMemsetAsync(L.ws.ctl, 0, L.ws.zero_bytes, stream);
