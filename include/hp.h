@@ -380,7 +380,8 @@ hp_status hp_reconstruct_device_noalloc(hp_ctx *ctx, uint32_t n_events, uint64_t
  * depend on the launch shape (how many (event, module) items, how many
  * digis per item):
  *   tile_slots     runs (horizontal stretches of surviving pixels) that a
- *                  block's shared memory holds: items with more are
+ *                  block's shared memory holds (of the largest tiles of
+ *                  small modules a few hundred fewer): items with more are
  *                  clustered in global scratch;
  *   blocks_per_sm  resident clustering blocks per SM, 1, 2 or 3: with 1 a
  *                  block is four groups of threads that cluster items of
@@ -438,9 +439,9 @@ hp_status hp_autotune(hp_ctx *ctx, uint32_t n_events, uint64_t n_digis, const ui
 
 /*
  * CUDA-graph form of the device-resident entry: hp_graph_capture records
- * one hp_reconstruct_device pass (a memset and six kernels; three kernels
- * for small launches) for fixed
- * arguments into an executable CUDA graph with its own scratch;
+ * one hp_reconstruct_device pass (a memset and six kernels; for small
+ * launches five, or three) for fixed arguments into an executable CUDA graph
+ * with its own scratch;
  * hp_graph_launch replays it on `stream` (one cudaGraphLaunch, no
  * allocation, no host work per launch).  The graph keeps the pointers and
  * sizes it was captured with: refill the same input buffers between

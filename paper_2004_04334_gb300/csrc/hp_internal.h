@@ -30,8 +30,8 @@ constexpr uint32_t kErrBadOffsets = 16u; // event offsets not 0 = o[0] <= o[1] <
 constexpr int kChunk = 4096;         // digis per histogram / scatter block
 constexpr int kHistThreads = 512;
 constexpr int kHistCap = 4096;       // (event, module) bins a block can histogram in shared memory
-constexpr int kCCThreads = 512;      // threads of a clustering block
-constexpr int kGroup = kCCThreads / 32; // most (event, module) items per work-queue ticket, one per warp
+constexpr int kCCThreads = 512;      // threads of a hash-store clustering block (the others: run_shape)
+constexpr int kGroup = 16;           // most (event, module) items per work-queue ticket
 constexpr int kWarpMax = 64;         // default of Tuning::warp_max
 constexpr int kSmemSlots = 4096;     // runs of an item a block clusters in shared memory (default tile)
 constexpr int kMaxTileSlots = 16384; // largest tile considered (one block per SM)
@@ -48,15 +48,16 @@ struct Tuning {
 };
 
 // Pixel lookup of the clustering items above the packed tier: module-sized
-// bitmaps (a group of threads an item), or an open-addressing hash table keyed by linear pixel index, sized by the item's digi count
-// (item_threads threads an item, several items of a block side by side).
+// bitmaps (a group of threads an item), or an open-addressing hash table keyed
+// by linear pixel index, sized by the item's digi count (item_threads threads
+// an item, several items of a block side by side).
 constexpr uint32_t kStoreBitmap = 0;
 constexpr uint32_t kStoreHash = 1;
 // Digi index bits of the hash store's packed keys (items of at most 4096 digis).
 constexpr uint32_t kHashIdxBits = 12;
 
-// Digis a clustering thread holds in registers in the register tier and
-// the hash store: fewer at three resident blocks per SM (40 registers).
+// Digis a thread of the hash store holds in registers: fewer at three resident
+// blocks per SM (40 registers).
 __host__ __device__ constexpr int cc_digis_per_thread(int blocks_per_sm) { return blocks_per_sm >= 3 ? 5 : 8; }
 
 // Largest item (digis) of the hash store: each of the block's
@@ -154,9 +155,12 @@ struct Outputs {
 // Output positions a copy_kernel warp writes per step (four a lane).
 constexpr uint32_t kOutChunk = 128;
 
-// Scratch of one launch.  The first `zero_bytes` bytes must be zero before
-// the first kernel (one memset): control words, per-event error bits,
-// per-item counts and the chained-scan state.
+// Scratch of one launch.  Before the first kernel hist_kernel the first
+// `zero_bytes` bytes are zeroed (one memset): control words, per-event error
+// bits, per-item counts and the chained-scan state.  Where bucket_kernel comes
+// first the control words and error bits alone are, by a memset up to `count`
+// or, for one event, by that kernel: it writes every count, and count2 and
+// chain, which nothing reads then, hold what an earlier launch left.
 struct Workspace {
     uint32_t *ctl;        // [16]: 0 item ticket, 1 launch error bits, 2 arena bump, 3 prefix frontier,
                           //       4 offsets chunk ticket, 5 large items and 7 their ticket,

@@ -706,8 +706,10 @@ __global__ void __launch_bounds__(kHistThreads, 2) scatter_kernel(const __grid_c
 // atomics (29.4M digis in 8 events: 281 -> 183 us; 171 us with the digis'
 // events looked up only in steps over several).  Bound by shared-memory
 // wavefronts (rank, placing and reading back each digi; half of their peak,
-// one block an SM) and by L2 writes.  A step over more keys than the tables
-// hold takes one atomic a digi, as scatter_kernel does.
+// one block an SM) and by L2 writes; a thread's 32 digi words and keys spill in
+// part (64 registers a thread: 180 bytes of stores, 156 of loads).  A step over
+// more keys than the tables hold takes one atomic a digi, as scatter_kernel
+// does.
 constexpr int kWideThreads = 1024;
 constexpr int kWidePer = 2 * kPerThread;                // digis a thread holds
 constexpr uint32_t kWideStep = kWideThreads * kWidePer; // digis a block sorts at a time
@@ -1287,7 +1289,7 @@ __device__ __forceinline__ uint32_t atoms_min(uint32_t a, uint32_t v)
 //
 // What bounds it: instruction issue and the latency of shared memory; an item
 // is a chain of ten barriers, so several groups a block work on items of
-// their own, every phase issues its loads four digis or two runs at a time,
+// their own, every phase issues its loads two digis or two runs at a time,
 // and the frequent conditions are predicates, not branches.  Runs, not
 // pixels, are the nodes because there are 0.6 of them a digi in blob-like
 // data (0.5 to 0.8): against a node and four atomics a pixel (the tier this
@@ -1493,10 +1495,10 @@ __device__ __forceinline__ uint32_t run_contacts(const RunView &v, uint32_t W, u
     return len;
 }
 
-// The item's digis, four at a time so that their loads overlap:
-// f(k, j, x) for the thread's digis j .. j + 3 with words x[kBatch] (kNoDigi for
-// those past the last), held in w[k] .. w[k + 3] with kSingle (all of them
-// loaded by load_digis), else loaded here.
+// The item's digis, kBatch at a time so that their loads overlap: f(k, j, x)
+// for the thread's digis from j on with words x[kBatch] (kNoDigi for those past
+// the last), held in w from w[k] on with kSingle (all of them loaded by
+// load_digis), else loaded here.
 constexpr int kBatch = 2; // (4: more slots past a thread's last digi; 27.7M digis 530 us, 2: 519, 1: 526)
 constexpr uint32_t kNoDigi = 0xFFFFFFFFu; // an invalid word (row 255, column 511)
 template <int GT>
@@ -2342,7 +2344,7 @@ __device__ __forceinline__ void pack_items(const Launch &L, uint32_t mem, unsign
 __device__ __forceinline__ uint32_t hash_home(uint32_t key, uint32_t H) { return __umulhi(key * 0x9E3779B1u, H); }
 
 // Find on packed keys with path halving (the index of a key is its low
-// bits); parents only ever decrease, as in uf_find_halving.
+// bits); parents only ever decrease, as in run_find.
 template <uint32_t kIdx>
 __device__ __forceinline__ uint32_t key_find(uint32_t *par, uint32_t x)
 {
@@ -2359,7 +2361,7 @@ __device__ __forceinline__ uint32_t key_find(uint32_t *par, uint32_t x)
 
 // Lock-free union of the trees of packed keys a and b (the root with the
 // larger key is linked under the smaller with atomicMin; a lost race retries
-// from the new parent), as uf_union on slots.
+// from the new parent), as run_union on runs.
 template <uint32_t kIdx>
 __device__ __forceinline__ void key_union(uint32_t *par, uint32_t a, uint32_t b)
 {
@@ -2884,7 +2886,9 @@ __device__ __forceinline__ void pack_ticket(const Launch &L, uint32_t mem, unsig
 // the whole block takes them one at a time, on all of its
 // shared memory, held in registers up to kRunDigis a thread (items of 4,500
 // digis: 24.9 -> 22.2 us a million digis, of 8,000: 20.7 -> 19.3; four items
-// of 2,500 at once: 17.2, which is why the groups have the rest).
+// of 2,500 at once: 17.2, which is why the groups have the rest).  64 registers
+// a thread, which 1,024 threads an SM leave, spill a little outside the inner
+// loops (80 to 90 bytes of stores and 52 of loads a thread).
 template <int kThreads, int kGroups, int kMinBlocks>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_constant__ Launch L)
 {
@@ -2896,7 +2900,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) cc_kernel(const __grid_c
     const uint32_t tid = threadIdx.x, gid = tid / GT, gt = tid - gid * GT, bar = 1 + gid;
     // the group's first ticket: its records before the previous kernel is done
     // (the launch's first kernel is an ordinary launch, so that the call's
-    // inputs are in place when this one starts; 760 -> 751 us for 256 events)
+    // inputs are in place when this one starts)
     const uint32_t ticket0 = gid * gridDim.x + blockIdx.x;
     TicketLane lane_of;
     if (gt < 32 && ticket0 < L.cc.tickets) load_record(L, ticket0, gt, &lane_of);
@@ -3625,7 +3629,7 @@ cudaError_t launch_reconstruct(const Launch &in, cudaStream_t stream, uint64_t *
     NvtxRange range("hp_launch_reconstruct");
     Launch L = in;
     L.cc = cluster_plan(L);
-    const bool finish = finish_fits(L), fused = finish && bucket_fits(L); // (the order chain is cleared for neither)
+    const bool finish = finish_fits(L), fused = finish && bucket_fits(L);
     L.bucket_parts = bucket_parts(L) ? L.E + (uint32_t)bucket_parts(L) : 0u;
     cudaError_t err = cudaSuccess;
     if (!fused)

@@ -1,5 +1,5 @@
 // Autotuner of libhp's clustering kernel: launch settings (shared-memory
-// tile, resident blocks, items per ticket, warp-tier limit, bitmap or hash
+// tile, resident blocks, items per ticket, warp_max, bitmap or hash
 // label store and the hash store's threads per item) per launch-shape
 // bucket, chosen by timing every candidate on device-resident inputs; an
 // optional cache file; untuned buckets take the nearest tuned entry.
