@@ -529,7 +529,7 @@ __device__ __forceinline__ void load_scatter(const Launch &L, uint64_t s0, uint6
 // digi, sorted by key in shared memory, and each key's run is written with
 // consecutive threads from the block's offset inside the bucket (reserved by
 // the histogram's flush), so no step needs a global atomic.  Bound by
-// shared-memory wavefronts (69% of the LSU pipe: rank, place and read back
+// shared-memory wavefronts (76% of the LSU pipe: rank, place and read back
 // each digi, the last two with the bank conflicts of a random order).  Against
 // steps of half the size with a histogram a warp and the event looked up for
 // every digi: 27.7M digis on 64 modules 153 -> 127 us.  Leaving the keys out
